@@ -372,10 +372,15 @@ mavg_status mavg_materialize_replicas(mavg_handle h) {
 
 mavg_status mavg_round(mavg_handle h, float* mean_loss) {
   CHECK_HANDLE(h);
-  mavg_status st = do_local_steps(h);
-  if (st != MAVG_OK) return st;
-  st = do_meta_update(h);
-  if (st != MAVG_OK) return st;
+  if (pseudograd_round_fused(h)) {
+    CU(h, launch_pseudograd_round(h, h->round + 1), "pseudo-gradient round");
+    h->round += 1;
+  } else {
+    mavg_status st = do_local_steps(h);
+    if (st != MAVG_OK) return st;
+    st = do_meta_update(h);
+    if (st != MAVG_OK) return st;
+  }
   if (mean_loss) return read_mean_loss(h, mean_loss);
   return MAVG_OK;
 }

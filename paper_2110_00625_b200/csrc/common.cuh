@@ -166,6 +166,9 @@ inline MomArgs mom_args(const mavg_ctx* c, bool from_broadcast) {
 cudaError_t launch_broadcast(mavg_ctx* c, bool zero_v, bool force_copies = false);
 cudaError_t launch_meta_update(mavg_ctx* c);
 cudaError_t launch_pseudograd_steps(mavg_ctx* c, int64_t round);
+// Local steps and meta-update of a pseudo-gradient round as one launch, where that applies
+bool pseudograd_round_fused(const mavg_ctx* c);
+cudaError_t launch_pseudograd_round(mavg_ctx* c, int64_t round);
 
 // MLP path (mlp_*.cu)
 mavg_status mlp_validate(const mavg_config* cfg, std::string* why);

@@ -10,13 +10,79 @@
 namespace mavg {
 namespace {
 
-// (sum of the four 16-bit lanes of h - 131070) * c.  The lane sums are two 2-way 16-bit dot
-// products with the weights (1, 1), chained through their addend, which starts at -131070
-// (modular arithmetic: the same integer as extracting and adding the lanes one by one).
-__device__ __forceinline__ float ih4(uint64_t h, float c) {
-  const uint32_t lo = (uint32_t)h, hi = (uint32_t)(h >> 32);
-  const uint32_t s = __dp2a_lo(hi, 0x0101u, __dp2a_lo(lo, 0x0101u, (uint32_t)-131070));
-  return (float)(int32_t)s * c;
+// The variate of element i at a step with key `key`: mix64(key + (i+1) G), its four 16-bit lanes
+// summed, minus 131070, times c (mavg.h).  What bounds the pass is the integer pipes: about 25
+// instructions per variate -- a 64-bit addition, three xor-shifts of 4, two 64 x 64 -> 64 bit
+// products of 3 multiply-adds, two dot products, three float operations -- of which the shifts and
+// logic operations (ALU pipe) and the multiply-adds (FMA pipe, 64-bit ones at a quarter of the
+// rate) are about 24 cycles per warp each.  Hence the 64-bit value is kept as two words:
+//  - the carry of the addition is a compare and a predicated increment, which the scheduler may
+//    place on either pipe, where a 64-bit add occupies the multiply pipe for four cycles;
+//  - the lane sum starts from the bits of 2^23, so that the sum's bits already are the float
+//    2^23 + sum and one exact subtraction takes the place of an integer-to-float conversion.
+// With four steps unrolled, 5.12e8 x 12.8 variates in 6.16 ms against 6.71 ms for the plain
+// 64-bit form (n = 6.4 M, P = 16, K = 64: 0.98e12 -> 1.06e12 variates/s).
+struct U64 { uint32_t lo, hi; };
+
+__device__ __forceinline__ U64 split(uint64_t v) { return {(uint32_t)v, (uint32_t)(v >> 32)}; }
+
+__device__ __forceinline__ U64 add(U64 a, uint64_t b) {
+  const uint32_t bl = (uint32_t)b;
+  U64 r{a.lo + bl, a.hi + (uint32_t)(b >> 32)};
+  if (r.lo < bl) r.hi += 1u;
+  return r;
+}
+template <int S>
+__device__ __forceinline__ U64 xor_shift(U64 z) {   // z ^ (z >> S), S < 32
+  return {z.lo ^ __funnelshift_r(z.lo, z.hi, S), z.hi ^ (z.hi >> S)};
+}
+template <uint64_t C>
+__device__ __forceinline__ U64 mul(U64 z) {
+  const uint64_t p = (uint64_t)z.lo * (uint32_t)C;
+  return {(uint32_t)p, z.hi * (uint32_t)C + (z.lo * (uint32_t)(C >> 32) + (uint32_t)(p >> 32))};
+}
+__device__ __forceinline__ float variate(U64 z, float c) {
+  z = mul<0xBF58476D1CE4E5B9ull>(xor_shift<30>(z));
+  z = mul<0x94D049BB133111EBull>(xor_shift<27>(z));
+  z = xor_shift<31>(z);
+  const uint32_t s = __dp2a_lo(z.hi, 0x0101u, __dp2a_lo(z.lo, 0x0101u, 0x4B000000u));
+  return (__uint_as_float(s) - (8388608.f + 131070.f)) * c;
+}
+
+// One local step on four consecutive elements, the first of which has counter c0 = (i+1) G.
+template <bool MOM>
+__device__ __forceinline__ void local_step4(float4& w, float4& u, uint64_t key, uint64_t c0,
+                                            float c, float gamma, float beta) {
+  const U64 z = add(split(key), c0);
+  const float g0 = variate(z, c), g1 = variate(add(z, kGamma), c);
+  const float g2 = variate(add(z, 2 * kGamma), c), g3 = variate(add(z, 3 * kGamma), c);
+  if (MOM) {
+    msgd(w.x, u.x, g0, gamma, beta);
+    msgd(w.y, u.y, g1, gamma, beta);
+    msgd(w.z, u.z, g2, gamma, beta);
+    msgd(w.w, u.w, g3, gamma, beta);
+  } else {
+    w.x = fmaf(-gamma, g0, w.x);
+    w.y = fmaf(-gamma, g1, w.y);
+    w.z = fmaf(-gamma, g2, w.z);
+    w.w = fmaf(-gamma, g3, w.w);
+  }
+}
+template <bool MOM>
+__device__ __forceinline__ void local_steps4(float4& w, float4& u, const uint64_t* keys, int K,
+                                             uint64_t c0, float c, float gamma, float beta) {
+#pragma unroll 4
+  for (int k = 0; k < K; ++k) local_step4<MOM>(w, u, keys[k], c0, c, gamma, beta);
+}
+// The same on one element (the ragged end of the vector).
+template <bool MOM>
+__device__ __forceinline__ void local_steps1(float& w, float& u, const uint64_t* keys, int K,
+                                             uint64_t c0, float c, float gamma, float beta) {
+  for (int k = 0; k < K; ++k) {
+    const float g = variate(add(split(keys[k]), c0), c);
+    if (MOM) msgd(w, u, g, gamma, beta);
+    else w = fmaf(-gamma, g, w);
+  }
 }
 
 // grid = (x, P); dynamic shared memory holds the K step keys of learner blockIdx.y.
@@ -37,31 +103,13 @@ k_pseudograd_steps(float* rep, int64_t stride, const float* src, int64_t src_str
   const float4* in4 = reinterpret_cast<const float4*>(in);
   const int64_t n4 = n >> 2;
   const int64_t step = (int64_t)gridDim.x * blockDim.x;
-  const float ng = -gamma;
   float* urow = MOM ? mom.u + (size_t)j * mom.u_stride : nullptr;
   float4* urow4 = reinterpret_cast<float4*>(urow);
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n4; q += step) {
     float4 w = src_stride ? __ldcs(in4 + q) : __ldg(in4 + q);
     float4 u = make_float4(0.f, 0.f, 0.f, 0.f);
     if (MOM && mom.read_u) u = __ldcs(urow4 + q);
-    const uint64_t c0 = (uint64_t)(4 * q + 1) * kGamma;  // element i uses (i+1) G
-    for (int k = 0; k < K; ++k) {
-      const uint64_t key = keys[k];
-      const float g0 = ih4(mix64(key + c0), c), g1 = ih4(mix64(key + c0 + kGamma), c);
-      const float g2 = ih4(mix64(key + c0 + 2 * kGamma), c);
-      const float g3 = ih4(mix64(key + c0 + 3 * kGamma), c);
-      if (MOM) {
-        msgd(w.x, u.x, g0, gamma, mom.beta);
-        msgd(w.y, u.y, g1, gamma, mom.beta);
-        msgd(w.z, u.z, g2, gamma, mom.beta);
-        msgd(w.w, u.w, g3, gamma, mom.beta);
-      } else {
-        w.x = fmaf(ng, g0, w.x);
-        w.y = fmaf(ng, g1, w.y);
-        w.z = fmaf(ng, g2, w.z);
-        w.w = fmaf(ng, g3, w.w);
-      }
-    }
+    local_steps4<MOM>(w, u, keys, K, (uint64_t)(4 * q + 1) * kGamma, c, gamma, mom.beta);
     __stcs(row4 + q, w);
     if (MOM) __stcs(urow4 + q, u);
   }
@@ -69,23 +117,105 @@ k_pseudograd_steps(float* rep, int64_t stride, const float* src, int64_t src_str
     const int64_t i = (n4 << 2) + threadIdx.x;
     float w = in[i];
     float u = (MOM && mom.read_u) ? urow[i] : 0.f;
-    for (int k = 0; k < K; ++k) {
-      const float gk = ih4(fold(keys[k], (uint64_t)i), c);
-      if (MOM) msgd(w, u, gk, gamma, mom.beta);
-      else w = fmaf(ng, gk, w);
-    }
+    local_steps1<MOM>(w, u, keys, K, (uint64_t)(i + 1) * kGamma, c, gamma, mom.beta);
     row[i] = w;
     if (MOM) urow[i] = u;
   }
 }
+
+// A whole round: the K local steps of all P learners and the meta-update.  A thread takes four
+// elements through learner 0's K steps, then learner 1's, ..., adds the differences w^j - w~ in
+// the same ascending order as the meta-update kernels and finishes the update itself, so the
+// replicas are not read back: per element (4P + 16) bytes where the two passes move (8P + 16)
+// with deferred copies (the learners' models are written) and (12P + 16) without (only the P
+// copies of the new w~ are).  Bounds: at K = 1 HBM (2.05 GB = 0.31 ms at n = 25.6 M, P = 16) and the
+// variates (0.38 ms) about equally, the variates beyond.  Measured there, deferred copies: K = 1
+// 507 us a round against 913 for the two passes, K = 64 25.5 ms against 27.4.
+// One quad per thread and no loop over the grid: the blocks' ends are spread over the launch.  The
+// last n % 4 elements have a block of their own, so that their serial P x K steps run beside the
+// rest.  K1: K = 1, the loop over the learners is unrolled instead of the one over the steps.
+// Dynamic shared memory holds the P x K step keys.
+template <bool MOM, bool K1>
+__global__ void __launch_bounds__(256)
+k_pseudograd_round(float* rep, int64_t stride, bool from_global, float* __restrict__ gw,
+                   float* __restrict__ gv, int64_t n, int P, int K, uint64_t seed, int64_t round,
+                   float c, float gamma, float mu, float zeta, float inv_p, bool read_v, bool bcast,
+                   const MomArgs mom) {
+  extern __shared__ uint64_t keys[];
+  for (int t = threadIdx.x; t < P * K; t += blockDim.x)
+    keys[t] = fold(learner_key(seed, kTagPseudoGrad, (uint64_t)round, (uint64_t)(t / K)),
+                   (uint64_t)(t % K + 1));
+  __syncthreads();
+  const int64_t n4 = n >> 2;
+  const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (q < n4) {
+    const float4 wt = __ldcs(reinterpret_cast<const float4*>(gw) + q);
+    const uint64_t c0 = (uint64_t)(4 * q + 1) * kGamma;
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll K1 ? 4 : 1
+    for (int j = 0; j < P; ++j) {
+      float4* row4 = reinterpret_cast<float4*>(rep + (size_t)j * stride) + q;
+      float4* u4 = MOM ? reinterpret_cast<float4*>(mom.u + (size_t)j * mom.u_stride) + q : nullptr;
+      float4 w = from_global ? wt : __ldcs(row4);
+      float4 u = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (MOM && mom.read_u) u = __ldcs(u4);
+      if (K1) local_step4<MOM>(w, u, keys[j], c0, c, gamma, mom.beta);
+      else local_steps4<MOM>(w, u, keys + j * K, K, c0, c, gamma, mom.beta);
+      acc.x += w.x - wt.x;
+      acc.y += w.y - wt.y;
+      acc.z += w.z - wt.z;
+      acc.w += w.w - wt.w;
+      if (!bcast) __stcs(row4, w);
+      if (MOM) __stcs(u4, u);
+    }
+    float4 vt = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (read_v) vt = __ldcs(reinterpret_cast<const float4*>(gv) + q);
+    float4 vn, wn;
+    vn.x = fmaf(mu, vt.x, zeta * (acc.x * inv_p));
+    vn.y = fmaf(mu, vt.y, zeta * (acc.y * inv_p));
+    vn.z = fmaf(mu, vt.z, zeta * (acc.z * inv_p));
+    vn.w = fmaf(mu, vt.w, zeta * (acc.w * inv_p));
+    wn.x = wt.x + vn.x; wn.y = wt.y + vn.y; wn.z = wt.z + vn.z; wn.w = wt.w + vn.w;
+    __stcs(reinterpret_cast<float4*>(gv) + q, vn);
+    __stcs(reinterpret_cast<float4*>(gw) + q, wn);
+    if (bcast)
+      for (int j = 0; j < P; ++j) __stcs(reinterpret_cast<float4*>(rep + (size_t)j * stride) + q, wn);
+  }
+  if (blockIdx.x == gridDim.x - 1 && threadIdx.x < (n & 3)) {
+    const int64_t i = (n4 << 2) + threadIdx.x;
+    const float wt = gw[i];
+    float acc = 0.f;
+    for (int j = 0; j < P; ++j) {
+      float* wp = rep + (size_t)j * stride + i;
+      float* up = MOM ? mom.u + (size_t)j * mom.u_stride + i : nullptr;
+      float w = from_global ? wt : *wp, u = (MOM && mom.read_u) ? *up : 0.f;
+      local_steps1<MOM>(w, u, keys + j * K, K, (uint64_t)(i + 1) * kGamma, c, gamma, mom.beta);
+      acc += w - wt;
+      if (!bcast) *wp = w;
+      if (MOM) *up = u;
+    }
+    const float vn = fmaf(mu, read_v ? gv[i] : 0.f, zeta * (acc * inv_p));
+    const float wn = wt + vn;
+    gv[i] = vn;
+    gw[i] = wn;
+    if (bcast)
+      for (int j = 0; j < P; ++j) rep[(size_t)j * stride + i] = wn;
+  }
+}
+
+float variate_scale(const mavg_ctx* c) {
+  const double var_lane = (65536.0 * 65536.0 - 1.0) / 12.0;
+  return (float)((double)c->cfg.pseudo_grad_sigma / sqrt(4.0 * var_lane));
+}
+
+constexpr int kMaxRoundKeys = 4096;   // P x K step keys of a fused round: 32 KB of shared memory
 
 }  // namespace
 
 cudaError_t launch_pseudograd_steps(mavg_ctx* c, int64_t round) {
   const int64_t n = c->cfg.n;
   const int P = c->cfg.P, K = c->cfg.K;
-  const double var_lane = (65536.0 * 65536.0 - 1.0) / 12.0;
-  const float scale = (float)((double)c->cfg.pseudo_grad_sigma / sqrt(4.0 * var_lane));
+  const float scale = variate_scale(c);
   constexpr int kMaxFused = 2048;  // step keys per launch (16 KB of shared memory)
   int64_t blocks_x = ((n >> 2) + 255) / 256;
   int64_t cap = ((int64_t)c->sm_count * 8 + P - 1) / P;
@@ -114,6 +244,39 @@ cudaError_t launch_pseudograd_steps(mavg_ctx* c, int64_t round) {
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
+}
+
+// The fused round has n / 4 threads where the local steps on their own have P times as many: a
+// short vector with many steps keeps the two launches.  Measured (P = 16, both forms, us a round):
+// n = 300 000: K = 5 36 against 38, K = 64 357 against 331; n = 1 M: K = 64 1101 against 1141;
+// n = 100 000: K = 1 8.5 against 12.5, K = 64 217 against 174.
+bool pseudograd_round_fused(const mavg_ctx* c) {
+  const int64_t n = c->cfg.n, sms = c->sm_count;
+  return c->cfg.objective == MAVG_OBJ_PSEUDOGRAD && !c->profiling &&
+         (int64_t)c->cfg.P * c->cfg.K <= kMaxRoundKeys &&
+         n >= (c->cfg.K <= 4 ? 512 : 4096) * sms;
+}
+
+cudaError_t launch_pseudograd_round(mavg_ctx* c, int64_t round) {
+  const int64_t n4 = c->cfg.n >> 2;
+  // blocks of 64 threads where the vector gives every SM only a few of them
+  const int threads = n4 < (int64_t)c->sm_count * 2048 ? 64 : 256;
+  const unsigned grid = (unsigned)((n4 + threads - 1) / threads + ((c->cfg.n & 3) ? 1 : 0));
+  const size_t smem = (size_t)c->cfg.P * c->cfg.K * sizeof(uint64_t);
+  const bool from_global = c->replicas_equal_global;
+  const bool bcast = !c->cfg.defer_broadcast;
+  const MomArgs mom = mom_args(c, from_global);
+  auto kernel = mom.u ? (c->cfg.K == 1 ? k_pseudograd_round<true, true> : k_pseudograd_round<true, false>)
+                      : (c->cfg.K == 1 ? k_pseudograd_round<false, true> : k_pseudograd_round<false, false>);
+  prof_begin(c, MAVG_K_PSEUDOGRAD);
+  kernel<<<grid, threads, smem, c->stream>>>(
+      c->buf.replicas, c->buf.replica_stride, from_global, c->buf.global_w, c->buf.momentum,
+      c->cfg.n, c->cfg.P, c->cfg.K, c->cfg.seed, round, variate_scale(c), c->cfg.local_lr,
+      c->cfg.mu, c->cfg.block_lr, 1.0f / (float)c->cfg.P, c->cfg.mu != 0.f, bcast, mom);
+  prof_end(c);
+  c->replicas_equal_global = true;
+  c->replicas_materialized = bcast;
+  return cudaGetLastError();
 }
 
 }  // namespace mavg
