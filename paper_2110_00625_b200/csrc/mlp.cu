@@ -37,7 +37,10 @@ mavg_status mlp_setup(mavg_ctx* c) {
     c->layers.push_back(ly);
   }
   if (use_tensor_cores(&cfg)) return tc_setup(c);
-  return MAVG_OK;
+  const cudaError_t e = simt_setup(c);
+  if (e == cudaSuccess) return MAVG_OK;
+  c->err = std::string("kernel attributes: ") + cudaGetErrorString(e);
+  return MAVG_ERR_CUDA;
 }
 
 void mlp_drop_graph(mavg_ctx* c);
@@ -132,14 +135,6 @@ cudaError_t mlp_local_steps(mavg_ctx* c, int64_t round) {
   // The usual round starts from the broadcast state and is replayed from a graph.  Rounds that
   // start elsewhere (local steps called twice in a row), profiled rounds and handles whose
   // capture failed once take the launch-by-launch path.
-  // The CUDA-core path reads every learner's own copy from the first step on: a deferred
-  // re-broadcast (Algorithm 1, "set w^j = w~") is carried out here, on the caller's stream and
-  // outside the recorded graph, so that a replay never depends on whether the copies happened to
-  // exist when the graph was recorded.
-  if (!use_tensor_cores(&c->cfg) && c->replicas_equal_global && !c->replicas_materialized) {
-    cudaError_t e = launch_broadcast(c, false, /*force_copies=*/true);
-    if (e != cudaSuccess) return e;
-  }
   const bool want_graph = !c->profiling && !c->graph_disabled && c->replicas_equal_global;
   if (!want_graph) return run_steps(c, round);
   if (!c->graph_exec || c->graph_K != c->cfg.K || c->graph_lr != c->cfg.local_lr ||
@@ -166,7 +161,7 @@ cudaError_t mlp_local_steps(mavg_ctx* c, int64_t round) {
 }
 
 cudaError_t mlp_indices_only(mavg_ctx* c, int64_t round, int learner, int step, int32_t* dev_out) {
-  return launch_batch_indices(c, round, step, learner, 1, dev_out, nullptr);
+  return launch_batch_indices(c, round, step, learner, dev_out);
 }
 
 }  // namespace mavg

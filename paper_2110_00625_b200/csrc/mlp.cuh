@@ -8,27 +8,22 @@ namespace mavg {
 // idx = lo_j + floor(u * len_j / 2^32), u = top 32 bits of the stream value (see mavg.h).
 __device__ __forceinline__ int32_t sample_index(uint64_t seed, int64_t round, int j, int step,
                                                 int s, int P, int64_t S) {
-  int64_t lo = (int64_t)(((unsigned __int128)j * (unsigned __int128)S) / (unsigned)P);
-  int64_t hi = (int64_t)(((unsigned __int128)(j + 1) * (unsigned __int128)S) / (unsigned)P);
+  // j < 2^31 and S < 2^31: the products fit in 64 bits
+  int64_t lo = (int64_t)((uint64_t)j * (uint64_t)S / (uint32_t)P);
+  int64_t hi = (int64_t)(((uint64_t)j + 1) * (uint64_t)S / (uint32_t)P);
   uint64_t key = fold(learner_key(seed, kTagBatch, (uint64_t)round, (uint64_t)j), (uint64_t)step);
   uint64_t u = fold(key, (uint64_t)s) >> 32;
   return (int32_t)(lo + (int64_t)((u * (uint64_t)(hi - lo)) >> 32));
 }
 
 // batch.cu
-cudaError_t launch_batch_indices(mavg_ctx* c, int64_t round, int step, int j_first, int j_count,
-                                 int32_t* idx, int32_t* labels);
-cudaError_t launch_gather(mavg_ctx* c, const int32_t* idx, int quant, float* out_f32,
-                          __nv_bfloat16* out_bf, __nv_bfloat16* out_bft);
+cudaError_t launch_batch_indices(mavg_ctx* c, int64_t round, int step, int j, int32_t* idx);
 cudaError_t launch_sample_gather(mavg_ctx* c, int64_t round, int step, int32_t* idx,
                                  int32_t* labels, __nv_bfloat16* out_bf, __nv_bfloat16* out_bft);
-cudaError_t launch_softmax_ce(mavg_ctx* c, const float* logits, int ldz, const int32_t* labels,
-                              float* loss_out, int loss_stride, float* dz_f32, int ld32,
-                              __nv_bfloat16* dz_bf, int ldbf, __nv_bfloat16* dz_bft, int ldbft,
-                              bool update_bias, const MomArgs& mom = MomArgs());
 
 // CUDA-core path (mlp_simt.cu): fp32 arithmetic, or bf16-rounded operands with fp32 FMAs.
 size_t simt_workspace_bytes(const mavg_config* cfg, size_t base, size_t* act_off);
+cudaError_t simt_setup(mavg_ctx* c);      // once per handle
 cudaError_t simt_step(mavg_ctx* c, int64_t round, int step);
 
 // Tensor-core path (mlp_tc.cu): tcgen05 GEMMs fed by TMA.

@@ -1,253 +1,732 @@
 // CUDA-core MLP learner step, batched over the P learners (blockIdx.z).
-//   forward   Z_l = act(A_{l-1}) W_l^T + b_l                      (A_0 = gathered minibatch)
-//   backward  dZ_{l-1} = (dZ_l W_l) .* [Z_{l-1} > 0];  dW_l = dZ_l^T act(A_{l-1});  db_l = colsum dZ_l
+//   forward   Z_l = A_{l-1} W_l^T + b_l,  A_l = act(Z_l)          (A_0 = gathered minibatch)
+//   backward  dA_{l-1} = (dZ_l W_l) .* [A_{l-1} > 0];  dW_l = dZ_l^T A_{l-1};  db_l = colsum dZ_l
 //   SGD       W_l <- W_l - gamma dW_l, b_l <- b_l - gamma db_l    (Algorithm 1's local update)
 // fp32 FMAs throughout.  With QUANT every matrix-product operand is first rounded to bf16
 // (nearest-even), which makes this path compute the same thing as the tensor-core path; it is the
 // path for true fp32 models and for layer widths the tensor-core path does not cover.
-// Buffers hold pre-activations Z_l and dZ_l in fp32; ReLU and rounding are applied on load.
+// A step is L-1 forward launches, one for the whole last layer up to its data gradient (which
+// also gathers the next step's minibatch), L-2 data gradients and one for the weight gradients,
+// bias gradients and SGD steps of all layers.  At the first step of a round the weights are read
+// from w~ and the results written to the replicas, so the P copies of a deferred re-broadcast are
+// never needed.
+#include <algorithm>
+
 #include "mlp.cuh"
+#include "tc_ptx.cuh"
 
 namespace mavg {
 namespace {
 
-constexpr int BM = 64, BN = 64, BK = 16, TM = 4, TN = 4;
-
 __device__ __forceinline__ float qbf(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
+template <bool QUANT>
+__device__ __forceinline__ float operand(float v) { return QUANT ? qbf(v) : v; }
 
-enum LoadOp { LD_PLAIN = 0, LD_RELU = 1 };
-
-template <bool QUANT, int OP>
-__device__ __forceinline__ float load_op(float v) {
-  if (OP == LD_RELU) v = v > 0.f ? v : 0.f;
-  return QUANT ? qbf(v) : v;
-}
-
-struct GemmArgs {
-  const float* A; int64_t a_batch; int64_t a_m, a_k;   // A(m,k) = A[p*a_batch + m*a_m + k*a_k]
-  const float* B; int64_t b_batch; int64_t b_n, b_k;   // B(n,k) = B[p*b_batch + n*b_n + k*b_k]
-  int M, N, K;
-  // epilogue operands
-  float* C; int64_t c_batch; int64_t c_m;               // C(m,n) = C[p*c_batch + m*c_m + n]
-  const float* aux; int64_t aux_batch; int64_t aux_m;   // bias [n] (fwd) or mask source Z (dgrad)
-  float gamma;
-  MomArgs mom;          // EPI_WGRAD_SGD: learner momentum slots at mom.u[p*u_stride + (C's offset)]
-  int64_t u_off;        // offset of C inside a replica (the same inside u^j)
-};
+// ------------------------------------------------------------------------------ matrix products
+// C(m,n) = sum_k A(m,k) B(n,k): one 64 x 64 tile per block of 128 threads, 8 x 4 outputs each.
+// Bound: the FMA pipe and the register ports that feed it (a product of ordinary size keeps its
+// operands in the L2).  Slabs of 16 k go through registers into two shared-memory buffers, so the
+// loads of a slab overlap the products of the one before; both operands are stored k-major, the
+// operands of k + 1 are read while k is multiplied, and an fma.f32x2 does the FMAs of two rows in
+// one issue slot, which leaves slots for the reads.  Where the tiles would leave SMs idle the
+// contraction is split over the blocks of a cluster, which add their partial tiles in rank order
+// through distributed shared memory.
+// First layer of a 3072-512-512-10 model, P = 4, B = 100: 53 us forward (21 us of FMAs at the peak
+// rate, padding of the batch to 128 included), weight gradients of all layers 55 us.  Measured on the
+// same case and not better: 8 x 8 outputs per thread (51 and 60 us, whole round 693 us against
+// 590: half as many warps), the same with one-element FMAs (76), and a ring of asynchronous copies in
+// the operands' own orientation (58, and twice as slow for rows that do not start on 16 bytes).
+constexpr int BM = 64, BN = 64, BK = 16, kThreads = 128;
+constexpr int kPitchA = BM + 4, kPitchB = BN + 4;
+constexpr int kMaxSplit = 8;
 
 enum Epi { EPI_FWD = 0, EPI_DGRAD = 1, EPI_WGRAD_SGD = 2 };
 
-// C(m,n) = sum_k opA(A(m,k)) * opB(B(n,k)), 64x64 tile, 256 threads, 4x4 outputs per thread.
-template <bool QUANT, int OPA, int OPB, bool A_KC, bool B_KC, int EPI>
-__global__ void __launch_bounds__(256) k_simt_gemm(GemmArgs g) {
-  __shared__ float As[BK][BM + 4];
-  __shared__ float Bs[BK][BN + 4];
-  const int p = blockIdx.z;
-  const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-  const float* A = g.A + (size_t)p * g.a_batch;
-  const float* B = g.B + (size_t)p * g.b_batch;
-  const int tid = threadIdx.x;
-  const int tx = tid % 16, ty = tid / 16;   // tx over n, ty over m
-  float acc[TM][TN];
-#pragma unroll
-  for (int i = 0; i < TM; ++i)
-#pragma unroll
-    for (int j = 0; j < TN; ++j) acc[i][j] = 0.f;
+// FWD:   A = activations [M, K], B = W [N, K];       C = A_l (hidden) or the logits; aux = bias [N]
+// DGRAD: A = dZ [M, K],          B = W [K, N];       C = dZ of the layer below; aux = A_{l-1} [M, N]
+// WGRAD: A = dZ [K, M],          B = A_{l-1} [K, N]; C = W [M, N], aux = W before the step
+struct GemmArgs {
+  const float* A; int64_t a_batch;
+  const float* B; int64_t b_batch;
+  int M, N, K;
+  float* C; int64_t c_batch;
+  const float* aux; int64_t aux_batch;
+  int vec_a, vec_b, vec_c;  // rows of the operand start on 16 bytes and hold whole groups of 4
+  int k_per_split;
+  int hidden;           // FWD: apply ReLU (and the operand rounding of the next products)
+  // WGRAD: bias after the step, before it, and what the local update needs
+  float* bias; const float* bias_in;
+  float gamma;
+  MomArgs mom;          // momentum slots at mom.u[p*u_stride + u_off (+ the bias offset ub_off)]
+  int64_t u_off, ub_off;
+};
 
-  for (int k0 = 0; k0 < g.K; k0 += BK) {
-    // 64 x 16 elements per operand, 4 per thread; consecutive threads follow the unit stride
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      int lin = tid + e * 256;
-      int mm, kk;
-      if (A_KC) { kk = lin % BK; mm = lin / BK; } else { mm = lin % BM; kk = lin / BM; }
-      int gm = m0 + mm, gk = k0 + kk;
-      float v = 0.f;
-      if (gm < g.M && gk < g.K) v = load_op<QUANT, OPA>(A[(size_t)gm * g.a_m + (size_t)gk * g.a_k]);
-      As[kk][mm] = v;
-      int nn;
-      if (B_KC) { kk = lin % BK; nn = lin / BK; } else { nn = lin % BN; kk = lin / BN; }
-      int gn = n0 + nn;
-      gk = k0 + kk;
-      v = 0.f;
-      if (gn < g.N && gk < g.K) v = load_op<QUANT, OPB>(B[(size_t)gn * g.b_n + (size_t)gk * g.b_k]);
-      Bs[kk][nn] = v;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      float a[TM], b[TN];
-#pragma unroll
-      for (int i = 0; i < TM; ++i) a[i] = As[kk][ty * TM + i];
-#pragma unroll
-      for (int j = 0; j < TN; ++j) b[j] = Bs[kk][tx * TN + j];
-#pragma unroll
-      for (int i = 0; i < TM; ++i)
-#pragma unroll
-        for (int j = 0; j < TN; ++j) acc[i][j] = fmaf(a[i], b[j], acc[i][j]);
-    }
-    __syncthreads();
-  }
+struct __align__(16) Slab { float a[BK][kPitchA], b[BK][kPitchB]; };
+union __align__(16) GemmShared {
+  Slab slab[2];
+  float c[BM][kPitchB];  // partial tile of a split contraction
+};
 
-  float* C = g.C + (size_t)p * g.c_batch;
-  float* U = (EPI == EPI_WGRAD_SGD && g.mom.u) ? g.mom.u + (size_t)p * g.mom.u_stride + g.u_off
-                                               : nullptr;
-  const float* aux = g.aux ? g.aux + (size_t)p * g.aux_batch : nullptr;
+// A ROWS x 16 piece of an operand through registers.  KC: memory is [row, k] (k contiguous), else
+// [k, row].  rows and k_end bound the operand; what lies outside is zero.  The way a thread's
+// elements lie depends on `vec` alone (uniform): groups of four or single elements.
+template <int ROWS, bool KC, bool ROUND>
+struct Piece {
+  static constexpr int N = ROWS * BK / kThreads;   // elements per thread
+  float r[N];
+  __device__ __forceinline__ void load(const float* __restrict__ p, int ld, int vec, int row0,
+                                       int rows, int k0, int k_end) {
+    const int t = threadIdx.x;
+    if (vec) {
 #pragma unroll
-  for (int i = 0; i < TM; ++i) {
-    int gm = m0 + ty * TM + i;
-    if (gm >= g.M) continue;
+      for (int e = 0; e < N / 4; ++e) {
+        const int row = row0 + (KC ? t / 4 + 32 * e : (t % (ROWS / 4)) * 4);
+        const int k = k0 + (KC ? (t % 4) * 4 : t / (ROWS / 4) + e * (kThreads * 4 / ROWS));
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (row < rows && k < k_end)
+          v = *reinterpret_cast<const float4*>(p + (KC ? (size_t)row * ld + k : (size_t)k * ld + row));
+        r[4 * e] = v.x; r[4 * e + 1] = v.y; r[4 * e + 2] = v.z; r[4 * e + 3] = v.w;
+      }
+    } else {
 #pragma unroll
-    for (int j = 0; j < TN; ++j) {
-      int gn = n0 + tx * TN + j;
-      if (gn >= g.N) continue;
-      float v = acc[i][j];
-      size_t ci = (size_t)gm * g.c_m + gn;
-      if (EPI == EPI_FWD) {
-        C[ci] = v + aux[gn];
-      } else if (EPI == EPI_DGRAD) {
-        C[ci] = aux[(size_t)gm * g.aux_m + gn] > 0.f ? v : 0.f;   // ReLU'(0) = 0
-      } else {
-        local_update(C + ci, C[ci], U ? U + ci : nullptr, g.mom.read_u, v, g.gamma, g.mom.beta);
+      for (int e = 0; e < N; ++e) {
+        const int row = row0 + (KC ? t / 16 + 8 * e : t % ROWS);
+        const int k = k0 + (KC ? t % 16 : t / ROWS + e * (kThreads / ROWS));
+        r[e] = (row < rows && k < k_end) ? p[KC ? (size_t)row * ld + k : (size_t)k * ld + row] : 0.f;
       }
     }
   }
-}
-
-// b[o] -= gamma * sum_b dZ[b, o], ascending b.  grid (ceil(out/256), P)
-__global__ void __launch_bounds__(256)
-k_simt_bias_sgd(const float* __restrict__ dz, int64_t dz_batch, int B, int out,
-                float* __restrict__ rep, int64_t rep_stride, int64_t b_off, float gamma,
-                const MomArgs mom) {
-  int o = blockIdx.x * blockDim.x + threadIdx.x;
-  if (o >= out) return;
-  const int p = blockIdx.y;
-  const float* d = dz + (size_t)p * dz_batch;
-  float s = 0.f;
-  for (int b = 0; b < B; ++b) s += d[(size_t)b * out + o];
-  float* bias = rep + (size_t)p * rep_stride + b_off;
-  float* ub = mom.u ? mom.u + (size_t)p * mom.u_stride + b_off : nullptr;
-  local_update(bias + o, bias[o], ub ? ub + o : nullptr, mom.read_u, s, gamma, mom.beta);
-}
-
-struct SimtBuffers {
-  float* xg;                      // [P, B, d0]
-  float* z[MAVG_MAX_LAYERS + 1];  // z[l]  [P, B, d_l], l = 1..L
-  float* dz[MAVG_MAX_LAYERS + 1]; // dz[l] [P, B, d_l]
+  template <int PITCH>
+  __device__ __forceinline__ void store(float (*s)[PITCH], int vec) const {
+    const int t = threadIdx.x;
+    if (vec) {
+#pragma unroll
+      for (int e = 0; e < N / 4; ++e) {
+        if (KC) {
+#pragma unroll
+          for (int i = 0; i < 4; ++i) s[(t % 4) * 4 + i][t / 4 + 32 * e] = operand<ROUND>(r[4 * e + i]);
+        } else {
+          *reinterpret_cast<float4*>(&s[t / (ROWS / 4) + e * (kThreads * 4 / ROWS)][(t % (ROWS / 4)) * 4]) =
+              make_float4(operand<ROUND>(r[4 * e]), operand<ROUND>(r[4 * e + 1]),
+                          operand<ROUND>(r[4 * e + 2]), operand<ROUND>(r[4 * e + 3]));
+        }
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < N; ++e) {
+        if (KC) s[t % 16][t / 16 + 8 * e] = operand<ROUND>(r[e]);
+        else s[t / ROWS + e * (kThreads / ROWS)][t % ROWS] = operand<ROUND>(r[e]);
+      }
+    }
+  }
 };
 
-SimtBuffers carve(const mavg_config* cfg, char* base) {
-  SimtBuffers sb{};
+__device__ __forceinline__ uint64_t dup2(float v) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %1};" : "=l"(r) : "f"(v));
+  return r;
+}
+__device__ __forceinline__ void fma2(uint64_t& d, uint64_t a, uint64_t b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ float half_of(uint64_t v, int hi) {
+  return __uint_as_float((uint32_t)(hi ? v >> 32 : v));
+}
+
+// acc[i][j] holds rows 8 ty + 2 i, + 1 of column 4 tx + j
+struct Fragment { ulonglong2 a0, a1; float4 b; };
+__device__ __forceinline__ void read(Fragment& f, const Slab& s, int k) {
+  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+  f.a0 = *reinterpret_cast<const ulonglong2*>(&s.a[k][8 * ty]);
+  f.a1 = *reinterpret_cast<const ulonglong2*>(&s.a[k][8 * ty + 4]);
+  f.b = *reinterpret_cast<const float4*>(&s.b[k][4 * tx]);
+}
+__device__ __forceinline__ void multiply(const Slab& s, uint64_t (&acc)[4][4]) {
+  Fragment f[2];
+  read(f[0], s, 0);
+#pragma unroll
+  for (int k = 0; k < BK; ++k) {
+    if (k + 1 < BK) read(f[(k + 1) & 1], s, k + 1);
+    const Fragment& c = f[k & 1];
+    const uint64_t a[4] = {c.a0.x, c.a0.y, c.a1.x, c.a1.y};
+    const float b[4] = {c.b.x, c.b.y, c.b.z, c.b.w};
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const uint64_t bb = dup2(b[j]);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) fma2(acc[i][j], a[i], bb);
+    }
+  }
+}
+
+// Four finished sums C(m, n .. n+3): the layer's tail and the store.
+template <bool QUANT, int EPI>
+__device__ __forceinline__ void emit(const GemmArgs& g, int p, int m, int n, float (&v)[4]) {
+  if (m >= g.M || n >= g.N) return;
+  const size_t ci = (size_t)m * g.N + n;
+  float* C = g.C + (size_t)p * g.c_batch + ci;
+  const float* aux = g.aux + (size_t)p * g.aux_batch + (EPI == EPI_FWD ? (size_t)n : ci);
+  float x[4] = {0.f, 0.f, 0.f, 0.f};
+  if (g.vec_c && EPI != EPI_FWD) {       // the bias vector may start anywhere
+    const float4 t = *reinterpret_cast<const float4*>(aux);
+    x[0] = t.x; x[1] = t.y; x[2] = t.z; x[3] = t.w;
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (n + i < g.N) x[i] = aux[i];
+  }
+  float* U = (EPI == EPI_WGRAD_SGD && g.mom.u)
+                 ? g.mom.u + (size_t)p * g.mom.u_stride + g.u_off + ci : nullptr;
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    if (EPI == EPI_FWD) {
+      v[i] += x[i];
+      if (g.hidden) v[i] = operand<QUANT>(v[i] > 0.f ? v[i] : 0.f);
+    } else if (EPI == EPI_DGRAD) {
+      v[i] = x[i] > 0.f ? v[i] : 0.f;    // ReLU'(0) = 0
+    } else if (U && n + i < g.N) {
+      float u = g.mom.read_u ? U[i] : 0.f;
+      msgd(x[i], u, v[i], g.gamma, g.mom.beta);
+      U[i] = u;
+      v[i] = x[i];
+    } else {
+      v[i] = fmaf(-g.gamma, v[i], x[i]);
+    }
+  }
+  if (g.vec_c) {
+    *reinterpret_cast<float4*>(C) = make_float4(v[0], v[1], v[2], v[3]);
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+      if (n + i < g.N) C[i] = v[i];
+  }
+}
+
+template <bool QUANT, int EPI>
+__device__ __forceinline__ void gemm_tile(const GemmArgs& g, int m0, int n0, int p, int rank,
+                                          int splits, GemmShared& sh) {
+  constexpr bool A_KC = EPI != EPI_WGRAD_SGD, B_KC = EPI == EPI_FWD;
+  // activations were rounded where they were produced; dZ is kept unrounded for the bias step
+  constexpr bool QA = QUANT && EPI != EPI_FWD, QB = QUANT && EPI != EPI_WGRAD_SGD;
+  const float* A = g.A + (size_t)p * g.a_batch;
+  const float* B = g.B + (size_t)p * g.b_batch;
+  const int lda = A_KC ? g.K : g.M, ldb = B_KC ? g.K : g.N;
+  const int k_begin = rank * g.k_per_split;
+  const int k_end = min(g.K, k_begin + g.k_per_split);
+  uint64_t acc[4][4] = {};
+  Piece<BM, A_KC, QA> pa;
+  Piece<BN, B_KC, QB> pb;
+  if (k_begin < k_end) {
+    pa.load(A, lda, g.vec_a, m0, g.M, k_begin, k_end);
+    pb.load(B, ldb, g.vec_b, n0, g.N, k_begin, k_end);
+    pa.store(sh.slab[0].a, g.vec_a);
+    pb.store(sh.slab[0].b, g.vec_b);
+  }
+  __syncthreads();
+  int buf = 0;
+  for (int k0 = k_begin; k0 < k_end; k0 += BK, buf ^= 1) {
+    const bool more = k0 + BK < k_end;
+    if (more) {
+      pa.load(A, lda, g.vec_a, m0, g.M, k0 + BK, k_end);
+      pb.load(B, ldb, g.vec_b, n0, g.N, k0 + BK, k_end);
+    }
+    multiply(sh.slab[buf], acc);
+    if (more) {
+      pa.store(sh.slab[buf ^ 1].a, g.vec_a);
+      pb.store(sh.slab[buf ^ 1].b, g.vec_b);
+    }
+    __syncthreads();
+  }
+  const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
+  if (splits == 1) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      float v[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) v[j] = half_of(acc[i / 2][j], i & 1);
+      emit<QUANT, EPI>(g, p, m0 + 8 * ty + i, n0 + 4 * tx, v);
+    }
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    *reinterpret_cast<float4*>(&sh.c[8 * ty + i][4 * tx]) =
+        make_float4(half_of(acc[i / 2][0], i & 1), half_of(acc[i / 2][1], i & 1),
+                    half_of(acc[i / 2][2], i & 1), half_of(acc[i / 2][3], i & 1));
+  tc::cluster_sync_all();
+  // this block finishes 64 / splits rows of the tile
+  for (int t = threadIdx.x; t < BM / splits * (BN / 4); t += kThreads) {
+    const int m = rank * (BM / splits) + t / (BN / 4), n = 4 * (t % (BN / 4));
+    const uint32_t own = tc::smem_u32(&sh.c[m][n]);
+    float v[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int q = 0; q < splits; ++q) {
+      float4 x;
+      asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                   : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w)
+                   : "r"(tc::mapa_u32(own, q)) : "memory");
+      v[0] += x.x; v[1] += x.y; v[2] += x.z; v[3] += x.w;
+    }
+    emit<QUANT, EPI>(g, p, m0 + m, n0 + n, v);
+  }
+  tc::cluster_sync_all();   // a peer may still be reading this block's partial tile
+}
+
+// Forward and data gradient: grid (splits x row tiles x column tiles, 1, P), clusters of `splits`.
+template <bool QUANT, int EPI>
+__global__ void __launch_bounds__(kThreads, 4)
+k_simt_gemm(const __grid_constant__ GemmArgs g, int splits) {
+  __shared__ GemmShared sh;
+  tc::grid_launch_dependents();
+  tc::grid_dependency_wait();
+  const int rank = blockIdx.x % splits, tile = blockIdx.x / splits;
+  const int n_tiles = (g.N + BN - 1) / BN;
+  gemm_tile<QUANT, EPI>(g, tile / n_tiles * BM, tile % n_tiles * BN, blockIdx.z, rank, splits, sh);
+}
+
+// Weight gradients + SGD of all layers in one launch: grid (tiles of layer 1, 2, ..., 1, P).  The
+// blocks of a layer's first column tile also take the bias step (ascending batch, unrounded dZ),
+// and the first block of a learner adds up its row losses.
+struct WgradArgs {
+  GemmArgs g[MAVG_MAX_LAYERS];
+  int tile0[MAVG_MAX_LAYERS + 1];
+  int L;
+  const float* row_loss;   // [P, B]
+  float* loss_out;
+  int loss_stride;
+};
+template <bool QUANT>
+__global__ void __launch_bounds__(kThreads, 4)
+k_simt_wgrad(const __grid_constant__ WgradArgs w) {
+  __shared__ GemmShared sh;
+  tc::grid_launch_dependents();
+  tc::grid_dependency_wait();
+  int l = 0;
+  while (l + 1 < w.L && (int)blockIdx.x >= w.tile0[l + 1]) ++l;
+  const GemmArgs& g = w.g[l];
+  const int tile = blockIdx.x - w.tile0[l], p = blockIdx.z;
+  const int n_tiles = (g.N + BN - 1) / BN;
+  const int m0 = tile / n_tiles * BM, n0 = tile % n_tiles * BN;
+  gemm_tile<QUANT, EPI_WGRAD_SGD>(g, m0, n0, p, 0, 1, sh);
+  const int o = m0 + threadIdx.x;
+  if (n0 == 0 && threadIdx.x < BM && o < g.M) {
+    const float* d = g.A + (size_t)p * g.a_batch + o;
+    float s = 0.f;
+#pragma unroll 8
+    for (int b = 0; b < g.K; ++b) s += d[(size_t)b * g.M];
+    float* ub = g.mom.u ? g.mom.u + (size_t)p * g.mom.u_stride + g.ub_off + o : nullptr;
+    local_update(g.bias + (size_t)p * g.c_batch + o, g.bias_in[(size_t)p * g.aux_batch + o], ub,
+                 g.mom.read_u, s, g.gamma, g.mom.beta);
+  }
+  if (blockIdx.x == 0 && threadIdx.x >= kThreads - 32) {
+    const int lane = threadIdx.x % 32;
+    float s = 0.f;
+    for (int b = lane; b < g.K; b += 32) s += w.row_loss[(size_t)p * g.K + b];
+    for (int q = 16; q > 0; q >>= 1) s += __shfl_xor_sync(0xffffffffu, s, q);
+    if (lane == 0) w.loss_out[(size_t)p * w.loss_stride] = s / (float)g.K;
+  }
+}
+
+// ------------------------------------------------------------------------- minibatch and loss
+struct GatherArgs {
+  const void* x; int x_bf16;
+  const int32_t* y;
+  uint64_t seed; int64_t round; const int64_t* round_ptr;
+  int step, P, B, d;
+  int64_t S;
+  float* out;            // [P, B, d]
+  int32_t* labels;       // [P, B]
+};
+
+// One sampled row: index, label and the row itself.
+template <bool QUANT>
+__device__ __forceinline__ void gather_row(const GatherArgs& g, int row) {
+  __shared__ int32_t sidx;
+  if (threadIdx.x == 0) {
+    const int64_t round = g.round_ptr ? *g.round_ptr : g.round;
+    sidx = sample_index(g.seed, round, row / g.B, g.step, row % g.B, g.P, g.S);
+    g.labels[row] = g.y[sidx];
+  }
+  __syncthreads();
+  const size_t src = (size_t)sidx * g.d;
+  float* dst = g.out + (size_t)row * g.d;
+  if (g.x_bf16) {
+    const __nv_bfloat16* x = (const __nv_bfloat16*)g.x + src;
+    for (int i = threadIdx.x; i < g.d; i += blockDim.x) dst[i] = __bfloat162float(x[i]);
+  } else if (g.d % 4 == 0) {
+    const float4* x = reinterpret_cast<const float4*>((const float*)g.x + src);
+    for (int i = threadIdx.x; i < g.d / 4; i += blockDim.x) {
+      const float4 v = x[i];
+      reinterpret_cast<float4*>(dst)[i] = make_float4(operand<QUANT>(v.x), operand<QUANT>(v.y),
+                                                      operand<QUANT>(v.z), operand<QUANT>(v.w));
+    }
+  } else {
+    const float* x = (const float*)g.x + src;
+    for (int i = threadIdx.x; i < g.d; i += blockDim.x) dst[i] = operand<QUANT>(x[i]);
+  }
+}
+
+template <bool QUANT>
+__global__ void __launch_bounds__(256) k_simt_gather(const __grid_constant__ GatherArgs g) {
+  tc::grid_launch_dependents();
+  tc::grid_dependency_wait();
+  gather_row<QUANT>(g, blockIdx.x);
+}
+
+// Softmax of one row z (C logits in shared or global memory) by a warp: writes dz and returns the loss.
+template <typename Put>
+__device__ __forceinline__ float softmax_row(const float* z, int C, int label, float inv_b, Put put) {
+  const int lane = threadIdx.x % 32;
+  float m = z[lane < C ? lane : 0];
+  for (int c = lane + 32; c < C; c += 32) m = fmaxf(m, z[c]);
+  for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+  float se = 0.f;
+  for (int c = lane; c < C; c += 32) se += expf(z[c] - m);
+  for (int o = 16; o > 0; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
+  const float lse = m + logf(se);
+  for (int c = lane; c < C; c += 32) put(c, (expf(z[c] - lse) - (c == label ? 1.f : 0.f)) * inv_b);
+  return lse - z[label];
+}
+
+// The last layer of 8 batch rows of a learner: logits, loss, dZ_L and the data gradient through the
+// layer, in one block of 512 threads; the remaining blocks gather the next step's minibatch.  A
+// layer of few classes is latency, not work: as a forward product, a loss and a data gradient it
+// takes three launches with one busy tile column (25 us for 512 x 10, P = 4, B = 100, against
+// 11 here).  The layer's weights are brought into shared memory at once, which exposes one
+// trip to the L2 where reading them class by class exposed a dozen.  For the logits a warp takes
+// two rows and every fourth group of four classes (lanes along the input width); for the data
+// gradient a thread takes two columns of the input and four rows.
+// Dynamic shared memory: dZ [C][8], logits [8][C], the rows of A_{L-1} [8][in], W_L [C][in].
+struct TailArgs {
+  const float* a;                          // A_{L-1} [P, B, in]
+  const float* w; const float* b; int64_t w_batch;
+  const int32_t* labels;
+  int P, B, in, C, row_blocks;
+  float* row_loss;                         // [P, B]
+  float* dz;                               // [P, B, C]
+  float* dzp;                              // dZ_{L-1} [P, B, in], null for a one-layer model
+};
+constexpr int kTailRows = 8, kTailThreads = 512;
+
+template <bool QUANT>
+__global__ void __launch_bounds__(kTailThreads)
+k_simt_tail(const __grid_constant__ TailArgs t, const __grid_constant__ GatherArgs next) {
+  extern __shared__ __align__(16) float sm[];
+  tc::grid_launch_dependents();
+  tc::grid_dependency_wait();
+  if ((int)blockIdx.x >= t.P * t.row_blocks) {
+    gather_row<QUANT>(next, blockIdx.x - t.P * t.row_blocks);
+    return;
+  }
+  const int p = blockIdx.x / t.row_blocks, r0 = blockIdx.x % t.row_blocks * kTailRows;
+  const int rows = min(kTailRows, t.B - r0), in = t.in, C = t.C;
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  float* dzq = sm;                         // [C][8], operand of the data gradient
+  float* z = dzq + kTailRows * C;          // [8][C]
+  float* a = z + kTailRows * C;            // [8][in]
+  const float* W = t.w + (size_t)p * t.w_batch;
+  const float* bias = t.b + (size_t)p * t.w_batch;
+  const float* arow = t.a + ((size_t)p * t.B + r0) * in;
+  float* w = a + kTailRows * in;
+#pragma unroll 8
+  for (int i = threadIdx.x; i < C * in; i += kTailThreads) w[i] = operand<QUANT>(W[i]);
+#pragma unroll 4
+  for (int i = threadIdx.x; i < kTailRows * in; i += kTailThreads) a[i] = i < rows * in ? arow[i] : 0.f;
+  __syncthreads();
+  {
+    const int r = warp % 4 * 2;
+    const float* x = a + r * in;
+    for (int c0 = warp / 4 * 4; c0 < C; c0 += kTailThreads / 32) {
+      float s[2][4] = {};
+      const int last = C - 1 - c0;         // classes beyond the last repeat it
+      const float* w0 = w + c0 * in;
+      const float* wr[4] = {w0, w0 + min(1, last) * in, w0 + min(2, last) * in, w0 + min(3, last) * in};
+#pragma unroll 4
+      for (int i = lane; i < in; i += 32) {
+        const float x0 = x[i], x1 = x[in + i];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float wv = wr[q][i];
+          s[0][q] = fmaf(x0, wv, s[0][q]);
+          s[1][q] = fmaf(x1, wv, s[1][q]);
+        }
+      }
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          for (int o = 16; o > 0; o >>= 1) s[h][q] += __shfl_xor_sync(0xffffffffu, s[h][q], o);
+          if (lane == 4 * h + q && q <= last) z[(r + h) * C + c0 + q] = s[h][q] + bias[c0 + q];
+        }
+    }
+  }
+  __syncthreads();
+  if (warp < rows) {
+    const size_t row = (size_t)p * t.B + r0 + warp;
+    const float loss = softmax_row(z + warp * C, C, t.labels[row], 1.0f / (float)t.B, [&](int c, float g) {
+      t.dz[row * C + c] = g;
+      dzq[c * kTailRows + warp] = operand<QUANT>(g);
+    });
+    if (lane == 0) t.row_loss[row] = loss;
+  } else if (warp < kTailRows) {
+    for (int c = lane; c < C; c += 32) dzq[c * kTailRows + warp] = 0.f;
+  }
+  if (!t.dzp) return;
+  __syncthreads();
+  constexpr int kCols = kTailThreads / 2;
+  const int rh = threadIdx.x / kCols * 4;            // first of this thread's four rows
+  for (int i0 = threadIdx.x % kCols; i0 < in; i0 += 2 * kCols) {
+    const int i1 = i0 + kCols < in ? i0 + kCols : i0;   // i0 again: stored once
+    float s[2][4] = {};
+#pragma unroll 4
+    for (int c = 0; c < C; ++c) {
+      const float wv[2] = {w[c * in + i0], w[c * in + i1]};
+      const float4 dv = *reinterpret_cast<const float4*>(dzq + c * kTailRows + rh);
+      const float d[4] = {dv.x, dv.y, dv.z, dv.w};
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+#pragma unroll
+        for (int r = 0; r < 4; ++r) s[h][r] = fmaf(d[r], wv[h], s[h][r]);
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int i = h ? i1 : i0;
+      if (h && i1 == i0) break;
+#pragma unroll
+      for (int r = 0; r < 4; ++r)                // ReLU'(0) = 0
+        if (rh + r < rows)
+          t.dzp[((size_t)p * t.B + r0 + rh + r) * in + i] = a[(rh + r) * in + i] > 0.f ? s[h][r] : 0.f;
+    }
+  }
+}
+
+// Loss and dZ_L from the logits, for last layers too large for k_simt_tail.  Blocks 0..P-1: a learner's B
+// rows, a warp per row; the remaining blocks gather the next step's minibatch.
+template <bool QUANT>
+__global__ void __launch_bounds__(1024)
+k_simt_loss(const float* __restrict__ logits, const int32_t* __restrict__ labels, int P, int B, int C,
+            float* __restrict__ row_loss, float* __restrict__ dz,
+            const __grid_constant__ GatherArgs next) {
+  tc::grid_launch_dependents();
+  tc::grid_dependency_wait();
+  if ((int)blockIdx.x >= P) {
+    gather_row<QUANT>(next, blockIdx.x - P);
+    return;
+  }
+  const int p = blockIdx.x;
+  for (int b = threadIdx.x / 32; b < B; b += 32) {
+    const size_t row = (size_t)p * B + b;
+    const float loss = softmax_row(logits + row * C, C, labels[row], 1.0f / (float)B, [&](int c, float g) {
+      dz[row * C + c] = g;
+    });
+    if (threadIdx.x % 32 == 0) row_loss[row] = loss;
+  }
+}
+
+// ---------------------------------------------------------------------------------- host side
+struct SimtBuffers {
+  float* xg[2];                     // [P, B, d0], alternate steps
+  int32_t* labels[2];               // [P, B]
+  float* row_loss;                  // [P, B]
+  float* a[MAVG_MAX_LAYERS + 1];    // a[l]  [P, B, d_l]: A_l, l < L; a[L]: the logits
+  float* dz[MAVG_MAX_LAYERS + 1];   // dz[l] [P, B, d_l]
+};
+
+size_t carve(const mavg_config* cfg, char* base, SimtBuffers* sb) {
   const size_t rows = (size_t)cfg->P * cfg->B;
   size_t off = 0;
-  auto take = [&](size_t floats) {
-    float* p = (float*)(base + off);
-    off += (floats * sizeof(float) + 255) / 256 * 256;
+  auto take = [&](size_t words) {
+    char* p = base + off;
+    off += (words * 4 + 255) / 256 * 256;
     return p;
   };
-  sb.xg = take(rows * cfg->dims[0]);
-  for (int l = 1; l <= cfg->n_layers; ++l) {
-    sb.z[l] = take(rows * cfg->dims[l]);
-    sb.dz[l] = take(rows * cfg->dims[l]);
+  for (int i = 0; i < 2; ++i) {
+    sb->xg[i] = (float*)take(rows * cfg->dims[0]);
+    sb->labels[i] = (int32_t*)take(rows);
   }
-  return sb;
+  sb->row_loss = (float*)take(rows);
+  for (int l = 1; l <= cfg->n_layers; ++l) {
+    sb->a[l] = (float*)take(rows * cfg->dims[l]);
+    sb->dz[l] = (float*)take(rows * cfg->dims[l]);
+  }
+  return off;
+}
+
+// Every launch of the chain may begin while its predecessor finishes; the kernels wait for it
+// before they touch memory.
+template <typename... Params, typename... Args>
+cudaError_t launch(mavg_ctx* c, int cls, void (*kernel)(Params...), dim3 grid, int threads,
+                   int cluster, size_t smem, Args... args) {
+  cudaLaunchConfig_t lc{};
+  lc.gridDim = grid;
+  lc.dynamicSmemBytes = smem;
+  lc.blockDim = dim3((unsigned)threads);
+  lc.stream = c->stream;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = (unsigned)cluster;
+  at[1].val.clusterDim.y = 1;
+  at[1].val.clusterDim.z = 1;
+  lc.attrs = at;
+  lc.numAttrs = cluster > 1 ? 2 : 1;
+  prof_begin(c, cls);
+  cudaError_t e = cudaLaunchKernelEx(&lc, kernel, args...);
+  prof_end(c);
+  return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+// The dense rows of `len` elements at p can be copied in groups of four.
+bool vec4(const float* p, int64_t batch, int len) {
+  return (uintptr_t)p % 16 == 0 && batch % 4 == 0 && len % 4 == 0;
+}
+
+int tiles_of(const GemmArgs& g) { return ((g.M + BM - 1) / BM) * ((g.N + BN - 1) / BN); }
+
+// Forward / data gradient.  The contraction is halved until there are two blocks per SM, but a
+// block keeps at least 64 of it (four slabs).
+template <bool QUANT, int EPI>
+cudaError_t launch_gemm(mavg_ctx* c, int cls, GemmArgs g) {
+  const int P = c->cfg.P, tiles = tiles_of(g);
+  int splits = 1;
+  while (splits < kMaxSplit && (int64_t)tiles * P * splits < 2 * c->sm_count && g.K >= 128 * splits)
+    splits *= 2;
+  g.k_per_split = ((g.K + splits - 1) / splits + BK - 1) / BK * BK;
+  return launch(c, cls, k_simt_gemm<QUANT, EPI>, dim3((unsigned)(tiles * splits), 1, (unsigned)P),
+                kThreads, splits, 0, g, splits);
+}
+
+// Last layer in one launch (k_simt_tail) where its weights fit in an SM's shared memory.
+constexpr size_t kTailSmem = 200 * 1024;
+size_t tail_smem(int in, int C) {
+  return ((size_t)kTailRows * in + 2 * (size_t)kTailRows * C + (size_t)in * C) * sizeof(float);
+}
+bool use_tail(int in, int C) { return tail_smem(in, C) <= kTailSmem; }
+
+// Every kernel of a step asks for the same split of the SM's memory: a launch that needs another
+// split than the kernel before it has to wait until the SM is empty.
+template <bool QUANT>
+cudaError_t set_attributes() {
+  const void* kernels[] = {
+      (const void*)k_simt_gemm<QUANT, EPI_FWD>, (const void*)k_simt_gemm<QUANT, EPI_DGRAD>,
+      (const void*)k_simt_wgrad<QUANT>, (const void*)k_simt_gather<QUANT>,
+      (const void*)k_simt_loss<QUANT>, (const void*)k_simt_tail<QUANT>};
+  for (const void* k : kernels) {
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
+                                         cudaSharedmemCarveoutMaxShared);
+    if (e != cudaSuccess) return e;
+  }
+  return cudaFuncSetAttribute(k_simt_tail<QUANT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)kTailSmem);
 }
 
 template <bool QUANT>
 cudaError_t step_impl(mavg_ctx* c, int64_t round, int step) {
   const mavg_config& cfg = c->cfg;
   const int P = cfg.P, B = cfg.B, L = cfg.n_layers;
-  SimtBuffers sb = carve(&cfg, ws_ptr(c, c->ws.act));
-  int32_t* idx = (int32_t*)ws_ptr(c, c->ws.idx);
-  int32_t* labels = (int32_t*)ws_ptr(c, c->ws.labels);
-  float* losses = (float*)ws_ptr(c, c->ws.losses);
+  SimtBuffers sb;
+  carve(&cfg, ws_ptr(c, c->ws.act), &sb);
+  const int cur = step & 1;
+  GatherArgs ga{};
+  ga.x = cfg.x; ga.x_bf16 = cfg.x_dtype == MAVG_X_BF16;
+  ga.y = cfg.y; ga.seed = cfg.seed; ga.round = round;
+  ga.round_ptr = c->capturing ? (const int64_t*)(ws_ptr(c, c->ws.status) + 64) : nullptr;
+  ga.step = step; ga.P = P; ga.B = B; ga.d = cfg.dims[0]; ga.S = cfg.n_samples;
+  ga.out = sb.xg[cur]; ga.labels = sb.labels[cur];
+  GatherArgs next = ga;
+  next.step = step + 1; next.out = sb.xg[cur ^ 1]; next.labels = sb.labels[cur ^ 1];
+  const int gather_rows = step < cfg.K ? P * B : 0;
   cudaError_t e;
-  if ((e = launch_batch_indices(c, round, step, 0, P, idx, labels)) != cudaSuccess) return e;
-  if ((e = launch_gather(c, idx, QUANT ? 1 : 0, sb.xg, nullptr, nullptr)) != cudaSuccess) return e;
+  if (step == 1 &&
+      (e = launch(c, MAVG_K_BATCH, k_simt_gather<QUANT>, dim3((unsigned)(P * B)), 256, 1, 0, ga)) != cudaSuccess)
+    return e;
+  // the weights before this step: w~ itself at the first one
   float* rep = c->buf.replicas;
   const int64_t rs = c->buf.replica_stride;
+  const float* win = c->replicas_equal_global ? c->buf.global_w : rep;
+  const int64_t ws = c->replicas_equal_global ? 0 : rs;
   const MomArgs mom = mom_args(c, c->replicas_equal_global);
-  // forward
-  for (int l = 1; l <= L; ++l) {
+  auto a_in = [&](int l) { return l == 1 ? sb.xg[cur] : sb.a[l - 1]; };
+  const MlpLayer& top = c->layers[L - 1];
+  const bool tail = use_tail(top.in, top.out);
+  for (int l = 1; l <= (tail ? L - 1 : L); ++l) {
     const MlpLayer& ly = c->layers[l - 1];
     GemmArgs g{};
-    g.A = l == 1 ? sb.xg : sb.z[l - 1]; g.a_batch = (int64_t)B * ly.in; g.a_m = ly.in; g.a_k = 1;
-    g.B = rep + ly.w_off; g.b_batch = rs; g.b_n = ly.in; g.b_k = 1;
+    g.A = a_in(l); g.a_batch = (int64_t)B * ly.in;
+    g.B = win + ly.w_off; g.b_batch = ws;
     g.M = B; g.N = ly.out; g.K = ly.in;
-    g.C = sb.z[l]; g.c_batch = (int64_t)B * ly.out; g.c_m = ly.out;
-    g.aux = rep + ly.b_off; g.aux_batch = rs; g.aux_m = 0;
-    dim3 grid((ly.out + BN - 1) / BN, (B + BM - 1) / BM, P);
-    prof_begin(c, MAVG_K_FWD);
-    if (l == 1)
-      k_simt_gemm<QUANT, LD_PLAIN, LD_PLAIN, true, true, EPI_FWD><<<grid, 256, 0, c->stream>>>(g);
-    else
-      k_simt_gemm<QUANT, LD_RELU, LD_PLAIN, true, true, EPI_FWD><<<grid, 256, 0, c->stream>>>(g);
-    prof_end(c);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    g.C = sb.a[l]; g.c_batch = (int64_t)B * ly.out;
+    g.aux = win + ly.b_off; g.aux_batch = ws;
+    g.vec_a = vec4(g.A, g.a_batch, g.K);
+    g.vec_b = vec4(g.B, g.b_batch, g.K);
+    g.vec_c = vec4(g.C, g.c_batch, g.N);
+    g.hidden = l < L;
+    if ((e = launch_gemm<QUANT, EPI_FWD>(c, MAVG_K_FWD, g)) != cudaSuccess) return e;
   }
-  // loss, dZ_L and the last bias
-  const int C = cfg.dims[L];
-  if ((e = launch_softmax_ce(c, sb.z[L], C, labels, losses + (step - 1), cfg.K, sb.dz[L], C,
-                             nullptr, 0, nullptr, 0, true, mom)) != cudaSuccess)
-    return e;
-  // backward + SGD, layer L down to 1; dgrad reads W_l before wgrad overwrites it
-  for (int l = L; l >= 1; --l) {
+  if (tail) {
+    TailArgs t{};
+    t.a = a_in(L); t.w = win + top.w_off; t.b = win + top.b_off; t.w_batch = ws;
+    t.labels = sb.labels[cur];
+    t.P = P; t.B = B; t.in = top.in; t.C = top.out; t.row_blocks = (B + kTailRows - 1) / kTailRows;
+    t.row_loss = sb.row_loss; t.dz = sb.dz[L];
+    if (L >= 2) t.dzp = sb.dz[L - 1];
+    if ((e = launch(c, MAVG_K_LOSS, k_simt_tail<QUANT>, dim3((unsigned)(P * t.row_blocks + gather_rows)),
+                    kTailThreads, 1, tail_smem(t.in, t.C), t, next)) != cudaSuccess)
+      return e;
+  } else {
+    if ((e = launch(c, MAVG_K_LOSS, k_simt_loss<QUANT>, dim3((unsigned)(P + gather_rows)), 1024, 1, 0,
+                    (const float*)sb.a[L], (const int32_t*)sb.labels[cur], P, B, top.out, sb.row_loss,
+                    sb.dz[L], next)) != cudaSuccess)
+      return e;
+  }
+  for (int l = tail ? L - 1 : L; l >= 2; --l) {
     const MlpLayer& ly = c->layers[l - 1];
-    if (l > 1) {
-      GemmArgs g{};
-      g.A = sb.dz[l]; g.a_batch = (int64_t)B * ly.out; g.a_m = ly.out; g.a_k = 1;
-      g.B = rep + ly.w_off; g.b_batch = rs; g.b_n = 1; g.b_k = ly.in;
-      g.M = B; g.N = ly.in; g.K = ly.out;
-      g.C = sb.dz[l - 1]; g.c_batch = (int64_t)B * ly.in; g.c_m = ly.in;
-      g.aux = sb.z[l - 1]; g.aux_batch = (int64_t)B * ly.in; g.aux_m = ly.in;
-      dim3 grid((ly.in + BN - 1) / BN, (B + BM - 1) / BM, P);
-      prof_begin(c, MAVG_K_DGRAD);
-      k_simt_gemm<QUANT, LD_PLAIN, LD_PLAIN, true, false, EPI_DGRAD><<<grid, 256, 0, c->stream>>>(g);
-      prof_end(c);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    {
-      GemmArgs g{};
-      g.A = sb.dz[l]; g.a_batch = (int64_t)B * ly.out; g.a_m = 1; g.a_k = ly.out;
-      g.B = l == 1 ? sb.xg : sb.z[l - 1]; g.b_batch = (int64_t)B * ly.in; g.b_n = 1; g.b_k = ly.in;
-      g.M = ly.out; g.N = ly.in; g.K = B;
-      g.C = rep + ly.w_off; g.c_batch = rs; g.c_m = ly.in;
-      g.gamma = cfg.local_lr;
-      g.mom = mom; g.u_off = ly.w_off;
-      dim3 grid((ly.in + BN - 1) / BN, (ly.out + BM - 1) / BM, P);
-      prof_begin(c, MAVG_K_WGRAD_SGD);
-      if (l == 1)
-        k_simt_gemm<QUANT, LD_PLAIN, LD_PLAIN, false, false, EPI_WGRAD_SGD><<<grid, 256, 0, c->stream>>>(g);
-      else
-        k_simt_gemm<QUANT, LD_PLAIN, LD_RELU, false, false, EPI_WGRAD_SGD><<<grid, 256, 0, c->stream>>>(g);
-      prof_end(c);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
-    if (l < L) {
-      dim3 grid((ly.out + 255) / 256, P);
-      prof_begin(c, MAVG_K_WGRAD_SGD);
-      k_simt_bias_sgd<<<grid, 256, 0, c->stream>>>(sb.dz[l], (int64_t)B * ly.out, B, ly.out, rep,
-                                                   rs, ly.b_off, cfg.local_lr, mom);
-      prof_end(c);
-      if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    }
+    GemmArgs g{};
+    g.A = sb.dz[l]; g.a_batch = (int64_t)B * ly.out;
+    g.B = win + ly.w_off; g.b_batch = ws;
+    g.M = B; g.N = ly.in; g.K = ly.out;
+    g.C = sb.dz[l - 1]; g.c_batch = (int64_t)B * ly.in;
+    g.aux = sb.a[l - 1]; g.aux_batch = g.c_batch;
+    g.vec_a = vec4(g.A, g.a_batch, g.K);
+    g.vec_b = vec4(g.B, g.b_batch, g.N);
+    g.vec_c = vec4(g.C, g.c_batch, g.N);
+    if ((e = launch_gemm<QUANT, EPI_DGRAD>(c, MAVG_K_DGRAD, g)) != cudaSuccess) return e;
   }
-  return cudaSuccess;
+  WgradArgs w{};
+  w.L = L;
+  for (int l = 1; l <= L; ++l) {
+    const MlpLayer& ly = c->layers[l - 1];
+    GemmArgs& g = w.g[l - 1];
+    g.A = sb.dz[l]; g.a_batch = (int64_t)B * ly.out;
+    g.B = a_in(l); g.b_batch = (int64_t)B * ly.in;
+    g.M = ly.out; g.N = ly.in; g.K = g.k_per_split = B;
+    g.C = rep + ly.w_off; g.c_batch = rs;
+    g.aux = win + ly.w_off; g.aux_batch = ws;
+    g.vec_a = vec4(g.A, g.a_batch, g.M);
+    g.vec_b = vec4(g.B, g.b_batch, g.N);
+    g.vec_c = vec4(g.C, g.c_batch, g.N) && vec4(g.aux, g.aux_batch, g.N);
+    g.bias = rep + ly.b_off; g.bias_in = win + ly.b_off;
+    g.gamma = cfg.local_lr;
+    g.mom = mom; g.u_off = ly.w_off; g.ub_off = ly.b_off;
+    w.tile0[l] = w.tile0[l - 1] + tiles_of(g);
+  }
+  w.row_loss = sb.row_loss;
+  w.loss_out = (float*)ws_ptr(c, c->ws.losses) + (step - 1);
+  w.loss_stride = cfg.K;
+  return launch(c, MAVG_K_WGRAD_SGD, k_simt_wgrad<QUANT>, dim3((unsigned)w.tile0[L], 1, (unsigned)P),
+                kThreads, 1, 0, w);
 }
 
 }  // namespace
 
 size_t simt_workspace_bytes(const mavg_config* cfg, size_t base, size_t* act_off) {
   *act_off = base;
-  const size_t rows = (size_t)cfg->P * cfg->B;
-  size_t off = base;
-  auto take = [&](size_t floats) { off += (floats * sizeof(float) + 255) / 256 * 256; };
-  take(rows * cfg->dims[0]);
-  for (int l = 1; l <= cfg->n_layers; ++l) {
-    take(rows * cfg->dims[l]);
-    take(rows * cfg->dims[l]);
-  }
-  return off;
+  SimtBuffers sb;
+  return base + carve(cfg, nullptr, &sb);
+}
+
+cudaError_t simt_setup(mavg_ctx* c) {
+  return c->cfg.gemm_bf16 ? set_attributes<true>() : set_attributes<false>();
 }
 
 cudaError_t simt_step(mavg_ctx* c, int64_t round, int step) {
