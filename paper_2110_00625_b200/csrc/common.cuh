@@ -131,6 +131,7 @@ struct mavg_ctx {
   int graph_schedule = 0;
   int graph_w16_cur = 0;      // state of the doubled bf16 copy after the recorded steps
   int64_t graph_nodes = 0;
+  int small_splits = 0;       // blocks per learner of the small-model kernel (mlp_small.cu), 0: not used
   // this handle holds a request on the context's persisting-L2 limit (given up by mavg_destroy)
   bool l2_keep = false;
   size_t l2_keep_want = 0;

@@ -37,7 +37,8 @@ mavg_status mlp_setup(mavg_ctx* c) {
     c->layers.push_back(ly);
   }
   if (use_tensor_cores(&cfg)) return tc_setup(c);
-  const cudaError_t e = simt_setup(c);
+  cudaError_t e = simt_setup(c);
+  if (e == cudaSuccess) e = small_setup(c);
   if (e == cudaSuccess) return MAVG_OK;
   c->err = std::string("kernel attributes: ") + cudaGetErrorString(e);
   return MAVG_ERR_CUDA;
@@ -135,6 +136,7 @@ cudaError_t mlp_local_steps(mavg_ctx* c, int64_t round) {
   // The usual round starts from the broadcast state and is replayed from a graph.  Rounds that
   // start elsewhere (local steps called twice in a row), profiled rounds and handles whose
   // capture failed once take the launch-by-launch path.
+  if (!c->profiling && c->small_splits) return small_local_steps(c, round);
   const bool want_graph = !c->profiling && !c->graph_disabled && c->replicas_equal_global;
   if (!want_graph) return run_steps(c, round);
   if (!c->graph_exec || c->graph_K != c->cfg.K || c->graph_lr != c->cfg.local_lr ||

@@ -5,12 +5,14 @@
 
 namespace mavg {
 
+// First sample of learner j's shard, floor(j S / P); j <= 2^31 and S < 2^31: 64 bits hold the product.
+__device__ __forceinline__ int64_t shard_begin(int64_t j, int P, int64_t S) {
+  return (int64_t)((uint64_t)j * (uint64_t)S / (uint32_t)P);
+}
 // idx = lo_j + floor(u * len_j / 2^32), u = top 32 bits of the stream value (see mavg.h).
 __device__ __forceinline__ int32_t sample_index(uint64_t seed, int64_t round, int j, int step,
                                                 int s, int P, int64_t S) {
-  // j < 2^31 and S < 2^31: the products fit in 64 bits
-  int64_t lo = (int64_t)((uint64_t)j * (uint64_t)S / (uint32_t)P);
-  int64_t hi = (int64_t)(((uint64_t)j + 1) * (uint64_t)S / (uint32_t)P);
+  const int64_t lo = shard_begin(j, P, S), hi = shard_begin((int64_t)j + 1, P, S);
   uint64_t key = fold(learner_key(seed, kTagBatch, (uint64_t)round, (uint64_t)j), (uint64_t)step);
   uint64_t u = fold(key, (uint64_t)s) >> 32;
   return (int32_t)(lo + (int64_t)((u * (uint64_t)(hi - lo)) >> 32));
@@ -25,6 +27,10 @@ cudaError_t launch_sample_gather(mavg_ctx* c, int64_t round, int step, int32_t* 
 size_t simt_workspace_bytes(const mavg_config* cfg, size_t base, size_t* act_off);
 cudaError_t simt_setup(mavg_ctx* c);      // once per handle
 cudaError_t simt_step(mavg_ctx* c, int64_t round, int step);
+
+// Small models on the CUDA cores (mlp_small.cu): all local steps of a round in one launch.
+cudaError_t small_setup(mavg_ctx* c);     // once per handle: c->small_splits > 0 where it is used
+cudaError_t small_local_steps(mavg_ctx* c, int64_t round);
 
 // Tensor-core path (mlp_tc.cu): tcgen05 GEMMs fed by TMA.
 bool tc_shapes_ok(const mavg_config* cfg, std::string* why);

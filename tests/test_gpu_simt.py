@@ -1,5 +1,6 @@
 """CUDA-core learner steps at the edges of their tiles and of the rules that choose between their
-launches, against the oracle: two local steps from identical replicas with learner momentum, whose
+launches, against the oracle, with all steps in one launch where a model is small enough and launch by
+launch (profiled rounds): two local steps from identical replicas with learner momentum, whose
 buffers hold the gradients without the cancellation of a weight difference."""
 import numpy as np
 import pytest
@@ -21,12 +22,19 @@ SHAPES = [
     ([96, 256, 600], 33, 2),               # many classes
     ([3072, 64, 10], 16, 1),               # contraction split over eight blocks
     ([130, 72, 40, 24, 16, 6], 9, 2),      # five layers
+    ([9, 1, 7], 3, 1),                     # a width of one, fewer samples than a group of rows
+    ([32, 64, 10], 32, 4),                 # eight blocks a learner, one group of rows each
+    ([33, 40, 40, 12], 29, 5),             # uneven rows and columns per block, padded rows
+    ([32, 64, 10], 50, 150),               # more learners than SMs: one block each
+    ([24, 30, 40], 70, 40),                # two blocks a learner, more than 32 classes
+    ([80, 128, 128, 16], 32, 3),           # the largest of its kind: four rows of W share a task
 ]
 
 
+@pytest.mark.parametrize("profiled", [False, True])
 @pytest.mark.parametrize("mode", [0, 2])
 @pytest.mark.parametrize("dims,B,P", SHAPES)
-def test_two_steps_against_the_oracle(oracle, mode, dims, B, P):
+def test_two_steps_against_the_oracle(oracle, mode, dims, B, P, profiled):
     import paper_2110_00625_b200 as m
     S = 40 * P + 3
     rng = np.random.default_rng(len(dims) * 1000 + B)
@@ -39,6 +47,7 @@ def test_two_steps_against_the_oracle(oracle, mode, dims, B, P):
     kw["x"] = g.x.float().cpu().numpy()
     o = oracle.Mavg(w1, gamma=0.01, objective=oracle.OBJ_MLP, bf16=mode != 0, beta=0.5,
                     stride=g.stride, **kw)
+    g.set_profiling(profiled)
     g.local_steps()
     losses, _ = o.local_steps()
     g.sync()
