@@ -172,6 +172,14 @@ GemmPlan plan_partial(int M, int N, int K, int P, int sm_count, bool tile_n) {
   return g;
 }
 
+// Whether the weight gradients are large enough to be launches of their own (more than 64 tiles per SM
+// in layer 1) and can take the next step's forward products along.
+bool rides(const mavg_config* cfg, int sm_count) {
+  const long m_tiles = (cfg->dims[1] + kWgradTileRows - 1) / kWgradTileRows;
+  const long n_tiles = (cfg->dims[0] + kWgradTileCols - 1) / kWgradTileCols;
+  return cfg->n_layers >= 2 && cfg->B <= 128 && cfg->P * m_tiles * n_tiles > 64L * sm_count;
+}
+
 TcLayout make_layout(const mavg_config* cfg, size_t base, int sm_count) {
   TcLayout t{};
   const int L = cfg->n_layers, P = cfg->P, B = cfg->B;
@@ -238,6 +246,12 @@ TcLayout make_layout(const mavg_config* cfg, size_t base, int sm_count) {
   }
   t.w16b_stride = L >= 3 ? (int64_t)up((size_t)cfg->dims[L - 2] * cfg->dims[L - 1], 64) : 0;
   t.w16b = take(L >= 3 ? (size_t)P * t.w16b_stride * 2 : 16);
+  if (rides(cfg, sm_count))
+    for (int l = 2; l < L; ++l) {
+      t.lo_off[l - 1] = t.n_lo;
+      t.n_lo += (int64_t)up((size_t)cfg->dims[l] * cfg->dims[l - 1], 64);
+    }
+  t.lo16 = take(std::max<size_t>((size_t)P * t.n_lo * 2, 16));
   t.end = off;
   return t;
 }
@@ -524,7 +538,7 @@ mavg_status tc_setup(mavg_ctx* c) {
     for (int l = 1; l < L; ++l) {
       const int in = cfg.dims[l - 1], out = cfg.dims[l];
       const WgradPlan w = plan_wgrad_stream(out, in, B, P, c->sm_count, st->wgrad_mom,
-                                            !masters_fit_l2(c), true);
+                                            !masters_fit_l2(c), true, l >= 2 && t.n_lo > 0);
       const size_t need = (size_t)P * w.m_tiles * w.n_chunks * B * kBM * sizeof(float);
       if (w.slots < 2 || need > t.zpart_bytes || (size_t)P * w.m_tiles * sizeof(int) > t.zcount_bytes)
         break;
@@ -534,6 +548,10 @@ mavg_status tc_setup(mavg_ctx* c) {
         enc = encode_any(st, &st->a_next[l][i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, bf(src), in, B,
                          P, in, (int64_t)B * in, kWgradTileCols, B, CU_TENSOR_MAP_SWIZZLE_64B, &why);
       }
+      if (enc && l >= 2 && t.n_lo)
+        enc = encode_any(st, &st->lo16[l], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
+                         (__nv_bfloat16*)bf(t.lo16) + t.lo_off[l - 1], in, out, P, in, t.n_lo,
+                         kWgradTileCols, kWgradTileRows, CU_TENSOR_MAP_SWIZZLE_64B, &why);
       if (!enc) break;
       st->wgrad_f[l] = w;
       st->fuse_upto = l;
@@ -683,6 +701,19 @@ cudaError_t tc_step(mavg_ctx* c, int64_t round, int step) {
   const int ride = (c->schedule == 0 && !merged && step < K) ? st->fuse_upto : 0;
   const int done = step == 1 ? 0 : st->fwd_done;
   st->fwd_done = 0;
+  const int was_split = step == 1 ? 0 : st->split_done;
+  st->split_done = 0;
+  auto split_of = [&](int l, bool out) {
+    WgradSplit sp;
+    sp.in = l >= 2 && l <= was_split;
+    sp.out = out && l >= 2 && t.n_lo > 0;
+    if (sp.in || sp.out) {
+      sp.lo = &st->lo16[l];
+      sp.master = c->buf.replicas + c->layers[l - 1].w_off;
+      sp.in_cols = c->layers[l - 1].in;
+    }
+    return sp;
+  };
   // activation buffers of this step and of the next
   const int ab = st->fuse_upto >= 1 ? (step & 1) : 0;
   auto act_of = [&](int l, int set) { return bfp(set ? t.act_b[l] : t.act[l]); };
@@ -834,12 +865,14 @@ cudaError_t tc_step(mavg_ctx* c, int64_t round, int step) {
       TC_TRY(cudaStreamWaitEvent(st->s_wgrad, st->ev_fork, 0));
       c->stream = st->s_wgrad;
       TC_TRY(launch_wgrad_stream(c, st->wgrad[l], st->dz_t[l], bm, st->w32[l], *w_st(l),
-                                 shared_w ? &st->w32g[l] : nullptr, &st->u32[l], mom));
+                                 shared_w ? &st->w32g[l] : nullptr, &st->u32[l], mom, nullptr,
+                                 split_of(l, false)));
       c->stream = main_s;
       side_used = true;
     } else {
       TC_TRY(launch_wgrad_stream(c, st->wgrad[l], st->dz_t[l], bm, st->w32[l], *w_st(l),
-                                 shared_w ? &st->w32g[l] : nullptr, &st->u32[l], mom));
+                                 shared_w ? &st->w32g[l] : nullptr, &st->u32[l], mom, nullptr,
+                                 split_of(l, false)));
     }
   }
   // Layers whose launch takes the next step's forward product along: layer l's needs A_{l-1} of
@@ -869,8 +902,10 @@ cudaError_t tc_step(mavg_ctx* c, int64_t round, int step) {
     fn.out_mb = act_t_of(l, nb);
     fn.store_w16 = l > 1;
     TC_TRY(launch_wgrad_stream(c, st->wgrad_f[l], st->dz_t[l], bm, st->w32[l], *w_st(l),
-                               shared_w ? &st->w32g[l] : nullptr, &st->u32[l], mom, &fn));
+                               shared_w ? &st->w32g[l] : nullptr, &st->u32[l], mom, &fn,
+                               split_of(l, true)));
     st->fwd_done = l;
+    if (t.n_lo) st->split_done = l;
   }
   if (merged) {
     // largest layer first, so that the small ones fill the ragged end of the launch

@@ -30,6 +30,10 @@ struct TcLayout {
                                              // layer at a time
   size_t w16b;                               // second bf16 copy of layer L-1's weights [P, w16b_stride]
   int64_t w16b_stride;
+  // low halves of the masters of layers 2..L-1 [P, n_lo], which are split between the steps of a call
+  // where forward products ride (0 elements: never); layer l at lo_off[l - 1]
+  size_t lo16;
+  int64_t n_lo, lo_off[MAVG_MAX_LAYERS];
   size_t end;
 };
 
@@ -79,6 +83,10 @@ struct TcState {
   // (l = 1: gather buffer i) as the riding product reads it.  fwd_done: how many leading
   // layers of the step about to be issued already have their activations; gathered_step: the
   // step whose batch has already been gathered by the launch-by-launch form.
+  // lo16: the low halves of split masters (layers 2..fuse_upto); split_done: the leading layers whose
+  // masters the previous step of this call left split (layer 1's never are).
+  CUtensorMap lo16[MAVG_MAX_LAYERS + 1];
+  int split_done = 0;
   int fuse_upto = 0;
   int fwd_done = 0;
   int gathered_step = 0;

@@ -8,9 +8,10 @@
 //                   of A^T into a ring of shared-memory slots; the 128 x B tile of dZ^T is loaded
 //                   once per work item (a run of column tiles of one learner and row tile);
 //   MMA warp        one thread issues tcgen05.mma (M=128, N=32, K=B) into one of two TMEM buffers;
-//   2 x 4 epilogue warps (one group per TMEM buffer, i.e. per tile parity) read the accumulator
-//                   (tcgen05.ld, one weight row per lane), update the master tile in place in
-//                   shared memory and write the bf16 tile beside it;
+//   2 x 8 epilogue warps (one group per TMEM buffer, i.e. per tile parity; four warps for each half
+//                   of a tile's columns) read the accumulator (tcgen05.ld, one weight row per
+//                   lane), update the master tile in place in shared memory and write the bf16
+//                   tile beside it;
 //   store warp      one thread sends the two finished tiles back with TMA stores and frees the
 //                   slot once they have left shared memory.
 // With learner-level momentum (MOM) the tile of u^j travels with the master tile: loaded into the
@@ -18,7 +19,7 @@
 // W <- W + u) and stored back, 18 bytes per weight instead of 10.
 // Edge tiles need no predicates: TMA zero-fills loads and clips stores at the tensor bounds.
 //
-// The 512-thread instantiation (FWD) lets the NEXT local step's forward product of the same layer
+// The 768-thread instantiation (FWD) lets the NEXT local step's forward product of the same layer
 // ride along: the epilogue has just put the updated bf16 tile W16[128, 32] into the slot, and the
 // producer has loaded the matching [B, 32] tile of the next step's input Xn beside it, so
 //   forward warp    one thread issues W16_tile . Xn_tile^T (M=128, N=B, K=32) into a third TMEM
@@ -31,6 +32,15 @@
 //                   partial sums in ascending run order and finishes the row.
 // Per weight and step this removes the forward product's read of the bf16 copy and, for a layer
 // without a dgrad product (layer 1), the copy itself.
+//
+// A layer whose dgrad product needs the copy keeps its masters split between the steps of a call
+// (join_master in wgrad_unit.cuh): the copy gives the upper half and an array of the same shape holds
+// the lower one, so a step moves 4 + 4 bytes per weight instead of 4 + 4 + 2, and no bit is lost.  The first riding launch
+// reads fp32 masters (or w~) and leaves the two halves, the call's last launch reads them and
+// writes fp32 masters and the copy, and in between nothing needs the fp32 array.
+// Per layer of 2048 x 2048, P = 32, B = 64: 270 -> 232 us a launch, with the deeper ring that the
+// smaller slots allow (see plan_wgrad_stream); as much arithmetic per weight takes an epilogue of 16
+// columns per thread (with 32, and half as many warps, the round took 17.15 ms against 15.9).
 #include <cuda.h>
 
 #include <algorithm>
@@ -47,7 +57,7 @@ using namespace tc;
 using namespace wgrad;
 
 template <bool MOM, bool FWD>
-__global__ void __launch_bounds__(FWD ? kThreadsFwd : kThreads)
+__global__ void __launch_bounds__(FWD ? kThreadsFwd : kThreads, 1)
 k_wgrad_sgd_stream(const __grid_constant__ CUtensorMap tm_dzt,   // bf16 [P, out, B]  load
                    const __grid_constant__ CUtensorMap tm_at,    // bf16 [P, in, B]   load
                    const __grid_constant__ CUtensorMap tm_w32,   // fp32 [P, out, in] store
@@ -57,6 +67,7 @@ k_wgrad_sgd_stream(const __grid_constant__ CUtensorMap tm_dzt,   // bf16 [P, out
                    const __grid_constant__ CUtensorMap tm_w16,   // bf16 [P, out, in] store
                    const __grid_constant__ CUtensorMap tm_u,     // fp32 [P, out, in] u^j, load + store (MOM)
                    const __grid_constant__ CUtensorMap tm_xn,    // bf16 [P, B, in] next step's input (fwd_next)
+                   const __grid_constant__ CUtensorMap tm_lo,    // [P, out, in] low halves of split masters
                    const WgradArgs g) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) WgradShared sh;
@@ -74,6 +85,7 @@ k_wgrad_sgd_stream(const __grid_constant__ CUtensorMap tm_dzt,   // bf16 [P, out
     tma_prefetch_desc(&tm_w16);
     if (MOM) tma_prefetch_desc(&tm_u);
     if (FWD && g.fwd_next) tma_prefetch_desc(&tm_xn);
+    if (g.in_split || g.out_split) tma_prefetch_desc(&tm_lo);
     wgrad_init_barriers(sh, g.slots);
     sh.abort_flag = 0;
     fence_barrier_init();
@@ -90,8 +102,8 @@ k_wgrad_sgd_stream(const __grid_constant__ CUtensorMap tm_dzt,   // bf16 [P, out
   tc_fence_after_sync();
   const uint32_t tmem_base = sh.tmem_slot;
   grid_dependency_wait();
-  wgrad_run<MOM, FWD>(tm_dzt, tm_at, tm_w32, tm_w32_in, tm_w16, tm_u, tm_xn, g, (int)blockIdx.x,
-                 (int)gridDim.x, smem, sh, tmem_base);
+  wgrad_run<MOM, FWD, true>(tm_dzt, tm_at, tm_w32, tm_w32_in, tm_w16, tm_u, tm_xn, tm_lo, g,
+                            (int)blockIdx.x, (int)gridDim.x, smem, sh, tmem_base);
   tc_fence_before_sync();
   __syncthreads();
   if (warp == 1) tmem_dealloc(tmem_base, tmem_cols);
@@ -110,7 +122,7 @@ struct WgradMultiParams {
 };
 
 template <bool MOM>
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 1)
 k_wgrad_sgd_multi(const __grid_constant__ WgradMultiParams mp) {
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(8) WgradShared sh;
@@ -137,8 +149,9 @@ k_wgrad_sgd_multi(const __grid_constant__ WgradMultiParams mp) {
   const int grid = (int)gridDim.x;
   for (int s = 0; s < mp.n; ++s) {
     const int vb = ((int)blockIdx.x + mp.rot[s]) % grid;
-    wgrad_run<MOM, false>(mp.dzt[s], mp.at[s], mp.w32[s], mp.w32_in[s], mp.w16[s], mp.u[s], mp.w16[s],
-                   mp.g[s], vb, grid, smem, sh, tmem_base, tiles, items);
+    wgrad_run<MOM, false, false>(mp.dzt[s], mp.at[s], mp.w32[s], mp.w32_in[s], mp.w16[s], mp.u[s],
+                                 mp.w16[s], mp.w16[s], mp.g[s], vb, grid, smem, sh, tmem_base, tiles,
+                                 items);
     wgrad_run_totals(mp.g[s], vb, grid, tiles, items);
   }
   tc_fence_before_sync();
@@ -148,32 +161,13 @@ k_wgrad_sgd_multi(const __grid_constant__ WgradMultiParams mp) {
 
 }  // namespace
 
-// longest run of column tiles of one work item
-#ifndef MAVG_WGRAD_CHUNK_CAP
-#define MAVG_WGRAD_CHUNK_CAP 16
-#endif
-constexpr long kWgradChunkCap = MAVG_WGRAD_CHUNK_CAP;
-// deepest ring the plan may choose (at most kMaxSlots)
-#ifndef MAVG_WGRAD_SLOT_CAP
-#define MAVG_WGRAD_SLOT_CAP 6
-#endif
-// the same two for a launch that streams its masters through HBM
-#ifndef MAVG_WGRAD_STREAM_CHUNK
-#define MAVG_WGRAD_STREAM_CHUNK 8
-#endif
-#ifndef MAVG_WGRAD_STREAM_SLOTS
-#define MAVG_WGRAD_STREAM_SLOTS 4
-#endif
-constexpr long kWgradStreamChunk = MAVG_WGRAD_STREAM_CHUNK;
-#ifndef MAVG_WGRAD_FWD_SLOTS
-#define MAVG_WGRAD_FWD_SLOTS 6
-#endif
-constexpr int kWgradFwdSlots = MAVG_WGRAD_FWD_SLOTS;
-constexpr int kWgradStreamSlots = MAVG_WGRAD_STREAM_SLOTS;
-constexpr int kWgradSlotCap = MAVG_WGRAD_SLOT_CAP < wgrad::kMaxSlots ? MAVG_WGRAD_SLOT_CAP : wgrad::kMaxSlots;
+// Longest run of column tiles of one work item and deepest ring of a launch without a riding forward
+// product; the same two where the masters stream through HBM.
+constexpr long kWgradChunkCap = 16, kWgradStreamChunk = 8;
+constexpr int kWgradSlotCap = 6, kWgradStreamSlots = 4;
 
 WgradPlan plan_wgrad_stream(int out, int in, int B, int P, int sm_count, bool momentum,
-                            bool streaming, bool fwd_next) {
+                            bool streaming, bool fwd_next, bool split) {
   WgradPlan w{};
   w.nkb = (B + kBK - 1) / kBK;
   w.m_tiles = (out + kBM - 1) / kBM;
@@ -221,20 +215,27 @@ WgradPlan plan_wgrad_stream(int out, int in, int B, int P, int sm_count, bool mo
   w.items = w.whole_rows + (P * w.m_tiles - w.whole_rows) * w.n_chunks;
   const int a_bytes = w.nkb * kBM * kBK * 2;
   const int b_bytes = w.nkb * kBN * kBK * 2;
-  w.w16_on_b = b_bytes >= kW16Bytes ? 1 : 0;   // the bf16 output tile reuses the A^T slabs' space
+  // Where in a slot the bf16 output tile lies: over the A^T slabs (read by then) if they are as large
+  // or a forward product rides along, behind them otherwise, nowhere if it is half of a split master.
+  const bool over = split || fwd_next || b_bytes >= kW16Bytes;
+  w.w16_off = over ? 0 : b_bytes;
+  w.b_room = split ? b_bytes : over ? std::max(b_bytes, kW16Bytes) : b_bytes + kW16Bytes;
   w.xn_bytes = fwd_next ? B * kBN * 2 : 0;
-  const int slot_bytes = kW32Bytes + (momentum ? kW32Bytes : 0) + (w.w16_on_b ? 0 : kW16Bytes) +
-                         b_bytes + w.xn_bytes;
+  const int slot_bytes = kW32Bytes + (momentum ? kW32Bytes : 0) + w.b_room + w.xn_bytes;
+  // With a riding forward product a slot lives through two more hand-overs (epilogue -> forward MMAs
+  // -> store), so it takes as many slots as fit: a second dZ^T buffer, which a long run uses once,
+  // makes room for one.  Large MLP, ms a round: 5 / 6 / 7 slots for split masters 16.1 / 15.7 / 15.3;
+  // bf16 tile over the slabs 15.5 -> 15.35; one dZ^T buffer (7 slots, 8 for split masters) 15.0.
   const int budget = 220 * 1024;
-  w.a_bufs = 2;
-  w.slots = (budget - 2 * a_bytes) / slot_bytes;
-  if (w.slots < 2) {
+  w.a_bufs = fwd_next ? 1 : 2;
+  w.slots = (budget - w.a_bufs * a_bytes) / slot_bytes;
+  if (w.slots < 2 && w.a_bufs == 2) {
     w.a_bufs = 1;
     w.slots = (budget - a_bytes) / slot_bytes;
   }
-  if (w.slots > kWgradSlotCap) w.slots = kWgradSlotCap;
-  const int stream_slots = fwd_next ? kWgradFwdSlots : kWgradStreamSlots;
-  if (streaming && w.slots > stream_slots) w.slots = stream_slots;
+  if (w.slots > wgrad::kMaxSlots) w.slots = wgrad::kMaxSlots;
+  if (!fwd_next && w.slots > kWgradSlotCap) w.slots = kWgradSlotCap;
+  if (!fwd_next && streaming && w.slots > kWgradStreamSlots) w.slots = kWgradStreamSlots;
   w.smem = (size_t)w.a_bufs * a_bytes + (size_t)w.slots * slot_bytes + 1024;
   w.grid = w.items < sm_count ? w.items : sm_count;
   return w;
@@ -267,7 +268,8 @@ WgradArgs make_args(mavg_ctx* c, const WgradPlan& w, bool shared, const MomArgs&
   g.whole_rows = w.whole_rows;
   g.slots = w.slots;
   g.a_bufs = w.a_bufs;
-  g.w16_on_b = w.w16_on_b;
+  g.b_room = w.b_room;
+  g.w16_off = w.w16_off;
   g.keep_w32 = c->l2_keep ? 1 : 0;
   g.gamma = c->cfg.local_lr;
   g.beta = mom.beta;
@@ -324,8 +326,14 @@ cudaError_t launch_wgrad_stream(mavg_ctx* c, const WgradPlan& w, const CUtensorM
                                 const CUtensorMap& at, const CUtensorMap& w32,
                                 const CUtensorMap& w16, const CUtensorMap* w32_shared,
                                 const CUtensorMap* u32, const MomArgs& mom,
-                                const WgradFwdNext* fn) {
+                                const WgradFwdNext* fn, const WgradSplit& split) {
   WgradArgs g = make_args(c, w, w32_shared != nullptr, mom);
+  g.master = split.master;
+  g.in_cols = split.in_cols;
+  g.rep_stride = c->buf.replica_stride;
+  g.in_split = split.in ? 1 : 0;
+  g.out_split = split.out ? 1 : 0;
+  const CUtensorMap& lo = split.lo ? *split.lo : w16;
   if (fn) {
     // the plan must have been made with fwd_next (room for the input tile in every slot)
     if (w.xn_bytes == 0 || !fn->xn) return cudaErrorInvalidValue;
@@ -358,11 +366,11 @@ cudaError_t launch_wgrad_stream(mavg_ctx* c, const WgradPlan& w, const CUtensorM
   prof_begin(c, MAVG_K_WGRAD_SGD);
   cudaError_t e;
   if (fn)
-    e = with_u ? cudaLaunchKernelEx(&lc, k_wgrad_sgd_stream<true, true>, dzt, at, w32, w32_in, w16, um, *fn->xn, g)
-               : cudaLaunchKernelEx(&lc, k_wgrad_sgd_stream<false, true>, dzt, at, w32, w32_in, w16, um, *fn->xn, g);
+    e = with_u ? cudaLaunchKernelEx(&lc, k_wgrad_sgd_stream<true, true>, dzt, at, w32, w32_in, w16, um, *fn->xn, lo, g)
+               : cudaLaunchKernelEx(&lc, k_wgrad_sgd_stream<false, true>, dzt, at, w32, w32_in, w16, um, *fn->xn, lo, g);
   else
-    e = with_u ? cudaLaunchKernelEx(&lc, k_wgrad_sgd_stream<true, false>, dzt, at, w32, w32_in, w16, um, w16, g)
-               : cudaLaunchKernelEx(&lc, k_wgrad_sgd_stream<false, false>, dzt, at, w32, w32_in, w16, um, w16, g);
+    e = with_u ? cudaLaunchKernelEx(&lc, k_wgrad_sgd_stream<true, false>, dzt, at, w32, w32_in, w16, um, w16, lo, g)
+               : cudaLaunchKernelEx(&lc, k_wgrad_sgd_stream<false, false>, dzt, at, w32, w32_in, w16, um, w16, lo, g);
   prof_end(c);
   return e != cudaSuccess ? e : cudaGetLastError();
 }

@@ -7,7 +7,8 @@
 namespace mavg {
 
 struct WgradPlan {
-  int nkb, m_tiles, n_tiles, chunk, n_chunks, items, slots, a_bufs, grid, w16_on_b;
+  int nkb, m_tiles, n_tiles, chunk, n_chunks, items, slots, a_bufs, grid;
+  int b_room, w16_off;  // a slot's room for A^T and the bf16 tile, and where in it the latter lies
   int whole_rows; // (learner, row tile) pairs taken as one run of all column tiles (plans made with
                   // fwd_next: whole waves of such items first, the remaining rows cut into runs)
   int xn_bytes;   // room in every slot for the next step's input tile (plans made with fwd_next)
@@ -24,8 +25,10 @@ constexpr int kWgradTileCols = 32;    // columns of in per tile
 // fwd_next: the launch may also take the next step's forward product of this layer along (see
 // launch_wgrad_stream): every slot gets room for a [B, 32] tile of the next step's input and the
 // runs of column tiles get long.
+// split: plans for launches that leave their masters split (WgradSplit); with fwd_next only.
 WgradPlan plan_wgrad_stream(int out, int in, int B, int P, int sm_count, bool momentum = false,
-                            bool streaming = false, bool fwd_next = false);
+                            bool streaming = false, bool fwd_next = false,
+                            bool split = false);
 cudaError_t wgrad_stream_prepare();
 // dzt: bf16 [P, out, B] box 64 x 128 (128B swizzle); at: bf16 [P, in, B] box 64 x 32 (128B swizzle);
 // w32: fp32 [P, out, in] box 32 x 128 (128B swizzle); w16: bf16 [P, out, in] box 32 x 128
@@ -51,11 +54,21 @@ struct WgradFwdNext {
                            // copy nothing else reads before the next launch that writes it:
                            // layer 1, which has no dgrad product)
 };
+// Masters kept as two halves between the steps of a call (wgrad_tc.cu): in: the launch reads them
+// split (the upper halves from w16), out: it leaves them so; lo: the low halves, bf16-typed
+// [P, out, in] with w16's box.
+struct WgradSplit {
+  const CUtensorMap* lo = nullptr;
+  float* master = nullptr;   // the layer's fp32 masters (of learner 0) and their row length
+  int in_cols = 0;
+  bool in = false, out = false;
+};
 cudaError_t launch_wgrad_stream(mavg_ctx* c, const WgradPlan& w, const CUtensorMap& dzt,
                                 const CUtensorMap& at, const CUtensorMap& w32,
                                 const CUtensorMap& w16, const CUtensorMap* w32_shared = nullptr,
                                 const CUtensorMap* u32 = nullptr, const MomArgs& mom = MomArgs(),
-                                const WgradFwdNext* fn = nullptr);
+                                const WgradFwdNext* fn = nullptr,
+                                const WgradSplit& split = WgradSplit());
 
 // Several layers' weight-gradient + SGD tiles in one persistent launch (layers listed in the
 // order their tiles should run).  All plans must come from the same batch size and momentum

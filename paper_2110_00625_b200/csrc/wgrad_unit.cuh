@@ -12,9 +12,13 @@ namespace wgrad {
 using namespace tc;
 
 constexpr int kBM = 128, kBN = 32, kBK = 64;
-constexpr int kThreads = 352;      // warp 0 producer, 1 MMA, 2-5 / 6-9 epilogue groups, 10 stores
-constexpr int kThreadsFwd = 512;   // + warp 11 forward MMAs, 12-15 forward accumulator (fwd_next)
-constexpr int kMaxSlots = 6;
+// Warp 0 producer, 1 MMA, 2-9 and the last eight epilogue, 10 stores; fwd_next: 11 forward MMAs, 12-15
+// forward accumulator.  Two epilogue groups take the tiles in turn; a group is eight warps, one set of
+// four for each half of a tile's columns.
+constexpr int kThreads = 608;
+constexpr int kThreadsFwd = 768;
+constexpr int kHalf = kBN / 2;
+constexpr int kMaxSlots = 8;
 constexpr int kW32Bytes = kBM * kBN * 4;  // 16 KB, rows of 128 bytes, 128-byte swizzle
 constexpr int kW16Bytes = kBM * kBN * 2;  //  8 KB, rows of  64 bytes,  64-byte swizzle
 enum { ERR_WG_PRODUCER = 21, ERR_WG_MMA = 22, ERR_WG_EPILOGUE = 23, ERR_WG_STORE = 24 };
@@ -59,7 +63,8 @@ struct WgradArgs {
                            // a riding forward product's long runs over the blocks)
   int slots;               // ring depth
   int a_bufs;              // 1 or 2 buffers for the dZ^T tile
-  int w16_on_b;            // 1: the bf16 output tile is written over the slot's A^T slabs
+  int b_room, w16_off;     // a slot's room for the A^T slabs and the bf16 output tile; where in it the
+                           // tile lies (0: over the slabs, which the MMA has read by then)
   int keep_w32;            // 1: master tiles are loaded and stored with the L2 evict-last hint
                            //    (all learners' masters together fit in half the L2: they are
                            //    read again one step later and should not go through HBM)
@@ -88,9 +93,25 @@ struct WgradArgs {
   int out_rows;            // rows of the layer (the last row tile may be ragged)
   __nv_bfloat16* out_bm;
   __nv_bfloat16* out_mb;
+  // The master tile comes in / goes out as two 16-bit halves, see join_master (a layer whose bf16 copy
+  // is kept between the steps of a call: 8 bytes per weight and step instead of 10).
+  int in_split, out_split;
+  float* master;           // the layer's fp32 masters [P, rep_stride] of in_cols columns, for ties
+  int in_cols;
   int* status;
 };
 
+// fp32 <-> (hi, lo): hi is the bf16 copy, rounded to nearest even, lo the low half of the fp32 bits.
+// The upper half is hi, or hi - 1 where lo says that hi was rounded up (lo > 0x8000).  On a tie (lo ==
+// 0x8000, one value in 65536) lo does not tell: those values are kept in the fp32 array as well.
+__device__ __forceinline__ uint32_t join_master(uint32_t hi_lo) {  // hi in the upper, lo in the lower half
+  return hi_lo - 2u * (hi_lo & 0x8000u);
+}
+// Non-zero if one of two low halves is a tie (and perhaps if one is next to it).
+__device__ __forceinline__ uint32_t maybe_tie(uint32_t lo) {
+  const uint32_t t = lo ^ 0x80008000u;
+  return (t - 0x00010001u) & ~t & 0x80008000u;
+}
 
 struct WgradShared {
   uint64_t slot_full[kMaxSlots], slot_empty[kMaxSlots], out_full[kMaxSlots];
@@ -98,6 +119,7 @@ struct WgradShared {
   uint64_t a_full[2], a_empty[2];
   uint64_t z_done[kMaxSlots];   // the forward MMAs that read this slot's bf16 tile have finished
   uint64_t z_full, z_empty;     // the item's forward accumulator is complete / has been read
+  uint64_t reshape[2];          // the group's warps have read a tile whose layout changes on the way out
   uint64_t z_part, z_flag;      // the item's partial sum is in global memory / z_last is set
   int z_last;                   // this item completed its row tile's product last
   uint32_t tmem_slot;
@@ -108,7 +130,7 @@ __device__ __forceinline__ void wgrad_init_barriers(WgradShared& sh, int slots) 
   for (int s = 0; s < slots; ++s) {
     mbar_init(&sh.slot_full[s], 1);
     mbar_init(&sh.slot_empty[s], 1);
-    mbar_init(&sh.out_full[s], 4);
+    mbar_init(&sh.out_full[s], 8);
     mbar_init(&sh.z_done[s], 1);
   }
   mbar_init(&sh.z_full, 1);
@@ -117,9 +139,10 @@ __device__ __forceinline__ void wgrad_init_barriers(WgradShared& sh, int slots) 
   mbar_init(&sh.z_flag, 1);
   for (int b = 0; b < 2; ++b) {
     mbar_init(&sh.tmem_full[b], 1);
-    mbar_init(&sh.tmem_empty[b], 4);
+    mbar_init(&sh.tmem_empty[b], 8);
     mbar_init(&sh.a_full[b], 1);
     mbar_init(&sh.a_empty[b], 1);
+    mbar_init(&sh.reshape[b], 8);
   }
 }
 
@@ -139,12 +162,13 @@ __device__ __forceinline__ void wgrad_run_totals(const WgradArgs& g, int vblock,
 // A block that makes several runs keeps using the same barriers (g.slots and g.a_bufs must not
 // change): tile_base and item_base are the tiles and items of its earlier runs, see
 // wgrad_run_totals.
-// FWD = false compiles the roles of the riding forward product out (g.fwd_next must be 0).
-template <bool MOM, bool FWD>
+// FWD = false compiles the roles of the riding forward product out (g.fwd_next must be 0), SPLIT =
+// false the split masters (g.in_split and g.out_split must be 0).
+template <bool MOM, bool FWD, bool SPLIT>
 __device__ __forceinline__ void wgrad_run(const CUtensorMap& tm_dzt, const CUtensorMap& tm_at,
                                           const CUtensorMap& tm_w32, const CUtensorMap& tm_w32_in,
                                           const CUtensorMap& tm_w16, const CUtensorMap& tm_u,
-                                          const CUtensorMap& tm_xn,
+                                          const CUtensorMap& tm_xn, const CUtensorMap& tm_lo,
                                           const WgradArgs& g, int vblock, int vgrid, uint8_t* smem,
                                           WgradShared& sh, uint32_t tmem_base,
                                           uint32_t tile_base = 0, uint32_t item_base = 0) {
@@ -152,15 +176,17 @@ __device__ __forceinline__ void wgrad_run(const CUtensorMap& tm_dzt, const CUten
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int a_bytes = g.nkb * kBM * kBK * 2;         // dZ^T tile: nkb slabs of 16 KB
   const int b_bytes = g.nkb * kBN * kBK * 2;         // A^T tile:  nkb slabs of 4 KB
-  // Slot: [master tile 16 KB][u tile 16 KB (MOM)][bf16 tile 8 KB][A^T slabs], or, when the A^T
-  // slabs are at least as large as the bf16 tile (g.w16_on_b), without a region of its own for the
-  // bf16 tile: the MMA has finished reading A^T when the epilogue writes, so the bf16 tile goes
-  // on top of it and more slots fit.
+  // Slot: [master tile 16 KB][u tile 16 KB (MOM)][A^T slabs, bf16 tile][next step's input].  The
+  // MMA has finished reading A^T when the epilogue writes the bf16 tile.
+  // A split master takes the master tile's 16 KB as [hi 8 KB][lo 8 KB], each laid out like the bf16
+  // tile; with out_split hi is the bf16 tile and its own region stays unused.
   constexpr int kUBytes = MOM ? kW32Bytes : 0;
-  const int w16_off = kW32Bytes + kUBytes;
-  const int b_off = g.w16_on_b ? w16_off : w16_off + kW16Bytes;
-  const int xn_off = b_off + b_bytes;                       // next step's input tile (fwd_next)
+  const bool in_split = SPLIT && g.in_split != 0, out_split = SPLIT && g.out_split != 0;
+  const int b_off = kW32Bytes + kUBytes;
+  const int w16_off = b_off + g.w16_off;
+  const int xn_off = b_off + g.b_room;                      // next step's input tile (fwd_next)
   const int slot_bytes = xn_off + g.xn_bytes;               // multiple of 1024
+  constexpr int kFirstHalf1 = FWD ? 16 : 11;                // first warp of the second column half
   constexpr uint32_t kZCol = 2 * kBN;                       // forward accumulator: B columns from here
   uint8_t* a_base = smem;
   uint8_t* slot_base = smem + (size_t)g.a_bufs * a_bytes;
@@ -213,7 +239,12 @@ __device__ __forceinline__ void wgrad_run(const CUtensorMap& tm_dzt, const CUten
                                 (uint32_t)(kW32Bytes + b_bytes + (load_u ? kUBytes : 0) +
                                            (fwd_next ? g.xn_bytes : 0)));
           if (fwd_next) tma_load_3d(sl + xn_off, &tm_xn, &sh.slot_full[s], i0, 0, p);
-          tma_load_3d_hint(sl, &tm_w32_in, &sh.slot_full[s], i0, m0, g.w32_in_batched ? p : 0, pol);
+          if (in_split) {
+            tma_load_3d(sl, &tm_w16, &sh.slot_full[s], i0, m0, p);
+            tma_load_3d(sl + kW16Bytes, &tm_lo, &sh.slot_full[s], i0, m0, p);
+          } else {
+            tma_load_3d_hint(sl, &tm_w32_in, &sh.slot_full[s], i0, m0, g.w32_in_batched ? p : 0, pol);
+          }
           if (load_u) tma_load_3d(sl + kW32Bytes, &tm_u, &sh.slot_full[s], i0, m0, p);
           for (int kb = 0; kb < g.nkb; ++kb)
             tma_load_3d(sl + b_off + (size_t)kb * (kBN * kBK * 2),
@@ -260,8 +291,9 @@ __device__ __forceinline__ void wgrad_run(const CUtensorMap& tm_dzt, const CUten
       }
     }
     __syncwarp();
-  } else if (warp < 10) {
-    const int grp = (warp - 2) >> 2;           // epilogue group = TMEM buffer = tile parity
+  } else if (warp < 10 || warp >= kFirstHalf1) {
+    const int cols = warp < 10 ? 0 : kHalf;    // this warp's half of a tile's columns
+    const int grp = (warp - (warp < 10 ? 2 : kFirstHalf1)) >> 2;   // group = TMEM buffer = tile parity
     const int q = warp & 3;                    // TMEM lane quarter this warp may read
     const int r = q * 32 + lane;               // weight row inside the tile
     uint32_t tile_ctr = tile_base;
@@ -281,8 +313,8 @@ __device__ __forceinline__ void wgrad_run(const CUtensorMap& tm_dzt, const CUten
           break;
         }
         tc_fence_after_sync();
-        uint32_t acc[32];
-        tmem_ld_32x32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(grp * kBN), acc);
+        uint32_t acc[kHalf];
+        tmem_ld_16cols(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(grp * kBN + cols), acc);
         tmem_ld_wait();
         tc_fence_before_sync();
         __syncwarp();
@@ -291,14 +323,13 @@ __device__ __forceinline__ void wgrad_run(const CUtensorMap& tm_dzt, const CUten
         uint8_t* sl = slot_base + (size_t)s * slot_bytes;
         uint8_t* w32 = sl + (size_t)r * 128;             // 8 chunks of 16 B, chunk c at c ^ (r & 7)
         uint8_t* w16 = sl + w16_off + (size_t)r * 64;    // 4 chunks, chunk c at c ^ ((r >> 1) & 3)
-        uint32_t hp[16];
-#pragma unroll
-        for (int c = 0; c < 8; ++c) {
-          float4* cell = reinterpret_cast<float4*>(w32 + ((c ^ (r & 7)) << 4));
-          float4 w = *cell;
+        uint8_t* half = sl + (size_t)r * 64;             // hi, laid out like w16; lo 8 KB behind it
+        auto at32 = [&](int c) { return (((cols >> 2) + c) ^ (r & 7)) << 4; };          // columns 4 c ..
+        auto at16 = [&](int c) { return (((cols >> 3) + c) ^ ((r >> 1) & 3)) << 4; };   // columns 8 c ..
+        auto step4 = [&](float4& w, int c) {             // columns 4 c .. 4 c + 3 of this half row
           if (MOM) {
             // the u tile has the master tile's shape and swizzle
-            float4* ucell = reinterpret_cast<float4*>(w32 + kW32Bytes + ((c ^ (r & 7)) << 4));
+            float4* ucell = reinterpret_cast<float4*>(w32 + kW32Bytes + at32(c));
             float4 u = g.read_u ? *ucell : make_float4(0.f, 0.f, 0.f, 0.f);
             msgd(w.x, u.x, __uint_as_float(acc[4 * c + 0]), g.gamma, g.beta);
             msgd(w.y, u.y, __uint_as_float(acc[4 * c + 1]), g.gamma, g.beta);
@@ -311,16 +342,103 @@ __device__ __forceinline__ void wgrad_run(const CUtensorMap& tm_dzt, const CUten
             w.z = fmaf(-g.gamma, __uint_as_float(acc[4 * c + 2]), w.z);
             w.w = fmaf(-g.gamma, __uint_as_float(acc[4 * c + 3]), w.w);
           }
-          *cell = w;
-          __nv_bfloat162 h0 = __floats2bfloat162_rn(w.x, w.y);
-          __nv_bfloat162 h1 = __floats2bfloat162_rn(w.z, w.w);
-          hp[2 * c] = *reinterpret_cast<uint32_t*>(&h0);
-          hp[2 * c + 1] = *reinterpret_cast<uint32_t*>(&h1);
-        }
+        };
+        if (SPLIT && (in_split || out_split)) {
+          // The half row goes through registers.  hi and lo of it are this thread's own bytes, as its
+          // fp32 values are; where one becomes the other, bytes change hands, and nobody writes
+          // before the group's eight warps have read.
+          uint32_t wv[kHalf];
+          float* exact = g.master + (size_t)p * g.rep_stride + (size_t)(m0 + r) * g.in_cols + (nt0 + j) * kBN + cols;
+          if (in_split) {
+            uint32_t tie = 0u;
 #pragma unroll
-        for (int c = 0; c < 4; ++c)
-          *reinterpret_cast<uint4*>(w16 + ((c ^ ((r >> 1) & 3)) << 4)) =
-              make_uint4(hp[4 * c], hp[4 * c + 1], hp[4 * c + 2], hp[4 * c + 3]);
+            for (int c = 0; c < 2; ++c) {                // 8 columns
+              const uint4 h4 = *reinterpret_cast<const uint4*>(half + at16(c));
+              const uint4 l4 = *reinterpret_cast<const uint4*>(half + kW16Bytes + at16(c));
+              const uint32_t h[4] = {h4.x, h4.y, h4.z, h4.w}, lo[4] = {l4.x, l4.y, l4.z, l4.w};
+#pragma unroll
+              for (int k = 0; k < 4; ++k) {
+                wv[8 * c + 2 * k] = join_master(__byte_perm(lo[k], h[k], 0x5410));
+                wv[8 * c + 2 * k + 1] = join_master(__byte_perm(lo[k], h[k], 0x7632));
+                tie |= maybe_tie(lo[k]);
+              }
+            }
+            if (tie) {
+#pragma unroll
+              for (int k = 0; k < kHalf; ++k)
+                if ((wv[k] & 0xffffu) == 0x8000u) wv[k] = __float_as_uint(__ldcg(exact + k));
+            }
+          } else {
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+              const uint4 v = *reinterpret_cast<const uint4*>(w32 + at32(c));
+              wv[4 * c] = v.x; wv[4 * c + 1] = v.y; wv[4 * c + 2] = v.z; wv[4 * c + 3] = v.w;
+            }
+          }
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            float4 w = make_float4(__uint_as_float(wv[4 * c]), __uint_as_float(wv[4 * c + 1]),
+                                   __uint_as_float(wv[4 * c + 2]), __uint_as_float(wv[4 * c + 3]));
+            step4(w, c);
+            wv[4 * c + 0] = __float_as_uint(w.x);
+            wv[4 * c + 1] = __float_as_uint(w.y);
+            wv[4 * c + 2] = __float_as_uint(w.z);
+            wv[4 * c + 3] = __float_as_uint(w.w);
+          }
+          if (in_split != out_split) {
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&sh.reshape[grp]);
+            if (!mbar_wait(&sh.reshape[grp], tuse & 1, abortp, g.status, ERR_WG_EPILOGUE)) {
+              ok = false;
+              break;
+            }
+          }
+          uint32_t tie = 0u;
+#pragma unroll
+          for (int c = 0; c < 2; ++c) {                  // 8 columns
+            uint32_t v[4], lo[4];
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const uint32_t b0 = wv[8 * c + 2 * k], b1 = wv[8 * c + 2 * k + 1];
+              __nv_bfloat162 hh = __floats2bfloat162_rn(__uint_as_float(b0), __uint_as_float(b1));
+              v[k] = *reinterpret_cast<uint32_t*>(&hh);
+              lo[k] = __byte_perm(b0, b1, 0x5410);
+              tie |= maybe_tie(lo[k]);
+            }
+            *reinterpret_cast<uint4*>((out_split ? half : w16) + at16(c)) = make_uint4(v[0], v[1], v[2], v[3]);
+            if (out_split) {
+              *reinterpret_cast<uint4*>(half + kW16Bytes + at16(c)) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
+            } else {
+#pragma unroll
+              for (int k = 0; k < 2; ++k)
+                *reinterpret_cast<uint4*>(w32 + at32(2 * c + k)) =
+                    make_uint4(wv[8 * c + 4 * k], wv[8 * c + 4 * k + 1], wv[8 * c + 4 * k + 2],
+                               wv[8 * c + 4 * k + 3]);
+            }
+          }
+          if (out_split && tie) {
+#pragma unroll
+            for (int k = 0; k < kHalf; ++k)
+              if ((wv[k] & 0xffffu) == 0x8000u) exact[k] = __uint_as_float(wv[k]);
+          }
+        } else {
+          uint32_t hp[kHalf / 2];
+#pragma unroll
+          for (int c = 0; c < 4; ++c) {
+            float4* cell = reinterpret_cast<float4*>(w32 + at32(c));
+            float4 w = *cell;
+            step4(w, c);
+            *cell = w;
+            __nv_bfloat162 h0 = __floats2bfloat162_rn(w.x, w.y);
+            __nv_bfloat162 h1 = __floats2bfloat162_rn(w.z, w.w);
+            hp[2 * c] = *reinterpret_cast<uint32_t*>(&h0);
+            hp[2 * c + 1] = *reinterpret_cast<uint32_t*>(&h1);
+          }
+#pragma unroll
+          for (int c = 0; c < 2; ++c)
+            *reinterpret_cast<uint4*>(w16 + at16(c)) =
+                make_uint4(hp[4 * c], hp[4 * c + 1], hp[4 * c + 2], hp[4 * c + 3]);
+        }
         fence_proxy_async();                   // generic-proxy writes -> visible to the TMA stores
         __syncwarp();                          // (and to the forward MMAs, fwd_next)
         if (lane == 0) mbar_arrive(&sh.out_full[s]);
@@ -345,8 +463,13 @@ __device__ __forceinline__ void wgrad_run(const CUtensorMap& tm_dzt, const CUten
           }
           uint8_t* sl = slot_base + (size_t)s * slot_bytes;
           const int i0 = (nt0 + j) * kBN;
-          tma_store_3d_hint(&tm_w32, sl, i0, m0, p, pol);
-          if (g.store_w16) tma_store_3d(&tm_w16, sl + w16_off, i0, m0, p);
+          if (out_split) {
+            tma_store_3d(&tm_w16, sl, i0, m0, p);
+            tma_store_3d(&tm_lo, sl + kW16Bytes, i0, m0, p);
+          } else {
+            tma_store_3d_hint(&tm_w32, sl, i0, m0, p, pol);
+            if (g.store_w16) tma_store_3d(&tm_w16, sl + w16_off, i0, m0, p);
+          }
           if (MOM) tma_store_3d(&tm_u, sl + kW32Bytes, i0, m0, p);
           tma_store_commit();
           // A slot is free once its stores have read shared memory.  If the next tile is already
@@ -410,7 +533,7 @@ __device__ __forceinline__ void wgrad_run(const CUtensorMap& tm_dzt, const CUten
           }
           tc_fence_after_sync();
           const uint32_t base = smem_u32(slot_base + (size_t)s * slot_bytes);
-          const uint64_t adesc = smem_desc_k_sw64(base + w16_off);
+          const uint64_t adesc = smem_desc_k_sw64(base + (out_split ? 0 : w16_off));
           const uint64_t bdesc = smem_desc_k_sw64(base + xn_off);
 #pragma unroll
           for (int k = 0; k < kBN / 16; ++k)
@@ -424,7 +547,7 @@ __device__ __forceinline__ void wgrad_run(const CUtensorMap& tm_dzt, const CUten
     __syncwarp();
   } else if (fwd_next) {
     // warps 12-15: the forward accumulator of every work item.  One weight row per lane (warp w
-    // reads TMEM lanes 32 (w % 4) ...), 32 batch columns at a time.
+    // reads TMEM lanes 32 (w % 4) ...), 16 batch columns at a time.
     const int q = warp & 3;
     const int r = q * 32 + lane;
     const size_t tile_floats = (size_t)g.batch * kBM;
@@ -438,48 +561,37 @@ __device__ __forceinline__ void wgrad_run(const CUtensorMap& tm_dzt, const CUten
       const int m = m0 + r;
       const bool row_ok = m < g.out_rows;
       const float bias = row_ok ? g.bias_rep[(size_t)p * g.rep_stride + g.bias_off + m] : 0.f;
-      // A_l of the next step from 32 (or the last 16) finished columns of this lane's row
+      // A_l of the next step from 16 finished columns of this lane's row
       auto emit = [&](int c0, const float* z) {
         if (!row_ok) return;
-        const int nc = min(32, g.batch - c0);
-        uint32_t h[16];
+        uint32_t h[8];
 #pragma unroll
-        for (int jj = 0; jj < 16; ++jj) {
+        for (int jj = 0; jj < 8; ++jj) {
           const float a0 = z[2 * jj] + bias, a1 = z[2 * jj + 1] + bias;
           __nv_bfloat162 h2 = __floats2bfloat162_rn(a0 > 0.f ? a0 : 0.f, a1 > 0.f ? a1 : 0.f);
           h[jj] = *reinterpret_cast<uint32_t*>(&h2);
         }
         uint4* dmb = reinterpret_cast<uint4*>(g.out_mb + ((size_t)p * g.out_rows + m) * g.batch + c0);
-#pragma unroll
-        for (int v = 0; v < 4; ++v)
-          if (8 * v < nc) dmb[v] = make_uint4(h[4 * v], h[4 * v + 1], h[4 * v + 2], h[4 * v + 3]);
+        dmb[0] = make_uint4(h[0], h[1], h[2], h[3]);
+        dmb[1] = make_uint4(h[4], h[5], h[6], h[7]);
         const __nv_bfloat16* hh = reinterpret_cast<const __nv_bfloat16*>(h);
         __nv_bfloat16* dbm = g.out_bm + ((size_t)p * g.batch + c0) * g.out_rows + m;
 #pragma unroll
-        for (int jj = 0; jj < 32; ++jj)
-          if (jj < nc) dbm[(size_t)jj * g.out_rows] = hh[jj];
+        for (int jj = 0; jj < 16; ++jj) dbm[(size_t)jj * g.out_rows] = hh[jj];
       };
       if (!mbar_wait_relaxed(&sh.z_full, item_ctr & 1, abortp, g.status, ERR_WG_EPILOGUE, 400)) break;
       tc_fence_after_sync();
       float* zbase = g.zpart + ((size_t)p * g.m_tiles + mt) * g.n_chunks * tile_floats + r;
       float* zp = zbase + (size_t)(nt0 / g.chunk) * tile_floats;
-      for (int c0 = 0; c0 < g.batch; c0 += 32) {
-        uint32_t acc[32];
-        if (c0 + 32 <= g.batch) {
-          tmem_ld_32x32(tmem_base + ((uint32_t)(q * 32) << 16) + kZCol + (uint32_t)c0, acc);
-        } else {                             // the batch is a multiple of 16
-          uint32_t h16[16];
-          tmem_ld_16cols(tmem_base + ((uint32_t)(q * 32) << 16) + kZCol + (uint32_t)c0, h16);
-#pragma unroll
-          for (int jj = 0; jj < 16; ++jj) { acc[jj] = h16[jj]; acc[16 + jj] = 0u; }
-        }
+      for (int c0 = 0; c0 < g.batch; c0 += 16) {     // the batch is a multiple of 16
+        uint32_t acc[16];
+        tmem_ld_16cols(tmem_base + ((uint32_t)(q * 32) << 16) + kZCol + (uint32_t)c0, acc);
         tmem_ld_wait();
         if (single) {
           emit(c0, reinterpret_cast<const float*>(acc));
         } else {
 #pragma unroll
-          for (int jj = 0; jj < 32; ++jj)
-            if (c0 + jj < g.batch) zp[(size_t)(c0 + jj) * kBM] = __uint_as_float(acc[jj]);
+          for (int jj = 0; jj < 16; ++jj) zp[(size_t)(c0 + jj) * kBM] = __uint_as_float(acc[jj]);
         }
       }
       tc_fence_before_sync();
@@ -507,23 +619,22 @@ __device__ __forceinline__ void wgrad_run(const CUtensorMap& tm_dzt, const CUten
       if (!mbar_wait(&sh.z_flag, split_ctr & 1, abortp, g.status, ERR_WG_EPILOGUE)) break;
       ++split_ctr;
       if (!sh.z_last) continue;
-      for (int c0 = 0; c0 < g.batch; c0 += 32) {
-        float z[32];
+      for (int c0 = 0; c0 < g.batch; c0 += 16) {
+        float z[16];
 #pragma unroll
-        for (int jj = 0; jj < 32; ++jj) z[jj] = 0.f;
+        for (int jj = 0; jj < 16; ++jj) z[jj] = 0.f;
         // two runs' loads in flight at a time; the sums are formed in ascending run order
         for (int nc = 0; nc < g.n_chunks; nc += 2) {
           const float* s0 = zbase + (size_t)nc * tile_floats + (size_t)c0 * kBM;
           const bool two = nc + 1 < g.n_chunks;
-          float a[32], b[32];
+          float a[16], b[16];
 #pragma unroll
-          for (int jj = 0; jj < 32; ++jj) {
-            const bool in = c0 + jj < g.batch;
-            a[jj] = in ? __ldcg(s0 + (size_t)jj * kBM) : 0.f;
-            b[jj] = in && two ? __ldcg(s0 + tile_floats + (size_t)jj * kBM) : 0.f;
+          for (int jj = 0; jj < 16; ++jj) {
+            a[jj] = __ldcg(s0 + (size_t)jj * kBM);
+            b[jj] = two ? __ldcg(s0 + tile_floats + (size_t)jj * kBM) : 0.f;
           }
 #pragma unroll
-          for (int jj = 0; jj < 32; ++jj) {
+          for (int jj = 0; jj < 16; ++jj) {
             z[jj] += a[jj];
             if (two) z[jj] += b[jj];
           }

@@ -1,0 +1,91 @@
+"""Masters kept as two 16-bit halves between the steps of a call (layers whose forward product rides on
+the weight-gradient launch and whose bf16 copy the data gradient reads): nothing of the fp32 value is
+lost, and the round is the one that keeps fp32 masters."""
+import numpy as np
+import pytest
+
+from tests.util import l2_rel
+
+pytestmark = pytest.mark.gpu
+P, B = 13, 32
+
+
+def _handle(dims, K, lr, w1=None, schedule=0, **kw):
+    import paper_2110_00625_b200 as m
+    rng = np.random.default_rng(7)
+    x = rng.standard_normal((1024, dims[0]), dtype=np.float32)
+    y = rng.integers(0, dims[-1], size=1024).astype(np.int32)
+    w1 = m.workloads.mlp_init(dims) if w1 is None else w1
+    g = m.Mavg(w1, P=P, K=K, local_lr=lr, mu=0.9, B=B, seed=3, objective=m.OBJ_MLP, dims=dims,
+               gemm_bf16=1, x=x, y=y, x_bf16=True, defer_broadcast=True, **kw)
+    g.set_schedule(schedule)
+    assert g.get_step_plan()["fwd_with_wgrad"] == len(dims) - 2
+    return g
+
+
+# whole tiles; ragged rows and columns in every layer, runs that end in a partial tile
+SHAPES = [[3072, 1024, 512, 10], [3048, 1000, 504, 264, 10]]
+
+
+@pytest.mark.parametrize("dims", SHAPES)
+@pytest.mark.parametrize("K", [1, 2, 5])
+@pytest.mark.parametrize("beta", [0.0, 0.9])
+def test_a_step_of_length_zero_keeps_every_bit(dims, K, beta):
+    # local_lr = 0: w <- w + (-0) g leaves every value as it is, whatever steps it goes through;
+    # values on and beside the ties of the bf16 rounding, subnormal ones and the largest below 1
+    import paper_2110_00625_b200 as m
+    w1 = m.workloads.mlp_init(dims)
+    bits = w1.view(np.uint32).copy()
+    rng = np.random.default_rng(1)
+    at = rng.permutation(bits.size)[:bits.size // 4]
+    low = np.array([0x8000, 0x7fff, 0x8001, 0xffff, 0, 1], dtype=np.uint32)
+    bits[at] = (bits[at] & np.uint32(0xffff0000)) | low[rng.integers(0, 6, at.size)]
+    bits[at[:64]] = np.uint32(0x00008000)
+    bits[at[64:128]] = np.uint32(0x3f7fffff)
+    bits[at[128:192]] = np.uint32(0x00000001)
+    # zeros of either sign become +0: keep them out
+    w1 = np.where(bits << 1 == 0, np.uint32(0x3c000000), bits).view(np.float32)
+    g = _handle(dims, K, 0.0, w1=w1, learner_momentum=beta)
+    g.local_steps()
+    g.sync()
+    rep = g.replicas[:, :g.n].cpu().numpy().view(np.uint32)
+    for j in range(P):
+        assert np.array_equal(rep[j], w1.view(np.uint32))
+    g.close()
+
+
+@pytest.mark.parametrize("dims", SHAPES)
+def test_same_round_as_with_fp32_masters(dims):
+    # the plain schedule keeps fp32 masters throughout; the two differ in summation orders: per-round
+    # drift bound of the bf16 path (5e-2), here three steps
+    a, b = _handle(dims, 3, 0.002), _handle(dims, 3, 0.002, schedule=2)
+    for _ in range(2):
+        la, lb = a.round(want_loss=True), b.round(want_loss=True)
+        assert abs(la - lb) <= 2e-2 * abs(lb)
+    a.local_steps(); a.local_steps()          # the second call starts from fp32 replicas
+    b.local_steps(); b.local_steps()
+    a.sync(); b.sync()
+    assert l2_rel(a.v.cpu().numpy(), b.v.cpu().numpy()) <= 5e-2
+    n = a.n
+    ra, rb = a.replicas[:, :n].cpu().numpy(), b.replicas[:, :n].cpu().numpy()
+    w = a.w.cpu().numpy()
+    for j in (0, P - 1):
+        assert l2_rel(ra[j] - w, rb[j] - w) <= 5e-2
+    a.close(); b.close()
+
+
+def test_a_weight_that_is_not_a_number_stays_one():
+    # and spreads exactly as far as it does with fp32 masters
+    import paper_2110_00625_b200 as m
+    dims = SHAPES[0]
+    w1 = m.workloads.mlp_init(dims)
+    at = dims[0] * dims[1] + dims[1] + 5 * dims[1] + 7          # in W_2
+    w1[at] = np.nan
+    nans = []
+    for schedule in (0, 2):
+        g = _handle(dims, 3, 0.002, w1=w1, schedule=schedule)
+        g.round()
+        g.sync()
+        nans.append(np.isnan(g.w.cpu().numpy()))
+        g.close()
+    assert nans[0][at] and np.array_equal(nans[0], nans[1])
