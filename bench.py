@@ -236,7 +236,7 @@ NCU_TRAFFIC = {
 
 
 def algorithmic_bytes(cfg, tensor_path, deferred=False, momentum=False, fwd_run_tiles=(),
-                      dense_layers=(), fwd_whole_rows=()):
+                      dense_layers=(), fwd_whole_rows=(), split_layers=()):
     """Bytes that must cross HBM per ROUND for each kernel class (weights streamed once per
     product, activations in and out), and their total.  fwd_run_tiles[l-1], layers l = 1..m: in
     steps 1..K-1 the weight-gradient launch of layer l also forms the next step's forward product
@@ -246,7 +246,9 @@ def algorithmic_bytes(cfg, tensor_path, deferred=False, momentum=False, fwd_run_
     per learner, row tile and run of fwd_run_tiles[l-1] column tiles (not for the fwd_whole_rows[l-1]
     (learner, row tile) pairs that are taken as one run); the flops move with them.
     dense_layers: hidden layers whose first-step forward is one dense product over all learners'
-    batch rows, reading the (shared) weights once instead of once per learner."""
+    batch rows, reading the (shared) weights once instead of once per learner.
+    split_layers: layers whose masters are the bf16 copy and an array of low halves between the steps
+    of a round: in steps 1..K-1 the copy is part of the master and not written on top of it."""
     dims, P, K, B = cfg["dims"], cfg["P"], cfg["K"], cfg["B"]
     L = len(dims) - 1
     nW = [dims[l] * dims[l + 1] for l in range(L)]
@@ -255,6 +257,8 @@ def algorithmic_bytes(cfg, tensor_path, deferred=False, momentum=False, fwd_run_
     fwd_delta = wgrad_delta = flop_delta = 0
     for l in dense_layers:
         fwd_delta -= 2 * (P - 1) * nW[l - 1]
+    for l in split_layers:
+        wgrad_delta -= (K - 1) * 2 * P * nW[l - 1]
     for i, run in enumerate(fwd_run_tiles if K > 1 else ()):
         n_tiles = -(-dims[i] // 32)
         runs = -(-n_tiles // run)
@@ -287,10 +291,10 @@ def algorithmic_bytes(cfg, tensor_path, deferred=False, momentum=False, fwd_run_
 
 
 def kernel_rooflines(cfg, prof, steps, peaks, tensor_path, deferred=False, momentum=False,
-                     fwd_run_tiles=(), dense_layers=(), fwd_whole_rows=()):
+                     fwd_run_tiles=(), dense_layers=(), fwd_whole_rows=(), split_layers=()):
     """Per kernel class: algorithmic bytes or flops of all its launches / its summed device time."""
     per_round = algorithmic_bytes(cfg, tensor_path, deferred, momentum, fwd_run_tiles, dense_layers,
-                                  fwd_whole_rows)
+                                  fwd_whole_rows, split_layers)
     out = {}
     for name, (ms, cnt) in prof.items():
         if cnt == 0 or ms <= 0:
@@ -370,7 +374,8 @@ def whole_job_value(units_per_step, steps, total_ms, world):
 
 def pseudograd_rounds(args, m, torch, peaks, Ks, steps):
     """Full round at the ResNet-50-sized vector (n = 25.6 M, P = 16) with seeded pseudo-gradients:
-    per K the local pass, the meta-update and the whole round."""
+    per K the local pass and the meta-update called one after the other, and the whole round as one
+    call, which takes both in one launch."""
     from paper_2110_00625_b200 import workloads as W
     cfg = W.CONFIGS["C5"]
     n, P = args.n or cfg["n"], cfg["P"]
@@ -386,7 +391,11 @@ def pseudograd_rounds(args, m, torch, peaks, Ks, steps):
         ev = [[torch.cuda.Event(enable_timing=True) for _ in range(3)] for _ in range(steps)]
         for a, b, c in ev:
             a.record(); g.local_steps(); b.record(); g.meta_update(); c.record()
+        rv = [[torch.cuda.Event(enable_timing=True) for _ in range(2)] for _ in range(steps)]
+        for a, b in rv:
+            a.record(); g.round(); b.record()
         torch.cuda.synchronize()
+        rnd = statistics.median(a.elapsed_time(b) for a, b in rv)
         loc = statistics.median(a.elapsed_time(b) for a, b, c in ev)
         met = statistics.median(b.elapsed_time(c) for a, b, c in ev)
         # the local pass reads w~ once (every learner starts from it) and writes P learner models;
@@ -394,8 +403,12 @@ def pseudograd_rounds(args, m, torch, peaks, Ks, steps):
         meta_b = ((8 if args.no_defer else 4) * P + 16) * n
         local_b = ((12 if args.beta else 4) * P + 4) * n
         var_rate = P * K * n / (loc * 1e-3)
-        out.append(dict(K=K, local_ms=loc, meta_ms=met, round_ms=loc + met,
-                        learner_steps_per_s=P * K / ((loc + met) * 1e-3),
+        # the one launch reads w~ and v and writes them and the P learner models (or copies of w~)
+        round_b = ((12 if args.beta else 4) * P + 16) * n
+        out.append(dict(K=K, local_ms=loc, meta_ms=met, round_ms=rnd,
+                        learner_steps_per_s=P * K / (rnd * 1e-3),
+                        round_gbs=round_b / rnd / 1e6,
+                        round_frac_hbm=round_b / rnd / 1e6 / peaks["hbm_gbs"],
                         local_gbs=local_b / loc / 1e6,
                         local_frac_hbm=local_b / loc / 1e6 / peaks["hbm_gbs"],
                         learner_momentum=args.beta,
@@ -524,9 +537,12 @@ def measure_mlp(name, args, m, torch, dist, peaks, world, rank, local, steps, wi
     fwd_run_tiles = tuple(plan["fwd_run_tiles"]) if args.schedule == 0 else ()
     dense_layers = tuple(plan["dense_first_step"]) if args.schedule == 0 else ()
     fwd_whole_rows = tuple(plan["fwd_whole_rows"]) if args.schedule == 0 else ()
+    # every riding layer but the first keeps its masters split within a round
+    split_layers = tuple(range(2, len(fwd_run_tiles) + 1))
     kern = kernel_rooflines(cfg, prof, psteps, peaks, mode == 1, deferred=not args.no_defer,
                             momentum=args.beta != 0.0, fwd_run_tiles=fwd_run_tiles,
-                            dense_layers=dense_layers, fwd_whole_rows=fwd_whole_rows)
+                            dense_layers=dense_layers, fwd_whole_rows=fwd_whole_rows,
+                            split_layers=split_layers)
     n = g.n
     g.close()
     del g, flush
@@ -560,7 +576,8 @@ def measure_mlp(name, args, m, torch, dist, peaks, world, rank, local, steps, wi
     # the whole round against the HBM roofline: every class's algorithmic bytes / the round's time
     per_round = algorithmic_bytes(cfg, mode == 1, deferred=not args.no_defer,
                                   momentum=args.beta != 0.0, fwd_run_tiles=fwd_run_tiles,
-                                  dense_layers=dense_layers, fwd_whole_rows=fwd_whole_rows)
+                                  dense_layers=dense_layers, fwd_whole_rows=fwd_whole_rows,
+                                  split_layers=split_layers)
     round_bytes = sum(v["bytes"] for v in per_round.values())
     ms_round = total_ms / steps
     return dict(

@@ -51,3 +51,13 @@ def test_riding_and_dense_forward_only_move_work_between_classes_and_remove_byte
     whole = b.algorithmic_bytes(CFG, tensor_path=True, fwd_run_tiles=(96, 64, 64),
                                 dense_layers=(1, 2, 3), fwd_whole_rows=(512, 512, 512))
     assert tot_b(plain) - tot_b(whole) == saved
+
+
+def test_split_masters_remove_the_copy_on_top_of_the_master():
+    b = _bench()
+    kw = dict(tensor_path=True, fwd_run_tiles=(48, 32, 32), dense_layers=(1, 2, 3),
+              fwd_whole_rows=(444, 444, 444))
+    fp32, split = b.algorithmic_bytes(CFG, **kw), b.algorithmic_bytes(CFG, split_layers=(2, 3), **kw)
+    saved = 15 * 32 * 2 * 2 * 2048 * 2048         # K - 1 steps, P learners, 2 bytes, two layers
+    assert fp32["wgrad_sgd_gemm"]["bytes"] - split["wgrad_sgd_gemm"]["bytes"] == saved
+    assert all(fp32[k] == split[k] for k in fp32 if k != "wgrad_sgd_gemm")
