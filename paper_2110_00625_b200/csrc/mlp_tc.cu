@@ -586,8 +586,8 @@ mavg_status tc_setup(mavg_ctx* c) {
   if (e == cudaSuccess && st->tail_ok) e = tail_fused_prepare();
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&st->s_wgrad, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&st->s_gather, cudaStreamNonBlocking);
-  cudaEvent_t* evs[] = {&st->ev_fork, &st->ev_wgrad_done, &st->ev_gather_done, &st->ev_x_free[0],
-                        &st->ev_x_free[1]};
+  cudaEvent_t* evs[] = {&st->ev_fork, &st->ev_wgrad_done, &st->ev_gather_done, &st->ev_tail_done,
+                        &st->ev_x_free[0], &st->ev_x_free[1]};
   for (cudaEvent_t* ev : evs)
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
   if (e == cudaSuccess)
@@ -607,8 +607,8 @@ void tc_teardown(mavg_ctx* c) {
   if (st) {
     if (st->s_wgrad) cudaStreamDestroy(st->s_wgrad);
     if (st->s_gather) cudaStreamDestroy(st->s_gather);
-    cudaEvent_t evs[] = {st->ev_fork, st->ev_wgrad_done, st->ev_gather_done, st->ev_x_free[0],
-                         st->ev_x_free[1]};
+    cudaEvent_t evs[] = {st->ev_fork, st->ev_wgrad_done, st->ev_gather_done, st->ev_tail_done,
+                         st->ev_x_free[0], st->ev_x_free[1]};
     for (cudaEvent_t ev : evs)
       if (ev) cudaEventDestroy(ev);
   }
@@ -816,6 +816,7 @@ cudaError_t tc_step(mavg_ctx* c, int64_t round, int step) {
         TC_TRY(launch_tail_finish(c, tl));
         c->stream = main_s;
         tail_on_side = true;
+        TC_TRY(cudaEventRecord(st->ev_tail_done, st->s_wgrad));
       } else {
         TC_TRY(launch_tail_finish(c, tl));
       }
@@ -891,6 +892,8 @@ cudaError_t tc_step(mavg_ctx* c, int64_t round, int step) {
         st->gathered_step = step + 1;
       }
     }
+    // the riding product adds the bias that the fused last layer steps on the side stream
+    if (l == L - 1 && tail_on_side) TC_TRY(cudaStreamWaitEvent(main_s, st->ev_tail_done, 0));
     const CUtensorMap& bm = l == 1 ? st->x_in_t[xb] : act_in_t(l);
     WgradFwdNext fn{};
     fn.xn = &st->a_next[l][nb];

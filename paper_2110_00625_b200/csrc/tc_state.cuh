@@ -104,6 +104,7 @@ struct TcState {
   // side streams and events for the branches of a step that may overlap
   cudaStream_t s_wgrad = nullptr, s_gather = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_wgrad_done = nullptr, ev_gather_done = nullptr,
+              ev_tail_done = nullptr,
               ev_x_free[2] = {nullptr, nullptr};
 };
 
