@@ -518,9 +518,6 @@ mavg_status tc_setup(mavg_ctx* c) {
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
   if (e == cudaSuccess) e = wgrad_stream_prepare();
-  // The fused CUDA-core last layer pays where the tensor-core products of that layer would leave
-  // most of the GPU idle (few learners, narrow layer below); with many tiles the tensor-core
-  // kernels are the faster ones.
   // Small problems (a few dozen weight tiles per SM in the largest layer): one persistent launch
   // takes the weight gradients of all layers, instead of one launch per layer on a side stream.
   {
@@ -581,8 +578,21 @@ mavg_status tc_setup(mavg_ctx* c) {
     c->shadow.total[l - 1] = (int64_t)c->layers[l - 1].in * c->layers[l - 1].out;
     c->shadow.sh_off[l - 1] = t.sh_off[l - 1];
   }
-  st->tail_ok = tail_fused_supported(&cfg) &&
-                P * ((cfg.dims[L - 1] + kBM - 1) / kBM) <= c->sm_count / 2;
+  // The fused CUDA-core last layer pays where the tensor-core products of that layer would leave most of
+  // the GPU idle (at most half a wave of tiles), and again where they take a wave or more of tiles that
+  // have little to do each: from three quarters of a wave on for layers of at most 16 K weights, at any
+  // number for at most 4 K, as long as the batch rows times the weights stay within 64 M.  Measured, us a round of 4 steps, fused / tensor tiles: 3072-512-512-10, B = 64:
+  // P = 48 923 / 978, P = 24 (96 tiles) 721 / 712; 1024-256-10, B = 32: P = 48 (96 tiles) 238 / 300;
+  // 600-800-800-16, B = 128: P = 24 555 / 628; 2048-768-32 (24 K weights), B = 128: P = 48 966 / 934;
+  // 512-128-24, B = 256: P = 100 (78 M) 471 / 424.
+  {
+    const long tiles = (long)P * ((cfg.dims[L - 1] + kBM - 1) / kBM);
+    const long weights = (long)cfg.dims[L - 1] * cfg.dims[L];
+    st->tail_ok = tail_fused_supported(&cfg) &&
+                  (2 * tiles <= c->sm_count ||
+                   ((weights <= 4096 || (4 * tiles >= 3 * c->sm_count && weights <= 16 * 1024)) &&
+                    (int64_t)P * B * weights <= 64 * 1024 * 1024));
+  }
   if (e == cudaSuccess && st->tail_ok) e = tail_fused_prepare();
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&st->s_wgrad, cudaStreamNonBlocking);
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&st->s_gather, cudaStreamNonBlocking);

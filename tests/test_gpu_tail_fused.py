@@ -42,6 +42,9 @@ SHAPES = [
     dict(dims=[512, 10], P=3, K=1, B=32),                  # one layer: no data gradient to take
     dict(dims=[256, 136, 32], P=5, K=1, B=16),             # 32 classes, one block per learner
     dict(dims=[3072, 2048, 10], P=2, K=1, B=48),           # wide last layer, ragged batch tiles
+    dict(dims=[256, 136, 10], P=40, K=1, B=32),            # few weights, more than half a wave of tiles
+    dict(dims=[256, 416, 10], P=28, K=1, B=32),            # just past three quarters of a wave of tiles
+    dict(dims=[128, 512, 32], P=30, K=1, B=16),            # the most weights that many tiles may have
 ]
 
 
