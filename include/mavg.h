@@ -101,7 +101,12 @@ typedef struct {
                         every w^j and writes each learner's own result, which is the same
                         assignment with 4P bytes per element less traffic.  Between a meta-update
                         and the next local step the replica array then holds the previous round's
-                        learner models; mavg_materialize_replicas writes the copies on request. */
+                        learner models; mavg_materialize_replicas writes the copies on request.
+                        What a program writes into the replica rows between two rounds: an MLP handle
+                        on the CUDA cores (gemm_bf16 0 or 2) starts its learners from the rows
+                        wherever they hold the copies (always with 0, after
+                        mavg_materialize_replicas with 1); a tensor-core or pseudo-gradient handle
+                        starts them from w~. */
   /* Learner-level momentum (the variant the paper names after Eq. 2 and in its conclusion:
    * momentum SGD inside each learner, under the block momentum of the meta level).  With
    * beta = learner_momentum != 0 the local step of Algorithm 1 becomes, in the form Eq. 2 uses,

@@ -137,7 +137,11 @@ cudaError_t mlp_local_steps(mavg_ctx* c, int64_t round) {
   // start elsewhere (local steps called twice in a row), profiled rounds and handles whose
   // capture failed once take the launch-by-launch path.
   if (!c->profiling && c->small_splits) return small_local_steps(c, round);
-  const bool want_graph = !c->profiling && !c->graph_disabled && c->replicas_equal_global;
+  // The graph of a CUDA-core handle reads w~ with defer_broadcast and the replica array without; a
+  // deferred round whose copies were written on request starts from them, outside the graph.
+  const bool usual_start = c->replicas_equal_global &&
+                           (use_tensor_cores(&c->cfg) || c->replicas_materialized == !c->cfg.defer_broadcast);
+  const bool want_graph = !c->profiling && !c->graph_disabled && usual_start;
   if (!want_graph) return run_steps(c, round);
   if (!c->graph_exec || c->graph_K != c->cfg.K || c->graph_lr != c->cfg.local_lr ||
       c->graph_beta != c->cfg.learner_momentum || c->graph_reset != c->cfg.learner_momentum_reset ||

@@ -18,6 +18,13 @@ __device__ __forceinline__ int32_t sample_index(uint64_t seed, int64_t round, in
   return (int32_t)(lo + (int64_t)((u * (uint64_t)(hi - lo)) >> 32));
 }
 
+// Where the CUDA-core paths find the learners' models at the start of a round: in w~ while a deferred
+// re-broadcast has not been carried out, in the replica array otherwise (whose rows a program may have
+// edited since they were written).
+inline bool starts_from_global(const mavg_ctx* c) {
+  return c->replicas_equal_global && !c->replicas_materialized;
+}
+
 // batch.cu
 cudaError_t launch_batch_indices(mavg_ctx* c, int64_t round, int step, int j, int32_t* idx);
 cudaError_t launch_sample_gather(mavg_ctx* c, int64_t round, int step, int32_t* idx,

@@ -7,9 +7,9 @@
 // path for true fp32 models and for layer widths the tensor-core path does not cover.
 // A step is L-1 forward launches, one for the whole last layer up to its data gradient (which
 // also gathers the next step's minibatch), L-2 data gradients and one for the weight gradients,
-// bias gradients and SGD steps of all layers.  At the first step of a round the weights are read
-// from w~ and the results written to the replicas, so the P copies of a deferred re-broadcast are
-// never needed.
+// bias gradients and SGD steps of all layers.  While a deferred re-broadcast is outstanding the first
+// step of a round reads the weights from w~ and writes the results to the replicas, so its P copies
+// are never needed.
 #include <algorithm>
 
 #include "mlp.cuh"
@@ -640,11 +640,11 @@ cudaError_t step_impl(mavg_ctx* c, int64_t round, int step) {
   if (step == 1 &&
       (e = launch(c, MAVG_K_BATCH, k_simt_gather<QUANT>, dim3((unsigned)(P * B)), 256, 1, 0, ga)) != cudaSuccess)
     return e;
-  // the weights before this step: w~ itself at the first one
+  // the weights before this step
   float* rep = c->buf.replicas;
   const int64_t rs = c->buf.replica_stride;
-  const float* win = c->replicas_equal_global ? c->buf.global_w : rep;
-  const int64_t ws = c->replicas_equal_global ? 0 : rs;
+  const float* win = starts_from_global(c) ? c->buf.global_w : rep;
+  const int64_t ws = starts_from_global(c) ? 0 : rs;
   const MomArgs mom = mom_args(c, c->replicas_equal_global);
   auto a_in = [&](int l) { return l == 1 ? sb.xg[cur] : sb.a[l - 1]; };
   const MlpLayer& top = c->layers[L - 1];

@@ -436,15 +436,14 @@ cudaError_t small_local_steps(mavg_ctx* c, int64_t round) {
     g.w_off[l] = (int)c->layers[l - 1].w_off;
     g.b_off[l] = (int)c->layers[l - 1].b_off;
   }
-  const bool from_global = c->replicas_equal_global;
-  g.src = from_global ? c->buf.global_w : c->buf.replicas;
-  g.src_stride = from_global ? 0 : c->buf.replica_stride;
+  g.src = starts_from_global(c) ? c->buf.global_w : c->buf.replicas;
+  g.src_stride = starts_from_global(c) ? 0 : c->buf.replica_stride;
   g.rep = c->buf.replicas; g.rep_stride = c->buf.replica_stride;
   g.x = cfg.x; g.x_bf16 = cfg.x_dtype == MAVG_X_BF16;
   g.y = cfg.y; g.S = cfg.n_samples;
   g.seed = cfg.seed; g.round = round;
   g.gamma = cfg.local_lr;
-  g.mom = mom_args(c, from_global);
+  g.mom = mom_args(c, c->replicas_equal_global);
   g.losses = (float*)ws_ptr(c, c->ws.losses);
   cudaLaunchAttribute at[2];
   const cudaLaunchConfig_t lc = launch_config(c, g.splits, at);

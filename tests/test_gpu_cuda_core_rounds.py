@@ -1,0 +1,67 @@
+"""Whole rounds on the CUDA cores, both forms of the learner level (all steps in one launch, and a launch
+per product replayed from a graph), against the oracle: where the learners start from."""
+import numpy as np
+import pytest
+import torch
+
+from tests.util import l2_rel
+
+pytestmark = pytest.mark.gpu
+
+# small: at most 4096 parameters, all K steps are one launch; large: a graph of launches per product
+SMALL, LARGE = [64, 48, 10], [300, 200, 10]
+
+
+def _pair(oracle, mode, dims, P=3, K=3, B=16, beta=0.0, **kw):
+    import paper_2110_00625_b200 as m
+    rng = np.random.default_rng(17)
+    x = rng.standard_normal((1000, dims[0]), dtype=np.float32)
+    y = rng.integers(0, dims[-1], size=1000).astype(np.int32)
+    w1 = m.workloads.mlp_init(dims)
+    common = dict(P=P, K=K, mu=0.9, B=B, seed=5, dims=dims, x=x, y=y)
+    g = m.Mavg(w1, local_lr=0.01, objective=m.OBJ_MLP, gemm_bf16=mode, learner_momentum=beta, **common, **kw)
+    o = oracle.Mavg(w1, gamma=0.01, objective=oracle.OBJ_MLP, bf16=mode != 0, beta=beta, stride=g.stride,
+                    **common)
+    return g, o
+
+
+def _tol(mode):
+    # a few steps of fp32 sums in another order / of bf16 operands that round to the other neighbour:
+    # the drift of the weights themselves stays a tenth of the 2e-5 / 2e-2 a step's gradient may have
+    return 2e-6 if mode == 0 else 2e-3
+
+
+def _steps_launches(g):
+    before = g.launch_count()
+    g.local_steps()
+    return g.launch_count() - before
+
+
+@pytest.mark.parametrize("defer", [False, True])
+@pytest.mark.parametrize("dims", [SMALL, LARGE])
+@pytest.mark.parametrize("mode", [0, 2])
+def test_rows_edited_between_rounds_are_where_the_learners_start(oracle, mode, dims, defer):
+    # a program that perturbs the learners' copies of w~ at a round boundary (written on request where
+    # the re-broadcast is deferred): in the first round, in a replayed one, and not after it
+    g, o = _pair(oracle, mode, dims, defer_broadcast=defer)
+    rng = np.random.default_rng(23)
+    for r in range(4):
+        if r != 2:
+            if defer:
+                g.materialize_replicas()
+            noise = 0.1 * rng.standard_normal((3, g.n), dtype=np.float32)
+            g.replicas[:, :g.n] += torch.from_numpy(noise).to(g.device)
+            o.replicas[:, :g.n] += noise
+        launches = _steps_launches(g)
+        assert (launches == 1) == (dims is SMALL)
+        losses, _ = o.local_steps()
+        g.sync()
+        rep = g.replicas[:, :g.n].cpu().numpy()
+        for j in range(3):
+            assert l2_rel(rep[j], o.replicas[j, :g.n]) <= (r + 1) * _tol(mode)
+        assert l2_rel(g.get_losses(), losses) <= 10 * (r + 1) * _tol(mode)
+        g.meta_update()
+        o.meta_update()
+        g.sync()
+        assert l2_rel(g.w.cpu().numpy(), o.w) <= (r + 1) * _tol(mode)
+    g.close()
