@@ -579,19 +579,33 @@ mavg_status tc_setup(mavg_ctx* c) {
     c->shadow.sh_off[l - 1] = t.sh_off[l - 1];
   }
   // The fused CUDA-core last layer pays where the tensor-core products of that layer would leave most of
-  // the GPU idle (at most half a wave of tiles), and again where they take a wave or more of tiles that
-  // have little to do each: from three quarters of a wave on for layers of at most 16 K weights, at any
-  // number for at most 4 K, as long as the batch rows times the weights stay within 64 M.  Measured, us a round of 4 steps, fused / tensor tiles: 3072-512-512-10, B = 64:
-  // P = 48 923 / 978, P = 24 (96 tiles) 721 / 712; 1024-256-10, B = 32: P = 48 (96 tiles) 238 / 300;
-  // 600-800-800-16, B = 128: P = 24 555 / 628; 2048-768-32 (24 K weights), B = 128: P = 48 966 / 934;
-  // 512-128-24, B = 256: P = 100 (78 M) 471 / 424.
+  // the GPU idle (at most half a wave of its data gradient's tiles), and again where these take more but
+  // its forward product, one tile per learner, is less than a wave with little to do: from three quarters
+  // of a wave of data-gradient tiles on for layers of at most 16 K weights, at any number for at most
+  // 4 K.  Its own work grows with the batch rows times the weights: up to 32 M of them, 48 M where the
+  // layer below is four row tiles wide or wider (that much less is left of the tensor form's advantage),
+  // and at most 32 K rows.  Measured, us a round of 4 steps, fused / tensor tiles:
+  //   128-24, B = 64: P = 148 262 / 291, P = 160 286 / 282, P = 300 532 / 506; 64-10, B = 128: P = 148
+  //   282 / 319, P = 200 357 / 335 (more than a wave of learners); 600-800-800-16, B = 32: P = 16 363 / 399;
+  //   200-16, B = 64: P = 148 (29 M) 357 / 367; 128-24, B = 128: P = 100 (38 M) 269 / 274, P = 148 (56 M)
+  //   376 / 365; four row tiles and more: 504-32, B = 128: P = 24 (47 M) 382 / 404, P = 28 (55 M) 447 / 443;
+  //   512-10, B = 64: P = 48 923 / 978, P = 100 (31 M) 1748 / 1761;
+  //   64-64-4, B = 256: P = 100 (26 K rows) 405 / 427, P = 148 (38 K) 562 / 549.
   {
-    const long tiles = (long)P * ((cfg.dims[L - 1] + kBM - 1) / kBM);
+    const int row_tiles = (cfg.dims[L - 1] + kBM - 1) / kBM;
+    const long tiles = (long)P * row_tiles;
     const long weights = (long)cfg.dims[L - 1] * cfg.dims[L];
+    const int64_t work = (int64_t)P * B * weights;
+    const bool few = 2 * tiles <= c->sm_count;
     st->tail_ok = tail_fused_supported(&cfg) &&
-                  (2 * tiles <= c->sm_count ||
-                   ((weights <= 4096 || (4 * tiles >= 3 * c->sm_count && weights <= 16 * 1024)) &&
-                    (int64_t)P * B * weights <= 64 * 1024 * 1024));
+                  (few || (P <= c->sm_count && (int64_t)P * B <= 32 * 1024 &&
+                           (weights <= 4096 || (4 * tiles >= 3 * c->sm_count && weights <= 16 * 1024)) &&
+                           work <= (row_tiles >= 4 ? 48 : 32) * 1024 * 1024));
+    // Beside the fused last layer the last two layers' weight gradients may run beside the data gradients
+    // that are left, on the SMs these do not take.  With more tiles than half a wave too few SMs are left:
+    // 600-800-800-16, B = 64, P = 16 (36 SMs) 615 us a round against 433 in one launch at the end of the
+    // step; 512-256-256-8, P = 56 (36 SMs) 363 against 295, P = 40 (68 SMs) 269 against 245.
+    st->wgrad_beside = few;
   }
   if (e == cudaSuccess && st->tail_ok) e = tail_fused_prepare();
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&st->s_wgrad, cudaStreamNonBlocking);
@@ -734,7 +748,7 @@ cudaError_t tc_step(mavg_ctx* c, int64_t round, int step) {
   // Weight gradients of the last two layers beside the remaining dgrad products (their dZ comes
   // out of the fused last-layer kernel): layer L-1 then writes the other of its two bf16 copies,
   // because dgrad through it still reads the current one.
-  const bool split_wg = merged && fused_tail && overlap && L >= 3 && st->dbl_layer == L - 1;
+  const bool split_wg = merged && fused_tail && st->wgrad_beside && overlap && L >= 3 && st->dbl_layer == L - 1;
   const int rd = st->w16_cur;                                  // copy read in this step
   const int wr = split_wg ? (shared_w ? 0 : 1 - rd) : rd;      // copy written in this step
   auto w_k = [&](int l) -> const CUtensorMap& {

@@ -72,6 +72,8 @@ struct TcState {
   int w16_cur = 0;
   CUtensorMap w_b, w_mn_b, w16_st_b;
   bool tail_ok = false;                       // the fused last-layer kernel covers the shape
+  bool wgrad_beside = false;                  // with it: the last two layers' weight gradients beside
+                                              // the remaining data gradients
   bool wgrad_merged = false;                  // all layers' weight gradients in one launch
   // Forward products of step k+1 formed inside step k's weight-gradient launches (see
   // wgrad_tc.cuh), for layers 1..fuse_upto (0: none; at most L-1).  Possible where those launches
