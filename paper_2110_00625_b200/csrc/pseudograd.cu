@@ -246,15 +246,22 @@ cudaError_t launch_pseudograd_steps(mavg_ctx* c, int64_t round) {
   return cudaSuccess;
 }
 
-// The fused round has n / 4 threads where the local steps on their own have P times as many: a
-// short vector with many steps keeps the two launches.  Measured (P = 16, both forms, us a round):
-// n = 300 000: K = 5 36 against 38, K = 64 357 against 331; n = 1 M: K = 64 1101 against 1141;
-// n = 100 000: K = 1 8.5 against 12.5, K = 64 217 against 174.
+// The fused round has n / 4 threads, each with P x K serial steps, where the local steps on their own have
+// P times as many: with more steps per learner the vector has to be longer for it to pay, and a block's
+// keys (32 KB of shared memory at 4096) leave few of them on an SM unless they are large.  Measured, us a
+// round with deferred copies, one launch / two:
+//   K = 1: n = 76 000 P = 16 6.4 / 12.5, P = 256 49 / 77; n = 303 000 P = 1000 395 / 696;
+//   K = 4: n = 76 000 P = 16 14.6 / 15.6, P = 64 49 / 39, P = 256 183 / 138; n = 100 000 P = 256 227 / 195;
+//          n = 152 000 P = 32 32 / 33, P = 400 352 / 409; n = 303 000 P = 512 758 / 844, P = 1000 1759 / 1602;
+//   K = 8: n = 606 000 P = 16 88 / 90, P = 256 1372 / 1432, P = 512 2986 / 2866 (K = 10, P = 16 111 / 109);
+//   K = 16: n = 1 M P = 16 286 / 281; n = 2 M P = 16 550.7 / 551.2; n = 2.4 M P = 16 627 / 660;
+//   K = 64: n = 2 M P = 16 2146 / 2084; n = 2.4 M P = 16 2447 / 2477; K = 256, P = 16 9726 / 9745.
 bool pseudograd_round_fused(const mavg_ctx* c) {
-  const int64_t n = c->cfg.n, sms = c->sm_count;
-  return c->cfg.objective == MAVG_OBJ_PSEUDOGRAD && !c->profiling &&
-         (int64_t)c->cfg.P * c->cfg.K <= kMaxRoundKeys &&
-         n >= (c->cfg.K <= 4 ? 512 : 4096) * sms;
+  if (c->cfg.objective != MAVG_OBJ_PSEUDOGRAD || c->profiling) return false;
+  const int64_t n = c->cfg.n, sms = c->sm_count, K = c->cfg.K, keys = c->cfg.P * K;
+  const int64_t per_sm = K == 1 || (K <= 4 && keys <= 64) ? 512 : K <= 4 ? 1024 : K <= 8 ? 4096
+                         : K <= 16 ? 12288 : 16384;
+  return n >= per_sm * sms && keys <= (n >= 16384 * sms ? kMaxRoundKeys : kMaxRoundKeys / 2);
 }
 
 cudaError_t launch_pseudograd_round(mavg_ctx* c, int64_t round) {

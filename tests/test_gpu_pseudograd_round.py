@@ -44,10 +44,29 @@ def test_round_is_local_steps_then_meta_update(n, K, kw):
 def test_more_step_keys_than_the_fused_round_holds():
     # P K = 4095, 4096 and 4100: the last takes the two launches
     for P, K in ((63, 65), (64, 64), (41, 100)):
-        a, b = _handle(4096 * SMS + 1, P, K, mu=0.9), _handle(4096 * SMS + 1, P, K, mu=0.9)
+        a, b = _handle(16384 * SMS + 1, P, K, mu=0.9), _handle(16384 * SMS + 1, P, K, mu=0.9)
+        before = a.launch_count()
         a.round()
+        assert a.launch_count() - before == (1 if P * K <= 4096 else 2)
         b.local_steps(); b.meta_update()
         for x, y in zip(_state(a), _state(b)):
             assert np.array_equal(x, y)
         a.close(); b.close()
         torch.cuda.empty_cache()
+
+
+# both sides of every line of the rule
+@pytest.mark.parametrize("n,P,K,launches", [
+    (512 * SMS - 1, 3, 1, 2), (512 * SMS, 3, 1, 1), (512 * SMS, 300, 1, 1),
+    (512 * SMS, 16, 4, 1), (512 * SMS, 17, 4, 2), (1024 * SMS - 1, 17, 4, 2), (1024 * SMS, 17, 4, 1),
+    (1024 * SMS, 512, 4, 1), (1024 * SMS, 513, 4, 2),
+    (4096 * SMS - 1, 2, 5, 2), (4096 * SMS, 2, 8, 1), (4096 * SMS, 2, 9, 2),
+    (12288 * SMS - 1, 2, 9, 2), (12288 * SMS, 2, 16, 1), (12288 * SMS, 2, 17, 2),
+    (16384 * SMS - 1, 2, 17, 2), (16384 * SMS, 2, 17, 1), (16384 * SMS - 1, 129, 16, 2)])
+def test_where_a_round_is_one_launch(n, P, K, launches):
+    g = _handle(n, P, K, mu=0.9, defer_broadcast=True)
+    before = g.launch_count()
+    g.round()
+    assert g.launch_count() - before == launches
+    g.close()
+    torch.cuda.empty_cache()
