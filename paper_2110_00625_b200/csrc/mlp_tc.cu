@@ -246,12 +246,28 @@ TcLayout make_layout(const mavg_config* cfg, size_t base, int sm_count) {
   }
   t.w16b_stride = L >= 3 ? (int64_t)up((size_t)cfg->dims[L - 2] * cfg->dims[L - 1], 64) : 0;
   t.w16b = take(L >= 3 ? (size_t)P * t.w16b_stride * 2 : 16);
-  if (rides(cfg, sm_count))
+  // Split masters take no room of their own (an array of low halves would be another 2 bytes per hidden
+  // weight and learner, 537 MB on the large MLP).  Where forward products ride, the second copy of layer
+  // L-1 is not used at all -- it belongs to the merged weight-gradient launch -- and layer 1's bf16 copy
+  // is not from the first step's forward product to the last step's weight gradient.  The halves lie
+  // there, lower layers in the former first; layers that find no room keep fp32 masters.
+  if (rides(cfg, sm_count)) {
+    const int64_t room_b = t.w16b_stride, room_1 = (int64_t)up((size_t)cfg->dims[0] * cfg->dims[1], 64);
+    int64_t at_b = 0, at_1 = 0;
     for (int l = 2; l < L; ++l) {
-      t.lo_off[l - 1] = t.n_lo;
-      t.n_lo += (int64_t)up((size_t)cfg->dims[l] * cfg->dims[l - 1], 64);
+      const int64_t size = (int64_t)up((size_t)cfg->dims[l] * cfg->dims[l - 1], 64);
+      if (at_b + size <= room_b) {
+        t.lo16[l] = t.w16b + (size_t)at_b * 2;
+        t.lo_stride[l] = t.w16b_stride;
+        at_b += size;
+      } else if (at_1 + size <= room_1) {
+        t.lo16[l] = t.w16 + (size_t)(t.sh_off[0] + at_1) * 2;
+        t.lo_stride[l] = t.n16;
+        at_1 += size;
+        if (!t.lo_on_w1) t.lo_on_w1 = l;
+      }
     }
-  t.lo16 = take(std::max<size_t>((size_t)P * t.n_lo * 2, 16));
+  }
   t.end = off;
   return t;
 }
@@ -535,7 +551,7 @@ mavg_status tc_setup(mavg_ctx* c) {
     for (int l = 1; l < L; ++l) {
       const int in = cfg.dims[l - 1], out = cfg.dims[l];
       const WgradPlan w = plan_wgrad_stream(out, in, B, P, c->sm_count, st->wgrad_mom,
-                                            !masters_fit_l2(c), true, l >= 2 && t.n_lo > 0);
+                                            !masters_fit_l2(c), true, t.lo_stride[l] > 0);
       const size_t need = (size_t)P * w.m_tiles * w.n_chunks * B * kBM * sizeof(float);
       if (w.slots < 2 || need > t.zpart_bytes || (size_t)P * w.m_tiles * sizeof(int) > t.zcount_bytes)
         break;
@@ -545,10 +561,10 @@ mavg_status tc_setup(mavg_ctx* c) {
         enc = encode_any(st, &st->a_next[l][i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, bf(src), in, B,
                          P, in, (int64_t)B * in, kWgradTileCols, B, CU_TENSOR_MAP_SWIZZLE_64B, &why);
       }
-      if (enc && l >= 2 && t.n_lo)
-        enc = encode_any(st, &st->lo16[l], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2,
-                         (__nv_bfloat16*)bf(t.lo16) + t.lo_off[l - 1], in, out, P, in, t.n_lo,
-                         kWgradTileCols, kWgradTileRows, CU_TENSOR_MAP_SWIZZLE_64B, &why);
+      if (enc && t.lo_stride[l] > 0)
+        enc = encode_any(st, &st->lo16[l], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, bf(t.lo16[l]), in, out, P,
+                         in, t.lo_stride[l], kWgradTileCols, kWgradTileRows, CU_TENSOR_MAP_SWIZZLE_64B,
+                         &why);
       if (!enc) break;
       st->wgrad_f[l] = w;
       st->fuse_upto = l;
@@ -729,8 +745,8 @@ cudaError_t tc_step(mavg_ctx* c, int64_t round, int step) {
   st->split_done = 0;
   auto split_of = [&](int l, bool out) {
     WgradSplit sp;
-    sp.in = l >= 2 && l <= was_split;
-    sp.out = out && l >= 2 && t.n_lo > 0;
+    sp.in = l <= was_split && t.lo_stride[l] > 0;
+    sp.out = out && t.lo_stride[l] > 0;
     if (sp.in || sp.out) {
       sp.lo = &st->lo16[l];
       sp.master = c->buf.replicas + c->layers[l - 1].w_off;
@@ -863,7 +879,7 @@ cudaError_t tc_step(mavg_ctx* c, int64_t round, int step) {
     TC_TRY(cudaEventRecord(st->ev_gather_done, st->s_gather));
   }
 
-  bool side_used = tail_on_side;
+  bool side_used = tail_on_side, lo_on_w1_read = false;
   for (int l = L; l >= 1; --l) {
     const MlpLayer& ly = c->layers[l - 1];
     if (l > 1 && !(fused_tail && l == L)) {
@@ -885,6 +901,9 @@ cudaError_t tc_step(mavg_ctx* c, int64_t round, int step) {
     const CUtensorMap& bm = l == 1 ? st->x_in_t[xb] : act_in_t(l);
     if (merged) continue;        // all layers' weight gradients follow in one launch
     if (l <= ride) continue;     // after the dgrad chain, in ascending order (below)
+    // layer 1's launch writes its bf16 copy again: the low halves that lie there have to be read first
+    // (the side stream takes the layers in descending order)
+    if (overlap && l == 1 && lo_on_w1_read) TC_TRY(cudaStreamWaitEvent(main_s, st->ev_wgrad_done, 0));
     if (overlap && l > 1) {
       TC_TRY(cudaEventRecord(st->ev_fork, main_s));
       TC_TRY(cudaStreamWaitEvent(st->s_wgrad, st->ev_fork, 0));
@@ -892,6 +911,10 @@ cudaError_t tc_step(mavg_ctx* c, int64_t round, int step) {
       TC_TRY(launch_wgrad_stream(c, st->wgrad[l], st->dz_t[l], bm, st->w32[l], *w_st(l),
                                  shared_w ? &st->w32g[l] : nullptr, &st->u32[l], mom, nullptr,
                                  split_of(l, false)));
+      if (l == t.lo_on_w1 && l <= was_split) {
+        TC_TRY(cudaEventRecord(st->ev_wgrad_done, st->s_wgrad));
+        lo_on_w1_read = true;
+      }
       c->stream = main_s;
       side_used = true;
     } else {
@@ -932,7 +955,7 @@ cudaError_t tc_step(mavg_ctx* c, int64_t round, int step) {
                                shared_w ? &st->w32g[l] : nullptr, &st->u32[l], mom, &fn,
                                split_of(l, true)));
     st->fwd_done = l;
-    if (t.n_lo) st->split_done = l;
+    st->split_done = l;
   }
   if (merged) {
     // largest layer first, so that the small ones fill the ragged end of the launch

@@ -30,10 +30,12 @@ struct TcLayout {
                                              // layer at a time
   size_t w16b;                               // second bf16 copy of layer L-1's weights [P, w16b_stride]
   int64_t w16b_stride;
-  // low halves of the masters of layers 2..L-1 [P, n_lo], which are split between the steps of a call
-  // where forward products ride (0 elements: never); layer l at lo_off[l - 1]
-  size_t lo16;
-  int64_t n_lo, lo_off[MAVG_MAX_LAYERS];
+  // Low halves of the masters of hidden layers l >= 2 that are split between the steps of a call, where
+  // forward products ride: at lo16[l], lo_stride[l] elements from learner to learner (0: fp32 masters
+  // throughout).  lo_on_w1: the lowest layer whose halves lie in layer 1's bf16 copy (0: none).
+  size_t lo16[MAVG_MAX_LAYERS + 1];
+  int64_t lo_stride[MAVG_MAX_LAYERS + 1];
+  int lo_on_w1;
   size_t end;
 };
 
@@ -85,8 +87,8 @@ struct TcState {
   // (l = 1: gather buffer i) as the riding product reads it.  fwd_done: how many leading
   // layers of the step about to be issued already have their activations; gathered_step: the
   // step whose batch has already been gathered by the launch-by-launch form.
-  // lo16: the low halves of split masters (layers 2..fuse_upto); split_done: the leading layers whose
-  // masters the previous step of this call left split (layer 1's never are).
+  // lo16: the low halves of split masters; split_done: the leading layers of which the previous step
+  // of this call left those split that the layout has room for (layer 1's never are).
   CUtensorMap lo16[MAVG_MAX_LAYERS + 1];
   int split_done = 0;
   int fuse_upto = 0;

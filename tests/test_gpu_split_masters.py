@@ -7,7 +7,12 @@ import pytest
 from tests.util import l2_rel
 
 pytestmark = pytest.mark.gpu
-P, B = 13, 32
+B = 32
+
+
+def _learners(dims):
+    """Enough for layer 1's weight gradients to be a launch of their own (64 tiles per SM)."""
+    return 13 if dims[0] > 3000 else 70
 
 
 def _handle(dims, K, lr, w1=None, schedule=0, **kw):
@@ -16,15 +21,17 @@ def _handle(dims, K, lr, w1=None, schedule=0, **kw):
     x = rng.standard_normal((1024, dims[0]), dtype=np.float32)
     y = rng.integers(0, dims[-1], size=1024).astype(np.int32)
     w1 = m.workloads.mlp_init(dims) if w1 is None else w1
-    g = m.Mavg(w1, P=P, K=K, local_lr=lr, mu=0.9, B=B, seed=3, objective=m.OBJ_MLP, dims=dims,
+    g = m.Mavg(w1, P=_learners(dims), K=K, local_lr=lr, mu=0.9, B=B, seed=3, objective=m.OBJ_MLP, dims=dims,
                gemm_bf16=1, x=x, y=y, x_bf16=True, defer_broadcast=True, **kw)
     g.set_schedule(schedule)
     assert g.get_step_plan()["fwd_with_wgrad"] == len(dims) - 2
     return g
 
 
-# whole tiles; ragged rows and columns in every layer, runs that end in a partial tile
-SHAPES = [[3072, 1024, 512, 10], [3048, 1000, 504, 264, 10]]
+# whole tiles; ragged rows and columns in every layer, runs that end in a partial tile, and layer 2's low
+# halves in layer 1's bf16 copy (in the others they take the place of the second copy of layer L-1); a
+# layer 2 that finds no room and keeps fp32 masters below a split layer 3
+SHAPES = [[3072, 1024, 512, 10], [3048, 1000, 504, 264, 10], [520, 1024, 1024, 512, 10]]
 
 
 @pytest.mark.parametrize("dims", SHAPES)
@@ -49,8 +56,8 @@ def test_a_step_of_length_zero_keeps_every_bit(dims, K, beta):
     g.local_steps()
     g.sync()
     rep = g.replicas[:, :g.n].cpu().numpy().view(np.uint32)
-    for j in range(P):
-        assert np.array_equal(rep[j], w1.view(np.uint32))
+    for row in rep:
+        assert np.array_equal(row, w1.view(np.uint32))
     g.close()
 
 
@@ -69,7 +76,7 @@ def test_same_round_as_with_fp32_masters(dims):
     n = a.n
     ra, rb = a.replicas[:, :n].cpu().numpy(), b.replicas[:, :n].cpu().numpy()
     w = a.w.cpu().numpy()
-    for j in (0, P - 1):
+    for j in (0, -1):
         assert l2_rel(ra[j] - w, rb[j] - w) <= 5e-2
     a.close(); b.close()
 
@@ -89,3 +96,20 @@ def test_a_weight_that_is_not_a_number_stays_one():
         nans.append(np.isnan(g.w.cpu().numpy()))
         g.close()
     assert nans[0][at] and np.array_equal(nans[0], nans[1])
+
+
+@pytest.mark.parametrize("dims", SHAPES)
+@pytest.mark.parametrize("K", [2, 3])
+def test_second_call_starts_from_a_whole_bf16_copy(dims, K):
+    # the last step's launches read the low halves that lie in layer 1's bf16 copy and write that copy
+    # anew; a second call without a meta-update reads it in its first forward product.  Launch by launch
+    # there is no side stream: the same bits mean that the one is read before the other is written.
+    out = []
+    for profiled in (False, True):
+        g = _handle(dims, K, 0.002)
+        g.set_profiling(profiled)
+        g.local_steps(); g.local_steps()
+        g.sync()
+        out.append((g.get_losses(), g.replicas[:, :g.n].cpu().numpy().view(np.uint32)))
+        g.close()
+    assert np.array_equal(out[0][0], out[1][0]) and np.array_equal(out[0][1], out[1][1])

@@ -144,3 +144,19 @@ def test_workloads_are_seeded_and_shaped():
     assert not reps[:, 10000:].any()
     assert not np.array_equal(reps[0], reps[1])
     assert not np.array_equal(reps, W.perturbed_replicas(np.zeros(10000, np.float32), 3, 0.1, update=1, stride=10016))
+
+
+@pytest.mark.parametrize("dims,P,B,total", [
+    ([3072, 2048, 2048, 2048, 10], 32, 64, 1476131840),
+    ([3072, 2048, 2048, 2048, 10], 8, 64, 386890752),
+    ([3048, 1000, 504, 264, 10], 13, 32, 135932928),
+    ([520, 1024, 2048, 1024, 10], 70, 16, 1035927552),
+    ([3072, 512, 512, 10], 48, 64, 338617344),
+])
+def test_split_masters_take_no_workspace(lib, dims, P, B, total):
+    # shapes whose forward products ride on the weight gradients and whose hidden layers' masters are split
+    # between steps: the bytes are those of the layout without an array for the low halves
+    n = sum(dims[i] * dims[i + 1] + dims[i + 1] for i in range(len(dims) - 1))
+    cfg = _cfg(P=P, K=8, n=n, B=B, objective=2, dims=dims, gemm_bf16=1, x_ptr=256, y_ptr=256, n_samples=50000)
+    nb = C.c_size_t()
+    assert lib.mavg_workspace_bytes(C.byref(cfg), C.byref(nb)) == 0 and nb.value == total
