@@ -38,10 +38,12 @@ mavg_status mlp_setup(mavg_ctx* c) {
   }
   if (use_tensor_cores(&cfg)) return tc_setup(c);
   cudaError_t e = simt_setup(c);
-  if (e == cudaSuccess) e = small_setup(c);
-  if (e == cudaSuccess) return MAVG_OK;
-  c->err = std::string("kernel attributes: ") + cudaGetErrorString(e);
-  return MAVG_ERR_CUDA;
+  if (e != cudaSuccess) {
+    c->err = std::string("kernel attributes: ") + cudaGetErrorString(e);
+    return MAVG_ERR_CUDA;
+  }
+  small_setup(c);
+  return MAVG_OK;
 }
 
 void mlp_drop_graph(mavg_ctx* c);

@@ -36,7 +36,7 @@ cudaError_t simt_setup(mavg_ctx* c);      // once per handle
 cudaError_t simt_step(mavg_ctx* c, int64_t round, int step);
 
 // Small models on the CUDA cores (mlp_small.cu): all local steps of a round in one launch.
-cudaError_t small_setup(mavg_ctx* c);     // once per handle: c->small_splits > 0 where it is used
+void small_setup(mavg_ctx* c);            // once per handle: c->small_splits > 0 where it is used
 cudaError_t small_local_steps(mavg_ctx* c, int64_t round);
 
 // Tensor-core path (mlp_tc.cu): tcgen05 GEMMs fed by TMA.

@@ -404,10 +404,11 @@ static bool small_fits(const mavg_config* cfg) {
 // 84 / 158, P = 300 226 / 358; 80-128-16, B = 32, P = 4 (8 blocks, 50 000) 66 / 84; 80-128-128-16,
 // B = 32, P = 4 (116 000) 109 / 147; beyond the line 80-128-16, B = 48, P = 16 (149 000) 105 / 100;
 // with one block a learner 80-128-16, B = 4 94 / 74, and 80-128-128-16, B = 16, P = 300 833 / 535.
-cudaError_t small_setup(mavg_ctx* c) {
+// A device or driver that refuses one of the calls here leaves the handle the launch per product.
+void small_setup(mavg_ctx* c) {
   const mavg_config& cfg = c->cfg;
   c->small_splits = 0;
-  if (!small_fits(&cfg)) return cudaSuccess;
+  if (!small_fits(&cfg)) return;
   auto kernel = cfg.gemm_bf16 ? k_small_steps<true> : k_small_steps<false>;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmallSmem);
   int splits = 1;
@@ -419,8 +420,11 @@ cudaError_t small_setup(mavg_ctx* c) {
     e = cudaOccupancyMaxActiveClusters(&resident, kernel, &lc);
     if (e == cudaSuccess && resident >= cfg.P) { splits = s; break; }
   }
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return;
+  }
   if (cfg.n <= 4096 || (splits >= 4 && cfg.n * cfg.B <= (int64_t)110000 * splits)) c->small_splits = splits;
-  return e;
 }
 
 cudaError_t small_local_steps(mavg_ctx* c, int64_t round) {
