@@ -240,12 +240,13 @@ mavg_status mavg_get_step_plan(mavg_handle h, int32_t *out);
 typedef enum {
   MAVG_K_META = 0,      /* fused meta-update + re-broadcast */
   MAVG_K_BROADCAST = 1, /* initial / resume broadcast */
-  MAVG_K_PSEUDOGRAD = 2,
+  MAVG_K_PSEUDOGRAD = 2, /* pseudo-gradient steps; a whole round where mavg_round takes one launch */
   MAVG_K_BATCH = 3,     /* index stream and gather */
   MAVG_K_FWD = 4,       /* forward GEMMs (+bias, ReLU) */
   MAVG_K_LOSS = 5,      /* softmax cross-entropy and loss reductions; the fused last-layer kernel */
   MAVG_K_DGRAD = 6,     /* backward-data GEMMs (+ReLU mask, bias step) */
-  MAVG_K_WGRAD_SGD = 7, /* backward-weight GEMMs fused with the SGD step */
+  MAVG_K_WGRAD_SGD = 7, /* backward-weight GEMMs fused with the SGD step; all K local steps of a
+                           small CUDA-core model, which are one launch */
   MAVG_K_AUX = 8,       /* operand copies (bf16 shadows) */
   MAVG_K_COUNT = 9
 } mavg_kernel_class;
@@ -259,7 +260,9 @@ mavg_status mavg_set_profiling(mavg_handle h, int32_t on);
  *   MAVG_SCHED_GRAPH_TC: the same graph with every product as plain one-tile-per-block
  *     tensor-core launches.  The two differ in the summation order of the products they run
  *     differently, nothing else; this one exists for comparison.
- * Profiled rounds (mavg_set_profiling) take the launch-by-launch form of the chosen schedule. */
+ * Profiled rounds (mavg_set_profiling) take the launch-by-launch form of the chosen schedule; what is
+ * one launch without profiling (the steps of a small CUDA-core model, a pseudo-gradient round) is one
+ * launch with it. */
 typedef enum { MAVG_SCHED_GRAPH = 0, MAVG_SCHED_GRAPH_TC = 2 } mavg_schedule;
 mavg_status mavg_set_schedule(mavg_handle h, int32_t mode);
 mavg_status mavg_get_profile(mavg_handle h, float *ms, int64_t *launches, int32_t reset);

@@ -138,7 +138,7 @@ cudaError_t mlp_local_steps(mavg_ctx* c, int64_t round) {
   // The usual round starts from the broadcast state and is replayed from a graph.  Rounds that
   // start elsewhere (local steps called twice in a row), profiled rounds and handles whose
   // capture failed once take the launch-by-launch path.
-  if (!c->profiling && c->small_splits) return small_local_steps(c, round);
+  if (c->small_splits) return small_local_steps(c, round);
   // The graph of a CUDA-core handle reads w~ with defer_broadcast and the replica array without; a
   // deferred round whose copies were written on request starts from them, outside the graph.
   const bool usual_start = c->replicas_equal_global &&

@@ -257,7 +257,7 @@ cudaError_t launch_pseudograd_steps(mavg_ctx* c, int64_t round) {
 //   K = 16: n = 1 M P = 16 286 / 281; n = 2 M P = 16 550.7 / 551.2; n = 2.4 M P = 16 627 / 660;
 //   K = 64: n = 2 M P = 16 2146 / 2084; n = 2.4 M P = 16 2447 / 2477; K = 256, P = 16 9726 / 9745.
 bool pseudograd_round_fused(const mavg_ctx* c) {
-  if (c->cfg.objective != MAVG_OBJ_PSEUDOGRAD || c->profiling) return false;
+  if (c->cfg.objective != MAVG_OBJ_PSEUDOGRAD) return false;
   const int64_t n = c->cfg.n, sms = c->sm_count, K = c->cfg.K, keys = c->cfg.P * K;
   const int64_t per_sm = K == 1 || (K <= 4 && keys <= 64) ? 512 : K <= 4 ? 1024 : K <= 8 ? 4096
                          : K <= 16 ? 12288 : 16384;
