@@ -1,5 +1,6 @@
 """Whole rounds on the CUDA cores, both forms of the learner level (all steps in one launch, and a launch
-per product replayed from a graph), against the oracle: where the learners start from."""
+per product replayed from a graph), against the oracle: where the learners start from, and local steps
+called twice in a row."""
 import numpy as np
 import pytest
 import torch
@@ -64,4 +65,31 @@ def test_rows_edited_between_rounds_are_where_the_learners_start(oracle, mode, d
         o.meta_update()
         g.sync()
         assert l2_rel(g.w.cpu().numpy(), o.w) <= (r + 1) * _tol(mode)
+    g.close()
+
+
+@pytest.mark.parametrize("beta", [0.0, 0.9])
+@pytest.mark.parametrize("defer", [False, True])
+@pytest.mark.parametrize("dims", [SMALL, LARGE])
+@pytest.mark.parametrize("mode", [0, 2])
+def test_local_steps_twice_in_a_row(oracle, mode, dims, defer, beta):
+    # the second call goes on from the learners' own models and momentum; two such rounds
+    g, o = _pair(oracle, mode, dims, beta=beta, defer_broadcast=defer)
+    for r in range(2):
+        for _ in range(2):
+            assert (_steps_launches(g) == 1) == (dims is SMALL)
+            losses, _ = o.local_steps()
+            g.sync()
+            assert l2_rel(g.get_losses(), losses) <= 10 * (r + 1) * _tol(mode)
+        rep = g.replicas[:, :g.n].cpu().numpy()
+        for j in range(3):
+            assert l2_rel(rep[j], o.replicas[j, :g.n]) <= (r + 1) * _tol(mode)
+            if beta:
+                # the buffers hold the gradients themselves
+                assert l2_rel(g.u[j, :g.n].cpu().numpy(), o.u[j, :g.n]) <= 10 * (r + 1) * _tol(mode)
+        g.meta_update()
+        o.meta_update()
+        g.sync()
+        assert l2_rel(g.w.cpu().numpy(), o.w) <= (r + 1) * _tol(mode)
+        assert l2_rel(g.v.cpu().numpy(), o.v) <= 10 * (r + 1) * _tol(mode)
     g.close()

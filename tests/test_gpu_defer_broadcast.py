@@ -109,8 +109,10 @@ def _mlp_pair(m, mode, dims, B, P, K, S=4000, **kw):
     (1, [512, 256, 128, 10], 64, 4, 3),      # tensor-core path, graph replay
     (1, [3072, 512, 512, 10], 128, 8, 2),    # the benchmark's shapes
     (1, [264, 200, 10], 48, 3, 1),           # ragged tiles, K = 1
-    (0, [40, 24, 10], 7, 3, 2),              # CUDA-core fp32 path
-    (2, [64, 48, 10], 16, 2, 2),             # CUDA-core path with rounded operands
+    (0, [40, 24, 10], 7, 3, 2),              # CUDA-core fp32 path, all steps in one launch
+    (2, [64, 48, 10], 16, 2, 2),             # the same with rounded operands
+    (0, [300, 200, 10], 16, 3, 2),           # a launch per product, graph replay
+    (2, [300, 200, 10], 16, 3, 2),
 ])
 def test_mlp_deferred_equals_eager(mode, dims, B, P, K):
     m = _mavg()
@@ -154,17 +156,18 @@ def test_mlp_deferred_launch_by_launch_and_round_host():
     a.close(); b.close()
 
 
-@pytest.mark.parametrize("mode", [0, 2])
-def test_cuda_core_graph_recorded_after_materialize(mode):
-    # CUDA-core path with deferred copies: the graph of a round's local steps is first recorded in
-    # a round whose copies had been written on request just before.  Every later replay must still
-    # start the learners from w~ (the copies are made outside the recorded graph), bit for bit
-    # like a handle that always writes them.
+@pytest.mark.parametrize("mode,dims", [(0, [40, 24, 10]), (2, [64, 48, 10]),
+                                       (0, [300, 200, 10]), (2, [300, 200, 10])])
+def test_cuda_core_graph_recorded_after_materialize(mode, dims):
+    # CUDA-core path with deferred copies: a round whose copies had been written on request just before
+    # starts from them (launch by launch where a round is not one launch), the first, before any graph is
+    # recorded, and one after; every other round must start the learners from w~, replayed or not,
+    # bit for bit like a handle that always writes the copies.
     m = _mavg()
-    dims = [40, 24, 10] if mode == 0 else [64, 48, 10]
     a, b = _mlp_pair(m, mode, dims, 16, 3, 2)
-    b.materialize_replicas()          # copies exist when the first round records the graph
-    for r in range(3):
+    for r in range(6):
+        if r in (0, 3):
+            b.materialize_replicas()
         a.round(); b.round()
         a.sync(); b.sync()
         assert _same(a.w, b.w) and _same(a.v, b.v), r
