@@ -114,8 +114,8 @@ __device__ __forceinline__ void gather(const SmallArgs& g, float* sm, uint64_t k
 enum Stage { FWD_HIDDEN = 0, FWD_LAST = 1, DGRAD = 2 };
 template <bool QUANT, int R>
 __device__ __forceinline__ void product(const float* a, const float* w, int sj, int sk, int J, int Kk,
-                                        uint32_t inv_j, int g0, int ng, int pitch, Stage stage, const float* aux,
-                                        float* out, int lanes, int splits, int t) {
+                                        uint32_t inv_j, int g0, int ng, int B, int pitch, Stage stage,
+                                        const float* aux, float* out, int lanes, int splits, int t) {
   const int part = t & (lanes - 1);
   const int tasks = J * ((ng + R - 1) / R);
   for (int e0 = 0; e0 < tasks; e0 += kCompute / lanes) {
@@ -164,8 +164,10 @@ __device__ __forceinline__ void product(const float* a, const float* w, int sj, 
         if (stage == FWD_LAST) {
           if (part == 0) *reinterpret_cast<float4*>(out + at) = v;   // logits stay in this block
         } else {
-          put4(out + at, operand4<QUANT>(make_float4(v.x > 0.f ? v.x : 0.f, v.y > 0.f ? v.y : 0.f,
-                                                     v.z > 0.f ? v.z : 0.f, v.w > 0.f ? v.w : 0.f)),
+          const int left = B - 4 * (gr + q);   // rows beyond the batch stay zero, whatever the weights are
+          put4(out + at, operand4<QUANT>(make_float4(v.x > 0.f ? v.x : 0.f, v.y > 0.f && left > 1 ? v.y : 0.f,
+                                                     v.z > 0.f && left > 2 ? v.z : 0.f,
+                                                     v.w > 0.f && left > 3 ? v.w : 0.f)),
                splits, part, lanes);
         }
       }
@@ -257,11 +259,11 @@ k_small_steps(const __grid_constant__ SmallArgs g) {
         const Stage stage = !fwd ? DGRAD : l < L ? FWD_HIDDEN : FWD_LAST;
         const int sj = fwd ? in | 1 : 1, sk = fwd ? 1 : in | 1;
         if (J * ng >= 4 * kCompute) {
-          product<QUANT, 2>(a, sm + g.s.w[l], sj, sk, J, Kk, g.inv[fwd ? l : l - 1], g0, ng, pitch, stage, aux, to, 1, splits, t);
+          product<QUANT, 2>(a, sm + g.s.w[l], sj, sk, J, Kk, g.inv[fwd ? l : l - 1], g0, ng, B, pitch, stage, aux, to, 1, splits, t);
         } else {
           int lanes = 1;
           while (lanes < 16 && J * ng * lanes * 2 <= kCompute && lanes * 4 <= Kk) lanes *= 2;
-          product<QUANT, 1>(a, sm + g.s.w[l], sj, sk, J, Kk, g.inv[fwd ? l : l - 1], g0, ng, pitch, stage, aux, to, lanes, splits, t);
+          product<QUANT, 1>(a, sm + g.s.w[l], sj, sk, J, Kk, g.inv[fwd ? l : l - 1], g0, ng, B, pitch, stage, aux, to, lanes, splits, t);
         }
         barrier<kCompute, 1>();
         if (st == L) {

@@ -93,3 +93,31 @@ def test_local_steps_twice_in_a_row(oracle, mode, dims, defer, beta):
         assert l2_rel(g.w.cpu().numpy(), o.w) <= (r + 1) * _tol(mode)
         assert l2_rel(g.v.cpu().numpy(), o.v) <= 10 * (r + 1) * _tol(mode)
     g.close()
+
+
+@pytest.mark.parametrize("mode", [0, 2])
+def test_rows_beyond_the_batch_take_no_part(oracle, mode):
+    # Hidden unit 0 is dead for every sample but would be alive for a row of zeros, and an infinite weight
+    # hangs on it: 0 x inf is no number, ReLU makes it zero, and everything stays finite.  The batch of 5
+    # leaves 3 rows of the last group of four that must not bring the infinity in.
+    import paper_2110_00625_b200 as m
+    dims, P, B = [4, 2, 2, 3], 2, 5
+    rng = np.random.default_rng(2)
+    x = np.abs(rng.standard_normal((40, 4), dtype=np.float32)) + 0.1
+    y = rng.integers(0, 3, size=40).astype(np.int32)
+    w1 = (0.3 * rng.standard_normal(10 + 6 + 9)).astype(np.float32)
+    w1[0:4] = -100.0                     # W_1's first row
+    w1[8] = 1.0                          # its bias
+    w1[10] = np.inf                      # W_2[0, 0]
+    kw = dict(P=P, K=2, mu=0.9, B=B, seed=4, dims=dims, x=x, y=y)
+    g = m.Mavg(w1, local_lr=0.01, objective=m.OBJ_MLP, gemm_bf16=mode, **kw)
+    o = oracle.Mavg(w1, gamma=0.01, objective=oracle.OBJ_MLP, bf16=mode != 0, stride=g.stride, **kw)
+    assert _steps_launches(g) == 1
+    losses, _ = o.local_steps()
+    g.sync()
+    assert np.isfinite(losses).all() and l2_rel(g.get_losses(), losses) <= 10 * _tol(mode)
+    rep, want = g.replicas[:, :g.n].cpu().numpy(), o.replicas[:, :g.n]
+    finite = np.isfinite(want)
+    assert np.array_equal(np.isfinite(rep), finite) and finite.sum() == P * (g.n - 1)
+    assert l2_rel(rep[finite], want[finite]) <= _tol(mode)
+    g.close()
