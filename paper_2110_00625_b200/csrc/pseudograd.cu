@@ -12,7 +12,7 @@ namespace {
 
 // The variate of element i at a step with key `key`: mix64(key + (i+1) G), its four 16-bit lanes
 // summed, minus 131070, times c (mavg.h).  What bounds the pass is the integer pipes: about 25
-// instructions per variate -- a 64-bit addition, three xor-shifts of 4, two 64 x 64 -> 64 bit
+// instructions of arithmetic per variate (29.3 executed, keys and loop included) -- a 64-bit addition, three xor-shifts of 4, two 64 x 64 -> 64 bit
 // products of 3 multiply-adds, two dot products, three float operations -- of which the shifts and
 // logic operations (ALU pipe) and the multiply-adds (FMA pipe, 64-bit ones at a quarter of the
 // rate) are about 24 cycles per warp each.  Hence the 64-bit value is kept as two words:
@@ -68,10 +68,10 @@ __device__ __forceinline__ void local_step4(float4& w, float4& u, uint64_t key, 
     w.w = fmaf(-gamma, g3, w.w);
   }
 }
-template <bool MOM>
+template <bool MOM, int U = 4>
 __device__ __forceinline__ void local_steps4(float4& w, float4& u, const uint64_t* keys, int K,
                                              uint64_t c0, float c, float gamma, float beta) {
-#pragma unroll 4
+#pragma unroll U
   for (int k = 0; k < K; ++k) local_step4<MOM>(w, u, keys[k], c0, c, gamma, beta);
 }
 // The same on one element (the ragged end of the vector).
@@ -87,8 +87,11 @@ __device__ __forceinline__ void local_steps1(float& w, float& u, const uint64_t*
 
 // grid = (x, P); dynamic shared memory holds the K step keys of learner blockIdx.y.
 // MOM: learner-level momentum, u^j read (unless mom.read_u == 0) and written once per pass like w^j.
-template <bool MOM>
-__global__ void __launch_bounds__(256)
+// U: steps unrolled, 4 (40 registers, six blocks on an SM) or, for one or two steps, where HBM counts as much as
+// the variates, 1 (32 registers, all eight): n = 25.6 M, P = 16, K = 1 570 us against 670, K = 2 982 against
+// 992, K = 3 1402 against 1380.
+template <bool MOM, int U>
+__global__ void __launch_bounds__(256, U == 1 ? 8 : 6)
 k_pseudograd_steps(float* rep, int64_t stride, const float* src, int64_t src_stride, int64_t n,
                    int K, uint64_t seed, int64_t round, int k_first, float c, float gamma,
                    const MomArgs mom) {
@@ -109,7 +112,7 @@ k_pseudograd_steps(float* rep, int64_t stride, const float* src, int64_t src_str
     float4 w = src_stride ? __ldcs(in4 + q) : __ldg(in4 + q);
     float4 u = make_float4(0.f, 0.f, 0.f, 0.f);
     if (MOM && mom.read_u) u = __ldcs(urow4 + q);
-    local_steps4<MOM>(w, u, keys, K, (uint64_t)(4 * q + 1) * kGamma, c, gamma, mom.beta);
+    local_steps4<MOM, U>(w, u, keys, K, (uint64_t)(4 * q + 1) * kGamma, c, gamma, mom.beta);
     __stcs(row4 + q, w);
     if (MOM) __stcs(urow4 + q, u);
   }
@@ -226,17 +229,13 @@ cudaError_t launch_pseudograd_steps(mavg_ctx* c, int64_t round) {
     dim3 grid((unsigned)blocks_x, (unsigned)P);
     const bool from_global = c->replicas_equal_global;
     const MomArgs mom = mom_args(c, from_global);
+    auto kernel = mom.u ? (kc <= 2 ? k_pseudograd_steps<true, 1> : k_pseudograd_steps<true, 4>)
+                        : (kc <= 2 ? k_pseudograd_steps<false, 1> : k_pseudograd_steps<false, 4>);
     prof_begin(c, MAVG_K_PSEUDOGRAD);
-    if (mom.u)
-      k_pseudograd_steps<true><<<grid, 256, (size_t)kc * sizeof(uint64_t), c->stream>>>(
-          c->buf.replicas, c->buf.replica_stride, from_global ? c->buf.global_w : c->buf.replicas,
-          from_global ? 0 : c->buf.replica_stride, n, kc, c->cfg.seed, round, k0 + 1, scale,
-          c->cfg.local_lr, mom);
-    else
-      k_pseudograd_steps<false><<<grid, 256, (size_t)kc * sizeof(uint64_t), c->stream>>>(
-          c->buf.replicas, c->buf.replica_stride, from_global ? c->buf.global_w : c->buf.replicas,
-          from_global ? 0 : c->buf.replica_stride, n, kc, c->cfg.seed, round, k0 + 1, scale,
-          c->cfg.local_lr, mom);
+    kernel<<<grid, 256, (size_t)kc * sizeof(uint64_t), c->stream>>>(
+        c->buf.replicas, c->buf.replica_stride, from_global ? c->buf.global_w : c->buf.replicas,
+        from_global ? 0 : c->buf.replica_stride, n, kc, c->cfg.seed, round, k0 + 1, scale,
+        c->cfg.local_lr, mom);
     prof_end(c);
     c->replicas_equal_global = false;
     c->replicas_materialized = true;
