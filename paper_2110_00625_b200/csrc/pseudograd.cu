@@ -213,6 +213,9 @@ float variate_scale(const mavg_ctx* c) {
 
 constexpr int kMaxRoundKeys = 4096;   // P x K step keys of a fused round: 32 KB of shared memory
 
+// Blocks of 64 threads in a fused round, where the vector gives every SM only a few blocks of 256.
+bool small_blocks(const mavg_ctx* c) { return (c->cfg.n >> 2) < (int64_t)c->sm_count * 2048; }
+
 }  // namespace
 
 cudaError_t launch_pseudograd_steps(mavg_ctx* c, int64_t round) {
@@ -246,27 +249,35 @@ cudaError_t launch_pseudograd_steps(mavg_ctx* c, int64_t round) {
 }
 
 // The fused round has n / 4 threads, each with P x K serial steps, where the local steps on their own have
-// P times as many: with more steps per learner the vector has to be longer for it to pay, and a block's
-// keys (32 KB of shared memory at 4096) leave few of them on an SM unless they are large.  Measured, us a
-// round with deferred copies, one launch / two:
-//   K = 1: n = 76 000 P = 16 6.4 / 12.5, P = 256 49 / 77; n = 303 000 P = 1000 395 / 696;
-//   K = 4: n = 76 000 P = 16 14.6 / 15.6, P = 64 49 / 39, P = 256 183 / 138; n = 100 000 P = 256 227 / 195;
-//          n = 152 000 P = 32 32 / 33, P = 400 352 / 409; n = 303 000 P = 512 758 / 844, P = 1000 1759 / 1602;
-//   K = 8: n = 606 000 P = 16 88 / 90, P = 256 1372 / 1432, P = 512 2986 / 2866 (K = 10, P = 16 111 / 109);
-//   K = 16: n = 1 M P = 16 286 / 281; n = 2 M P = 16 550.7 / 551.2; n = 2.4 M P = 16 627 / 660;
-//   K = 64: n = 2 M P = 16 2146 / 2084; n = 2.4 M P = 16 2447 / 2477; K = 256, P = 16 9726 / 9745.
+// P times as many: with more steps per learner the vector has to be longer for it to pay.  Learner momentum
+// adds a read per learner to the serial part.  Blocks of 64 threads (launch_pseudograd_round) with more than
+// 2048 step keys leave too few warps on an SM.  Measured, us a round with deferred copies, one launch / two
+// (n = 76 000 is 512 per SM; the eager form differs by a few per cent in favour of one launch):
+//   K = 1: n = 76 000 P = 16 6.7 / 12.7, P = 256 50 / 94; n = 303 000 P = 1000 395 / 696;
+//   K = 2: n = 76 000 P = 256 103 / 95; n = 100 000 P = 64 35.2 / 35.3, P = 256 127 / 142;
+//   K = 3: n = 100 000 P = 64 47 / 43; n = 152 000 P = 32 25 / 29;
+//   K = 4: n = 76 000 P = 16 14.9 / 16.8, P = 64 50 / 39; n = 152 000 P = 256 228 / 258;
+//   K = 8: n = 606 000 P = 16 89 / 90;  K = 24: n = 606 000 P = 16 251 / 240, n = 2.4 M 932 / 955;
+//   K = 38: n = 606 000 P = 16 394 / 371, n = 909 000 575 / 554;  K = 64: n = 1.2 M P = 5 397 / 412;
+//   P x K = 4096: n = 606 000, K = 256 2833 / 2440, K = 8 2986 / 2866; n = 2.4 M, K = 64 9767 / 10776;
+//   with momentum, K = 1: n = 76 000 P = 64 27.1 / 27.1, P = 256 179 / 118; n = 303 000 P = 256 241 / 260;
+//   K = 3: n = 76 000 P = 16 15.2 / 15.7, P = 64 51 / 39;  K = 4: n = 76 000 P = 16 18.9 / 16.8; n = 152 000
+//   P = 16 22.9 / 22.9, P = 64 79 / 72; n = 303 000 P = 64 124 / 138.
+// At these lines the two are within 5 % of one another but for n = 455 000, P = 32, K = 4 (83 / 76).
 bool pseudograd_round_fused(const mavg_ctx* c) {
   if (c->cfg.objective != MAVG_OBJ_PSEUDOGRAD) return false;
   const int64_t n = c->cfg.n, sms = c->sm_count, K = c->cfg.K, keys = c->cfg.P * K;
-  const int64_t per_sm = K == 1 || (K <= 4 && keys <= 64) ? 512 : K <= 4 ? 1024 : K <= 8 ? 4096
-                         : K <= 16 ? 12288 : 16384;
-  return n >= per_sm * sms && keys <= (n >= 16384 * sms ? kMaxRoundKeys : kMaxRoundKeys / 2);
+  if (keys > (K <= 3 || !small_blocks(c) ? kMaxRoundKeys : kMaxRoundKeys / 2)) return false;
+  if (K > 4) return n >= (K <= 24 ? 4096 : 6144) * sms;
+  if (c->cfg.learner_momentum != 0.f)
+    return n >= 2048 * sms || (n >= 1024 * sms && keys <= 64) ||
+           (n >= 512 * sms && keys <= (K == 4 ? 32 : 48));
+  return n >= (K == 1 ? 512 : K == 2 ? 640 : 1024) * sms || (n >= 512 * sms && keys <= 64);
 }
 
 cudaError_t launch_pseudograd_round(mavg_ctx* c, int64_t round) {
   const int64_t n4 = c->cfg.n >> 2;
-  // blocks of 64 threads where the vector gives every SM only a few of them
-  const int threads = n4 < (int64_t)c->sm_count * 2048 ? 64 : 256;
+  const int threads = small_blocks(c) ? 64 : 256;
   const unsigned grid = (unsigned)((n4 + threads - 1) / threads + ((c->cfg.n & 3) ? 1 : 0));
   const size_t smem = (size_t)c->cfg.P * c->cfg.K * sizeof(uint64_t);
   const bool from_global = c->replicas_equal_global;

@@ -44,7 +44,7 @@ def test_round_is_local_steps_then_meta_update(n, K, kw):
 def test_more_step_keys_than_the_fused_round_holds():
     # P K = 4095, 4096 and 4100: the last takes the two launches
     for P, K in ((63, 65), (64, 64), (41, 100)):
-        a, b = _handle(16384 * SMS + 1, P, K, mu=0.9), _handle(16384 * SMS + 1, P, K, mu=0.9)
+        a, b = _handle(8192 * SMS + 1, P, K, mu=0.9), _handle(8192 * SMS + 1, P, K, mu=0.9)
         before = a.launch_count()
         a.round()
         assert a.launch_count() - before == (1 if P * K <= 4096 else 2)
@@ -55,16 +55,22 @@ def test_more_step_keys_than_the_fused_round_holds():
         torch.cuda.empty_cache()
 
 
-# both sides of every line of the rule
-@pytest.mark.parametrize("n,P,K,launches", [
-    (512 * SMS - 1, 3, 1, 2), (512 * SMS, 3, 1, 1), (512 * SMS, 300, 1, 1),
-    (512 * SMS, 16, 4, 1), (512 * SMS, 17, 4, 2), (1024 * SMS - 1, 17, 4, 2), (1024 * SMS, 17, 4, 1),
-    (1024 * SMS, 512, 4, 1), (1024 * SMS, 513, 4, 2),
-    (4096 * SMS - 1, 2, 5, 2), (4096 * SMS, 2, 8, 1), (4096 * SMS, 2, 9, 2),
-    (12288 * SMS - 1, 2, 9, 2), (12288 * SMS, 2, 16, 1), (12288 * SMS, 2, 17, 2),
-    (16384 * SMS - 1, 2, 17, 2), (16384 * SMS, 2, 17, 1), (16384 * SMS - 1, 129, 16, 2)])
-def test_where_a_round_is_one_launch(n, P, K, launches):
-    g = _handle(n, P, K, mu=0.9, defer_broadcast=True)
+# both sides of every line of the rule: n, P, K, learner momentum, launches
+@pytest.mark.parametrize("n,P,K,beta,launches", [
+    (512 * SMS - 1, 3, 1, 0.0, 2), (512 * SMS, 3, 1, 0.0, 1), (512 * SMS, 300, 1, 0.0, 1),
+    (512 * SMS, 32, 2, 0.0, 1), (640 * SMS - 1, 33, 2, 0.0, 2), (640 * SMS, 33, 2, 0.0, 1),
+    (512 * SMS, 16, 4, 0.0, 1), (512 * SMS, 17, 4, 0.0, 2), (1024 * SMS - 1, 17, 4, 0.0, 2),
+    (1024 * SMS, 17, 4, 0.0, 1), (1024 * SMS, 512, 4, 0.0, 1), (1024 * SMS, 513, 4, 0.0, 2),
+    (1024 * SMS, 1001, 3, 0.0, 1),
+    (4096 * SMS - 1, 2, 5, 0.0, 2), (4096 * SMS, 2, 24, 0.0, 1), (4096 * SMS, 2, 25, 0.0, 2),
+    (6144 * SMS - 1, 2, 25, 0.0, 2), (6144 * SMS, 2, 25, 0.0, 1),
+    (6144 * SMS, 32, 64, 0.0, 1), (6144 * SMS, 33, 64, 0.0, 2), (8192 * SMS, 33, 64, 0.0, 1),
+    (512 * SMS, 48, 1, 0.9, 1), (512 * SMS, 49, 1, 0.9, 2), (512 * SMS, 16, 3, 0.9, 1), (512 * SMS, 17, 3, 0.9, 2),
+    (512 * SMS, 8, 4, 0.9, 1), (512 * SMS, 9, 4, 0.9, 2), (1024 * SMS, 16, 4, 0.9, 1),
+    (1024 * SMS, 17, 4, 0.9, 2), (2048 * SMS - 1, 17, 4, 0.9, 2), (2048 * SMS, 17, 4, 0.9, 1),
+    (4096 * SMS, 2, 5, 0.9, 1)])
+def test_where_a_round_is_one_launch(n, P, K, beta, launches):
+    g = _handle(n, P, K, mu=0.9, defer_broadcast=True, learner_momentum=beta)
     before = g.launch_count()
     g.round()
     assert g.launch_count() - before == launches
