@@ -231,7 +231,7 @@ NCU_TRAFFIC = {
     "C2": {"wgrad_sgd_gemm": None, "fwd_gemm": None, "dgrad_gemm": None},
     # profiles/step_kernels_c4_p8.md: sums over a middle step's launches of the class at P = 8,
     # times 4, divided by the launches of the class (4 weight-gradient, 1 forward, 3 dgrad)
-    "C4": {"wgrad_sgd_gemm": 945.9e6, "fwd_gemm": 10.2e6, "dgrad_gemm": 198.2e6},
+    "C4": {"wgrad_sgd_gemm": 809.5e6, "fwd_gemm": 10.2e6, "dgrad_gemm": 197.4e6},
 }
 
 
@@ -424,11 +424,11 @@ def pseudograd_rounds(args, m, torch, peaks, Ks, steps):
 
 
 # Peak rate of the K-fused pseudo-gradient pass when instruction issue binds (variates/s): the
-# kernel executes 29.5 instructions per variate (ncu: 4.717e8 warp instructions for 5.12e8
+# kernel executes 29.3 instructions per variate (ncu: 4.684e8 warp instructions for 5.12e8
 # variates at n = 2 M, P = 16, K = 16, profiles/pseudograd_k16.md; 64-bit SplitMix64 arithmetic on
 # 32-bit ALUs), against an issue rate of 148 SMs x 4 schedulers x 1 warp instruction (32 lanes)
 # per clock at the maximum SM clock of 1965 MHz.
-PSEUDOGRAD_INSTR_PER_VARIATE = 29.5
+PSEUDOGRAD_INSTR_PER_VARIATE = 29.3
 PSEUDOGRAD_ALU_PEAK_VARIATES = 148 * 4 * 32 * 1.965e9 / PSEUDOGRAD_INSTR_PER_VARIATE
 
 

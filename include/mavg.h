@@ -254,9 +254,10 @@ mavg_status mavg_set_profiling(mavg_handle h, int32_t on);
 /* Schedule of the tensor-core MLP learner level (the paper has no counterpart).
  *   MAVG_SCHED_GRAPH (default): one launch per matrix product, the K steps of a round replayed
  *     from a CUDA graph; where the last layer's tensor-core tiles would leave most of the GPU idle
- *     (at most 32 classes, few learners) that layer -- forward, loss, dZ_L, its data gradient and
- *     the bias steps -- runs as one CUDA-core kernel, and hidden-layer forward products may split
- *     their contraction over a thread-block cluster.
+ *     or have little to do each (at most 32 classes and either few tiles, or fewer learners than SMs
+ *     and few weights and batch rows) that layer -- forward, loss, dZ_L, its data gradient and the
+ *     bias steps -- runs as one CUDA-core kernel, and hidden-layer forward products may split their
+ *     contraction over a thread-block cluster.
  *   MAVG_SCHED_GRAPH_TC: the same graph with every product as plain one-tile-per-block
  *     tensor-core launches.  The two differ in the summation order of the products they run
  *     differently, nothing else; this one exists for comparison.

@@ -133,7 +133,7 @@ k_pseudograd_steps(float* rep, int64_t stride, const float* src, int64_t src_str
 // with deferred copies (the learners' models are written) and (12P + 16) without (only the P
 // copies of the new w~ are).  Bounds: at K = 1 HBM (2.05 GB = 0.31 ms at n = 25.6 M, P = 16) and the
 // variates (0.38 ms) about equally, the variates beyond.  Measured there, deferred copies: K = 1
-// 507 us a round against 913 for the two passes, K = 64 25.5 ms against 27.4.
+// 492 us a round against 887 for the two passes, K = 64 25.5 ms against 25.8.
 // One quad per thread and no loop over the grid: the blocks' ends are spread over the launch.  The
 // last n % 4 elements have a block of their own, so that their serial P x K steps run beside the
 // rest.  K1: K = 1, the loop over the learners is unrolled instead of the one over the steps.

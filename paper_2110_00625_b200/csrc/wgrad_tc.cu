@@ -224,8 +224,10 @@ WgradPlan plan_wgrad_stream(int out, int in, int B, int P, int sm_count, bool mo
   const int slot_bytes = kW32Bytes + (momentum ? kW32Bytes : 0) + w.b_room + w.xn_bytes;
   // With a riding forward product a slot lives through two more hand-overs (epilogue -> forward MMAs
   // -> store), so it takes as many slots as fit: a second dZ^T buffer, which a long run uses once,
-  // makes room for one.  Large MLP, ms a round: 5 / 6 / 7 slots for split masters 16.1 / 15.7 / 15.3;
-  // bf16 tile over the slabs 15.5 -> 15.35; one dZ^T buffer (7 slots, 8 for split masters) 15.0.
+  // makes room for one.  Large MLP, ms a round, taken with a form of the split masters that rounded ties
+  // away from zero and had a cheaper epilogue (16.0 with the exact one): 5 / 6 / 7 slots for split masters
+  // 16.1 / 15.7 / 15.3; bf16 tile over the slabs 15.5 -> 15.35; one dZ^T buffer (7 slots, 8 for split
+  // masters) 15.0.
   const int budget = 220 * 1024;
   w.a_bufs = fwd_next ? 1 : 2;
   w.slots = (budget - w.a_bufs * a_bytes) / slot_bytes;
