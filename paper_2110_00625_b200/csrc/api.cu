@@ -95,6 +95,7 @@ void carve_workspace(const mavg_config* cfg, Workspace* ws) {
     off = mlp_workspace_bytes(cfg, ws, off);
   }
   ws->total = off;
+  if (cfg->objective != MAVG_OBJ_MLP) ws->least = off;
 }
 
 mavg_status set_err(mavg_ctx* c, mavg_status st, const std::string& msg) {
@@ -291,7 +292,7 @@ mavg_status mavg_create(const mavg_config* cfg, const mavg_buffers* buf, mavg_ha
     return fail(&g_create_error, MAVG_ERR_BAD_BUFFER, "learner_u must be 16-byte aligned");
   Workspace ws;
   carve_workspace(cfg, &ws);
-  if (buf->workspace_bytes < ws.total)
+  if (buf->workspace_bytes < ws.least)
     return fail(&g_create_error, MAVG_ERR_BAD_BUFFER, "workspace is smaller than mavg_workspace_bytes");
 
   int dev = 0;

@@ -84,6 +84,7 @@ struct Workspace {           // byte offsets into the caller's scratch buffer
   size_t idx = 0;            // int32 [P*B] sample indices of the current step
   size_t labels = 0;         // int32 [P*B]
   size_t act = 0;            // activations and their gradients (see mlp files)
+  size_t least = 0;          // a buffer of this size is accepted; `total` is what mavg_workspace_bytes reports
   size_t total = 0;
 };
 

@@ -1,0 +1,67 @@
+// Factored local steps of the tensor-core MLP path (factored.cu).
+//
+// Within a round every learner starts from w~, so its weights after k steps are
+//   W_l(k) = W~_l - gamma sum_{i<k} dZ_l(i)^T A_{l-1}(i),
+// and the products of step k can be taken from w~ and the factors without forming W_l(k):
+//   forward   Z = A W~^T - gamma sum_i (A A(i)^T) dZ(i)
+//   dgrad     dA = dZ W~  - gamma sum_i (dZ dZ(i)^T) A(i)
+// The hidden layers' weights are formed once, at the end of the call.
+#pragma once
+#include <cuda.h>
+
+#include <string>
+
+#include "common.cuh"
+
+namespace mavg {
+
+// Byte offsets of the path's scratch.  Rows of a learner are ordered (step, slot): K * B of them.
+struct FacLayout {
+  int64_t kb = 0;                            // rows of a learner: fac_steps() * B
+  int64_t s_ld = 0;                          // row length of the Gram arrays: kb rounded up to 64
+  size_t h[MAVG_MAX_LAYERS] = {};            // A_l, l = 0..L-1: bf16 [P, kb, d_l]
+  size_t g[MAVG_MAX_LAYERS] = {};            // dZ_l, l = 1..L-1: bf16 [P, kb, d_l]
+  // X W~_1^T, fp32 [kb, d_1] per learner, and -gamma X X^T below the step diagonal, bf16 [kb, s_ld] per
+  // learner.  Where they fit they lie in the learner's rows of the replica array, on W_1, which no
+  // factored step reads or writes before the last (in_rows; zbase and s1 are then byte offsets in a row).
+  bool in_rows = false;
+  size_t zbase = 0, s1 = 0;
+  size_t s[2] = {0, 0};                      // one step's -gamma A A(i)^T and -gamma dZ dZ(i)^T: bf16 [P, B, s_ld]
+  size_t labels = 0;                         // int32 [K, P, B]
+  size_t w_lo = 0;                           // low parts of w~'s last hidden layer: bf16 [d_{L-1}, d_{L-2}]
+  size_t end = 0;
+};
+
+// Learners per block, columns per learner and block, column tiles per learner (more than 1 with nl 1 only).
+struct FacCols { int nl = 1, cols = 0, c_tiles = 1; };
+
+struct FacState {
+  FacLayout lay;
+  int K = 0;                                 // steps the scratch has room for
+  int row_tile = 0;                          // rows of X per tile where all steps' rows are one operand
+  char *z_ptr = nullptr, *s1_ptr = nullptr;  // zbase and s1 of learner 0; strides in elements
+  int64_t z_stride = 0, s1_stride = 0;
+  // How the columns of the forward product of layer l, the data gradient through it and the Gram
+  // products are cut; the first two's batch operands (box 64 x cols x nl) and Gram operands (64 x cols)
+  FacCols fwd[MAVG_MAX_LAYERS + 1], dgrad[MAVG_MAX_LAYERS + 1], gram;
+  CUtensorMap in[MAVG_MAX_LAYERS + 1], dz_in[MAVG_MAX_LAYERS + 1];
+  CUtensorMap s_f[MAVG_MAX_LAYERS + 1], s_d[MAVG_MAX_LAYERS + 1];
+  CUtensorMap w_lo;                          // low parts of w~'s last hidden layer, box 64 x 128
+  // Row arrays [P, kb, d_l]: A_l (h) and dZ_l (g) with boxes of 64 x 64 rows (_mn: features are the MMA's
+  // row dimension, rows the contraction), 64 x 128 (_k) and 64 x gram.cols (_b; A_0: 64 x row_tile).
+  CUtensorMap h_mn[MAVG_MAX_LAYERS], g_mn[MAVG_MAX_LAYERS];
+  CUtensorMap h_k[MAVG_MAX_LAYERS], g_k[MAVG_MAX_LAYERS];
+  CUtensorMap h_b[MAVG_MAX_LAYERS], g_b[MAVG_MAX_LAYERS];
+};
+
+// The most steps of a call that a handle's calls may take in this form (0: never; at most the K it was made
+// for), and the scratch for them from `base` on.
+int fac_steps(const mavg_config* cfg);
+FacLayout fac_layout(const mavg_config* cfg, size_t base);
+struct TcState;
+mavg_status fac_setup(mavg_ctx* c, TcState* st, std::string* why);
+// This call's steps can take the factored form (they start from w~, the scratch is there).
+bool fac_usable(const mavg_ctx* c);
+cudaError_t fac_local_steps(mavg_ctx* c, int64_t round);
+
+}  // namespace mavg

@@ -41,11 +41,13 @@ cudaError_t small_local_steps(mavg_ctx* c, int64_t round);
 
 // Tensor-core path (mlp_tc.cu): tcgen05 GEMMs fed by TMA.
 bool tc_shapes_ok(const mavg_config* cfg, std::string* why);
-size_t tc_workspace_bytes(const mavg_config* cfg, size_t base, size_t* act_off);
+// least: what the path cannot do without (a smaller figure where factored steps would need more).
+size_t tc_workspace_bytes(const mavg_config* cfg, size_t base, size_t* act_off, size_t* least);
 mavg_status tc_setup(mavg_ctx* c);
 void tc_teardown(mavg_ctx* c);
 cudaError_t tc_refresh_shared_operands(mavg_ctx* c);
 cudaError_t tc_step(mavg_ctx* c, int64_t round, int step);
+cudaError_t tc_local_steps(mavg_ctx* c, int64_t round);      // all K of them
 
 // Fused last layer on CUDA cores (tail_fused.cu): forward, loss, dZ_L, dgrad through the layer
 // and the bias steps of the last two layers, for the tensor-core path's bf16 operands.
@@ -71,7 +73,10 @@ cudaError_t launch_tail_finish(mavg_ctx* c, const TailLaunch& t);   // bias step
 
 void tc_reset_counters(mavg_ctx* c);          // after an abandoned device-side wait
 void tc_step_plan(mavg_ctx* c, int32_t* out);  // entries of mavg_plan_entry
-int tc_get_w16_cur(mavg_ctx* c);            // which bf16 copy of the doubled layer is current
+// State of the learners' bf16 copies between calls: which copy of the doubled layer is current, or
+// kW16Stale: none (factored steps keep none; the next step that reads them writes them anew).
+constexpr int kW16Stale = -1;
+int tc_get_w16_cur(mavg_ctx* c);
 void tc_set_w16_cur(mavg_ctx* c, int cur);
 
 inline bool use_tensor_cores(const mavg_config* cfg) { return cfg->gemm_bf16 == 1; }

@@ -23,6 +23,7 @@
 
 #include <algorithm>
 
+#include "factored.cuh"
 #include "gemm_unit.cuh"
 #include "mlp.cuh"
 #include "tc_ptx.cuh"
@@ -134,6 +135,18 @@ k_shadow_from_global(const float* __restrict__ w, __nv_bfloat16* __restrict__ w1
     dst[t] = __float2bfloat16_rn(src[t]);
 }
 
+// The learners' own bf16 copies from their masters: grid (x, layers, P).
+__global__ void __launch_bounds__(256)
+k_copies_from_replicas(const float* __restrict__ rep, int64_t rep_stride, __nv_bfloat16* __restrict__ w16,
+                       int64_t n16, const ShadowArgs a) {
+  const int l = blockIdx.y;
+  const float* src = rep + (size_t)blockIdx.z * rep_stride + a.w_off[l];
+  __nv_bfloat16* dst = w16 + (size_t)blockIdx.z * n16 + a.sh_off[l];
+  for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < a.total[l];
+       t += (int64_t)gridDim.x * blockDim.x)
+    dst[t] = __float2bfloat16_rn(src[t]);
+}
+
 // ---------------------------------------------------------------------------------- host side
 size_t up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
@@ -194,25 +207,9 @@ TcLayout make_layout(const mavg_config* cfg, size_t base, int sm_count) {
   t.n16 = o16;
   size_t off = up(base, 1024);
   auto take = [&](size_t bytes) { size_t r = off; off = up(off + bytes, 1024); return r; };
-  for (int i = 0; i < 2; ++i) {
-    t.xg[i] = take(rows * cfg->dims[0] * 2);
-    t.xt[i] = take(rows * cfg->dims[0] * 2);
-  }
   int max_m_tiles = 1;
-  for (int l = 1; l <= L; ++l) {
-    const int d = cfg->dims[l];
-    if (l < L) {
-      t.act[l] = take(rows * d * 2);
-      t.act_t[l] = take(rows * d * 2);
-      t.act_b[l] = take(rows * d * 2);
-      t.act_t_b[l] = take(rows * d * 2);
-      t.dz[l] = take(rows * d * 2);
-    } else {
-      t.dz[l] = take(rows * t.cpad * 2);
-    }
-    t.dz_t[l] = take(rows * d * 2);
-    max_m_tiles = std::max(max_m_tiles, 8 * ((d + kBM - 1) / kBM));   // up to 8 column tiles
-  }
+  for (int l = 1; l <= L; ++l)
+    max_m_tiles = std::max(max_m_tiles, 8 * ((cfg->dims[l] + kBM - 1) / kBM));   // up to 8 column tiles
   size_t pb = 1024;
   for (int l = 1; l <= L; ++l) {
     GemmPlan f = plan_partial(cfg->dims[l], B, cfg->dims[l - 1], P, sm_count, l < L);
@@ -226,24 +223,38 @@ TcLayout make_layout(const mavg_config* cfg, size_t base, int sm_count) {
   t.part = take(pb);
   t.counters_bytes = (size_t)P * max_m_tiles * sizeof(int);
   t.counters = take(t.counters_bytes);
-  t.w16 = take((size_t)P * t.n16 * 2);
   t.w16g = take((size_t)t.n16 * 2);
   t.tail_part = take(tail_fused_supported(cfg) ? tail_fused_part_bytes(cfg) : 16);
-  {
-    // partial sums of a forward product that rides along with a weight-gradient launch: one
-    // 128 x B fp32 tile per (learner, row tile, run of column tiles) of that launch's plan; the
-    // layers use the space one after the other
-    t.zpart_bytes = 16;
-    t.zcount_bytes = 16;
-    if (B <= 128)
-      for (int l = 1; l < L; ++l) {
-        const WgradPlan w = plan_wgrad_stream(cfg->dims[l], cfg->dims[l - 1], B, P, sm_count, false, true, true);
-        t.zpart_bytes = std::max(t.zpart_bytes, (size_t)P * w.m_tiles * w.n_chunks * B * kBM * sizeof(float));
-        t.zcount_bytes = std::max(t.zcount_bytes, (size_t)P * w.m_tiles * sizeof(int));
-      }
-    t.zcount = take(t.zcount_bytes);
-    t.zpart = take(t.zpart_bytes);
+  t.dz[L] = take(rows * t.cpad * 2);
+  t.dz_t[L] = take(rows * cfg->dims[L] * 2);
+  t.zpart_bytes = 16;
+  t.zcount_bytes = 16;
+  if (B <= 128)
+    for (int l = 1; l < L; ++l) {
+      const WgradPlan w = plan_wgrad_stream(cfg->dims[l], cfg->dims[l - 1], B, P, sm_count, false, true, true);
+      t.zpart_bytes = std::max(t.zpart_bytes, (size_t)P * w.m_tiles * w.n_chunks * B * kBM * sizeof(float));
+      t.zcount_bytes = std::max(t.zcount_bytes, (size_t)P * w.m_tiles * sizeof(int));
+    }
+  t.zcount = take(t.zcount_bytes);
+  t.shared_end = off;
+  for (int i = 0; i < 2; ++i) {
+    t.xg[i] = take(rows * cfg->dims[0] * 2);
+    t.xt[i] = take(rows * cfg->dims[0] * 2);
   }
+  for (int l = 1; l < L; ++l) {
+    const int d = cfg->dims[l];
+    t.act[l] = take(rows * d * 2);
+    t.act_t[l] = take(rows * d * 2);
+    t.act_b[l] = take(rows * d * 2);
+    t.act_t_b[l] = take(rows * d * 2);
+    t.dz[l] = take(rows * d * 2);
+    t.dz_t[l] = take(rows * d * 2);
+  }
+  t.w16 = take((size_t)P * t.n16 * 2);
+  // partial sums of a forward product that rides along with a weight-gradient launch: one 128 x B fp32
+  // tile per (learner, row tile, run of column tiles) of that launch's plan; the layers use the space
+  // one after the other
+  t.zpart = take(t.zpart_bytes);
   t.w16b_stride = L >= 3 ? (int64_t)up((size_t)cfg->dims[L - 2] * cfg->dims[L - 1], 64) : 0;
   t.w16b = take(L >= 3 ? (size_t)P * t.w16b_stride * 2 : 16);
   // Split masters take no room of their own (an array of low halves would be another 2 bytes per hidden
@@ -275,30 +286,6 @@ TcLayout make_layout(const mavg_config* cfg, size_t base, int sm_count) {
 // SM count the plans (and with them the size of the partial buffer) are made for, so that the
 // workspace size does not depend on the device that later runs the problem.
 constexpr int kPlanSmCount = 148;
-
-// Tensor [batch, rows, inner] with the given strides (in elements) and box inner x box_rows.
-bool encode_any(TcState* st, CUtensorMap* m, CUtensorMapDataType dt, int esize, void* ptr,
-                int inner, int rows, int batch, int64_t row_stride, int64_t batch_stride,
-                int box_inner, int box_rows, CUtensorMapSwizzle swz, std::string* why) {
-  cuuint64_t dims[3] = {(cuuint64_t)inner, (cuuint64_t)rows, (cuuint64_t)batch};
-  cuuint64_t strides[2] = {(cuuint64_t)row_stride * esize, (cuuint64_t)batch_stride * esize};
-  cuuint32_t box[3] = {(cuuint32_t)box_inner, (cuuint32_t)box_rows, 1};
-  cuuint32_t es[3] = {1, 1, 1};
-  CUresult r = st->encode(m, dt, 3, ptr, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
-                          CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r != CUDA_SUCCESS) {
-    if (why) *why = "cuTensorMapEncodeTiled failed with code " + std::to_string((int)r);
-    return false;
-  }
-  return true;
-}
-
-// bf16 operand of an MMA: 64-element K slabs, 128-byte swizzle.
-bool encode_map(TcState* st, CUtensorMap* m, void* ptr, int inner, int rows, int batch,
-                int64_t row_stride, int64_t batch_stride, int box_rows, std::string* why) {
-  return encode_any(st, m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, ptr, inner, rows, batch, row_stride,
-                    batch_stride, kBK, box_rows, CU_TENSOR_MAP_SWIZZLE_128B, why);
-}
 
 template <int EPI>
 cudaError_t launch_gemm(mavg_ctx* c, int cls, const CUtensorMap& a, const CUtensorMap& b,
@@ -419,10 +406,13 @@ bool tc_shapes_ok(const mavg_config* cfg, std::string* why) {
   return true;
 }
 
-size_t tc_workspace_bytes(const mavg_config* cfg, size_t base, size_t* act_off) {
+size_t tc_workspace_bytes(const mavg_config* cfg, size_t base, size_t* act_off, size_t* least) {
   *act_off = base;
-  return make_layout(cfg, base, kPlanSmCount).end;
+  const TcLayout t = make_layout(cfg, base, kPlanSmCount);
+  *least = t.end;
+  return fac_steps(cfg) ? std::max(t.end, fac_layout(cfg, t.shared_end).end) : t.end;
 }
+
 
 mavg_status tc_setup(mavg_ctx* c) {
   const mavg_config& cfg = c->cfg;
@@ -630,6 +620,14 @@ mavg_status tc_setup(mavg_ctx* c) {
                         &st->ev_x_free[0], &st->ev_x_free[1]};
   for (cudaEvent_t* ev : evs)
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
+  if (e == cudaSuccess && fac_steps(&cfg) &&
+      c->buf.workspace_bytes >= std::max(t.end, fac_layout(&cfg, t.shared_end).end)) {
+    const mavg_status fs = fac_setup(c, st, &why);
+    if (fs != MAVG_OK) {
+      c->err = why;
+      return fs;
+    }
+  }
   if (e == cudaSuccess)
     e = cudaMemsetAsync(ws + t.counters, 0, t.counters_bytes, c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(ws + t.zcount, 0, t.zcount_bytes, c->stream);
@@ -651,6 +649,7 @@ void tc_teardown(mavg_ctx* c) {
                          st->ev_x_free[0], st->ev_x_free[1]};
     for (cudaEvent_t ev : evs)
       if (ev) cudaEventDestroy(ev);
+    delete st->fac;
   }
   delete st;
   c->mlp = nullptr;
@@ -686,26 +685,60 @@ void tc_step_plan(mavg_ctx* c, int32_t* out) {
     if (st->dense[l].ok) out[MAVG_PLAN_DENSE_FIRST_STEP] |= 1 << (l - 1);
 }
 
-cudaError_t tc_refresh_shared_operands(mavg_ctx* c) {
-  TcState* st = (TcState*)c->mlp;
-  const TcLayout& t = st->lay;
-  char* ws = (char*)c->buf.workspace;
+namespace {
+ShadowArgs copy_args(const mavg_ctx* c, int64_t* most) {
+  const TcLayout& t = ((const TcState*)c->mlp)->lay;
   ShadowArgs a{};
-  int64_t most = 0;
+  *most = 0;
   for (int l = 1; l <= c->cfg.n_layers; ++l) {
     const MlpLayer& ly = c->layers[l - 1];
     a.w_off[l - 1] = ly.w_off;
     a.total[l - 1] = (int64_t)ly.in * ly.out;
     a.sh_off[l - 1] = t.sh_off[l - 1];
-    most = std::max(most, a.total[l - 1]);
+    *most = std::max(*most, a.total[l - 1]);
   }
+  return a;
+}
+
+// The learners' bf16 copies (copy 0 of the doubled layer), which factored steps leave behind unwritten.
+cudaError_t rebuild_copies(mavg_ctx* c) {
+  const TcLayout& t = ((const TcState*)c->mlp)->lay;
+  int64_t most = 0;
+  const ShadowArgs a = copy_args(c, &most);
+  const int gx = (int)std::min<int64_t>((most + 1023) / 1024, std::max(1, c->sm_count * 16 / c->cfg.P));
+  prof_begin(c, MAVG_K_AUX);
+  k_copies_from_replicas<<<dim3((unsigned)gx, (unsigned)c->cfg.n_layers, (unsigned)c->cfg.P), 256, 0, c->stream>>>(
+      c->buf.replicas, c->buf.replica_stride, (__nv_bfloat16*)ws_ptr(c, t.w16), t.n16, a);
+  prof_end(c);
+  return cudaGetLastError();
+}
+}  // namespace
+
+cudaError_t tc_refresh_shared_operands(mavg_ctx* c) {
+  const TcLayout& t = ((const TcState*)c->mlp)->lay;
+  int64_t most = 0;
+  const ShadowArgs a = copy_args(c, &most);
   const int gx = (int)std::min<int64_t>((most + 255) / 256, (int64_t)c->sm_count * 4);
   prof_begin(c, MAVG_K_AUX);
   k_shadow_from_global<<<dim3((unsigned)gx, (unsigned)c->cfg.n_layers), 256, 0, c->stream>>>(
-      c->buf.global_w, (__nv_bfloat16*)(ws + t.w16g), a);
+      c->buf.global_w, (__nv_bfloat16*)ws_ptr(c, t.w16g), a);
   prof_end(c);
-  cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
+  return cudaGetLastError();
+}
+
+cudaError_t tc_local_steps(mavg_ctx* c, int64_t round) {
+  if (fac_usable(c)) {
+    cudaError_t e = fac_local_steps(c, round);
+    if (e != cudaSuccess) return e;
+    tc_set_w16_cur(c, kW16Stale);
+    c->replicas_equal_global = false;
+    return cudaSuccess;
+  }
+  for (int k = 1; k <= c->cfg.K; ++k) {
+    cudaError_t e = tc_step(c, round, k);
+    if (e != cudaSuccess) return e;
+    c->replicas_equal_global = false;
+  }
   return cudaSuccess;
 }
 
@@ -764,6 +797,13 @@ cudaError_t tc_step(mavg_ctx* c, int64_t round, int step) {
   // Weight gradients of the last two layers beside the remaining dgrad products (their dZ comes
   // out of the fused last-layer kernel): layer L-1 then writes the other of its two bf16 copies,
   // because dgrad through it still reads the current one.
+  if (st->w16_cur == kW16Stale) {
+    if (!shared_w) {
+      cudaError_t er = rebuild_copies(c);
+      if (er != cudaSuccess) return er;
+    }
+    st->w16_cur = 0;
+  }
   const bool split_wg = merged && fused_tail && st->wgrad_beside && overlap && L >= 3 && st->dbl_layer == L - 1;
   const int rd = st->w16_cur;                                  // copy read in this step
   const int wr = split_wg ? (shared_w ? 0 : 1 - rd) : rd;      // copy written in this step

@@ -159,6 +159,14 @@ __device__ __forceinline__ void st_cluster_f4(uint32_t addr, float a, float b, f
                "f"(c), "f"(d)
                : "memory");
 }
+__device__ __forceinline__ void st_cluster_u32(uint32_t addr, uint32_t v) {
+  asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+__device__ __forceinline__ float ld_cluster_f32(uint32_t addr) {
+  float v;
+  asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(addr) : "memory");
+  return v;
+}
 // One arrival on an mbarrier of another block of the cluster; releases this thread's earlier
 // writes (its distributed-shared-memory stores included) at cluster scope.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t remote_bar_addr) {
@@ -298,10 +306,11 @@ __device__ __forceinline__ uint64_t smem_desc_k_sw64(uint32_t smem_addr) {
   d |= (uint64_t)4 << 61;
   return d;
 }
-// Instruction descriptor, kind::f16: fp32 accumulator, bf16 A and B, both K-major, M x N tile.
-__host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N, int a_mn_major = 0) {
+// Instruction descriptor, kind::f16: fp32 accumulator, bf16 A and B, K-major unless said otherwise,
+// M x N tile.
+__host__ __device__ constexpr uint32_t idesc_bf16_f32(int M, int N, int a_mn_major = 0, int b_mn_major = 0) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(a_mn_major & 1) << 15) |
-         ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
+         ((uint32_t)(b_mn_major & 1) << 16) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
 }  // namespace tc

@@ -3,8 +3,12 @@
 #pragma once
 #include <cuda.h>
 
+#include <string>
+
 #include "common.cuh"
+#include "factored.cuh"
 #include "fwd_dense.cuh"
+#include "gemm_unit.cuh"
 #include "wgrad_tc.cuh"
 
 namespace mavg {
@@ -36,6 +40,8 @@ struct TcLayout {
   size_t lo16[MAVG_MAX_LAYERS + 1];
   int64_t lo_stride[MAVG_MAX_LAYERS + 1];
   int lo_on_w1;
+  size_t shared_end;                         // what lies behind here is dead while factored steps run,
+                                             // whose scratch begins here too
   size_t end;
 };
 
@@ -105,6 +111,7 @@ struct TcState {
   CUtensorMap in2d[MAVG_MAX_LAYERS + 1][2];
   GemmPlan fwd[MAVG_MAX_LAYERS + 1], dgrad[MAVG_MAX_LAYERS + 1];
   WgradPlan wgrad[MAVG_MAX_LAYERS + 1];
+  FacState* fac = nullptr;                    // factored steps (factored.cuh), null: not for this handle
   // side streams and events for the branches of a step that may overlap
   cudaStream_t s_wgrad = nullptr, s_gather = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_wgrad_done = nullptr, ev_gather_done = nullptr,
@@ -113,7 +120,28 @@ struct TcState {
 };
 
 
-int tc_get_w16_cur(mavg_ctx* c);
-void tc_set_w16_cur(mavg_ctx* c, int cur);
+// Tensor [batch, rows, inner] with the given strides (in elements) and box inner x box_rows x box_batch.
+inline bool encode_any(TcState* st, CUtensorMap* m, CUtensorMapDataType dt, int esize, void* ptr,
+                int inner, int rows, int batch, int64_t row_stride, int64_t batch_stride,
+                int box_inner, int box_rows, CUtensorMapSwizzle swz, std::string* why, int box_batch = 1) {
+  cuuint64_t dims[3] = {(cuuint64_t)inner, (cuuint64_t)rows, (cuuint64_t)batch};
+  cuuint64_t strides[2] = {(cuuint64_t)row_stride * esize, (cuuint64_t)batch_stride * esize};
+  cuuint32_t box[3] = {(cuuint32_t)box_inner, (cuuint32_t)box_rows, (cuuint32_t)box_batch};
+  cuuint32_t es[3] = {1, 1, 1};
+  CUresult r = st->encode(m, dt, 3, ptr, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
+                          CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  if (r != CUDA_SUCCESS) {
+    if (why) *why = "cuTensorMapEncodeTiled failed with code " + std::to_string((int)r);
+    return false;
+  }
+  return true;
+}
+
+// bf16 operand of an MMA: 64-element K slabs, 128-byte swizzle.
+inline bool encode_map(TcState* st, CUtensorMap* m, void* ptr, int inner, int rows, int batch,
+                int64_t row_stride, int64_t batch_stride, int box_rows, std::string* why, int box_batch = 1) {
+  return encode_any(st, m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, ptr, inner, rows, batch, row_stride,
+                    batch_stride, gemm::kBK, box_rows, CU_TENSOR_MAP_SWIZZLE_128B, why, box_batch);
+}
 
 }  // namespace mavg
