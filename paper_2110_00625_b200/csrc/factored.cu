@@ -324,68 +324,73 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     float* colsum = reinterpret_cast<float*>(smem + (size_t)stages * stage_bytes);   // [2][nl][128]
     if (EPI == PROD_DGRAD)
       for (int q = 0; q < nl; ++q) colsum[(half * nl + q) * kBM + row] = 0.f;
+    // What a group of columns needs besides the accumulator (the fp32 base of layer 1, the activations that
+    // gate dZ) is in flight while the group before it, or the main loop, is still at work.
+    const int end = EPI == PROD_RAW ? min(g.cols, g.row_end - r0) : nl * g.cols;
+    const bool add_base = EPI == PROD_FWD && g.zbase != nullptr;
+    float zb[16], bias_next = 0.f;
+    __nv_bfloat16 act[16];
+    auto locate = [&](int c0, size_t& at, size_t& z_at, int& q) {
+      q = EPI == PROD_RAW ? 0 : c0 / g.cols;
+      const int r = r0 + c0 - q * g.cols;
+      at = ((size_t)(p0 + q) * g.kb + r) * g.M + m;                    // element of column c0
+      z_at = (size_t)(p0 + q) * g.z_stride + (size_t)r * g.M + m;
+    };
+    auto fetch = [&](int c0) {
+      size_t at, z_at;
+      int q;
+      if (!m_ok || c0 >= end) return;
+      locate(c0, at, z_at, q);
+      if (EPI == PROD_FWD) bias_next = g.bias_in[(size_t)(p0 + q) * g.bias_in_stride + g.bias_off + m];
+      if (add_base) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) zb[j] = __ldg(g.zbase + z_at + (size_t)j * g.M);
+      }
+      if (EPI == PROD_DGRAD) {
+#pragma unroll
+        for (int j = 0; j < 16; ++j) act[j] = g.act[at + (size_t)j * g.M];
+      }
+    };
+#pragma unroll
+    for (int j = 0; j < 16; ++j) { zb[j] = 0.f; act[j] = __float2bfloat16_rn(0.f); }
+    fetch(half * 16);
     const bool ok = !any || mbar_wait(&sh.acc_bar, 0, abortp, g.status, ERR_EPILOGUE);
     if (ok) {
       tc_fence_after_sync();
       const uint32_t lane_addr = tmem_base + ((uint32_t)(q4 * 32) << 16);
-      int bias_q = -1;
-      float bias = 0.f;
 #pragma unroll 1
-      for (int c0 = half * 16; c0 < nl * g.cols; c0 += 32) {
-        const int q = EPI == PROD_RAW ? 0 : c0 / g.cols;
-        const int b = c0 - q * g.cols;
-        if (EPI == PROD_RAW && r0 + b >= g.row_end) break;
-        const size_t at = ((size_t)(p0 + q) * g.kb + r0 + b) * g.M + m;    // element of column c0
-        const size_t z_at = (size_t)(p0 + q) * g.z_stride + (size_t)(r0 + b) * g.M + m;
+      for (int c0 = half * 16; c0 < end; c0 += 32) {
+        size_t at, z_at;
+        int q;
+        locate(c0, at, z_at, q);
         float z[16];
+        __syncwarp();
+        load16(lane_addr + (uint32_t)c0, any, z);
         if (EPI == PROD_FWD) {
-          float zb[16];
-          if (g.zbase) {
 #pragma unroll
-            for (int j = 0; j < 16; ++j) zb[j] = m_ok ? __ldg(g.zbase + z_at + (size_t)j * g.M) : 0.f;
-          }
-          if (q != bias_q) {
-            bias = m_ok ? g.bias_in[(size_t)(p0 + q) * g.bias_in_stride + g.bias_off + m] : 0.f;
-            bias_q = q;
-          }
-          load16(lane_addr + (uint32_t)c0, any, z);
-          uint32_t h[8];
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            float a0 = z[2 * j], a1 = z[2 * j + 1];
-            if (g.zbase) { a0 += zb[2 * j]; a1 += zb[2 * j + 1]; }
-            a0 += bias; a1 += bias;
-            __nv_bfloat162 h2 = __floats2bfloat162_rn(a0 > 0.f ? a0 : 0.f, a1 > 0.f ? a1 : 0.f);
-            h[j] = *reinterpret_cast<uint32_t*>(&h2);
-          }
+          for (int j = 0; j < 16; ++j) z[j] = (add_base ? z[j] + zb[j] : z[j]) + bias_next;
+          fetch(c0 + 32);
           if (m_ok) {
-            const __nv_bfloat16* hh = reinterpret_cast<const __nv_bfloat16*>(h);
 #pragma unroll
-            for (int j = 0; j < 16; ++j) g.out[at + (size_t)j * g.M] = hh[j];
+            for (int j = 0; j < 16; ++j) g.out[at + (size_t)j * g.M] = __float2bfloat16_rn(z[j] > 0.f ? z[j] : 0.f);
           }
         } else if (EPI == PROD_DGRAD) {
-          float live[16];
-#pragma unroll
-          for (int j = 0; j < 16; ++j) live[j] = m_ok ? __bfloat162float(g.act[at + (size_t)j * g.M]) : 0.f;
-          load16(lane_addr + (uint32_t)c0, any, z);
           float s = 0.f;
 #pragma unroll
           for (int j = 0; j < 16; ++j) {
-            z[j] = live[j] > 0.f ? z[j] : 0.f;                       // ReLU'(0) = 0
+            z[j] = __bfloat162float(act[j]) > 0.f ? z[j] : 0.f;      // ReLU'(0) = 0
             s += z[j];
           }
+          fetch(c0 + 32);
           if (m_ok) {
 #pragma unroll
             for (int j = 0; j < 16; ++j) g.out[at + (size_t)j * g.M] = __float2bfloat16_rn(z[j]);
           }
           colsum[(half * nl + q) * kBM + row] += s;
-        } else {
-          load16(lane_addr + (uint32_t)c0, any, z);
-          if (m_ok) {
+        } else if (m_ok) {
 #pragma unroll
-            for (int j = 0; j < 16; ++j)
-              if (r0 + b + j < g.row_end) g.raw[z_at + (size_t)j * g.M] = z[j];
-          }
+          for (int j = 0; j < 16; ++j)
+            if (c0 + j < end) g.raw[z_at + (size_t)j * g.M] = z[j];
         }
       }
     }
