@@ -2,9 +2,10 @@
 //   forward   Z_l = A_{l-1} W_l^T + b_l,  A_l = act(Z_l)          (A_0 = gathered minibatch)
 //   backward  dA_{l-1} = (dZ_l W_l) .* [A_{l-1} > 0];  dW_l = dZ_l^T A_{l-1};  db_l = colsum dZ_l
 //   SGD       W_l <- W_l - gamma dW_l, b_l <- b_l - gamma db_l    (Algorithm 1's local update)
-// fp32 FMAs throughout.  With QUANT every matrix-product operand is first rounded to bf16
-// (nearest-even), which makes this path compute the same thing as the tensor-core path; it is the
-// path for true fp32 models and for layer widths the tensor-core path does not cover.
+// fp32 FMAs.  With QUANT every matrix-product operand is first rounded to bf16
+// (nearest-even), which makes this path compute the same thing as the tensor-core path, and the products run
+// on warp-level MMAs (fp32 sums); it is the path for true fp32 models and for layer widths the tensor-core
+// path does not cover.
 // A step is L-1 forward launches, one for the whole last layer up to its data gradient (which
 // also gathers the next step's minibatch), L-2 data gradients and one for the weight gradients,
 // bias gradients and SGD steps of all layers.  While a deferred re-broadcast is outstanding the first
@@ -70,7 +71,7 @@ union __align__(16) GemmShared {
 // A ROWS x 16 piece of an operand through registers.  KC: memory is [row, k] (k contiguous), else
 // [k, row].  rows and k_end bound the operand; what lies outside is zero.  The way a thread's
 // elements lie depends on `vec` alone (uniform): groups of four or single elements.
-template <int ROWS, bool KC, bool ROUND>
+template <int ROWS, bool KC>
 struct Piece {
   static constexpr int N = ROWS * BK / kThreads;   // elements per thread
   float r[N];
@@ -104,18 +105,17 @@ struct Piece {
       for (int e = 0; e < N / 4; ++e) {
         if (KC) {
 #pragma unroll
-          for (int i = 0; i < 4; ++i) s[(t % 4) * 4 + i][t / 4 + 32 * e] = operand<ROUND>(r[4 * e + i]);
+          for (int i = 0; i < 4; ++i) s[(t % 4) * 4 + i][t / 4 + 32 * e] = r[4 * e + i];
         } else {
           *reinterpret_cast<float4*>(&s[t / (ROWS / 4) + e * (kThreads * 4 / ROWS)][(t % (ROWS / 4)) * 4]) =
-              make_float4(operand<ROUND>(r[4 * e]), operand<ROUND>(r[4 * e + 1]),
-                          operand<ROUND>(r[4 * e + 2]), operand<ROUND>(r[4 * e + 3]));
+              make_float4(r[4 * e], r[4 * e + 1], r[4 * e + 2], r[4 * e + 3]);
         }
       }
     } else {
 #pragma unroll
       for (int e = 0; e < N; ++e) {
-        if (KC) s[t % 16][t / 16 + 8 * e] = operand<ROUND>(r[e]);
-        else s[t / ROWS + e * (kThreads / ROWS)][t % ROWS] = operand<ROUND>(r[e]);
+        if (KC) s[t % 16][t / 16 + 8 * e] = r[e];
+        else s[t / ROWS + e * (kThreads / ROWS)][t % ROWS] = r[e];
       }
     }
   }
@@ -157,6 +157,140 @@ __device__ __forceinline__ void multiply(const Slab& s, uint64_t (&acc)[4][4]) {
       for (int i = 0; i < 4; ++i) fma2(acc[i][j], a[i], bb);
     }
   }
+}
+
+// ---- bf16 operands: the same tile on warp-level MMAs, 4 warps of 32 x 32 each.  They take operands from any row
+// length and start, which tiled copies do not (B200's rate for them, 144 TFLOP/s measured, is twice the FMA
+// pipe's; as sums of three bf16 numbers fp32 operands would need six of them: 76 us for the 53 of the first
+// layer above).  Bound by the way through registers and the latency of a few slabs: 1000-333-100, P = 6, B = 50:
+// forward product of layer 1 14 us (19 with FMAs), weight gradients of
+// both layers 16 us (26, of which a last wave that was nearly empty and four loads at a time in the epilogue).
+// A slab's sum starts from zero and is added to the tile's in fp32, rounded to nearest: the tensor cores cut a
+// sum off where they add to it.
+constexpr int QK = 32;                             // k per slab
+// An operand's slab: [64 rows][32 k] in rows of 40 elements, or [32 k][64 rows] in rows of 72: eight
+// consecutive rows start in different banks.
+constexpr int kPitchK = QK + 8, kPitchR = BM + 8;
+constexpr int kSlab = BM * kPitchK;                // elements, the larger of the two
+static_assert(QK * kPitchR <= kSlab && BM == BN, "");
+union __align__(16) MmaShared {
+  __nv_bfloat16 slab[2][2][kSlab];                 // buffer, operand
+  float c[BM][kPitchB];
+};
+
+// A 64 x 32 piece of an operand through registers.  KC: memory is [row, k] (k contiguous), else
+// [k, row].  rows and k_end bound the operand; what lies outside is zero.  The way a thread's
+// elements lie depends on `vec` alone (uniform): groups of four or single elements.
+template <bool KC>
+struct MmaPiece {
+  static constexpr int N = BM * QK / kThreads;   // elements per thread
+  float r[N];
+  __device__ __forceinline__ void load(const float* __restrict__ p, int ld, int vec, int row0,
+                                       int rows, int k0, int k_end) {
+    const int t = threadIdx.x;
+    if (vec) {
+#pragma unroll
+      for (int e = 0; e < N / 4; ++e) {
+        const int row = row0 + (KC ? t / 8 + 16 * e : (t % 16) * 4);
+        const int k = k0 + (KC ? (t % 8) * 4 : t / 16 + 8 * e);
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (row < rows && k < k_end)
+          v = *reinterpret_cast<const float4*>(p + (KC ? (size_t)row * ld + k : (size_t)k * ld + row));
+        r[4 * e] = v.x; r[4 * e + 1] = v.y; r[4 * e + 2] = v.z; r[4 * e + 3] = v.w;
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < N; ++e) {
+        const int row = row0 + (KC ? t / 32 + 4 * e : t % 64);
+        const int k = k0 + (KC ? t % 32 : t / 64 + 2 * e);
+        r[e] = (row < rows && k < k_end) ? p[KC ? (size_t)row * ld + k : (size_t)k * ld + row] : 0.f;
+      }
+    }
+  }
+  __device__ __forceinline__ void store(__nv_bfloat16* s, int vec) const {
+    const int t = threadIdx.x;
+    if (vec) {
+#pragma unroll
+      for (int e = 0; e < N / 4; ++e) {
+        const int at = KC ? (t / 8 + 16 * e) * kPitchK + (t % 8) * 4 : (t / 16 + 8 * e) * kPitchR + (t % 16) * 4;
+        __nv_bfloat162 h[2] = {__floats2bfloat162_rn(r[4 * e], r[4 * e + 1]), __floats2bfloat162_rn(r[4 * e + 2], r[4 * e + 3])};
+        *reinterpret_cast<uint2*>(s + at) = *reinterpret_cast<uint2*>(h);
+      }
+    } else {
+#pragma unroll
+      for (int e = 0; e < N; ++e)
+        s[KC ? (t / 32 + 4 * e) * kPitchK + t % 32 : (t / 64 + 2 * e) * kPitchR + t % 64] = __float2bfloat16_rn(r[e]);
+    }
+  }
+};
+
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const __nv_bfloat16* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(tc::smem_u32(p)) : "memory");
+}
+__device__ __forceinline__ void ldsm4_t(uint32_t (&r)[4], const __nv_bfloat16* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(tc::smem_u32(p)) : "memory");
+}
+__device__ __forceinline__ void ldsm2(uint32_t (&r)[2], const __nv_bfloat16* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0, %1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(tc::smem_u32(p)) : "memory");
+}
+__device__ __forceinline__ void ldsm2_t(uint32_t (&r)[2], const __nv_bfloat16* p) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0, %1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(tc::smem_u32(p)) : "memory");
+}
+__device__ __forceinline__ void mma(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
+      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// 16 rows x 16 k of the MMA's row operand, 16 columns x 16 k (two of its column operands) from a plane.
+template <bool KC>
+__device__ __forceinline__ void row_operand(uint32_t (&r)[4], const __nv_bfloat16* pl, int row, int k) {
+  const int i = threadIdx.x % 32 / 8, j = threadIdx.x % 8;
+  if (KC) ldsm4(r, pl + (row + (i & 1) * 8 + j) * kPitchK + k + (i >> 1) * 8);
+  else ldsm4_t(r, pl + (k + (i >> 1) * 8 + j) * kPitchR + row + (i & 1) * 8);
+}
+template <bool KC>
+__device__ __forceinline__ void col_operands(uint32_t (&r)[4], const __nv_bfloat16* pl, int row, int k) {
+  const int i = threadIdx.x % 32 / 8, j = threadIdx.x % 8;
+  if (KC) ldsm4(r, pl + (row + (i >> 1) * 8 + j) * kPitchK + k + (i & 1) * 8);
+  else ldsm4_t(r, pl + (k + (i & 1) * 8 + j) * kPitchR + row + (i >> 1) * 8);
+}
+// One slab of the tile.  acc[mt][nt]: 16 x 8 results at rows 32 wm + 16 mt, columns 32 wn + 8 nt; mts, nps: how
+// many 16-row and 16-column groups of the warp's lie inside the result.
+// FRESH: the slab's sum on its own first (not for weight gradients, whose contraction is a few slabs long).
+template <bool A_KC, bool B_KC, bool FRESH>
+__device__ __forceinline__ void multiply_mma(const __nv_bfloat16* a, const __nv_bfloat16* b, int mts, int nps,
+                                             float (&acc)[2][4][4]) {
+  const int warp = threadIdx.x / 32, wm = warp & 1, wn = warp >> 1;
+  float own[2][4][4] = {};
+  float (&d)[2][4][4] = FRESH ? own : acc;
+#pragma unroll
+  for (int k = 0; k < QK; k += 16) {
+    uint32_t fa[2][4];
+#pragma unroll
+    for (int mt = 0; mt < 2; ++mt) row_operand<A_KC>(fa[mt], a, 32 * wm + 16 * mt, k);
+#pragma unroll
+    for (int np = 0; np < 2; ++np) {
+      if (np >= nps) break;
+      uint32_t fb[4];
+      col_operands<B_KC>(fb, b, 32 * wn + 16 * np, k);
+#pragma unroll
+      for (int mt = 0; mt < 2; ++mt) {
+        if (mt >= mts) break;
+        mma(d[mt][2 * np], fa[mt], fb[0], fb[1]);
+        mma(d[mt][2 * np + 1], fa[mt], fb[2], fb[3]);
+      }
+    }
+  }
+  if (!FRESH) return;
+#pragma unroll
+  for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[mt][nt][i] += own[mt][nt][i];
 }
 
 // Four finished sums C(m, n .. n+3): the layer's tail and the store.
@@ -202,20 +336,40 @@ __device__ __forceinline__ void emit(const GemmArgs& g, int p, int m, int n, flo
   }
 }
 
+// The blocks of a cluster have left their partial tiles in c: this block finishes 64 / splits rows of the tile.
 template <bool QUANT, int EPI>
-__device__ __forceinline__ void gemm_tile(const GemmArgs& g, int m0, int n0, int p, int rank,
-                                          int splits, GemmShared& sh) {
+__device__ __forceinline__ void finish_split(const GemmArgs& g, int m0, int n0, int p, int rank, int splits,
+                                             float (*c)[kPitchB]) {
+  tc::cluster_sync_all();
+  for (int t = threadIdx.x; t < BM / splits * (BN / 4); t += kThreads) {
+    const int m = rank * (BM / splits) + t / (BN / 4), n = 4 * (t % (BN / 4));
+    const uint32_t own = tc::smem_u32(&c[m][n]);
+    float v[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int q = 0; q < splits; ++q) {
+      float4 x;
+      asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
+                   : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w)
+                   : "r"(tc::mapa_u32(own, q)) : "memory");
+      v[0] += x.x; v[1] += x.y; v[2] += x.z; v[3] += x.w;
+    }
+    emit<QUANT, EPI>(g, p, m0 + m, n0 + n, v);
+  }
+  __syncwarp();
+  tc::cluster_sync_all();   // a peer may still be reading this block's partial tile
+}
+
+template <int EPI>
+__device__ __forceinline__ void fma_tile(const GemmArgs& g, int m0, int n0, int p, int rank,
+                                         int splits, GemmShared& sh) {
   constexpr bool A_KC = EPI != EPI_WGRAD_SGD, B_KC = EPI == EPI_FWD;
-  // activations were rounded where they were produced; dZ is kept unrounded for the bias step
-  constexpr bool QA = QUANT && EPI != EPI_FWD, QB = QUANT && EPI != EPI_WGRAD_SGD;
   const float* A = g.A + (size_t)p * g.a_batch;
   const float* B = g.B + (size_t)p * g.b_batch;
   const int lda = A_KC ? g.K : g.M, ldb = B_KC ? g.K : g.N;
   const int k_begin = rank * g.k_per_split;
   const int k_end = min(g.K, k_begin + g.k_per_split);
   uint64_t acc[4][4] = {};
-  Piece<BM, A_KC, QA> pa;
-  Piece<BN, B_KC, QB> pb;
+  Piece<BM, A_KC> pa;
+  Piece<BN, B_KC> pb;
   if (k_begin < k_end) {
     pa.load(A, lda, g.vec_a, m0, g.M, k_begin, k_end);
     pb.load(B, ldb, g.vec_b, n0, g.N, k_begin, k_end);
@@ -244,7 +398,7 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& g, int m0, int n0, int
       float v[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) v[j] = half_of(acc[i / 2][j], i & 1);
-      emit<QUANT, EPI>(g, p, m0 + 8 * ty + i, n0 + 4 * tx, v);
+      emit<false, EPI>(g, p, m0 + 8 * ty + i, n0 + 4 * tx, v);
     }
     return;
   }
@@ -253,29 +407,81 @@ __device__ __forceinline__ void gemm_tile(const GemmArgs& g, int m0, int n0, int
     *reinterpret_cast<float4*>(&sh.c[8 * ty + i][4 * tx]) =
         make_float4(half_of(acc[i / 2][0], i & 1), half_of(acc[i / 2][1], i & 1),
                     half_of(acc[i / 2][2], i & 1), half_of(acc[i / 2][3], i & 1));
-  tc::cluster_sync_all();
-  // this block finishes 64 / splits rows of the tile
-  for (int t = threadIdx.x; t < BM / splits * (BN / 4); t += kThreads) {
-    const int m = rank * (BM / splits) + t / (BN / 4), n = 4 * (t % (BN / 4));
-    const uint32_t own = tc::smem_u32(&sh.c[m][n]);
-    float v[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int q = 0; q < splits; ++q) {
-      float4 x;
-      asm volatile("ld.shared::cluster.v4.f32 {%0, %1, %2, %3}, [%4];"
-                   : "=f"(x.x), "=f"(x.y), "=f"(x.z), "=f"(x.w)
-                   : "r"(tc::mapa_u32(own, q)) : "memory");
-      v[0] += x.x; v[1] += x.y; v[2] += x.z; v[3] += x.w;
-    }
-    emit<QUANT, EPI>(g, p, m0 + m, n0 + n, v);
+  finish_split<false, EPI>(g, m0, n0, p, rank, splits, sh.c);
+}
+
+template <int EPI>
+__device__ __forceinline__ void mma_tile(const GemmArgs& g, int m0, int n0, int p, int rank, int splits,
+                                         MmaShared& sh) {
+  constexpr bool A_KC = EPI != EPI_WGRAD_SGD, B_KC = EPI == EPI_FWD;
+  const float* A = g.A + (size_t)p * g.a_batch;
+  const float* B = g.B + (size_t)p * g.b_batch;
+  const int lda = A_KC ? g.K : g.M, ldb = B_KC ? g.K : g.N;
+  const int k_begin = rank * g.k_per_split;
+  const int k_end = min(g.K, k_begin + g.k_per_split);
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32, wm = warp & 1, wn = warp >> 1;
+  const int mts = (g.M - m0 - 32 * wm + 15) / 16, nps = (g.N - n0 - 32 * wn + 15) / 16;
+  float acc[2][4][4] = {};
+  MmaPiece<A_KC> pa;
+  MmaPiece<B_KC> pb;
+  if (k_begin < k_end) {
+    pa.load(A, lda, g.vec_a, m0, g.M, k_begin, k_end);
+    pb.load(B, ldb, g.vec_b, n0, g.N, k_begin, k_end);
+    pa.store(sh.slab[0][0], g.vec_a);
+    pb.store(sh.slab[0][1], g.vec_b);
   }
-  tc::cluster_sync_all();   // a peer may still be reading this block's partial tile
+  __syncthreads();
+  int buf = 0;
+  for (int k0 = k_begin; k0 < k_end; k0 += QK, buf ^= 1) {
+    const bool more = k0 + QK < k_end;
+    if (more) {
+      pa.load(A, lda, g.vec_a, m0, g.M, k0 + QK, k_end);
+      pb.load(B, ldb, g.vec_b, n0, g.N, k0 + QK, k_end);
+    }
+    multiply_mma<A_KC, B_KC, EPI != EPI_WGRAD_SGD>(sh.slab[buf][0], sh.slab[buf][1], mts, nps, acc);
+    if (more) {
+      pa.store(sh.slab[buf ^ 1][0], g.vec_a);
+      pb.store(sh.slab[buf ^ 1][1], g.vec_b);
+    }
+    __syncthreads();
+  }
+  // through shared memory, so that a thread finishes four neighbours of a row
+#pragma unroll
+  for (int mt = 0; mt < 2; ++mt)
+#pragma unroll
+    for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+      for (int h = 0; h < 2; ++h)
+        *reinterpret_cast<float2*>(&sh.c[32 * wm + 16 * mt + lane / 4 + 8 * h][32 * wn + 8 * nt + 2 * (lane % 4)]) =
+            make_float2(acc[mt][nt][2 * h], acc[mt][nt][2 * h + 1]);
+  __syncthreads();
+  if (splits > 1) {
+    finish_split<true, EPI>(g, m0, n0, p, rank, splits, sh.c);
+    return;
+  }
+#pragma unroll
+  for (int i = 0; i < BM * (BN / 4) / kThreads; ++i) {
+    const int t = threadIdx.x + i * kThreads;
+    const float4 x = *reinterpret_cast<const float4*>(&sh.c[t / (BN / 4)][4 * (t % (BN / 4))]);
+    float v[4] = {x.x, x.y, x.z, x.w};
+    emit<true, EPI>(g, p, m0 + t / (BN / 4), n0 + 4 * (t % (BN / 4)), v);
+  }
+}
+
+template <bool QUANT> struct TileShared { using type = GemmShared; };
+template <> struct TileShared<true> { using type = MmaShared; };
+template <bool QUANT, int EPI>
+__device__ __forceinline__ void gemm_tile(const GemmArgs& g, int m0, int n0, int p, int rank, int splits,
+                                          typename TileShared<QUANT>::type& sh) {
+  if constexpr (QUANT) mma_tile<EPI>(g, m0, n0, p, rank, splits, sh);
+  else fma_tile<EPI>(g, m0, n0, p, rank, splits, sh);
 }
 
 // Forward and data gradient: grid (splits x row tiles x column tiles, 1, P), clusters of `splits`.
 template <bool QUANT, int EPI>
 __global__ void __launch_bounds__(kThreads, 4)
 k_simt_gemm(const __grid_constant__ GemmArgs g, int splits) {
-  __shared__ GemmShared sh;
+  __shared__ typename TileShared<QUANT>::type sh;
   tc::grid_launch_dependents();
   tc::grid_dependency_wait();
   const int rank = blockIdx.x % splits, tile = blockIdx.x / splits;
@@ -295,9 +501,9 @@ struct WgradArgs {
   int loss_stride;
 };
 template <bool QUANT>
-__global__ void __launch_bounds__(kThreads, 4)
+__global__ void __launch_bounds__(kThreads, QUANT ? 5 : 4)
 k_simt_wgrad(const __grid_constant__ WgradArgs w) {
-  __shared__ GemmShared sh;
+  __shared__ typename TileShared<QUANT>::type sh;
   tc::grid_launch_dependents();
   tc::grid_dependency_wait();
   int l = 0;
@@ -311,7 +517,7 @@ k_simt_wgrad(const __grid_constant__ WgradArgs w) {
   if (n0 == 0 && threadIdx.x < BM && o < g.M) {
     const float* d = g.A + (size_t)p * g.a_batch + o;
     float s = 0.f;
-#pragma unroll 8
+#pragma unroll 16
     for (int b = 0; b < g.K; ++b) s += d[(size_t)b * g.M];
     float* ub = g.mom.u ? g.mom.u + (size_t)p * g.mom.u_stride + g.ub_off + o : nullptr;
     local_update(g.bias + (size_t)p * g.c_batch + o, g.bias_in[(size_t)p * g.aux_batch + o], ub,
@@ -387,6 +593,39 @@ __device__ __forceinline__ float softmax_row(const float* z, int C, int label, f
   return lse - z[label];
 }
 
+constexpr int kTailRows = 8, kTailThreads = 512;
+
+// `count` contiguous floats into shared memory, 16 bytes per load wherever the source starts, eight loads of a
+// thread in flight.
+template <bool QUANT>
+__device__ __forceinline__ void copy_floats(float* dst, const float* __restrict__ src, int count) {
+  const int head = min(count, (int)((16 - ((uintptr_t)src & 15)) & 15) / 4), n4 = (count - head) / 4;
+  const int t = threadIdx.x;
+  const float4* s4 = reinterpret_cast<const float4*>(src + head);
+  for (int i0 = t; i0 < n4; i0 += 8 * kTailThreads) {
+    float4 v[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (i0 + u * kTailThreads < n4) v[u] = s4[i0 + u * kTailThreads];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int i = i0 + u * kTailThreads;
+      if (i >= n4) break;
+      float* d = dst + head + 4 * i;
+      d[0] = operand<QUANT>(v[u].x);
+      d[1] = operand<QUANT>(v[u].y);
+      d[2] = operand<QUANT>(v[u].z);
+      d[3] = operand<QUANT>(v[u].w);
+    }
+  }
+  const int rest = count - head - 4 * n4;
+  if (t < head) dst[t] = operand<QUANT>(src[t]);
+  if (t < rest) dst[head + 4 * n4 + t] = operand<QUANT>(src[head + 4 * n4 + t]);
+}
+
+// Elements of a bf16 row in shared memory: whole groups of 16, then an odd number of 16-byte units.
+__host__ __device__ constexpr int bf_pitch(int n) { return (((n + 15) / 16 * 16 >> 3) | 1) << 3; }
+
 // The last layer of 8 batch rows of a learner: logits, loss, dZ_L and the data gradient through the
 // layer, in one block of 512 threads; the remaining blocks gather the next step's minibatch.  A
 // layer of few classes is latency, not work: as a forward product, a loss and a data gradient it
@@ -396,6 +635,8 @@ __device__ __forceinline__ float softmax_row(const float* z, int C, int label, f
 // two rows and every fourth group of four classes (lanes along the input width); for the data
 // gradient a thread takes two columns of the input and four rows.
 // Dynamic shared memory: dZ [C][8], logits [8][C], the rows of A_{L-1} [8][in], W_L [C][in].
+// With bf16 operands the two products are warp-level MMAs on bf16 copies (mma_tail): their reads of shared
+// memory were what bounded the launch (333 x 100, P = 6, B = 50: 24 us, 13 now).
 struct TailArgs {
   const float* a;                          // A_{L-1} [P, B, in]
   const float* w; const float* b; int64_t w_batch;
@@ -404,8 +645,102 @@ struct TailArgs {
   float* row_loss;                         // [P, B]
   float* dz;                               // [P, B, C]
   float* dzp;                              // dZ_{L-1} [P, B, in], null for a one-layer model
+  bool mma;                                // bf16 operands on warp-level MMAs (mma_tail)
 };
-constexpr int kTailRows = 8, kTailThreads = 512;
+
+// k_simt_tail's block with bf16 operands.  Dynamic shared memory: W_L [C, to a multiple of 16][in], the rows of
+// A_{L-1} [16][in] (the last eight are zero), dZ [16][C], all bf16; logits [8][C].
+__device__ __forceinline__ void mma_tail(const TailArgs& t, int p, int r0, uint8_t* smem) {
+  const int rows = min(kTailRows, t.B - r0), in = t.in, C = t.C;
+  const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
+  const int ip = bf_pitch(in), dp = bf_pitch(C), c16 = (C + 15) / 16 * 16, in16 = (in + 15) / 16 * 16;
+  __nv_bfloat16* w = reinterpret_cast<__nv_bfloat16*>(smem);
+  __nv_bfloat16* a = w + (size_t)c16 * ip;
+  __nv_bfloat16* dq = a + 16 * ip;
+  float* z = reinterpret_cast<float*>(dq + 16 * dp);
+  const float* W = t.w + (size_t)p * t.w_batch;
+  const float* bias = t.b + (size_t)p * t.w_batch;
+  const int n16 = ((c16 + 16) * ip + 16 * dp) / 8;
+  for (int i = threadIdx.x; i < n16; i += kTailThreads) reinterpret_cast<uint4*>(w)[i] = make_uint4(0, 0, 0, 0);
+  __syncthreads();
+  // rows of `in` floats, contiguous from src on, to rows of ip
+  auto fill = [&](__nv_bfloat16* dst, const float* __restrict__ src, int count) {
+    const int head = min(count, (int)((16 - ((uintptr_t)src & 15)) & 15) / 4), n4 = (count - head) / 4;
+    const float4* s4 = reinterpret_cast<const float4*>(src + head);
+    for (int i0 = threadIdx.x; i0 < n4; i0 += 8 * kTailThreads) {
+      float4 v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (i0 + u * kTailThreads < n4) v[u] = s4[i0 + u * kTailThreads];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int i = i0 + u * kTailThreads;
+        if (i >= n4) break;
+        const int at = head + 4 * i;
+        int r = at / in, k = at - r * in;
+        const float x[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          dst[r * ip + k] = __float2bfloat16_rn(x[j]);
+          if (++k == in) { k = 0; ++r; }
+        }
+      }
+    }
+    const int rest = count - head - 4 * n4, x = threadIdx.x;
+    if (x < head) dst[x / in * ip + x % in] = __float2bfloat16_rn(src[x]);
+    if (x < rest) {
+      const int at = head + 4 * n4 + x;
+      dst[at / in * ip + at % in] = __float2bfloat16_rn(src[at]);
+    }
+  };
+  fill(w, W, C * in);
+  fill(a, t.a + ((size_t)p * t.B + r0) * in, rows * in);
+  __syncthreads();
+  const int i8 = lane / 8, j8 = lane % 8, qr = lane / 4, qc = 2 * (lane % 4);
+  for (int nt = warp; nt < (C + 7) / 8; nt += kTailThreads / 32) {
+    float s[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int k0 = 0; k0 < in16; k0 += 64) {            // 64 inputs' sum on its own: see multiply_mma
+      float d[4] = {0.f, 0.f, 0.f, 0.f};
+      for (int k = k0; k < min(in16, k0 + 64); k += 16) {
+        uint32_t fa[4], fb[2];
+        ldsm4(fa, a + ((i8 & 1) * 8 + j8) * ip + k + (i8 >> 1) * 8);
+        ldsm2(fb, w + (size_t)(nt * 8 + j8) * ip + k + (i8 & 1) * 8);
+        mma(d, fa, fb[0], fb[1]);
+      }
+      s[0] += d[0];
+      s[1] += d[1];
+    }
+    const int c = nt * 8 + qc;
+    if (c < C) z[qr * C + c] = s[0] + bias[c];
+    if (c + 1 < C) z[qr * C + c + 1] = s[1] + bias[c + 1];
+  }
+  __syncthreads();
+  if (warp < rows) {
+    const size_t row = (size_t)p * t.B + r0 + warp;
+    const float loss = softmax_row(z + warp * C, C, t.labels[row], 1.0f / (float)t.B, [&](int c, float g) {
+      t.dz[row * C + c] = g;
+      dq[warp * dp + c] = __float2bfloat16_rn(g);
+    });
+    if (lane == 0) t.row_loss[row] = loss;
+  }
+  if (!t.dzp) return;
+  __syncthreads();
+  for (int nt = warp; nt < (in + 7) / 8; nt += kTailThreads / 32) {
+    float d[4] = {0.f, 0.f, 0.f, 0.f};
+    for (int k = 0; k < c16; k += 16) {
+      uint32_t fa[4], fb[2];
+      ldsm4(fa, dq + ((i8 & 1) * 8 + j8) * dp + k + (i8 >> 1) * 8);
+      ldsm2_t(fb, w + (size_t)(k + (i8 & 1) * 8 + j8) * ip + nt * 8);
+      mma(d, fa, fb[0], fb[1]);
+    }
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int i = nt * 8 + qc + h;
+      if (qr < rows && i < in)                         // ReLU'(0) = 0
+        t.dzp[((size_t)p * t.B + r0 + qr) * in + i] = __bfloat162float(a[qr * ip + i]) > 0.f ? d[h] : 0.f;
+    }
+  }
+}
 
 template <bool QUANT>
 __global__ void __launch_bounds__(kTailThreads)
@@ -418,6 +753,10 @@ k_simt_tail(const __grid_constant__ TailArgs t, const __grid_constant__ GatherAr
     return;
   }
   const int p = blockIdx.x / t.row_blocks, r0 = blockIdx.x % t.row_blocks * kTailRows;
+  if (QUANT && t.mma) {
+    mma_tail(t, p, r0, reinterpret_cast<uint8_t*>(sm));
+    return;
+  }
   const int rows = min(kTailRows, t.B - r0), in = t.in, C = t.C;
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   float* dzq = sm;                         // [C][8], operand of the data gradient
@@ -427,10 +766,9 @@ k_simt_tail(const __grid_constant__ TailArgs t, const __grid_constant__ GatherAr
   const float* bias = t.b + (size_t)p * t.w_batch;
   const float* arow = t.a + ((size_t)p * t.B + r0) * in;
   float* w = a + kTailRows * in;
-#pragma unroll 8
-  for (int i = threadIdx.x; i < C * in; i += kTailThreads) w[i] = operand<QUANT>(W[i]);
-#pragma unroll 4
-  for (int i = threadIdx.x; i < kTailRows * in; i += kTailThreads) a[i] = i < rows * in ? arow[i] : 0.f;
+  copy_floats<QUANT>(w, W, C * in);
+  copy_floats<false>(a, arow, rows * in);
+  for (int i = rows * in + threadIdx.x; i < kTailRows * in; i += kTailThreads) a[i] = 0.f;
   __syncthreads();
   {
     const int r = warp % 4 * 2;
@@ -598,10 +936,13 @@ cudaError_t launch_gemm(mavg_ctx* c, int cls, GemmArgs g) {
 
 // Last layer in one launch (k_simt_tail) where its weights fit in an SM's shared memory.
 constexpr size_t kTailSmem = 200 * 1024;
-size_t tail_smem(int in, int C) {
+size_t tail_smem(int in, int C, bool quant) {
+  if (quant)
+    return ((size_t)((C + 15) / 16 * 16 + 16) * bf_pitch(in) + (size_t)16 * bf_pitch(C)) * 2 +
+           (size_t)kTailRows * C * sizeof(float);
   return ((size_t)kTailRows * in + 2 * (size_t)kTailRows * C + (size_t)in * C) * sizeof(float);
 }
-bool use_tail(int in, int C) { return tail_smem(in, C) <= kTailSmem; }
+bool use_tail(int in, int C) { return tail_smem(in, C, false) <= kTailSmem; }
 
 // Every kernel of a step asks for the same split of the SM's memory: a launch that needs another
 // split than the kernel before it has to wait until the SM is empty.
@@ -670,8 +1011,10 @@ cudaError_t step_impl(mavg_ctx* c, int64_t round, int step) {
     t.P = P; t.B = B; t.in = top.in; t.C = top.out; t.row_blocks = (B + kTailRows - 1) / kTailRows;
     t.row_loss = sb.row_loss; t.dz = sb.dz[L];
     if (L >= 2) t.dzp = sb.dz[L - 1];
+    // few classes on very wide rows: their padding to 16 would not fit
+    t.mma = QUANT && tail_smem(t.in, t.C, true) <= kTailSmem;
     if ((e = launch(c, MAVG_K_LOSS, k_simt_tail<QUANT>, dim3((unsigned)(P * t.row_blocks + gather_rows)),
-                    kTailThreads, 1, tail_smem(t.in, t.C), t, next)) != cudaSuccess)
+                    kTailThreads, 1, tail_smem(t.in, t.C, t.mma), t, next)) != cudaSuccess)
       return e;
   } else {
     if ((e = launch(c, MAVG_K_LOSS, k_simt_loss<QUANT>, dim3((unsigned)(P + gather_rows)), 1024, 1, 0,
