@@ -161,6 +161,10 @@ struct ProdArgs {
   int64_t bias_in_stride;
   float* bias_rep;          // dgrad: stepped bias written at bias_rep[p * rep_stride + bias_off + m]
   int64_t rep_stride, bias_off;
+  // GRAM: contraction slabs of the Gram product, its rows [cols of the batch, history] per learner
+  int gram_nkb;
+  __nv_bfloat16* gram_out;
+  int64_t gram_stride, gram_ld;
   float gamma;
   int* status;
 };
@@ -189,10 +193,15 @@ __device__ __forceinline__ void load16(uint32_t taddr, bool any, float (&z)[16])
 // whose first block adds their bias gradients in rank order.
 // TILES: 16 KB tiles of the MMA's row operand per stage.  LOW (two tiles): the product with w~ reads its low
 // parts as well.
-template <int EPI, int TILES, bool LOW>
+// GRAM: the Gram rows are formed here too, instead of by a launch of k_fac_gram before.  The blocks of a
+// learner are a cluster; those of a column tile share its Gram tiles out among themselves (128 history
+// rows each, row tile m_tile, m_tile + m_tiles, ...), write them to global memory and tell each other, while
+// the product with w~ runs; the tiles come back through the L2 as an operand.  A launch less on the chain of
+// a step for models whose launches are short.
+template <int EPI, int TILES, bool LOW, bool GRAM>
 __global__ void __launch_bounds__(kFacThreads, 2)
 k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ CUtensorMap tm_lo,
-              const __grid_constant__ CUtensorMap tm_in,
+              const __grid_constant__ CUtensorMap tm_in, const __grid_constant__ CUtensorMap tm_gram,
               const __grid_constant__ CUtensorMap tm_hist, const __grid_constant__ CUtensorMap tm_s,
               const ProdArgs g) {
   extern __shared__ uint8_t smem_raw[];
@@ -208,9 +217,15 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
   constexpr bool kMn = EPI == PROD_DGRAD;          // w~ is read MN-major
   constexpr int kBOff = TILES * kATileBytes;
   const int stage_bytes = product_stage_bytes(TILES, g.nl, g.cols), s_bytes = g.cols * kBK * 2;
+  __shared__ __align__(8) uint64_t gram_bar, rows_bar;     // GRAM: Gram sums complete; Gram rows in global memory
 
   if (threadIdx.x == 0) {
     if (LOW) tma_prefetch_desc(&tm_lo);
+    if (GRAM) {
+      tma_prefetch_desc(&tm_gram);
+      mbar_init(&gram_bar, 1);
+      mbar_init(&rows_bar, 8u * g.m_tiles);        // the epilogue warps of the column tile's blocks
+    }
     tma_prefetch_desc(&tm_w);
     tma_prefetch_desc(&tm_in);
     tma_prefetch_desc(&tm_hist);
@@ -227,6 +242,7 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
   tc_fence_before_sync();
   __syncthreads();
   tc_fence_after_sync();
+  if (GRAM) cluster_sync_all();                    // every block's barriers exist before anyone arrives on them
   const uint32_t tmem_base = sh.tmem_slot;
   grid_launch_dependents();   // not before the tensor memory is this block's: see the head of the file
   grid_dependency_wait();
@@ -239,14 +255,25 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
   const int nslab = (g.hist + kBK - 1) / kBK;
   volatile int* abortp = &sh.abort_flag;
   const bool any = g.nkb > 0 || g.hist > 0;
+  const int gram_step = kBM * g.m_tiles;           // from one of this block's Gram tiles to the next, in rows
 
   if (warp == 0) {
     if (lane == 0) {
       Ring ring;
       int issued = 0;
       bool ok = true;
+      if (GRAM)
+        for (int s0 = m0; s0 < g.hist && ok; s0 += gram_step)
+          for (int i = 0; i < g.gram_nkb; ++i, ++issued, ring.next(stages)) {
+            uint64_t* full = &sh.full_bar[ring.s];
+            if (!(ok = mbar_wait(&sh.empty_bar[ring.s], ring.ph ^ 1, abortp, g.status, ERR_PRODUCER))) break;
+            uint8_t* sa = smem + (size_t)ring.s * stage_bytes;
+            mbar_arrive_expect_tx(full, (uint32_t)(kATileBytes + s_bytes));
+            tma_load_3d(sa, &tm_gram, full, i * kBK, s0, p0);
+            tma_load_3d(sa + kBOff, &tm_in, full, i * kBK, r0, p0);
+          }
       const uint32_t base_bytes = (uint32_t)((LOW ? 2 : 1) * kATileBytes + N * kBK * 2);
-      for (int i = 0; i < g.nkb; ++i, ++issued, ring.next(stages)) {
+      for (int i = 0; i < g.nkb && ok; ++i, ++issued, ring.next(stages)) {
         uint64_t* full = &sh.full_bar[ring.s];
         if (!(ok = mbar_wait(&sh.empty_bar[ring.s], ring.ph ^ 1, abortp, g.status, ERR_PRODUCER))) break;
         uint8_t* sa = smem + (size_t)ring.s * stage_bytes;
@@ -259,6 +286,10 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
         }
         if (LOW) tma_load_3d(sa + kATileBytes, &tm_lo, full, i * kBK, m0, 0);
         tma_load_3d(sa + kBOff, &tm_in, full, i * kBK, r0, p0);
+      }
+      if (GRAM && ok) {
+        ok = mbar_wait_cluster(&rows_bar, 0, abortp, g.status, ERR_PRODUCER);
+        fence_proxy_async_all();                   // the rows were written by ordinary stores
       }
       for (int q = 0; q < nl && ok; ++q)
         for (int i = 0; i < nslab; i += TILES, ++issued, ring.next(stages)) {
@@ -286,7 +317,21 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
       const uint64_t b_base = smem_desc_k_sw128(base + kBOff);
       constexpr uint32_t kStepA = kMn ? kStepMn : kStepK;
       const uint32_t unit = (uint32_t)stage_bytes >> 4;
-      for (int i = 0; i < g.nkb; ++i, ring.next(stages)) {
+      if (GRAM) {
+        const uint32_t idesc_gram = idesc_bf16_f32(kBM, g.cols);
+        const uint64_t a_gram = smem_desc_k_sw128(base);
+        uint32_t d = tmem_base + (uint32_t)N;
+        for (int s0 = m0; s0 < g.hist && ok; s0 += gram_step, d += (uint32_t)g.cols)
+          for (int i = 0; i < g.gram_nkb; ++i, ring.next(stages)) {
+            if (!(ok = mbar_wait(&sh.full_bar[ring.s], ring.ph, abortp, g.status, ERR_MMA))) break;
+            tc_fence_after_sync();
+            const uint32_t off = (uint32_t)ring.s * unit;
+            slab_mma(d, a_gram + off, kStepK, b_base + off, kStepK, idesc_gram, i > 0);
+            umma_commit(&sh.empty_bar[ring.s]);
+          }
+        if (ok && m0 < g.hist) umma_commit(&gram_bar);
+      }
+      for (int i = 0; i < g.nkb && ok; ++i, ring.next(stages)) {
         if (!(ok = mbar_wait(&sh.full_bar[ring.s], ring.ph, abortp, g.status, ERR_MMA))) break;
         tc_fence_after_sync();
         const uint32_t off = (uint32_t)ring.s * unit;
@@ -321,6 +366,30 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     const int q4 = warp & 3, half = (warp - 2) >> 2;
     const int row = q4 * 32 + lane, m = m0 + row;
     const bool m_ok = m < g.M;
+    if (GRAM) {
+      if (m0 < g.hist && mbar_wait(&gram_bar, 0, abortp, g.status, ERR_EPILOGUE)) {
+        tc_fence_after_sync();
+        uint32_t d = tmem_base + ((uint32_t)(q4 * 32) << 16) + (uint32_t)N;
+        for (int s0 = m0; s0 < g.hist; s0 += gram_step, d += (uint32_t)g.cols) {
+          const int s = s0 + row;
+#pragma unroll 1
+          for (int c0 = half * 16; c0 < g.cols; c0 += 32) {
+            float z[16];
+            __syncwarp();
+            load16(d + (uint32_t)c0, true, z);
+            if (s >= g.hist) continue;
+            __nv_bfloat16* dst = g.gram_out + (size_t)p0 * g.gram_stride + (size_t)(s_row + c0) * g.gram_ld + s;
+#pragma unroll
+            for (int j = 0; j < 16; ++j) dst[(size_t)j * g.gram_ld] = __float2bfloat16_rn(-g.gamma * z[j]);
+          }
+        }
+      }
+      __threadfence();
+      fence_proxy_async_all();
+      __syncwarp();
+      if (lane < g.m_tiles) mbar_arrive_cluster(mapa_u32(smem_u32(&rows_bar), (uint32_t)(lane * g.c_tiles + c_tile)));
+      __syncwarp();
+    }
     float* colsum = reinterpret_cast<float*>(smem + (size_t)stages * stage_bytes);   // [2][nl][128]
     if (EPI == PROD_DGRAD)
       for (int q = 0; q < nl; ++q) colsum[(half * nl + q) * kBM + row] = 0.f;
@@ -412,15 +481,18 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
   if (EPI == PROD_DGRAD && g.c_tiles > 1) {
     __syncthreads();
     cluster_sync_all();
-    const int row = (int)threadIdx.x, m = m0 + row;
+    const int row = (int)threadIdx.x, m = m0 + row, rank0 = GRAM ? m_tile * g.c_tiles : 0;
     if (c_tile == 0 && row < kBM && m < g.M) {
       float s = 0.f;
-      for (int r = 0; r < g.c_tiles; ++r) s += ld_cluster_f32(mapa_u32(smem_u32(&sh.colsum[0][row]), (uint32_t)r));
+      for (int r = 0; r < g.c_tiles; ++r) s += ld_cluster_f32(mapa_u32(smem_u32(&sh.colsum[0][row]), (uint32_t)(rank0 + r)));
       const float w_in = g.bias_in[(size_t)p0 * g.bias_in_stride + g.bias_off + m];
       local_update(g.bias_rep + (size_t)p0 * g.rep_stride + g.bias_off + m, w_in, nullptr, 0, s, g.gamma, 0.f);
     }
     __syncwarp();
     cluster_sync_all();           // nobody leaves while its sums may still be read
+  } else if (GRAM) {
+    __syncwarp();
+    cluster_sync_all();           // nobody leaves while a peer may still arrive on its barrier
   }
   tc_fence_before_sync();
   __syncthreads();
@@ -1052,15 +1124,34 @@ int row_tile_of(int64_t rows) {
 // How a product's columns are cut into blocks, given its row tiles: several learners to a block, up to 256
 // columns (they share the w~ tile), while the blocks still take four fifths of the SMs; with fewer row
 // tiles a learner's batch in pieces, of 32 columns at least.
-FacCols cols_for(int P, int B, long row_tiles, int sm_count, int most_learners = 16) {
+FacCols cols_for(int P, int B, long row_tiles, int sm_count, int most_learners = 16, int most_tiles = 8) {
   FacCols c{std::min({std::max(1, 256 / B), P, most_learners}), B, 1};
   auto few = [&] { return row_tiles * ((P + c.nl - 1) / c.nl) * c.c_tiles * 5 < 4L * sm_count; };
   while (c.nl > 1 && few()) c.nl = (c.nl + 1) / 2;
-  while (few() && c.cols % 32 == 0 && c.cols > 32 && c.c_tiles < 8) {
+  while (few() && c.cols % 32 == 0 && c.cols > 32 && 2 * c.c_tiles <= most_tiles) {
     c.cols /= 2;
     c.c_tiles *= 2;
   }
   return c;
+}
+
+// Cut of a product that forms its own Gram rows where it can: short launches (a learner per block at most, so
+// that the blocks take the SMs) of at most four row tiles, which with the column tiles are one cluster.
+// us a round with the Gram rows in launches of their own / in the product's: 3072-512-512-10, K = 8, P = 8,
+// B = 128 479 / 455, P = 48, B = 64 861 / 844; 520-200-136-12, P = 20, K = 9, B = 48 367 / 334; six row tiles:
+// 1504-672-672-11, P = 10, K = 8, B = 176 788 / 793; eight: 3072-1024-1024-1024-10, P = 16, K = 8, B = 64
+// 977 / 1288 (clusters of eight blocks of one per SM).
+FacCols product_cols(int P, int B, int rows, int sm_count) {
+  const int m_tiles = (rows + kBM - 1) / kBM;
+  FacCols c = cols_for(P, B, m_tiles, sm_count);
+  if (c.nl > 1 || m_tiles > 4) return c;
+  c = cols_for(P, B, m_tiles, sm_count, 1, 8 / m_tiles);
+  c.own_gram = true;
+  return c;
+}
+// Tensor memory of a block that does: its sums and its Gram tiles'.
+int gram_columns(const FacCols& c, int m_tiles, int hist) {
+  return c.cols * (1 + ((hist + kBM - 1) / kBM + m_tiles - 1) / m_tiles);
 }
 
 struct PdlLaunch {
@@ -1093,9 +1184,9 @@ int stages_for(int slabs, int stage_bytes, long blocks, int sm_count) {
   return std::max(2, std::min({kMaxStages, slabs, (blocks > sm_count ? 96 : 196) * 1024 / stage_bytes}));
 }
 
-template <int EPI, int TILES, bool LOW = false>
+template <int EPI, int TILES, bool LOW = false, bool GRAM = false>
 cudaError_t launch_product(mavg_ctx* c, int cls, const CUtensorMap& w, const CUtensorMap& lo, const CUtensorMap& in,
-                           const CUtensorMap& hist, const CUtensorMap& s, ProdArgs g) {
+                           const CUtensorMap& hist, const CUtensorMap& s, ProdArgs g, const CUtensorMap* gram = nullptr) {
   g.m_tiles = (g.M + kBM - 1) / kBM;
   g.P = c->cfg.P;
   g.gamma = c->cfg.local_lr;
@@ -1105,13 +1196,14 @@ cudaError_t launch_product(mavg_ctx* c, int cls, const CUtensorMap& w, const CUt
   const int stage_bytes = product_stage_bytes(TILES, g.nl, g.cols);
   const dim3 grid((unsigned)(g.m_tiles * g.c_tiles), (unsigned)((g.P + g.nl - 1) / g.nl));
   const int hist_stages = ((g.hist + kBK - 1) / kBK + TILES - 1) / TILES;
-  g.stages = stages_for(std::max(1, g.nkb + g.nl * hist_stages), stage_bytes, (long)grid.x * grid.y, c->sm_count);
-  g.tmem_cols = tmem_columns(g.nl * g.cols);
+  g.stages = stages_for(std::max(1, g.gram_nkb + g.nkb + g.nl * hist_stages), stage_bytes, (long)grid.x * grid.y,
+                        c->sm_count);
+  g.tmem_cols = tmem_columns(GRAM ? gram_columns({1, g.cols, g.c_tiles}, g.m_tiles, g.hist) : g.nl * g.cols);
   const size_t smem = (size_t)g.stages * stage_bytes + 1024 +
                       (EPI == PROD_DGRAD ? (size_t)2 * g.nl * kBM * sizeof(float) : 0);
-  PdlLaunch l(grid, kFacThreads, smem, c->stream, EPI == PROD_DGRAD ? g.c_tiles : 1);
+  PdlLaunch l(grid, kFacThreads, smem, c->stream, GRAM ? (int)grid.x : EPI == PROD_DGRAD ? g.c_tiles : 1);
   prof_begin(c, cls);
-  cudaError_t e = cudaLaunchKernelEx(&l.lc, k_fac_product<EPI, TILES, LOW>, w, lo, in, hist, s, g);
+  cudaError_t e = cudaLaunchKernelEx(&l.lc, k_fac_product<EPI, TILES, LOW, GRAM>, w, lo, in, gram ? *gram : in, hist, s, g);
   prof_end(c);
   return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -1240,7 +1332,8 @@ mavg_status fac_setup(mavg_ctx* c, TcState* st, std::string* why) {
   f->z_stride = t.in_rows ? c->buf.replica_stride : t.kb * cfg.dims[1];
   for (int l = 1; l < L && ok; ++l) {
     // forward product of layer l; data gradient through layer l
-    f->fwd[l] = cols_for(P, B, (cfg.dims[l] + kBM - 1) / kBM, c->sm_count);
+    f->fwd[l] = l == 1 ? cols_for(P, B, (cfg.dims[l] + kBM - 1) / kBM, c->sm_count)
+                       : product_cols(P, B, cfg.dims[l], c->sm_count);
     if (l > 1 && l == L - 1)
       ok = ok && encode_map(st, &f->w_lo, bf(t.w_lo), cfg.dims[l - 1], cfg.dims[l], 1, cfg.dims[l - 1],
                             (int64_t)cfg.dims[l - 1] * cfg.dims[l], kBM, why);
@@ -1249,7 +1342,7 @@ mavg_status fac_setup(mavg_ctx* c, TcState* st, std::string* why) {
       continue;
     }
     const int in = cfg.dims[l - 1], out = cfg.dims[l];
-    f->dgrad[l] = cols_for(P, B, (in + kBM - 1) / kBM, c->sm_count);
+    f->dgrad[l] = product_cols(P, B, in, c->sm_count);
     ok = ok && encode_map(st, &f->in[l], bf(t.h[l - 1]), in, kb, P, in, t.kb * in, f->fwd[l].cols, why, f->fwd[l].nl);
     ok = ok && encode_map(st, &f->dz_in[l], bf(t.g[l]), out, kb, P, out, t.kb * out, f->dgrad[l].cols, why,
                           f->dgrad[l].nl);
@@ -1257,11 +1350,13 @@ mavg_status fac_setup(mavg_ctx* c, TcState* st, std::string* why) {
     ok = ok && encode_map(st, &f->s_d[l], bf(t.s[1]), (int)t.s_ld, B, P, t.s_ld, B * t.s_ld, f->dgrad[l].cols, why);
   }
   if (!ok) return MAVG_ERR_CUDA;
-  const void* kernels[] = {(const void*)k_fac_product<PROD_FWD, 2, false>, (const void*)k_fac_product<PROD_FWD, 2, true>,
-                           (const void*)k_fac_product<PROD_FWD, 1, false>, (const void*)k_fac_product<PROD_DGRAD, 1, false>,
-                           (const void*)k_fac_product<PROD_RAW, 1, false>, (const void*)k_fac_gram, (const void*)k_fac_last<1>,
-                           (const void*)k_fac_last<2>, 
-                           (const void*)k_fac_apply<kApplyStages, kApplyPieces>};
+  const void* kernels[] = {
+      (const void*)k_fac_product<PROD_FWD, 2, false, false>, (const void*)k_fac_product<PROD_FWD, 2, true, false>,
+      (const void*)k_fac_product<PROD_FWD, 1, false, false>, (const void*)k_fac_product<PROD_DGRAD, 1, false, false>,
+      (const void*)k_fac_product<PROD_RAW, 1, false, false>, (const void*)k_fac_product<PROD_FWD, 2, true, true>,
+      (const void*)k_fac_product<PROD_FWD, 1, false, true>,  (const void*)k_fac_product<PROD_DGRAD, 1, false, true>,
+      (const void*)k_fac_gram, (const void*)k_fac_last<1>, (const void*)k_fac_last<2>,
+      (const void*)k_fac_apply<kApplyStages, kApplyPieces>};
   for (const void* k : kernels) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024);
     if (e != cudaSuccess) {
@@ -1281,7 +1376,7 @@ bool fac_usable(const mavg_ctx* c) {
 // The K steps of a round.  Chain of a step, layers L:
 //   F_1 -> (S_2 -> F_2) -> ... -> last layer -> (T_{L-1} -> D_{L-1}) -> ... -> D_2
 // S_l, T_l: the Gram products that the forward product F_l and the data gradient D_l through layer l
-// need (none in the first step).
+// need (none in the first step); a launch of their own or part of F_l and D_l.
 cudaError_t fac_local_steps(mavg_ctx* c, int64_t round) {
   TcState* st = (TcState*)c->mlp;
   FacState* f = st->fac;
@@ -1371,23 +1466,42 @@ cudaError_t fac_local_steps(mavg_ctx* c, int64_t round) {
       g.bias_in_stride = w_in_stride;
       return g;
     };
+    // the product forms its Gram rows itself
+    auto own_gram = [&](const FacCols& cols, int M) {
+      return k > 1 && cols.own_gram && gram_columns(cols, (M + kBM - 1) / kBM, hist) <= 256;
+    };
+    auto with_gram = [&](ProdArgs& g, int dim, int i) {
+      g.gram_nkb = (dim + kBK - 1) / kBK;
+      g.gram_out = bfp(t.s[i]);
+      g.gram_stride = B * t.s_ld;
+      g.gram_ld = t.s_ld;
+    };
     for (int l = 1; l < L; ++l) {
-      if (l > 1 && k > 1) FAC_TRY(gram(MAVG_K_FWD, f->h_k[l - 1], f->h_b[l - 1], cfg.dims[l - 1], 0, k));
       ProdArgs g = product(cfg.dims[l], l, f->fwd[l]);
+      g.out = bfp(t.h[l]);
       if (l == 1) {
         g.s_row0 = hist;
         g.zbase = (const float*)f->z_ptr;
         g.z_stride = f->z_stride;
-      } else {
-        g.nkb = (cfg.dims[l - 1] + kBK - 1) / kBK;
-      }
-      g.out = bfp(t.h[l]);
-      if (l == 1)
         FAC_TRY((launch_product<PROD_FWD, 2>(c, MAVG_K_FWD, st->wg[1], st->wg[1], f->h_b[0], f->g_mn[1], f->s_f[1], g)));
-      else if (l == L - 1)
-        FAC_TRY((launch_product<PROD_FWD, 2, true>(c, MAVG_K_FWD, st->wg[l], f->w_lo, f->in[l], f->g_mn[l], f->s_f[l], g)));
+        continue;
+      }
+      const int in = cfg.dims[l - 1];
+      const CUtensorMap &w = st->wg[l], &a = f->in[l], &d = f->g_mn[l], &s = f->s_f[l];
+      g.nkb = (in + kBK - 1) / kBK;
+      if (own_gram(f->fwd[l], cfg.dims[l])) {
+        with_gram(g, in, 0);
+        if (l == L - 1)
+          FAC_TRY((launch_product<PROD_FWD, 2, true, true>(c, MAVG_K_FWD, w, f->w_lo, a, d, s, g, &f->h_k[l - 1])));
+        else
+          FAC_TRY((launch_product<PROD_FWD, 1, false, true>(c, MAVG_K_FWD, w, w, a, d, s, g, &f->h_k[l - 1])));
+        continue;
+      }
+      if (k > 1) FAC_TRY(gram(MAVG_K_FWD, f->h_k[l - 1], f->h_b[l - 1], in, 0, k));
+      if (l == L - 1)
+        FAC_TRY((launch_product<PROD_FWD, 2, true>(c, MAVG_K_FWD, w, f->w_lo, a, d, s, g)));
       else
-        FAC_TRY((launch_product<PROD_FWD, 1>(c, MAVG_K_FWD, st->wg[l], st->wg[l], f->in[l], f->g_mn[l], f->s_f[l], g)));
+        FAC_TRY((launch_product<PROD_FWD, 1>(c, MAVG_K_FWD, w, w, a, d, s, g)));
     }
     {
       LastArgs g{};
@@ -1419,13 +1533,18 @@ cudaError_t fac_local_steps(mavg_ctx* c, int64_t round) {
       FAC_TRY(cudaGetLastError());
     }
     for (int l = L - 1; l > 1; --l) {
-      if (k > 1) FAC_TRY(gram(MAVG_K_DGRAD, f->g_k[l], f->g_b[l], cfg.dims[l], 1, k));
       ProdArgs g = product(cfg.dims[l - 1], l - 1, f->dgrad[l]);
+      const CUtensorMap &w = st->wg_mn[l], &dz = f->dz_in[l], &a = f->h_mn[l - 1], &s = f->s_d[l];
       g.nkb = (cfg.dims[l] + kBK - 1) / kBK;
       g.out = bfp(t.g[l - 1]);
       g.act = bfp(t.h[l - 1]);
-      FAC_TRY((launch_product<PROD_DGRAD, 1>(c, MAVG_K_DGRAD, st->wg_mn[l], st->wg_mn[l], f->dz_in[l], f->h_mn[l - 1],
-                                             f->s_d[l], g)));
+      if (own_gram(f->dgrad[l], cfg.dims[l - 1])) {
+        with_gram(g, cfg.dims[l], 1);
+        FAC_TRY((launch_product<PROD_DGRAD, 1, false, true>(c, MAVG_K_DGRAD, w, w, dz, a, s, g, &f->g_k[l])));
+        continue;
+      }
+      if (k > 1) FAC_TRY(gram(MAVG_K_DGRAD, f->g_k[l], f->g_b[l], cfg.dims[l], 1, k));
+      FAC_TRY((launch_product<PROD_DGRAD, 1>(c, MAVG_K_DGRAD, w, w, dz, a, s, g)));
     }
   }
   {

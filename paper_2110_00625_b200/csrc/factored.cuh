@@ -33,7 +33,8 @@ struct FacLayout {
 };
 
 // Learners per block, columns per learner and block, column tiles per learner (more than 1 with nl 1 only).
-struct FacCols { int nl = 1, cols = 0, c_tiles = 1; };
+// own_gram: the product may form its Gram rows itself.
+struct FacCols { int nl = 1, cols = 0, c_tiles = 1; bool own_gram = false; };
 
 struct FacState {
   FacLayout lay;
