@@ -290,11 +290,43 @@ def algorithmic_bytes(cfg, tensor_path, deferred=False, momentum=False, fwd_run_
     return per_round
 
 
-def kernel_rooflines(cfg, prof, steps, peaks, tensor_path, deferred=False, momentum=False,
-                     fwd_run_tiles=(), dense_layers=(), fwd_whole_rows=(), split_layers=()):
+def factored_bytes(cfg, deferred=False, x_bytes=2):
+    """Bytes and flops per ROUND and kernel class of a round in factored form: products take w~ (read once
+    for all learners; the last hidden layer's forward product its low parts too) and the rows of the earlier
+    steps; the hidden layers' weights are written once, at the end."""
+    dims, P, K, B = cfg["dims"], cfg["P"], cfg["K"], cfg["B"]
+    L = len(dims) - 1
+    nW = [dims[l] * dims[l + 1] for l in range(L)]
+    n = sum(nW) + sum(dims[1:])
+    rows, all_rows = P * B, P * K * B
+    hist = P * B * K * (K - 1) // 2                       # history rows over all steps and learners
+    pairs = hist * B                                      # (batch row, history row) pairs
+    fwd = dict(bytes=2 * nW[0] + 2 * 2 * all_rows * dims[0] + 2 * 4 * all_rows * dims[1],   # X W~_1^T, X X^T, base
+               flops=2 * all_rows * nW[0] + 2 * pairs * (dims[0] + dims[1]))
+    fwd["bytes"] += 2 * 2 * pairs + 2 * (hist + all_rows) * dims[1]                          # F_1
+    dgrad = dict(bytes=0, flops=0)
+    for l in range(1, L - 1):                             # layer l + 1: dims[l] -> dims[l + 1]
+        parts = 2 if l == L - 2 else 1
+        fwd["bytes"] += (K * 2 * parts * nW[l] + 2 * all_rows * (2 * dims[l] + dims[l + 1])
+                         + 2 * hist * (dims[l] + dims[l + 1]) + 2 * 2 * pairs)
+        fwd["flops"] += 2 * all_rows * nW[l] * parts + 2 * pairs * (dims[l] + dims[l + 1])
+        dgrad["bytes"] += (K * 2 * nW[l] + 2 * all_rows * (2 * dims[l + 1] + 2 * dims[l])
+                           + 2 * hist * (dims[l] + dims[l + 1]) + 2 * 2 * pairs)
+        dgrad["flops"] += 2 * all_rows * nW[l] + 2 * pairs * (dims[l] + dims[l + 1])
+    hidden = nW[:-1]
+    return {
+        "meta_update": dict(bytes=((4 if deferred else 8) * P + 16) * n, flops=0),
+        "batch_gather": dict(bytes=all_rows * dims[0] * (x_bytes + 2), flops=0),
+        "fwd_gemm": fwd,
+        "loss": dict(bytes=2 * 2 * all_rows * dims[L - 1] + K * 8 * P * nW[-1], flops=6 * all_rows * nW[-1]),
+        "dgrad_gemm": dgrad,
+        "wgrad_sgd_gemm": dict(bytes=2 * all_rows * (sum(dims[:-2]) + sum(dims[1:-1])) + 4 * (1 + P) * sum(hidden),
+                               flops=2 * all_rows * sum(hidden)),
+    }
+
+
+def kernel_rooflines(per_round, prof, steps, peaks):
     """Per kernel class: algorithmic bytes or flops of all its launches / its summed device time."""
-    per_round = algorithmic_bytes(cfg, tensor_path, deferred, momentum, fwd_run_tiles, dense_layers,
-                                  fwd_whole_rows, split_layers)
     out = {}
     for name, (ms, cnt) in prof.items():
         if cnt == 0 or ms <= 0:
@@ -539,10 +571,16 @@ def measure_mlp(name, args, m, torch, dist, peaks, world, rank, local, steps, wi
     fwd_whole_rows = tuple(plan["fwd_whole_rows"]) if args.schedule == 0 else ()
     # every riding layer but the first keeps its masters split within a round
     split_layers = tuple(range(2, len(fwd_run_tiles) + 1))
-    kern = kernel_rooflines(cfg, prof, psteps, peaks, mode == 1, deferred=not args.no_defer,
-                            momentum=args.beta != 0.0, fwd_run_tiles=fwd_run_tiles,
-                            dense_layers=dense_layers, fwd_whole_rows=fwd_whole_rows,
-                            split_layers=split_layers)
+    factored = g.factored()
+    if factored:
+        fwd_run_tiles = dense_layers = fwd_whole_rows = ()
+        per_round = factored_bytes(cfg, deferred=not args.no_defer)
+    else:
+        per_round = algorithmic_bytes(cfg, mode == 1, deferred=not args.no_defer,
+                                      momentum=args.beta != 0.0, fwd_run_tiles=fwd_run_tiles,
+                                      dense_layers=dense_layers, fwd_whole_rows=fwd_whole_rows,
+                                      split_layers=split_layers)
+    kern = kernel_rooflines(per_round, prof, psteps, peaks)
     n = g.n
     g.close()
     del g, flush
@@ -571,17 +609,13 @@ def measure_mlp(name, args, m, torch, dist, peaks, world, rank, local, steps, wi
         roof["peak_source"] = peaks["source"]
         roof["bytes_per_launch"] = e["bytes_per_launch"]
         roof["ms_per_launch"] = e["ms_per_launch"]
-        if mode == 1 and not args.learners and not args.beta:
+        if mode == 1 and not args.learners and not args.beta and not factored:
             roof["traffic"] = NCU_TRAFFIC.get(name, {}).get(dom)
     # the whole round against the HBM roofline: every class's algorithmic bytes / the round's time
-    per_round = algorithmic_bytes(cfg, mode == 1, deferred=not args.no_defer,
-                                  momentum=args.beta != 0.0, fwd_run_tiles=fwd_run_tiles,
-                                  dense_layers=dense_layers, fwd_whole_rows=fwd_whole_rows,
-                                  split_layers=split_layers)
     round_bytes = sum(v["bytes"] for v in per_round.values())
     ms_round = total_ms / steps
     return dict(
-        cfg=cfg, n=n, units=units, fwd_run_tiles=fwd_run_tiles, dense_layers=dense_layers,
+        cfg=cfg, n=n, units=units, factored=factored, fwd_run_tiles=fwd_run_tiles, dense_layers=dense_layers,
         fwd_whole_rows=fwd_whole_rows, total_ms=total_ms, e2e_ms=e2e_ms, launches=launches,
         clocks=clocks, cpu=cpu, kern=kern, roof=roof, t_wall=t_wall, mode=mode,
         meta_in_round={"ms": statistics.median(meta_ms),
@@ -647,6 +681,8 @@ def run_mavg(args):
                        "l2_keep": bool(args.l2_keep),
                        "schedule": {0: "CUDA graph of per-product launches",
                                     2: "CUDA graph of per-product launches, plain tensor-core tiles"}[args.schedule],
+                       "local_steps": ("factored: products from w~ and the rows of the earlier steps, hidden weights "
+                                       "formed once per round" if r["factored"] else "weights stepped in place"),
                        "forward_products": (f"layers 1..{len(r['fwd_run_tiles'])} inside their weight-gradient "
                                             "launch of the step before (steps 2..K; partial sums per "
                                             f"{list(r['fwd_run_tiles'])} column tiles, after {list(r['fwd_whole_rows'])} "
@@ -654,6 +690,7 @@ def run_mavg(args):
                                             if r["fwd_run_tiles"] else "launches of their own"),
                        "first_step_forward": (f"layers {list(r['dense_layers'])}: one dense product over the "
                                               "batch rows of all learners" if r["dense_layers"]
+                                              else "all steps' rows as one dense product for layer 1" if r["factored"]
                                               else "per-learner tiles reading the one bf16 copy of the global model"),
                        "l2": "flushed between steps by a 256 MiB memset, outside the step's events",
                        "kernel_timing": "second pass over the same steps with one event pair per launch"},

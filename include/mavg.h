@@ -233,6 +233,10 @@ typedef enum {
 } mavg_plan_entry;
 mavg_status mavg_get_step_plan(mavg_handle h, int32_t *out);
 
+/* Measurement aid: whether the handle's next local steps, if they start from w~, run in factored form
+ * (MAVG_SCHED_GRAPH below), in which case the step plan above describes only calls that do not. */
+mavg_status mavg_get_factored(mavg_handle h, int32_t *factored);
+
 /* Measurement aid (the paper has no counterpart).  While profiling is on, every kernel launch of
  * this handle is bracketed by a pair of CUDA events on the stream.  mavg_get_profile waits for the
  * stream and returns, per kernel class, the summed device time in milliseconds and the number of
@@ -257,10 +261,16 @@ mavg_status mavg_set_profiling(mavg_handle h, int32_t on);
  *     or have little to do each (at most 32 classes and either few tiles, or fewer learners than SMs
  *     and few weights and batch rows) that layer -- forward, loss, dZ_L, its data gradient and the
  *     bias steps -- runs as one CUDA-core kernel, and hidden-layer forward products may split their
- *     contraction over a thread-block cluster.
+ *     contraction over a thread-block cluster.  Large rounds that start from w~ (8192 batch rows P K B
+ *     or more, at least two steps, no learner momentum, rows of a learner few against its weights) run
+ *     in factored form: W_l(k) = w~_l - gamma sum_{i<k} dZ_l(i)^T A_{l-1}(i) is not formed until the last
+ *     step, products take w~ and the factors instead.  w~ enters as bf16 (the last hidden layer's forward
+ *     product and the last layer: as two bf16 parts), the sums over the factors through bf16 Gram rows; the
+ *     plain form rounds W_l(k) to bf16 at every step.  mavg_workspace_bytes has room for it; a buffer
+ *     with room for the plain form only is accepted and keeps that.
  *   MAVG_SCHED_GRAPH_TC: the same graph with every product as plain one-tile-per-block
- *     tensor-core launches.  The two differ in the summation order of the products they run
- *     differently, nothing else; this one exists for comparison.
+ *     tensor-core launches.  Apart from factored rounds the two differ in the
+ *     summation order of the products they run differently, nothing else; this one exists for comparison.
  * Profiled rounds (mavg_set_profiling) take the launch-by-launch form of the chosen schedule; what is
  * one launch without profiling (the steps of a small CUDA-core model, a pseudo-gradient round) is one
  * launch with it. */

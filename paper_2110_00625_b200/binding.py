@@ -21,7 +21,7 @@ EXPORTS = ["mavg_workspace_bytes", "mavg_create", "mavg_local_steps", "mavg_meta
            "mavg_materialize_replicas", "mavg_round", "mavg_round_host", "mavg_set_hparams",
            "mavg_set_learner_momentum", "mavg_get_batch_indices",
            "mavg_get_losses", "mavg_get_round", "mavg_set_round", "mavg_get_launch_count",
-           "mavg_get_step_plan", "mavg_set_profiling", "mavg_set_schedule", "mavg_get_profile", "mavg_sync",
+           "mavg_get_step_plan", "mavg_get_factored", "mavg_set_profiling", "mavg_set_schedule", "mavg_get_profile", "mavg_sync",
            "mavg_set_wait_limit", "mavg_selftest_wait", "mavg_cache_release", "mavg_last_error",
            "mavg_batch_indices_noalloc", "mavg_destroy"]
 KERNEL_CLASSES = ["meta_update", "broadcast", "pseudograd_steps", "batch_gather", "fwd_gemm",
@@ -92,6 +92,7 @@ def load_library():
     L.mavg_set_round.argtypes = [H, C.c_int64]
     L.mavg_get_launch_count.argtypes = [H, C.POINTER(C.c_int64)]
     L.mavg_get_step_plan.argtypes = [H, C.POINTER(C.c_int32)]
+    L.mavg_get_factored.argtypes = [H, C.POINTER(C.c_int32)]
     L.mavg_set_profiling.argtypes = [H, C.c_int32]
     L.mavg_set_schedule.argtypes = [H, C.c_int32]
     L.mavg_get_profile.argtypes = [H, C.c_void_p, C.c_void_p, C.c_int32]
@@ -279,6 +280,12 @@ class Mavg:
                 "fwd_run_tiles": list(out[3:3 + out[2]]),
                 "fwd_whole_rows": list(out[4 + MAX_LAYERS:4 + MAX_LAYERS + out[2]]),
                 "dense_first_step": [l + 1 for l in range(MAX_LAYERS) if out[3 + MAX_LAYERS] >> l & 1]}
+
+    def factored(self):
+        """Whether the next local steps run in factored form if they start from w~ (see mavg_set_schedule)."""
+        r = C.c_int32()
+        self._check(self.lib.mavg_get_factored(self.handle, C.byref(r)))
+        return bool(r.value)
 
     def set_profiling(self, on):
         self._check(self.lib.mavg_set_profiling(self.handle, int(bool(on))))

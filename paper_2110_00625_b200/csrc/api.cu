@@ -511,6 +511,12 @@ mavg_status mavg_get_step_plan(mavg_handle h, int32_t* out) {
   return MAVG_OK;
 }
 
+mavg_status mavg_get_factored(mavg_handle h, int32_t* factored) {
+  if (!h || !factored) return MAVG_ERR_INVALID_ARG;
+  *factored = h->cfg.objective == MAVG_OBJ_MLP && mlp_factored(h) ? 1 : 0;
+  return MAVG_OK;
+}
+
 mavg_status mavg_set_profiling(mavg_handle h, int32_t on) {
   CHECK_HANDLE(h);
   h->profiling = on != 0;

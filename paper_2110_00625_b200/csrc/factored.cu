@@ -930,7 +930,8 @@ __device__ __forceinline__ bool group_any(bool pred, int id) {
 // before it is subtracted from w~ and stored.
 // Bound by what an SM takes in (48 KB of operands per 4.2 Mflop, w~ once more per learner): 1.01 ms at
 // n = 14.7 M, P = 32, 1024 rows = 950 TFLOP/s; the weight-gradient launches it replaces took 12 ms there.
-// Two stages and four pieces per group: 156 us against 131 at n = 1.84 M, P = 48, 512 rows.
+// n = 1.84 M, P = 48, 512 rows: 131 us.  Two stages and four pieces per group: 156 there; tiles of 256 x 256,
+// which take in a third less but leave no room for a second accumulator or a third stage: 185 and 1.26 ms.
 // STAGES operand slabs of 64 rows; PIECES buffers per epilogue group, of which a piece is worked on, one or
 // two are being fetched and the rest is being stored.
 template <int STAGES, int PIECES>
@@ -1199,8 +1200,11 @@ cudaError_t launch_product(mavg_ctx* c, int cls, const CUtensorMap& w, const CUt
   g.stages = stages_for(std::max(1, g.gram_nkb + g.nkb + g.nl * hist_stages), stage_bytes, (long)grid.x * grid.y,
                         c->sm_count);
   g.tmem_cols = tmem_columns(GRAM ? gram_columns({1, g.cols, g.c_tiles}, g.m_tiles, g.hist) : g.nl * g.cols);
-  const size_t smem = (size_t)g.stages * stage_bytes + 1024 +
-                      (EPI == PROD_DGRAD ? (size_t)2 * g.nl * kBM * sizeof(float) : 0);
+  size_t smem = (size_t)g.stages * stage_bytes + 1024 +
+                (EPI == PROD_DGRAD ? (size_t)2 * g.nl * kBM * sizeof(float) : 0);
+  // Blocks that wait on one another must all get their tensor memory: no more of them on an SM than it has
+  // columns for, or two clusters could each hold what the other's last block is waiting for.
+  if (GRAM) smem = std::max(smem, (size_t)228 * 1024 / (512 / g.tmem_cols + 1) + 1024);
   PdlLaunch l(grid, kFacThreads, smem, c->stream, GRAM ? (int)grid.x : EPI == PROD_DGRAD ? g.c_tiles : 1);
   prof_begin(c, cls);
   cudaError_t e = cudaLaunchKernelEx(&l.lc, k_fac_product<EPI, TILES, LOW, GRAM>, w, lo, in, gram ? *gram : in, hist, s, g);
@@ -1369,7 +1373,7 @@ mavg_status fac_setup(mavg_ctx* c, TcState* st, std::string* why) {
 
 bool fac_usable(const mavg_ctx* c) {
   const TcState* st = (const TcState*)c->mlp;
-  return st->fac && c->replicas_equal_global && c->schedule == 0 && c->cfg.learner_momentum == 0.f &&
+  return st && st->fac && c->schedule == 0 && c->cfg.learner_momentum == 0.f &&
          c->cfg.K <= st->fac->K && enough_rows(&c->cfg, c->cfg.K);
 }
 

@@ -671,6 +671,8 @@ void tc_reset_counters(mavg_ctx* c) {
   cudaMemsetAsync(ws + st->lay.zcount, 0, st->lay.zcount_bytes, c->stream);
 }
 
+bool tc_factored(const mavg_ctx* c) { return fac_usable(c); }
+
 void tc_step_plan(mavg_ctx* c, int32_t* out) {
   const TcState* st = (const TcState*)c->mlp;
   if (!st) return;
@@ -727,7 +729,7 @@ cudaError_t tc_refresh_shared_operands(mavg_ctx* c) {
 }
 
 cudaError_t tc_local_steps(mavg_ctx* c, int64_t round) {
-  if (fac_usable(c)) {
+  if (c->replicas_equal_global && fac_usable(c)) {
     cudaError_t e = fac_local_steps(c, round);
     if (e != cudaSuccess) return e;
     tc_set_w16_cur(c, kW16Stale);

@@ -61,3 +61,21 @@ def test_split_masters_remove_the_copy_on_top_of_the_master():
     saved = 15 * 32 * 2 * 2 * 2048 * 2048         # K - 1 steps, P learners, 2 bytes, two layers
     assert fp32["wgrad_sgd_gemm"]["bytes"] - split["wgrad_sgd_gemm"]["bytes"] == saved
     assert all(fp32[k] == split[k] for k in fp32 if k != "wgrad_sgd_gemm")
+
+
+def test_factored_rounds_write_the_weights_once_and_grow_with_the_history():
+    b = _bench()
+    per = b.factored_bytes(CFG, deferred=True)
+    nW = [3072 * 2048, 2048 * 2048, 2048 * 2048]
+    P, K, B = 32, 16, 64
+    R = P * K * B
+    assert per["wgrad_sgd_gemm"] == dict(bytes=2 * R * (3072 + 3 * 2048 + 2 * 2048) + 4 * 33 * sum(nW),
+                                         flops=2 * R * sum(nW))
+    # a round of one step has no history: the products of the plain form's first step, read once for all
+    one = b.factored_bytes(dict(CFG, K=1))
+    assert one["fwd_gemm"]["flops"] == 2 * P * B * (nW[0] + nW[1] + 2 * nW[2])
+    assert one["dgrad_gemm"]["flops"] == 2 * P * B * (nW[1] + nW[2])
+    # the history of step k is (k - 1) B rows a learner: K (K - 1) / 2 batches in all
+    two, four = (b.factored_bytes(dict(CFG, K=k))["dgrad_gemm"]["flops"] for k in (2, 4))
+    extra = lambda k, f: f - k * one["dgrad_gemm"]["flops"]
+    assert extra(4, four) == 6 * extra(2, two) == 6 * 2 * P * B * B * 2 * (2048 + 2048)

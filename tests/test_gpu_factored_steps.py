@@ -165,3 +165,25 @@ def test_where_the_form_is_taken():
         ([400, 400, 10], 8, 8, 128, {}, False), ([1000, 10], 32, 2, 128, {}, False),
     ]:
         assert _factored(dims, P, K, B, **kw) == want, (dims, P, K, B, kw)
+
+
+def test_a_workspace_of_the_plain_forms_size_keeps_that_form():
+    # buffers sized before the form existed: a handle of one step has no use for more than the plain form needs
+    import ctypes as C
+    from paper_2110_00625_b200 import binding
+    dims, P, K, B = SHAPES[-1]
+    g, _ = _handle(dims, P, K, B)
+    assert g.factored()
+    one, plain = binding.Config.from_buffer_copy(g.cfg), C.c_size_t()
+    one.K = 1
+    assert g.lib.mavg_workspace_bytes(C.byref(one), C.byref(plain)) == 0
+    buf = binding.Buffers.from_buffer_copy(g.buf)
+    buf.workspace_bytes = plain.value + 4 * P * K + 256          # the losses of K steps
+    assert buf.workspace_bytes < g.workspace.numel()
+    h, used = C.c_void_p(), C.c_int32(-1)
+    assert g.lib.mavg_create(C.byref(g.cfg), C.byref(buf), C.byref(h)) == 0
+    assert g.lib.mavg_get_factored(h, C.byref(used)) == 0 and used.value == 0
+    assert g.lib.mavg_round(h, None) == 0 and g.lib.mavg_sync(h) == 0
+    assert torch.isfinite(g.w).all()
+    g.lib.mavg_destroy(h)
+    g.close()
