@@ -405,7 +405,9 @@ mavg_status mavg_round_host(mavg_handle h, float* w_host, float* v_host, float* 
   CU(h, cudaStreamWaitEvent(h->s_copy, h->ev_copy_fork, 0), "copy fork");
   CU(h, cudaMemcpyAsync(h->buf.momentum, v_host, bytes, cudaMemcpyHostToDevice, h->s_copy), "v upload");
   CU(h, cudaEventRecord(h->ev_copy_done, h->s_copy), "copy join");
-  CU(h, launch_broadcast(h, false), "re-broadcast");
+  // the tensor-core path's local steps read w~ itself: P copies would be overwritten unread
+  if (h->cfg.objective == MAVG_OBJ_MLP && h->cfg.gemm_bf16 == 1) h->replicas_materialized = false;
+  else CU(h, launch_broadcast(h, false), "re-broadcast");
   h->replicas_equal_global = true;
   if (h->cfg.objective == MAVG_OBJ_MLP)
     CU(h, mlp_refresh_shared_operands(h), "operand refresh");
