@@ -379,7 +379,12 @@ cudaError_t launch_meta_update(mavg_ctx* c) {
   prof_begin(c, MAVG_K_META);
   cudaError_t e = cudaSuccess;
   c->shadow_fresh = false;
-  if (big && n >= (int64_t)4096 * c->sm_count * 4) {
+  // Shorter vectors leave its blocks few tiles each.  Where the copies are written it still pays for many
+  // replicas (us, register / bulk kernel: n = 1.84 M, P = 24 70 / 68, P = 48 136 / 125; n = 2.1 M, P = 64 203 / 182;
+  // n = 1.2 M, P = 32 57 / 57, P = 48 88 / 82), not for fewer or below (n = 1.84 M, P = 16 48 / 52; n = 0.9 M, P = 64
+  // 76 / 81) and not with deferred copies (n = 1.84 M, P = 48 63 / 69).
+  const bool many = bcast && P >= 24 && n >= 1200000 && (int64_t)P * n >= 44000000;
+  if (big && (many || n >= (int64_t)4096 * c->sm_count * 4)) {
     if (P <= 4) e = launch_bulk<2048, 4, 3, 256>(c, mu, zeta, inv_p, read_v, bcast);
     else if (P <= 8 || P >= 24) e = launch_bulk<2048, 6, 2, 512>(c, mu, zeta, inv_p, read_v, bcast);
     else e = launch_bulk<4096, 3, 2, 512>(c, mu, zeta, inv_p, read_v, bcast);

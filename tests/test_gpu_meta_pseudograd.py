@@ -107,6 +107,26 @@ def test_meta_update_bulk_kernel_rings_and_ragged_end(oracle, n, P, mu, defer):
     g.close()
 
 
+@pytest.mark.parametrize("n,P", [(1_200_000, 37), (1_833_335, 24), (1_200_003, 65)])
+def test_meta_update_bulk_kernel_on_short_vectors_with_many_replicas(oracle, n, P):
+    # few tiles per block: fewer than the ring holds, and ragged ends of 0 and 3
+    m = _mavg()
+    w1 = m.workloads.global_model(n, seed=9)
+    g = m.Mavg(w1, P=P, K=1, local_lr=0.1, mu=0.9, objective=m.OBJ_NONE)
+    o = oracle.Mavg(w1, P=P, K=1, gamma=0.1, mu=0.9, stride=g.stride)
+    for u in range(2):
+        reps = m.workloads.perturbed_replicas(o.w, P, 0.1, update=u, seed=21, stride=g.stride)
+        o.replicas[:] = reps
+        g.replicas.copy_(torch.from_numpy(reps))
+        g.meta_update()
+        o.meta_update()
+    g.sync()
+    assert rel_err(g.w.cpu().numpy(), o.w) <= META_TOL
+    assert rel_err(g.v.cpu().numpy(), o.v) <= META_TOL
+    assert (g.replicas[:, :n] == g.w).all()
+    g.close()
+
+
 @pytest.mark.parametrize("K", [1, 4, 16, 64])
 @pytest.mark.parametrize("mu", [0.0, 0.9])
 def test_pseudograd_rounds(oracle, K, mu):
