@@ -1256,11 +1256,13 @@ bool enough_rows(const mavg_config* cfg, int K) { return K >= 2 && (int64_t)cfg-
 // Speed: what it saves goes with the weights (none is read or written per learner and step), what it adds
 // with the square of a learner's rows K B: the Gram products and the products with them,
 // K B (d_0 + d_1 + 2 sum_{l>=2} (d_{l-1} + d_l)) multiply-adds per row against one per hidden weight and
-// product.  Taken below a ratio of 5 (plain / factored, us a round): 3072-2048-2048-2048-10, P = 32,
-// K = 16, B = 64 (ratio 1.6) 15180 / 5600; 3072-512-512-10, P = 48, K = 8, B = 64 (1.6) 1860 / 848, P = 8,
-// B = 128 (3.2) 623 / 486; 2344-344-344-4, P = 15, K = 5, B = 176 (3.9) 588 / 505; 1504-672-672-11, P = 10,
-// K = 8, B = 176 (4.7) 951 / 758; beyond: 1200-272-272-6, P = 10, K = 5, B = 176 (5.6) 324 / 355;
-// 560-648-2, P = 5, K = 7, B = 240 (5.6) 232 / 271; 2232-128-128-13, P = 7, K = 9, B = 208 (18) 602 / 800.
+// product.  Taken below a ratio of 5, from 11 learners on (whose launches fill the chip) below 6 (plain /
+// factored, us a round): 3072-2048-2048-2048-10, P = 32, K = 16, B = 64 (ratio 1.6) 15180 / 5600;
+// 3072-512-512-10, P = 48, K = 8, B = 64 (1.6) 1860 / 848, P = 8, B = 128 (3.2) 623 / 457.
+// 17 drawn models of ratios 3.6 to 6, P >= 8: all faster, least 1584-168-168-11, P = 36, K = 5, B = 128 (5.3)
+// 436 / 415, 720-688-688-21, P = 11, K = 14, B = 96 (5.8) 1092 / 933; beyond: few learners 560-648-2, P = 5, K = 7,
+// B = 240 (5.6) 232 / 271, 1584-528-528-7, P = 6, K = 7, B = 240 (6.4) 627 / 715; many, either way: 784-232-2,
+// P = 34, K = 8, B = 176 (7.9) 405 / 486, 2432-512-512-27, P = 26, K = 10, B = 240 (7.9) 2807 / 1949.
 // Models of fewer than 48 K hidden weights keep the plain form: a round is a chain of short launches either
 // way (128-128-128-10, P = 148, B = 32: K = 2 124 / 103, K = 8 371 / 371; 256-128-10, P = 64, K = 4 119 / 110).
 // Results: the plain form rounds W_l(k) to bf16 at every step, this one rounds w~ and the Gram rows.  Both are
@@ -1278,7 +1280,7 @@ int fac_steps(const mavg_config* cfg) {
     weights += (int64_t)cfg->dims[l - 1] * cfg->dims[l];
   }
   if (weights < 48 * 1024) return 0;
-  const int most = (int)std::min<int64_t>({cfg->K, 4096 / B, (5 * weights - 1) / (span * B)});
+  const int most = (int)std::min<int64_t>({cfg->K, 4096 / B, ((cfg->P >= 11 ? 6 : 5) * weights - 1) / (span * B)});
   return enough_rows(cfg, most) && last_plan(cfg).smem <= kLastSmem ? most : 0;
 }
 

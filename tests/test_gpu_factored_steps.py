@@ -158,11 +158,12 @@ def test_steps_of_length_zero_keep_every_bit(dims, P, K, B):
 
 
 def test_where_the_form_is_taken():
-    # both sides of its lines: 8192 rows a round, five times the weights, two steps, learner momentum
+    # both sides of its lines: 8192 rows a round, the added work (P = 8: 5 times the weights, P = 11: 6), two steps, momentum
     for dims, P, K, B, kw, want in [
         ([1000, 312, 10], 32, 2, 128, {}, True), ([1000, 312, 10], 31, 2, 128, {}, False),
         ([1000, 312, 10], 64, 1, 128, {}, False), ([1000, 312, 10], 32, 2, 128, dict(learner_momentum=0.9), False),
-        ([400, 400, 10], 8, 8, 128, {}, False), ([1000, 10], 32, 2, 128, {}, False),
+        ([400, 400, 10], 8, 8, 128, {}, False),
+    ([400, 400, 10], 11, 9, 128, {}, True), ([400, 400, 10], 11, 10, 128, {}, False), ([1000, 10], 32, 2, 128, {}, False),
     ]:
         assert _factored(dims, P, K, B, **kw) == want, (dims, P, K, B, kw)
 
