@@ -367,7 +367,7 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     const int row = q4 * 32 + lane, m = m0 + row;
     const bool m_ok = m < g.M;
     if (GRAM) {
-      if (m0 < g.hist && mbar_wait(&gram_bar, 0, abortp, g.status, ERR_EPILOGUE)) {
+      if (m0 < g.hist && mbar_wait_warp(&gram_bar, 0, abortp, g.status, ERR_EPILOGUE)) {
         tc_fence_after_sync();
         uint32_t d = tmem_base + ((uint32_t)(q4 * 32) << 16) + (uint32_t)N;
         for (int s0 = m0; s0 < g.hist; s0 += gram_step, d += (uint32_t)g.cols) {
@@ -375,7 +375,6 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
 #pragma unroll 1
           for (int c0 = half * 16; c0 < g.cols; c0 += 32) {
             float z[16];
-            __syncwarp();
             load16(d + (uint32_t)c0, true, z);
             if (s >= g.hist) continue;
             __nv_bfloat16* dst = g.gram_out + (size_t)p0 * g.gram_stride + (size_t)(s_row + c0) * g.gram_ld + s;
@@ -423,7 +422,7 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
 #pragma unroll
     for (int j = 0; j < 16; ++j) { zb[j] = 0.f; act[j] = __float2bfloat16_rn(0.f); }
     fetch(half * 16);
-    const bool ok = !any || mbar_wait(&sh.acc_bar, 0, abortp, g.status, ERR_EPILOGUE);
+    const bool ok = !any || mbar_wait_warp(&sh.acc_bar, 0, abortp, g.status, ERR_EPILOGUE);
     if (ok) {
       tc_fence_after_sync();
       const uint32_t lane_addr = tmem_base + ((uint32_t)(q4 * 32) << 16);
@@ -433,7 +432,6 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
         int q;
         locate(c0, at, z_at, q);
         float z[16];
-        __syncwarp();
         load16(lane_addr + (uint32_t)c0, any, z);
         if (EPI == PROD_FWD) {
 #pragma unroll
@@ -589,7 +587,7 @@ k_fac_gram(const __grid_constant__ CUtensorMap tm_hist, const __grid_constant__ 
   } else {
     const int q4 = warp & 3, half = (warp - 2) >> 2;
     const int s = s0 + q4 * 32 + lane;
-    if (mbar_wait(&sh.acc_bar, 0, abortp, g.status, ERR_EPILOGUE)) {
+    if (mbar_wait_warp(&sh.acc_bar, 0, abortp, g.status, ERR_EPILOGUE)) {
       tc_fence_after_sync();
       const uint32_t lane_addr = tmem_base + ((uint32_t)(q4 * 32) << 16);
 #pragma unroll 1
@@ -1075,11 +1073,9 @@ k_fac_apply(const __grid_constant__ ApplyArgs g) {
           asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kStores) : "memory");
           fetch();
         }
-        __syncwarp();
         uint32_t acc[32];
         tmem_ld_32x32(tmem_base + ((uint32_t)(q4 * 32) << 16) + b * kApplyBN + (uint32_t)(c * kApplyChunk), acc);
         if (!mbar_wait(&sh.piece_full[grp][s], (pn / PIECES) & 1, abortp, g.status, ERR_EPILOGUE)) failed = true;
-        __syncwarp();
         tmem_ld_wait();
         uint8_t* wrow = mine + (size_t)s * kPieceBytes + (size_t)row * 128;
 #pragma unroll

@@ -112,7 +112,7 @@ k_fwd_dense(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
     const int m = m0 + q * 32 + lane;
     const bool m_ok = m < g.M;
     const float bias = m_ok ? g.bias[m] : 0.f;
-    if (mbar_wait(&sh.acc_bar, 0, abortp, g.status, ERR_EPILOGUE)) {
+    if (mbar_wait_warp(&sh.acc_bar, 0, abortp, g.status, ERR_EPILOGUE)) {
       tc_fence_after_sync();
       const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
       for (int c0 = half * 32; c0 < kDenseCols; c0 += 64) {

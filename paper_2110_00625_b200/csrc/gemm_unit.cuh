@@ -215,7 +215,7 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
     int label_pre = 0;
     if (EPI == EPI_FWD_LAST && ew * 32 + lane < g.N)
       label_pre = g.labels[(size_t)p * g.N + ew * 32 + lane];
-    const bool ok = mbar_wait(&sh.acc_bar, acc_phase & 1, abortp, g.status, ERR_EPILOGUE);
+    const bool ok = mbar_wait_warp(&sh.acc_bar, acc_phase & 1, abortp, g.status, ERR_EPILOGUE);
     tc_fence_after_sync();
     const uint32_t lane_addr = tmem_base + ((uint32_t)(q * 32) << 16);
     {
@@ -256,6 +256,7 @@ __device__ __forceinline__ void gemm_tile(const CUtensorMap& tmA, const CUtensor
               }
             }
           }
+          got = __all_sync(0xffffffffu, got);
           if (got) {
             // eight columns at a time in a loop that is not unrolled (see the note on the compact
             // tails below); partials added in ascending rank order, this block's own from TMEM

@@ -307,8 +307,8 @@ __device__ __forceinline__ void wgrad_run(const CUtensorMap& tm_dzt, const CUten
         const uint32_t use = tile_ctr / g.slots;
         const uint32_t tuse = tile_ctr >> 1;
         // the master tile landed with the same barrier the MMA waited on; the accumulator next
-        if (!mbar_wait(&sh.slot_full[s], use & 1, abortp, g.status, ERR_WG_EPILOGUE) ||
-            !mbar_wait(&sh.tmem_full[grp], tuse & 1, abortp, g.status, ERR_WG_EPILOGUE)) {
+        if (!mbar_wait_warp(&sh.slot_full[s], use & 1, abortp, g.status, ERR_WG_EPILOGUE) ||
+            !mbar_wait_warp(&sh.tmem_full[grp], tuse & 1, abortp, g.status, ERR_WG_EPILOGUE)) {
           ok = false;
           break;
         }
@@ -388,7 +388,7 @@ __device__ __forceinline__ void wgrad_run(const CUtensorMap& tm_dzt, const CUten
           if (in_split != out_split) {
             __syncwarp();
             if (lane == 0) mbar_arrive(&sh.reshape[grp]);
-            if (!mbar_wait(&sh.reshape[grp], tuse & 1, abortp, g.status, ERR_WG_EPILOGUE)) {
+            if (!mbar_wait_warp(&sh.reshape[grp], tuse & 1, abortp, g.status, ERR_WG_EPILOGUE)) {
               ok = false;
               break;
             }
@@ -579,7 +579,7 @@ __device__ __forceinline__ void wgrad_run(const CUtensorMap& tm_dzt, const CUten
 #pragma unroll
         for (int jj = 0; jj < 16; ++jj) dbm[(size_t)jj * g.out_rows] = hh[jj];
       };
-      if (!mbar_wait_relaxed(&sh.z_full, item_ctr & 1, abortp, g.status, ERR_WG_EPILOGUE, 400)) break;
+      if (!__all_sync(0xffffffffu, mbar_wait_relaxed(&sh.z_full, item_ctr & 1, abortp, g.status, ERR_WG_EPILOGUE, 400))) break;
       tc_fence_after_sync();
       float* zbase = g.zpart + ((size_t)p * g.m_tiles + mt) * g.n_chunks * tile_floats + r;
       float* zp = zbase + (size_t)(nt0 / g.chunk) * tile_floats;
@@ -616,7 +616,7 @@ __device__ __forceinline__ void wgrad_run(const CUtensorMap& tm_dzt, const CUten
         mbar_arrive(&sh.z_flag);
       }
       __syncwarp();
-      if (!mbar_wait(&sh.z_flag, split_ctr & 1, abortp, g.status, ERR_WG_EPILOGUE)) break;
+      if (!mbar_wait_warp(&sh.z_flag, split_ctr & 1, abortp, g.status, ERR_WG_EPILOGUE)) break;
       ++split_ctr;
       if (!sh.z_last) continue;
       for (int c0 = 0; c0 < g.batch; c0 += 16) {
