@@ -264,9 +264,9 @@ mavg_status mavg_set_profiling(mavg_handle h, int32_t on);
  *     contraction over a thread-block cluster.  Large rounds that start from w~ (8192 batch rows P K B
  *     or more, at least two steps, no learner momentum, rows of a learner few against its weights) run
  *     in factored form: W_l(k) = w~_l - gamma sum_{i<k} dZ_l(i)^T A_{l-1}(i) is not formed until the last
- *     step, products take w~ and the factors instead.  w~ enters as bf16 (the last hidden layer's forward
- *     product and the last layer: as two bf16 parts), the sums over the factors through bf16 Gram rows; the
- *     plain form rounds W_l(k) to bf16 at every step.  mavg_workspace_bytes has room for it; a buffer
+ *     step, products take w~ and the factors instead.  w~ enters the forward products and the last layer as
+ *     two bf16 parts and the data gradients as one, the sums over the factors through bf16 Gram rows; the plain
+ *     form rounds W_l(k) to bf16 at every step.  mavg_workspace_bytes has room for it; a buffer
  *     with room for the plain form only is accepted and keeps that.
  *   MAVG_SCHED_GRAPH_TC: the same graph with every product as plain one-tile-per-block
  *     tensor-core launches.  Apart from factored rounds the two differ in the

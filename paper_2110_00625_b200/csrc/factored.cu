@@ -79,18 +79,23 @@ __device__ __forceinline__ uint4 load8_bf16<float>(const float* src) {
   return *reinterpret_cast<uint4*>(h);
 }
 
-// What the bf16 copy of w~'s last hidden layer leaves over, as bf16: that layer's forward product and the last
-// layer read both parts (16 bits of the weights).  A rounding of the weights is the same for every sample and
-// learner, so it is what the error of a round's mean loss consists of; two layers next to the loss carry most
-// of it.  Root mean square against 64 bits, 14 seeds (plain form / this one without / with the low
-// parts): 3072-512-512-10, P = 8, K = 8, B = 128 8.1e-5 / 9.2e-5 / 2.0e-5; 1000-200-200-20, P = 20, K = 5,
-// B = 96 5.8e-5 / 8.2e-5 / 1.7e-5; one hidden layer (2000-400-10, P = 16, K = 4, B = 128), where only the last
-// layer takes them, 6.6e-5 / 6.5e-5 / 1.4e-5.  Layer 1's would not help (1.5e-5 for 2.0e-5 above) and cost most.
+// What the bf16 copy of w~'s hidden layers leaves over, as bf16: the forward products and the last layer read
+// both parts (16 bits of the weights).  A rounding of the weights is the same for every sample, step and learner
+// here, where the plain form rounds each learner's own weights at every step, so it does not average out: with
+// one bf16 part v or the mean loss can be further from 64 bits than the plain form's.  Root mean square of
+// v's relative error and of the mean loss's error over 12 seeds, plain / one part / both parts in every hidden layer:
+//   1000-312-10, P = 40, K = 4, B = 80:            v 3.6e-3 / 3.9e-3 / 0.4e-3, loss 1.1e-4 / 0.7e-4 / 0.4e-4
+//   the same, inputs in [0, 1]:                    v 1.8e-3 / 2.0e-3 / 0.6e-3, loss 2.9e-4 / 3.3e-4 / 0.1e-4
+//   520-200-136-12, P = 20, K = 9, B = 48, [0, 1]: v 3.0e-3 / 3.2e-3 / 2.1e-3, loss 2.1e-4 / 2.4e-4 / 0.3e-4
+//   3072-512-512-10, P = 8, K = 8, B = 128:        v 7.9e-3 / 7.7e-3 / 4.7e-3, loss 2.5e-4 / 0.7e-4 / 0.5e-4
+//   2048-1024-1024-1024-10, P = 8, K = 8, B = 128, inputs >= 0: v 6.3e-3 / 6.2e-3 / 4.5e-3, loss 1.6e-4 / 1.4e-4 / 0.3e-4
+// (the last with low parts in the first and last hidden layer only: loss 1.6e-4).  Low parts in the data gradients
+// and Gram rows of two parts change none of these by more than a tenth.
 struct LowArgs {
-  const float* w;           // the layer in w~
-  __nv_bfloat16* dst;
-  int64_t total;            // weights, a multiple of 8
-  int blocks;               // blocks of the launch that do this
+  const float* w[MAVG_MAX_LAYERS - 1];            // the hidden layers in w~
+  __nv_bfloat16* dst[MAVG_MAX_LAYERS - 1];
+  int64_t total[MAVG_MAX_LAYERS - 1];             // weights, a multiple of 8
+  int layers, blocks;                             // blocks of the launch that do this
 };
 __device__ __forceinline__ uint32_t low_pair(float a, float b) {
   const __nv_bfloat162 hi = __floats2bfloat162_rn(a, b);
@@ -108,10 +113,11 @@ template <typename TIN>
 __global__ void __launch_bounds__(256)
 k_fac_gather(const TIN* __restrict__ x, const int32_t* __restrict__ y, uint64_t seed, int64_t round,
              const int64_t* __restrict__ round_ptr, int P, int K, int B, int64_t kb, int64_t S, int d,
-             int32_t* __restrict__ labels, __nv_bfloat16* __restrict__ out, const LowArgs la) {
+             int32_t* __restrict__ labels, __nv_bfloat16* __restrict__ out, const __grid_constant__ LowArgs la) {
   if ((int)blockIdx.x < la.blocks) {
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < la.total >> 3; t += (int64_t)la.blocks * blockDim.x)
-      reinterpret_cast<uint4*>(la.dst)[t] = low8(la.w + 8 * t);
+    for (int l = 0; l < la.layers; ++l)
+      for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < la.total[l] >> 3; t += (int64_t)la.blocks * blockDim.x)
+        reinterpret_cast<uint4*>(la.dst[l])[t] = low8(la.w[l] + 8 * t);
     return;
   }
   const int64_t row = (int64_t)(blockIdx.x - la.blocks) * 8 + (threadIdx.x >> 5);
@@ -169,8 +175,9 @@ struct ProdArgs {
   int* status;
 };
 
-__host__ __device__ __forceinline__ int product_stage_bytes(int tiles, int nl, int cols) {
-  return tiles * kATileBytes + (nl > tiles ? nl : tiles) * cols * kBK * 2;      // one batch operand or Gram rows per tile
+// One batch operand, or Gram rows for each of `grams` history tiles.
+__host__ __device__ __forceinline__ int product_stage_bytes(int tiles, int grams, int nl, int cols) {
+  return tiles * kATileBytes + (nl > grams ? nl : grams) * cols * kBK * 2;
 }
 
 __device__ __forceinline__ void load16(uint32_t taddr, bool any, float (&z)[16]) {
@@ -216,7 +223,7 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
   static_assert(!LOW || TILES == 2, "");
   constexpr bool kMn = EPI == PROD_DGRAD;          // w~ is read MN-major
   constexpr int kBOff = TILES * kATileBytes;
-  const int stage_bytes = product_stage_bytes(TILES, g.nl, g.cols), s_bytes = g.cols * kBK * 2;
+  const int stage_bytes = product_stage_bytes(TILES, EPI == PROD_RAW ? 1 : TILES, g.nl, g.cols), s_bytes = g.cols * kBK * 2;
   __shared__ __align__(8) uint64_t gram_bar, rows_bar;     // GRAM: Gram sums complete; Gram rows in global memory
 
   if (threadIdx.x == 0) {
@@ -1176,9 +1183,11 @@ uint32_t tmem_columns(int n) {
   return c;
 }
 
-// Two blocks share an SM where there are more blocks than SMs.
+// Two blocks share an SM where there are more blocks than SMs and two stages leave room for them: not with
+// two tiles to a stage and 128 columns or more (64 KB).
 int stages_for(int slabs, int stage_bytes, long blocks, int sm_count) {
-  return std::max(2, std::min({kMaxStages, slabs, (blocks > sm_count ? 96 : 196) * 1024 / stage_bytes}));
+  const int budget = (blocks > sm_count && stage_bytes <= 48 * 1024 ? 96 : 196) * 1024;
+  return std::max(2, std::min({kMaxStages, slabs, budget / stage_bytes}));
 }
 
 template <int EPI, int TILES, bool LOW = false, bool GRAM = false>
@@ -1190,7 +1199,7 @@ cudaError_t launch_product(mavg_ctx* c, int cls, const CUtensorMap& w, const CUt
   g.rep_stride = c->buf.replica_stride;
   g.bias_rep = c->buf.replicas;
   g.status = (int*)ws_ptr(c, c->ws.status);
-  const int stage_bytes = product_stage_bytes(TILES, g.nl, g.cols);
+  const int stage_bytes = product_stage_bytes(TILES, EPI == PROD_RAW ? 1 : TILES, g.nl, g.cols);
   const dim3 grid((unsigned)(g.m_tiles * g.c_tiles), (unsigned)((g.P + g.nl - 1) / g.nl));
   const int hist_stages = ((g.hist + kBK - 1) / kBK + TILES - 1) / TILES;
   g.stages = stages_for(std::max(1, g.gram_nkb + g.nkb + g.nl * hist_stages), stage_bytes, (long)grid.x * grid.y,
@@ -1298,7 +1307,7 @@ FacLayout fac_layout(const mavg_config* cfg, size_t base) {
   t.s1 = t.in_rows ? z_bytes : take(P * s_bytes);
   for (size_t& s : t.s) s = take((size_t)P * B * t.s_ld * 2);
   t.labels = take(rows * sizeof(int32_t));
-  t.w_lo = take(L > 2 ? (size_t)cfg->dims[L - 2] * cfg->dims[L - 1] * 2 : 16);
+  for (int l = 1; l < L; ++l) t.w_lo[l] = take((size_t)cfg->dims[l - 1] * cfg->dims[l] * 2);
   t.end = off;
   return t;
 }
@@ -1336,9 +1345,8 @@ mavg_status fac_setup(mavg_ctx* c, TcState* st, std::string* why) {
     // forward product of layer l; data gradient through layer l
     f->fwd[l] = l == 1 ? cols_for(P, B, (cfg.dims[l] + kBM - 1) / kBM, c->sm_count)
                        : product_cols(P, B, cfg.dims[l], c->sm_count);
-    if (l > 1 && l == L - 1)
-      ok = ok && encode_map(st, &f->w_lo, bf(t.w_lo), cfg.dims[l - 1], cfg.dims[l], 1, cfg.dims[l - 1],
-                            (int64_t)cfg.dims[l - 1] * cfg.dims[l], kBM, why);
+    ok = ok && encode_map(st, &f->w_lo[l], bf(t.w_lo[l]), cfg.dims[l - 1], cfg.dims[l], 1, cfg.dims[l - 1],
+                          (int64_t)cfg.dims[l - 1] * cfg.dims[l], kBM, why);
     if (l == 1) {
       ok = ok && encode_map(st, &f->s_f[1], f->s1_ptr, (int)t.s_ld, kb, P, t.s_ld, f->s1_stride, f->fwd[1].cols, why);
       continue;
@@ -1354,9 +1362,8 @@ mavg_status fac_setup(mavg_ctx* c, TcState* st, std::string* why) {
   if (!ok) return MAVG_ERR_CUDA;
   const void* kernels[] = {
       (const void*)k_fac_product<PROD_FWD, 2, false, false>, (const void*)k_fac_product<PROD_FWD, 2, true, false>,
-      (const void*)k_fac_product<PROD_FWD, 1, false, false>, (const void*)k_fac_product<PROD_DGRAD, 1, false, false>,
-      (const void*)k_fac_product<PROD_RAW, 1, false, false>, (const void*)k_fac_product<PROD_FWD, 2, true, true>,
-      (const void*)k_fac_product<PROD_FWD, 1, false, true>,  (const void*)k_fac_product<PROD_DGRAD, 1, false, true>,
+      (const void*)k_fac_product<PROD_RAW, 2, true, false>,  (const void*)k_fac_product<PROD_DGRAD, 1, false, false>,
+      (const void*)k_fac_product<PROD_FWD, 2, true, true>,   (const void*)k_fac_product<PROD_DGRAD, 1, false, true>,
       (const void*)k_fac_gram, (const void*)k_fac_last<1>, (const void*)k_fac_last<2>,
       (const void*)k_fac_apply<kApplyStages, kApplyPieces>};
   for (const void* k : kernels) {
@@ -1393,13 +1400,15 @@ cudaError_t fac_local_steps(mavg_ctx* c, int64_t round) {
   {
     const int64_t* rp = c->capturing ? (const int64_t*)(ws_ptr(c, c->ws.status) + 64) : nullptr;
     LowArgs la{};
-    if (L > 2) {
-      const MlpLayer& ly = c->layers[L - 2];
-      la.w = c->buf.global_w + ly.w_off;
-      la.dst = bfp(t.w_lo);
-      la.total = (int64_t)ly.in * ly.out;
-      la.blocks = (int)std::min<int64_t>((la.total + 8191) / 8192, 2 * c->sm_count);
+    int64_t all = 0;
+    la.layers = L - 1;
+    for (int l = 1; l < L; ++l) {
+      const MlpLayer& ly = c->layers[l - 1];
+      la.w[l - 1] = c->buf.global_w + ly.w_off;
+      la.dst[l - 1] = bfp(t.w_lo[l]);
+      all += la.total[l - 1] = (int64_t)ly.in * ly.out;
     }
+    la.blocks = (int)std::min<int64_t>((all + 8191) / 8192, 2 * c->sm_count);
     const unsigned grid = (unsigned)(((int64_t)P * rows + 7) / 8 + la.blocks);
     prof_begin(c, MAVG_K_BATCH);
     if (cfg.x_dtype == MAVG_X_BF16)
@@ -1424,7 +1433,7 @@ cudaError_t fac_local_steps(mavg_ctx* c, int64_t round) {
     g.nkb = (cfg.dims[0] + kBK - 1) / kBK;
     g.raw = (float*)f->z_ptr;
     g.z_stride = f->z_stride;
-    FAC_TRY((launch_product<PROD_RAW, 1>(c, MAVG_K_FWD, st->wg[1], st->wg[1], f->h_b[0], f->g_mn[1], f->s_f[1], g)));
+    FAC_TRY((launch_product<PROD_RAW, 2, true>(c, MAVG_K_FWD, st->wg[1], f->w_lo[1], f->h_b[0], f->g_mn[1], f->s_f[1], g)));
   }
   {
     GramArgs g{};
@@ -1493,17 +1502,11 @@ cudaError_t fac_local_steps(mavg_ctx* c, int64_t round) {
       g.nkb = (in + kBK - 1) / kBK;
       if (own_gram(f->fwd[l], cfg.dims[l])) {
         with_gram(g, in, 0);
-        if (l == L - 1)
-          FAC_TRY((launch_product<PROD_FWD, 2, true, true>(c, MAVG_K_FWD, w, f->w_lo, a, d, s, g, &f->h_k[l - 1])));
-        else
-          FAC_TRY((launch_product<PROD_FWD, 1, false, true>(c, MAVG_K_FWD, w, w, a, d, s, g, &f->h_k[l - 1])));
+        FAC_TRY((launch_product<PROD_FWD, 2, true, true>(c, MAVG_K_FWD, w, f->w_lo[l], a, d, s, g, &f->h_k[l - 1])));
         continue;
       }
       if (k > 1) FAC_TRY(gram(MAVG_K_FWD, f->h_k[l - 1], f->h_b[l - 1], in, 0, k));
-      if (l == L - 1)
-        FAC_TRY((launch_product<PROD_FWD, 2, true>(c, MAVG_K_FWD, w, f->w_lo, a, d, s, g)));
-      else
-        FAC_TRY((launch_product<PROD_FWD, 1>(c, MAVG_K_FWD, w, w, a, d, s, g)));
+      FAC_TRY((launch_product<PROD_FWD, 2, true>(c, MAVG_K_FWD, w, f->w_lo[l], a, d, s, g)));
     }
     {
       LastArgs g{};

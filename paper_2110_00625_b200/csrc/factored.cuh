@@ -28,7 +28,7 @@ struct FacLayout {
   size_t zbase = 0, s1 = 0;
   size_t s[2] = {0, 0};                      // one step's -gamma A A(i)^T and -gamma dZ dZ(i)^T: bf16 [P, B, s_ld]
   size_t labels = 0;                         // int32 [K, P, B]
-  size_t w_lo = 0;                           // low parts of w~'s last hidden layer: bf16 [d_{L-1}, d_{L-2}]
+  size_t w_lo[MAVG_MAX_LAYERS] = {};         // low parts of w~'s hidden layers, l = 1..L-1: bf16 [d_l, d_{l-1}]
   size_t end = 0;
 };
 
@@ -47,7 +47,7 @@ struct FacState {
   FacCols fwd[MAVG_MAX_LAYERS + 1], dgrad[MAVG_MAX_LAYERS + 1], gram;
   CUtensorMap in[MAVG_MAX_LAYERS + 1], dz_in[MAVG_MAX_LAYERS + 1];
   CUtensorMap s_f[MAVG_MAX_LAYERS + 1], s_d[MAVG_MAX_LAYERS + 1];
-  CUtensorMap w_lo;                          // low parts of w~'s last hidden layer, box 64 x 128
+  CUtensorMap w_lo[MAVG_MAX_LAYERS];         // low parts of w~'s hidden layers, box 64 x 128
   // Row arrays [P, kb, d_l]: A_l (h) and dZ_l (g) with boxes of 64 x 64 rows (_mn: features are the MMA's
   // row dimension, rows the contraction), 64 x 128 (_k) and 64 x gram.cols (_b; A_0: 64 x row_tile).
   CUtensorMap h_mn[MAVG_MAX_LAYERS], g_mn[MAVG_MAX_LAYERS];

@@ -72,7 +72,7 @@ def _reference(dims, P, K, B, w1, x, y, idx):
             for l in range(L):
                 ai = _q(a[l])
                 w = W0[l] if l < L - 1 else W[l]
-                z = ai @ (_both(w) if l == L - 1 or l == L - 2 > 0 else _q(w)).T + b[l]
+                z = ai @ _both(w).T + b[l]
                 if k and l < L - 1:
                     z = z + _q(-LR * (ai @ torch.cat(A[l]).T)) @ torch.cat(D[l])
                 a.append(torch.relu(z) if l < L - 1 else z)
