@@ -107,6 +107,11 @@ __device__ __forceinline__ uint4 low8(const float* src) {
   return make_uint4(low_pair(a.x, a.y), low_pair(a.z, a.w), low_pair(b.x, b.y), low_pair(b.z, b.w));
 }
 
+// A sum and what the low parts add to it.  An infinite operand (a diverging model's weight or activation) has an
+// infinite product with the high part and with the low one, of either sign: the former alone is the result, as in
+// the plain form.  Added up they would be NaN, which ReLU makes 0.
+__device__ __forceinline__ float with_low(float high, float low) { return fabsf(high) <= 3.402823466e38f ? high + low : high; }
+
 // A warp per row (learner p, step k, slot s): its sample's index, its label and its d inputs as bf16.  The
 // first la.blocks blocks write the low parts of w~ instead.
 template <typename TIN>
@@ -158,6 +163,7 @@ struct ProdArgs {
   int s_row0;               // row of the batch inside a learner's Gram rows
   int stages;
   uint32_t tmem_cols;
+  uint32_t low_col;         // LOW: first column of the low parts' sums
   const float* zbase;       // added to the result: fp32 [kb, M] per learner (null: nothing)
   float* raw;               // RAW: the result, laid out like zbase
   int64_t z_stride;         // floats from learner to learner of either
@@ -199,7 +205,7 @@ __device__ __forceinline__ void load16(uint32_t taddr, bool any, float (&z)[16])
 // grid (column tiles x m_tiles, learner groups).  dgrad with several column tiles: these are a cluster,
 // whose first block adds their bias gradients in rank order.
 // TILES: 16 KB tiles of the MMA's row operand per stage.  LOW (two tiles): the product with w~ reads its low
-// parts as well.
+// parts as well, into columns of their own.
 // GRAM: the Gram rows are formed here too, instead of by a launch of k_fac_gram before.  The blocks of a
 // learner are a cluster; those of a column tile share its Gram tiles out among themselves (128 history
 // rows each, row tile m_tile, m_tile + m_tiles, ...), write them to global memory and tell each other, while
@@ -343,7 +349,7 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
         tc_fence_after_sync();
         const uint32_t off = (uint32_t)ring.s * unit;
         slab_mma(tmem_base, a_base + off, kStepA, b_base + off, kStepK, idesc_base, i > 0);
-        if (LOW) slab_mma(tmem_base, a_base + off + (kATileBytes >> 4), kStepA, b_base + off, kStepK, idesc_base, true);
+        if (LOW) slab_mma(tmem_base + g.low_col, a_base + off + (kATileBytes >> 4), kStepA, b_base + off, kStepK, idesc_base, i > 0);
         umma_commit(&sh.empty_bar[ring.s]);
       }
       const uint32_t idesc_hist = idesc_bf16_f32(kBM, g.cols, 1);
@@ -440,6 +446,12 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
         locate(c0, at, z_at, q);
         float z[16];
         load16(lane_addr + (uint32_t)c0, any, z);
+        if (LOW) {
+          float low[16];
+          load16(lane_addr + g.low_col + (uint32_t)c0, any, low);
+#pragma unroll
+          for (int j = 0; j < 16; ++j) z[j] = with_low(z[j], low[j]);
+        }
         if (EPI == PROD_FWD) {
 #pragma unroll
           for (int j = 0; j < 16; ++j) z[j] = (add_base ? z[j] + zb[j] : z[j]) + bias_next;
@@ -738,7 +750,7 @@ k_fac_last(const LastArgs g) {
   // partial logits: 16 rows x 8 classes per warp and turn
   for (int t = warp; t < (B >> 4) * (CP >> 3); t += kLastThreads / 32) {
     const int mt = t / (CP >> 3), nt = t - mt * (CP >> 3);
-    float d[4] = {0.f, 0.f, 0.f, 0.f};
+    float d[4] = {0.f, 0.f, 0.f, 0.f}, dl[4] = {0.f, 0.f, 0.f, 0.f};
     const __nv_bfloat16* arow_s = As + (size_t)(mt * 16 + (mi & 1) * 8 + mr) * ap + (mi >> 1) * 8;
     const __nv_bfloat16* wrow_s = Ws + (size_t)(nt * 8 + mr) * ap + (mi & 1) * 8;
     for (int k = 0; k < g.cw; k += 16) {
@@ -747,8 +759,10 @@ k_fac_last(const LastArgs g) {
       ldsm_x2(b, wrow_s + k);
       ldsm_x2(bl, wrow_s + k + (size_t)CP * ap);
       mma16816(d, a, b);
-      mma16816(d, a, bl);
+      mma16816(dl, a, bl);
     }
+#pragma unroll
+    for (int i = 0; i < 4; ++i) d[i] = with_low(d[i], dl[i]);
     float* z = zp + (size_t)(mt * 16 + qr) * CP + nt * 8 + qc;
     *reinterpret_cast<float2*>(z) = make_float2(d[0], d[1]);
     *reinterpret_cast<float2*>(z + 8 * CP) = make_float2(d[2], d[3]);
@@ -1153,9 +1167,10 @@ FacCols product_cols(int P, int B, int rows, int sm_count) {
   c.own_gram = true;
   return c;
 }
-// Tensor memory of a block that does: its sums and its Gram tiles'.
-int gram_columns(const FacCols& c, int m_tiles, int hist) {
-  return c.cols * (1 + ((hist + kBM - 1) / kBM + m_tiles - 1) / m_tiles);
+// Tensor memory of a block that does: its sums and its Gram tiles' (and as many columns again as its sums where
+// the low parts' are apart).
+int gram_columns(int cols, int m_tiles, int hist) {
+  return cols * (1 + ((hist + kBM - 1) / kBM + m_tiles - 1) / m_tiles);
 }
 
 struct PdlLaunch {
@@ -1204,7 +1219,8 @@ cudaError_t launch_product(mavg_ctx* c, int cls, const CUtensorMap& w, const CUt
   const int hist_stages = ((g.hist + kBK - 1) / kBK + TILES - 1) / TILES;
   g.stages = stages_for(std::max(1, g.gram_nkb + g.nkb + g.nl * hist_stages), stage_bytes, (long)grid.x * grid.y,
                         c->sm_count);
-  g.tmem_cols = tmem_columns(GRAM ? gram_columns({1, g.cols, g.c_tiles}, g.m_tiles, g.hist) : g.nl * g.cols);
+  g.low_col = (uint32_t)(GRAM ? gram_columns(g.cols, g.m_tiles, g.hist) : g.nl * g.cols);
+  g.tmem_cols = tmem_columns((int)g.low_col + (LOW ? g.nl * g.cols : 0));
   size_t smem = (size_t)g.stages * stage_bytes + 1024 +
                 (EPI == PROD_DGRAD ? (size_t)2 * g.nl * kBM * sizeof(float) : 0);
   // Blocks that wait on one another must all get their tensor memory: no more of them on an SM than it has
@@ -1478,8 +1494,8 @@ cudaError_t fac_local_steps(mavg_ctx* c, int64_t round) {
       return g;
     };
     // the product forms its Gram rows itself
-    auto own_gram = [&](const FacCols& cols, int M) {
-      return k > 1 && cols.own_gram && gram_columns(cols, (M + kBM - 1) / kBM, hist) <= 256;
+    auto own_gram = [&](const FacCols& cols, int M, bool low) {
+      return k > 1 && cols.own_gram && gram_columns(cols.cols, (M + kBM - 1) / kBM, hist) + (low ? cols.cols : 0) <= 256;
     };
     auto with_gram = [&](ProdArgs& g, int dim, int i) {
       g.gram_nkb = (dim + kBK - 1) / kBK;
@@ -1500,7 +1516,7 @@ cudaError_t fac_local_steps(mavg_ctx* c, int64_t round) {
       const int in = cfg.dims[l - 1];
       const CUtensorMap &w = st->wg[l], &a = f->in[l], &d = f->g_mn[l], &s = f->s_f[l];
       g.nkb = (in + kBK - 1) / kBK;
-      if (own_gram(f->fwd[l], cfg.dims[l])) {
+      if (own_gram(f->fwd[l], cfg.dims[l], true)) {
         with_gram(g, in, 0);
         FAC_TRY((launch_product<PROD_FWD, 2, true, true>(c, MAVG_K_FWD, w, f->w_lo[l], a, d, s, g, &f->h_k[l - 1])));
         continue;
@@ -1543,7 +1559,7 @@ cudaError_t fac_local_steps(mavg_ctx* c, int64_t round) {
       g.nkb = (cfg.dims[l] + kBK - 1) / kBK;
       g.out = bfp(t.g[l - 1]);
       g.act = bfp(t.h[l - 1]);
-      if (own_gram(f->dgrad[l], cfg.dims[l - 1])) {
+      if (own_gram(f->dgrad[l], cfg.dims[l - 1], false)) {
         with_gram(g, cfg.dims[l], 1);
         FAC_TRY((launch_product<PROD_DGRAD, 1, false, true>(c, MAVG_K_DGRAD, w, w, dz, a, s, g, &f->g_k[l])));
         continue;

@@ -188,3 +188,24 @@ def test_a_workspace_of_the_plain_forms_size_keeps_that_form():
     assert torch.isfinite(g.w).all()
     g.lib.mavg_destroy(h)
     g.close()
+
+
+@pytest.mark.parametrize("dims,P,K,B", [SHAPES[0], SHAPES[1], SHAPES[4]])
+@pytest.mark.parametrize("value", [np.inf, -np.inf, 3.4e38, np.nan])
+@pytest.mark.parametrize("layer", [1, 2])
+def test_a_weight_that_is_not_finite_spreads_as_in_the_plain_form(dims, P, K, B, value, layer):
+    # an infinite weight makes activations infinite, and those whatever they meet: the loss and every weight are
+    # finite, or not, as without the form (3.4e38 rounds to infinity as bf16)
+    if layer > len(dims) - 2:
+        pytest.skip("one hidden layer")
+    out = []
+    for schedule in (0, 2):
+        g, w1 = _handle(dims, P, K, B, schedule=schedule)
+        at = sum(dims[i] * dims[i + 1] + dims[i + 1] for i in range(layer - 1)) + 3 * dims[layer - 1] + 5
+        g.w[at] = value
+        g.set_round(0)
+        assert g.factored() == (schedule == 0)
+        out.append((np.isfinite(g.round(want_loss=True)), np.isfinite(g.w.cpu().numpy())))
+        g.close()
+    assert out[0][0] == out[1][0]
+    assert np.array_equal(out[0][1], out[1][1]), (out[0][1].mean(), out[1][1].mean())
