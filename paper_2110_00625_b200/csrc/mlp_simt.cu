@@ -259,7 +259,11 @@ __device__ __forceinline__ void col_operands(uint32_t (&r)[4], const __nv_bfloat
 }
 // One slab of the tile.  acc[mt][nt]: 16 x 8 results at rows 32 wm + 16 mt, columns 32 wn + 8 nt; mts, nps: how
 // many 16-row and 16-column groups of the warp's lie inside the result.
-// FRESH: the slab's sum on its own first (not for weight gradients, whose contraction is a few slabs long).
+// FRESH: the slab's sum on its own first.  Not for weight gradients over batches of up to kChainRows samples, whose
+// chains are short (the sums apart need the registers of a fifth block on the SM: 3000-801-99, P = 8, B = 128 513 us
+// for two steps, 582 with spills).  A chain's cut-offs all go the same way, an fp32 sum's roundings either way: relative
+// to 2^-24 of a sum of like terms, root mean square, chain / fp32 sum / FRESH: 1000 samples 7.5 / 9.2 / 1.7; 3000
+// samples 133 / 14 / 2.5; 12000 samples 1082 / 30 / 5.0.
 template <bool A_KC, bool B_KC, bool FRESH>
 __device__ __forceinline__ void multiply_mma(const __nv_bfloat16* a, const __nv_bfloat16* b, int mts, int nps,
                                              float (&acc)[2][4][4]) {
@@ -410,7 +414,7 @@ __device__ __forceinline__ void fma_tile(const GemmArgs& g, int m0, int n0, int 
   finish_split<false, EPI>(g, m0, n0, p, rank, splits, sh.c);
 }
 
-template <int EPI>
+template <int EPI, bool FRESH>
 __device__ __forceinline__ void mma_tile(const GemmArgs& g, int m0, int n0, int p, int rank, int splits,
                                          MmaShared& sh) {
   constexpr bool A_KC = EPI != EPI_WGRAD_SGD, B_KC = EPI == EPI_FWD;
@@ -438,7 +442,7 @@ __device__ __forceinline__ void mma_tile(const GemmArgs& g, int m0, int n0, int 
       pa.load(A, lda, g.vec_a, m0, g.M, k0 + QK, k_end);
       pb.load(B, ldb, g.vec_b, n0, g.N, k0 + QK, k_end);
     }
-    multiply_mma<A_KC, B_KC, EPI != EPI_WGRAD_SGD>(sh.slab[buf][0], sh.slab[buf][1], mts, nps, acc);
+    multiply_mma<A_KC, B_KC, FRESH>(sh.slab[buf][0], sh.slab[buf][1], mts, nps, acc);
     if (more) {
       pa.store(sh.slab[buf ^ 1][0], g.vec_a);
       pb.store(sh.slab[buf ^ 1][1], g.vec_b);
@@ -470,10 +474,10 @@ __device__ __forceinline__ void mma_tile(const GemmArgs& g, int m0, int n0, int 
 
 template <bool QUANT> struct TileShared { using type = GemmShared; };
 template <> struct TileShared<true> { using type = MmaShared; };
-template <bool QUANT, int EPI>
+template <bool QUANT, int EPI, bool FRESH = true>
 __device__ __forceinline__ void gemm_tile(const GemmArgs& g, int m0, int n0, int p, int rank, int splits,
                                           typename TileShared<QUANT>::type& sh) {
-  if constexpr (QUANT) mma_tile<EPI>(g, m0, n0, p, rank, splits, sh);
+  if constexpr (QUANT) mma_tile<EPI, FRESH>(g, m0, n0, p, rank, splits, sh);
   else fma_tile<EPI>(g, m0, n0, p, rank, splits, sh);
 }
 
@@ -500,8 +504,10 @@ struct WgradArgs {
   float* loss_out;
   int loss_stride;
 };
-template <bool QUANT>
-__global__ void __launch_bounds__(kThreads, QUANT ? 5 : 4)
+// FRESH (bf16 operands): see multiply_mma.
+constexpr int kChainRows = 512;
+template <bool QUANT, bool FRESH>
+__global__ void __launch_bounds__(kThreads, QUANT && !FRESH ? 5 : 4)
 k_simt_wgrad(const __grid_constant__ WgradArgs w) {
   __shared__ typename TileShared<QUANT>::type sh;
   tc::grid_launch_dependents();
@@ -512,7 +518,7 @@ k_simt_wgrad(const __grid_constant__ WgradArgs w) {
   const int tile = blockIdx.x - w.tile0[l], p = blockIdx.z;
   const int n_tiles = (g.N + BN - 1) / BN;
   const int m0 = tile / n_tiles * BM, n0 = tile % n_tiles * BN;
-  gemm_tile<QUANT, EPI_WGRAD_SGD>(g, m0, n0, p, 0, 1, sh);
+  gemm_tile<QUANT, EPI_WGRAD_SGD, FRESH>(g, m0, n0, p, 0, 1, sh);
   const int o = m0 + threadIdx.x;
   if (n0 == 0 && threadIdx.x < BM && o < g.M) {
     const float* d = g.A + (size_t)p * g.a_batch + o;
@@ -726,18 +732,23 @@ __device__ __forceinline__ void mma_tail(const TailArgs& t, int p, int r0, uint8
   if (!t.dzp) return;
   __syncthreads();
   for (int nt = warp; nt < (in + 7) / 8; nt += kTailThreads / 32) {
-    float d[4] = {0.f, 0.f, 0.f, 0.f};
-    for (int k = 0; k < c16; k += 16) {
-      uint32_t fa[4], fb[2];
-      ldsm4(fa, dq + ((i8 & 1) * 8 + j8) * dp + k + (i8 >> 1) * 8);
-      ldsm2_t(fb, w + (size_t)(k + (i8 & 1) * 8 + j8) * ip + nt * 8);
-      mma(d, fa, fb[0], fb[1]);
+    float s[2] = {0.f, 0.f};
+    for (int k0 = 0; k0 < c16; k0 += 64) {             // 64 classes' sum on its own, likewise
+      float d[4] = {0.f, 0.f, 0.f, 0.f};
+      for (int k = k0; k < min(c16, k0 + 64); k += 16) {
+        uint32_t fa[4], fb[2];
+        ldsm4(fa, dq + ((i8 & 1) * 8 + j8) * dp + k + (i8 >> 1) * 8);
+        ldsm2_t(fb, w + (size_t)(k + (i8 & 1) * 8 + j8) * ip + nt * 8);
+        mma(d, fa, fb[0], fb[1]);
+      }
+      s[0] += d[0];
+      s[1] += d[1];
     }
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
       const int i = nt * 8 + qc + h;
       if (qr < rows && i < in)                         // ReLU'(0) = 0
-        t.dzp[((size_t)p * t.B + r0 + qr) * in + i] = __bfloat162float(a[qr * ip + i]) > 0.f ? d[h] : 0.f;
+        t.dzp[((size_t)p * t.B + r0 + qr) * in + i] = __bfloat162float(a[qr * ip + i]) > 0.f ? s[h] : 0.f;
     }
   }
 }
@@ -950,7 +961,7 @@ template <bool QUANT>
 cudaError_t set_attributes() {
   const void* kernels[] = {
       (const void*)k_simt_gemm<QUANT, EPI_FWD>, (const void*)k_simt_gemm<QUANT, EPI_DGRAD>,
-      (const void*)k_simt_wgrad<QUANT>, (const void*)k_simt_gather<QUANT>,
+      (const void*)k_simt_wgrad<QUANT, false>, (const void*)k_simt_wgrad<QUANT, QUANT>, (const void*)k_simt_gather<QUANT>,
       (const void*)k_simt_loss<QUANT>, (const void*)k_simt_tail<QUANT>};
   for (const void* k : kernels) {
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -1056,8 +1067,8 @@ cudaError_t step_impl(mavg_ctx* c, int64_t round, int step) {
   w.row_loss = sb.row_loss;
   w.loss_out = (float*)ws_ptr(c, c->ws.losses) + (step - 1);
   w.loss_stride = cfg.K;
-  return launch(c, MAVG_K_WGRAD_SGD, k_simt_wgrad<QUANT>, dim3((unsigned)w.tile0[L], 1, (unsigned)P),
-                kThreads, 1, 0, w);
+  return launch(c, MAVG_K_WGRAD_SGD, B > kChainRows ? k_simt_wgrad<QUANT, QUANT> : k_simt_wgrad<QUANT, false>,
+                dim3((unsigned)w.tile0[L], 1, (unsigned)P), kThreads, 1, 0, w);
 }
 
 }  // namespace
