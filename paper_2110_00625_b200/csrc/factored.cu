@@ -1223,10 +1223,9 @@ cudaError_t launch_product(mavg_ctx* c, int cls, const CUtensorMap& w, const CUt
   g.tmem_cols = tmem_columns((int)g.low_col + (LOW ? g.nl * g.cols : 0));
   size_t smem = (size_t)g.stages * stage_bytes + 1024 +
                 (EPI == PROD_DGRAD ? (size_t)2 * g.nl * kBM * sizeof(float) : 0);
-  // Blocks that wait on one another must all get their tensor memory: no more of them on an SM than it has
-  // columns for, or two clusters could each hold what the other's last block is waiting for.
-  if (GRAM) smem = std::max(smem, (size_t)228 * 1024 / (512 / g.tmem_cols + 1) + 1024);
-  PdlLaunch l(grid, kFacThreads, smem, c->stream, GRAM ? (int)grid.x : EPI == PROD_DGRAD ? g.c_tiles : 1);
+  const int cluster = GRAM ? (int)grid.x : EPI == PROD_DGRAD ? g.c_tiles : 1;
+  if (cluster > 1) smem = std::max(smem, tmem_share_bytes(g.tmem_cols, sizeof(GemmShared) + (GRAM ? 2 * sizeof(uint64_t) : 0)));
+  PdlLaunch l(grid, kFacThreads, smem, c->stream, cluster);
   prof_begin(c, cls);
   cudaError_t e = cudaLaunchKernelEx(&l.lc, k_fac_product<EPI, TILES, LOW, GRAM>, w, lo, in, gram ? *gram : in, hist, s, g);
   prof_end(c);

@@ -365,8 +365,8 @@ cudaError_t launch_gemm_ks(mavg_ctx* c, const CUtensorMap& a, const CUtensorMap&
   g.rep_stride = c->buf.replica_stride;
   g.gamma = c->cfg.local_lr;
   g.status = (int*)ws_ptr(c, c->ws.status);
-  const size_t smem = (size_t)pl.stages * (kATileBytes + pl.BN * kBK * 2) +
-                      (size_t)pl.splits * kBM * 32 * 4 + 1024;
+  const size_t smem = std::max((size_t)pl.stages * (kATileBytes + pl.BN * kBK * 2) + (size_t)pl.splits * kBM * 32 * 4 + 1024,
+                               tmem_share_bytes(pl.tmem_cols, sizeof(GemmShared)));
   cudaLaunchConfig_t lc{};
   lc.gridDim = dim3((unsigned)(pl.m_tiles * pl.splits), (unsigned)c->cfg.P);
   lc.blockDim = dim3(kThreads);

@@ -1,0 +1,49 @@
+"""Cluster launches that hold tensor memory: whatever mix of their blocks an SM's shared memory admits, its 512
+columns of tensor memory are enough for all of them.  Otherwise blocks of two handles on two streams could hold what
+the other's cluster is waiting for, and neither wait has a time limit.  Host arithmetic only."""
+import os
+import re
+import subprocess
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_2110_00625_b200", "csrc")
+MAIN = r'''
+#include <cstdio>
+#include "gemm_unit.cuh"
+int main() {
+  for (unsigned c = 32; c <= 256; c *= 2)
+    for (size_t fixed : {sizeof(mavg::gemm::GemmShared), sizeof(mavg::gemm::GemmShared) + 16})
+      printf("%u %zu %zu\n", c, fixed, mavg::gemm::tmem_share_bytes(c, fixed));
+}
+'''
+
+
+def test_no_mix_of_blocks_runs_out_of_columns(tmp_path):
+    from paper_2110_00625_b200 import build as B
+    if not os.path.exists(B.NVCC):
+        pytest.skip("no nvcc")
+    src, exe = tmp_path / "main.cu", tmp_path / "main"
+    src.write_text(MAIN)
+    subprocess.run([B.NVCC, *B.FLAGS, "-I", CSRC, str(src), "-o", str(exe)], check=True)
+    kinds = [tuple(map(int, line.split())) for line in subprocess.run([str(exe)], capture_output=True, text=True,
+                                                                      check=True).stdout.splitlines()]
+    assert len(kinds) == 8
+
+    def most_columns(room, left):              # over all mixes that fit `room` bytes of an SM's shared memory
+        if not left:
+            return 0
+        columns, fixed, dynamic = left[0]
+        held = fixed + dynamic + 1024          # 1 KB of it is reserved per block
+        return max(n * columns + most_columns(room - n * held, left[1:]) for n in range(room // held + 1))
+
+    assert most_columns(228 * 1024, kinds) <= 512
+    # and the share is no more than needed: as many blocks of one kind as there are columns for do fit
+    for columns, fixed, dynamic in kinds:
+        assert 228 * 1024 // (fixed + dynamic + 1024) == 512 // columns
+
+
+def test_every_cluster_launch_that_holds_tensor_memory_asks_for_its_share():
+    for name, launches in (("factored.cu", 1), ("mlp_tc.cu", 1)):
+        text = open(os.path.join(CSRC, name)).read()
+        assert len(re.findall(r"tmem_share_bytes\(", text)) == launches, name
