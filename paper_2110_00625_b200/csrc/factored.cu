@@ -9,9 +9,7 @@
 //   k_fac_apply     W_l = w~_l - gamma dZ_l^T A_{l-1} over all steps' rows, every learner and hidden layer
 //   k_fac_last      the last layer (at most 32 classes), which keeps its own weights and steps
 //
-// All are launched with programmatic stream serialisation.  A block lets the next kernel begin only when
-// it holds its tensor memory: a successor's block on the same SM could otherwise take the columns first
-// and then wait for this grid, which waits for the columns.
+// All are launched with programmatic stream serialisation.
 #include <cuda.h>
 
 #include <algorithm>
@@ -257,7 +255,7 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
   tc_fence_after_sync();
   if (GRAM) cluster_sync_all();                    // every block's barriers exist before anyone arrives on them
   const uint32_t tmem_base = sh.tmem_slot;
-  grid_launch_dependents();   // not before the tensor memory is this block's: see the head of the file
+  grid_launch_dependents();   // not before the tensor memory is this block's: see tc_ptx.cuh
   grid_dependency_wait();
 
   const int c_tile = (int)blockIdx.x % g.c_tiles, m_tile = (int)blockIdx.x / g.c_tiles;
@@ -569,7 +567,7 @@ k_fac_gram(const __grid_constant__ CUtensorMap tm_hist, const __grid_constant__ 
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = sh.tmem_slot;
-  grid_launch_dependents();   // not before the tensor memory is this block's: see the head of the file
+  grid_launch_dependents();   // not before the tensor memory is this block's: see tc_ptx.cuh
   grid_dependency_wait();
   volatile int* abortp = &sh.abort_flag;
   if (warp == 0) {
@@ -987,7 +985,7 @@ k_fac_apply(const __grid_constant__ ApplyArgs g) {
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = sh.tmem_slot;
-  grid_launch_dependents();   // not before the tensor memory is this block's: see the head of the file
+  grid_launch_dependents();   // not before the tensor memory is this block's: see tc_ptx.cuh
   grid_dependency_wait();
   volatile int* abortp = &sh.abort_flag;
   const int nslab = (g.rows + kBK - 1) / kBK;

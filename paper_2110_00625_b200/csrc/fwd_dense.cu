@@ -40,7 +40,6 @@ k_fwd_dense(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
                                              ~(uintptr_t)1023);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
 
-  grid_launch_dependents();
   if (threadIdx.x == 0) {
     tma_prefetch_desc(&tmW);
     tma_prefetch_desc(&tmX);
@@ -57,6 +56,7 @@ k_fwd_dense(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUt
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = sh.tmem_slot;
+  grid_launch_dependents();   // not before the tensor memory is this block's: see tc_ptx.cuh
   grid_dependency_wait();
 
   const int n_tile = (int)blockIdx.x % g.n_tiles, m_tile = (int)blockIdx.x / g.n_tiles;

@@ -51,7 +51,6 @@ k_tc_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
                                              ~(uintptr_t)1023);
   const int warp = threadIdx.x >> 5;
 
-  grid_launch_dependents();   // the next kernel may begin its own set-up early
   if (threadIdx.x == 0) {
     tma_prefetch_desc(&tmA);
     tma_prefetch_desc(&tmB);
@@ -71,6 +70,7 @@ k_tc_gemm(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUten
   // Everything above touched only this block's own shared and tensor memory.  When the launch
   // allowed it, that much ran while the previous kernel of the stream was still finishing; from
   // here on its results are read, so wait for it to complete (returns at once otherwise).
+  grid_launch_dependents();   // not before the tensor memory is this block's: see tc_ptx.cuh
   grid_dependency_wait();
   // the split path is compiled out of the register-capped build, which is never used with a split
   gemm_tile<EPI, MINB == 1>(tmA, tmB, g, (int)blockIdx.x, (int)blockIdx.y, smem, sh, tmem_base);
@@ -89,7 +89,6 @@ k_tc_gemm_ks(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~(uintptr_t)1023);
   const int warp = threadIdx.x >> 5;
-  grid_launch_dependents();
   if (threadIdx.x == 0) {
     tma_prefetch_desc(&tmA);
     tma_prefetch_desc(&tmB);
@@ -109,6 +108,7 @@ k_tc_gemm_ks(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CU
   tc_fence_after_sync();
   cluster_sync_all();           // every block's barriers exist before anyone arrives on them
   const uint32_t tmem_base = sh.tmem_slot;
+  grid_launch_dependents();   // not before the tensor memory is this block's: see tc_ptx.cuh
   grid_dependency_wait();
   gemm_tile<EPI_FWD_HIDDEN, false, true>(tmA, tmB, g, (int)blockIdx.x, (int)blockIdx.y, smem, sh,
                                          tmem_base);

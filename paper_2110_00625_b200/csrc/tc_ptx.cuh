@@ -141,7 +141,9 @@ __device__ __forceinline__ void tma_load_3d_hint(void* dst, const CUtensorMap* m
 // Programmatic dependent launch: a kernel launched with the stream-serialisation attribute may
 // start before its predecessor in the stream has finished; it must not read the predecessor's
 // results before grid_dependency_wait() returns (which it does once that grid has completed and
-// its writes are visible).  grid_launch_dependents() lets the successor start early.
+// its writes are visible).  grid_launch_dependents() lets the successor start early.  A block that takes tensor
+// memory does so first: a successor's block on its SM could otherwise have the columns before it and then wait for
+// this grid, which waits for the columns.
 __device__ __forceinline__ void grid_dependency_wait() {
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }

@@ -76,7 +76,6 @@ k_wgrad_sgd_stream(const __grid_constant__ CUtensorMap tm_dzt,   // bf16 [P, out
                                              ~(uintptr_t)1023);
   const int warp = threadIdx.x >> 5;
 
-  grid_launch_dependents();
   if (threadIdx.x == 0) {
     tma_prefetch_desc(&tm_dzt);
     tma_prefetch_desc(&tm_at);
@@ -101,6 +100,7 @@ k_wgrad_sgd_stream(const __grid_constant__ CUtensorMap tm_dzt,   // bf16 [P, out
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = sh.tmem_slot;
+  grid_launch_dependents();   // not before the tensor memory is this block's: see tc_ptx.cuh
   grid_dependency_wait();
   wgrad_run<MOM, FWD, true>(tm_dzt, tm_at, tm_w32, tm_w32_in, tm_w16, tm_u, tm_xn, tm_lo, g,
                             (int)blockIdx.x, (int)gridDim.x, smem, sh, tmem_base);
@@ -129,7 +129,6 @@ k_wgrad_sgd_multi(const __grid_constant__ WgradMultiParams mp) {
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~(uintptr_t)1023);
   const int warp = threadIdx.x >> 5;
-  grid_launch_dependents();
   if (threadIdx.x == 0) {
     wgrad_init_barriers(sh, mp.g[0].slots);
     sh.abort_flag = 0;
@@ -144,6 +143,7 @@ k_wgrad_sgd_multi(const __grid_constant__ WgradMultiParams mp) {
   __syncthreads();
   tc_fence_after_sync();
   const uint32_t tmem_base = sh.tmem_slot;
+  grid_launch_dependents();   // not before the tensor memory is this block's: see tc_ptx.cuh
   grid_dependency_wait();
   uint32_t tiles = 0, items = 0;
   const int grid = (int)gridDim.x;

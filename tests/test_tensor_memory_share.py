@@ -47,3 +47,19 @@ def test_every_cluster_launch_that_holds_tensor_memory_asks_for_its_share():
     for name, launches in (("factored.cu", 1), ("mlp_tc.cu", 1)):
         text = open(os.path.join(CSRC, name)).read()
         assert len(re.findall(r"tmem_share_bytes\(", text)) == launches, name
+
+
+def test_the_next_kernel_begins_after_a_block_has_its_columns():
+    # in every kernel that takes tensor memory: alloc, then the trigger, then the wait for the kernel before
+    for name in ("factored.cu", "fwd_dense.cu", "mlp_tc.cu", "wgrad_tc.cu"):
+        text = open(os.path.join(CSRC, name)).read()
+        allocs = [m.start() for m in re.finditer(r"\btmem_alloc\(", text)]
+        assert allocs, name
+        for at in allocs:
+            kernel = text[text.rindex("__global__", 0, at):]
+            body = kernel[:kernel.index("tmem_dealloc(")]
+            first = body.index("tmem_alloc(")
+            early = [m.start() for m in re.finditer(r"grid_launch_dependents\(\)", body) if m.start() < first]
+            # (a block that returns at once takes none)
+            assert all("return;" in body[e:e + 60] for e in early), name
+            assert first < body.index("grid_launch_dependents()", first) < body.index("grid_dependency_wait()"), name
