@@ -1274,31 +1274,44 @@ bool enough_rows(const mavg_config* cfg, int K) { return K >= 2 && (int64_t)cfg-
 // Speed: what it saves goes with the weights (none is read or written per learner and step), what it adds
 // with the square of a learner's rows K B: the Gram products and the products with them,
 // K B (d_0 + d_1 + 2 sum_{l>=2} (d_{l-1} + d_l)) multiply-adds per row against one per hidden weight and
-// product.  Taken below a ratio of 5, from 11 learners on (whose launches fill the chip) below 6 (plain /
-// factored, us a round): 3072-2048-2048-2048-10, P = 32, K = 16, B = 64 (ratio 1.6) 15180 / 5600;
-// 3072-512-512-10, P = 48, K = 8, B = 64 (1.6) 1860 / 848, P = 8, B = 128 (3.2) 623 / 457.
-// 17 drawn models of ratios 3.6 to 6, P >= 8: all faster, least 1584-168-168-11, P = 36, K = 5, B = 128 (5.3)
-// 436 / 415, 720-688-688-21, P = 11, K = 14, B = 96 (5.8) 1092 / 933; beyond: few learners 560-648-2, P = 5, K = 7,
-// B = 240 (5.6) 232 / 271, 1584-528-528-7, P = 6, K = 7, B = 240 (6.4) 627 / 715; many, either way: 784-232-2,
-// P = 34, K = 8, B = 176 (7.9) 405 / 486, 2432-512-512-27, P = 26, K = 10, B = 240 (7.9) 2807 / 1949.
+// product.  The lines are drawn through 860 measured models of 0.05 to 60 M hidden weights, P = 2 to 64, K = 2 to 24
+// (plain / factored, us a round).  Never from a ratio of 5.5 on: 2024-424-408-88-32, P = 9, K = 9, B = 144 (6.2)
+// 910 / 1142, 752-688-688-2, P = 34, K = 8, B = 176 (6.0) 1337 / 1482 (most large ones are faster still:
+// 3048-1536-1536-10, P = 6, K = 19, B = 208 (6.0) 5757 / 3749).  Below it
+//   - where the learners' weights are many for the launches of a step, P x weights / hidden layers = V:
+//     ratio < 0.5 + 0.6 V / 10^6.  3072-2048-2048-2048-10, P = 32, K = 16, B = 64 (1.5, V = 154 M) 15380 / 6360,
+//     3072-512-512-10, P = 48, K = 8, B = 64 (1.6, 44 M) 1845 / 862, P = 8, B = 128 (3.1, 7 M) 621 / 470; beyond
+//     784-640-3, P = 8, K = 9, B = 176 (4.5, 4 M) 311 / 357, 1752-600-600-16, P = 8, K = 10, B = 144 (4.9, 6 M) 862 / 948,
+//     2968-240-240-240-11, P = 16, K = 4, B = 128 (3.2, 4 M) 389 / 441;
+//   - batches of up to 96 from V = 2 M on, 3 M with three hidden layers, and below a ratio of 5 with fewer from 1 M on (a
+//     step's products then have few columns a learner): 1720-360-13, P = 10, K = 18, B = 80 (4.8, 6 M) 796 / 479,
+//     520-200-136-12, P = 20, K = 9, B = 48 (4.6, 1.3 M) 342 / 338; not P = 16, K = 7, B = 80 of the latter (5.9, 1.0 M)
+//     275 / 309 nor 336-296-296-296-27, P = 22, K = 5, B = 80 (4.4, 2.0 M) 346 / 364;
+//   - one hidden layer, whose step is two launches, up to B = 128 and from V = 2 M on: 664-672-29, P = 7, K = 17, B = 96
+//     (4.9, 3 M) 609 / 476; not 536-296-19, P = 10, K = 8, B = 128 (5.4, 1.6 M) 229 / 241.
+// Within the lines 3 of 630 models are slower, by 2 to 4 %; 102 beyond them would be faster by a tenth or more.
 // Models of fewer than 48 K hidden weights keep the plain form: a round is a chain of short launches either
 // way (128-128-128-10, P = 148, B = 32: K = 2 124 / 103, K = 8 371 / 371; 256-128-10, P = 64, K = 4 119 / 110).
-// Results: the plain form rounds W_l(k) to bf16 at every step, this one rounds w~ and the Gram rows.  Both are
-// equally far from the 64-bit result (3072-512-512-10, P = 8, K = 8, B = 128: 4.5e-3 and 4.6e-3 of v), by
-// roundings and ReLU branches that differ from row to row, so a round's mean agrees the better the more rows
-// it has: v of the two forms differs by 4e-3 to 1e-2 from 8192 rows P K B on (6e-3 to 1.6e-2 with three
-// hidden layers and 16 steps), by 1.5e-2 to 3e-2 at 500 to 800 rows.  Below 8192 rows the learners keep
-// the rounding of their own weights.
+// Results: the plain form rounds W_l(k) to bf16 at every step, this one rounds w~ (to 16 bits in the forward
+// products, see LowArgs) and the Gram rows; its error against 64 bits is the smaller one, at 2048 rows P K B as at
+// 30000.  The two differ from each other by roundings and ReLU branches that vary from row to row: v by 4e-3 to
+// 1e-2 from 8192 rows on (6e-3 to 1.6e-2 with three hidden layers and 16 steps), by 1.5e-2 to 3e-2 at 500 to
+// 800.  Below 8192 rows the learners keep the rounding of their own weights: a cautious line, not one that the
+// error draws.
 int fac_steps(const mavg_config* cfg) {
-  const int B = cfg->B;
-  if (cfg->n_layers < 2) return 0;
+  const int B = cfg->B, hidden = cfg->n_layers - 1;
+  if (hidden < 1) return 0;
   int64_t span = cfg->dims[0] + cfg->dims[1], weights = (int64_t)cfg->dims[0] * cfg->dims[1];
-  for (int l = 2; l < cfg->n_layers; ++l) {
+  for (int l = 2; l <= hidden; ++l) {
     span += 2 * ((int64_t)cfg->dims[l - 1] + cfg->dims[l]);
     weights += (int64_t)cfg->dims[l - 1] * cfg->dims[l];
   }
   if (weights < 48 * 1024) return 0;
-  const int most = (int)std::min<int64_t>({cfg->K, 4096 / B, ((cfg->P >= 11 ? 6 : 5) * weights - 1) / (span * B)});
+  const double v = 1e-6 * (double)cfg->P * (double)weights / hidden;
+  double line = std::min(5.5, 0.5 + 0.6 * v);
+  if (v >= (hidden < 3 ? 2.0 : 3.0) && (B <= 96 || (B <= 128 && hidden == 1))) line = 5.5;
+  else if (v >= 1.0 && B <= 96 && hidden < 3) line = std::max(line, 5.0);
+  const int most = (int)std::min<int64_t>({cfg->K, 4096 / B, ((int64_t)(line * (double)weights) - 1) / (span * B)});
   return enough_rows(cfg, most) && last_plan(cfg).smem <= kLastSmem ? most : 0;
 }
 

@@ -158,12 +158,18 @@ def test_steps_of_length_zero_keep_every_bit(dims, P, K, B):
 
 
 def test_where_the_form_is_taken():
-    # both sides of its lines: 8192 rows a round, the added work (P = 8: 5 times the weights, P = 11: 6), two steps, momentum
+    # both sides of its lines: 8192 rows a round, two steps, momentum, a hidden layer; the added work (K) below 5.5 times
+    # the weights, where they are few for a step's launches (P) only for small batches or one hidden layer
     for dims, P, K, B, kw, want in [
         ([1000, 312, 10], 32, 2, 128, {}, True), ([1000, 312, 10], 31, 2, 128, {}, False),
         ([1000, 312, 10], 64, 1, 128, {}, False), ([1000, 312, 10], 32, 2, 128, dict(learner_momentum=0.9), False),
-        ([400, 400, 10], 8, 8, 128, {}, False),
-    ([400, 400, 10], 11, 9, 128, {}, True), ([400, 400, 10], 11, 10, 128, {}, False), ([1000, 10], 32, 2, 128, {}, False),
+        ([1000, 10], 32, 2, 128, {}, False),
+        ([1000, 312, 10], 16, 5, 144, {}, True), ([1000, 312, 10], 16, 6, 144, {}, False),
+        ([400, 400, 10], 13, 8, 128, {}, True), ([400, 400, 10], 13, 9, 128, {}, False),
+        ([400, 400, 10], 12, 8, 128, {}, False), ([400, 400, 10], 13, 7, 144, {}, False),
+        ([520, 200, 136, 12], 19, 9, 48, {}, True), ([520, 200, 136, 12], 19, 10, 48, {}, False),
+        ([376, 136, 19], 20, 14, 32, {}, True), ([376, 136, 19], 19, 14, 32, {}, False),
+        ([616, 192, 80, 80, 30], 65, 4, 96, {}, True), ([616, 192, 80, 80, 30], 64, 4, 96, {}, False),
     ]:
         assert _factored(dims, P, K, B, **kw) == want, (dims, P, K, B, kw)
 
