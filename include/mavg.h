@@ -134,7 +134,7 @@ typedef struct {
   int64_t replica_stride; /* floats between rows, >= n and a multiple of 4 */
   float *global_w;        /* [n] w~; on entry to mavg_create it holds w~_1 */
   float *momentum;        /* [n] v */
-  void *workspace;        /* scratch, at least mavg_workspace_bytes() bytes */
+  void *workspace;        /* scratch of mavg_workspace_bytes() bytes, or at least mavg_workspace_least_bytes() */
   size_t workspace_bytes;
   float *learner_u;       /* [P, replica_stride] fp32 learner momentum buffers u^j, same layout as
                              replicas; required iff learner_momentum != 0 (else ignored, may be
@@ -144,6 +144,10 @@ typedef struct {
 /* Bytes of scratch the configuration needs (activations, bf16 operand copies, batch indices,
  * loss accumulators, the device status word).  Checks the configuration like mavg_create. */
 mavg_status mavg_workspace_bytes(const mavg_config *cfg, size_t *out_bytes);
+
+/* The least that mavg_create accepts: smaller where rounds run in factored form (MAVG_SCHED_GRAPH below), which
+ * needs room for the rows of all K steps; a handle with less than mavg_workspace_bytes keeps the plain form. */
+mavg_status mavg_workspace_least_bytes(const mavg_config *cfg, size_t *out_bytes);
 
 /* Algorithm 1, the two initialisation lines and the first "set w^j = w~": v <- 0, w^j <- w~_1
  * (the copies are skipped with defer_broadcast, see there).
@@ -266,8 +270,9 @@ mavg_status mavg_set_profiling(mavg_handle h, int32_t on);
  *     in factored form: W_l(k) = w~_l - gamma sum_{i<k} dZ_l(i)^T A_{l-1}(i) is not formed until the last
  *     step, products take w~ and the factors instead.  w~ enters the forward products and the last layer as
  *     two bf16 parts and the data gradients as one, the sums over the factors through bf16 Gram rows; the plain
- *     form rounds W_l(k) to bf16 at every step.  mavg_workspace_bytes has room for it; a buffer
- *     with room for the plain form only is accepted and keeps that.
+ *     form rounds W_l(k) to bf16 at every step.  mavg_workspace_bytes has room for it if
+ *     the handle's own K and momentum take it; a buffer with room for the plain form only
+ *     (mavg_workspace_least_bytes) is accepted and keeps that.
  *   MAVG_SCHED_GRAPH_TC: the same graph with every product as plain one-tile-per-block
  *     tensor-core launches.  Apart from factored rounds the two differ in the
  *     summation order of the products they run differently, nothing else; this one exists for comparison.

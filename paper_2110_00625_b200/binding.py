@@ -17,7 +17,7 @@ MAX_LAYERS = 8
 STATUS = {0: "MAVG_OK", 1: "MAVG_ERR_INVALID_ARG", 2: "MAVG_ERR_BAD_BUFFER", 3: "MAVG_ERR_STATE",
           4: "MAVG_ERR_UNSUPPORTED", 5: "MAVG_ERR_CUDA", 6: "MAVG_ERR_TIMEOUT"}
 
-EXPORTS = ["mavg_workspace_bytes", "mavg_create", "mavg_local_steps", "mavg_meta_update",
+EXPORTS = ["mavg_workspace_bytes", "mavg_workspace_least_bytes", "mavg_create", "mavg_local_steps", "mavg_meta_update",
            "mavg_materialize_replicas", "mavg_round", "mavg_round_host", "mavg_set_hparams",
            "mavg_set_learner_momentum", "mavg_get_batch_indices",
            "mavg_get_losses", "mavg_get_round", "mavg_set_round", "mavg_get_launch_count",
@@ -79,6 +79,7 @@ def load_library():
     L = C.CDLL(path)
     H = C.c_void_p
     L.mavg_workspace_bytes.argtypes = [C.POINTER(Config), C.POINTER(C.c_size_t)]
+    L.mavg_workspace_least_bytes.argtypes = [C.POINTER(Config), C.POINTER(C.c_size_t)]
     L.mavg_create.argtypes = [C.POINTER(Config), C.POINTER(Buffers), C.POINTER(H)]
     L.mavg_local_steps.argtypes = [H]
     L.mavg_meta_update.argtypes = [H]
@@ -198,7 +199,15 @@ class Mavg:
         st = self.lib.mavg_workspace_bytes(C.byref(self.cfg), C.byref(nbytes))
         if st != 0:
             raise MavgError(st, self.lib.mavg_last_error(None).decode())
-        self.workspace = torch.empty(max(nbytes.value, 256), dtype=torch.uint8, device=self.device)
+        try:
+            self.workspace = torch.empty(max(nbytes.value, 256), dtype=torch.uint8, device=self.device)
+        except torch.cuda.OutOfMemoryError:
+            # room for the plain form of the local steps, if that is less (factored() then says False)
+            full = nbytes.value
+            self.lib.mavg_workspace_least_bytes(C.byref(self.cfg), C.byref(nbytes))
+            if nbytes.value == full:
+                raise
+            self.workspace = torch.empty(max(nbytes.value, 256), dtype=torch.uint8, device=self.device)
         self.buf = Buffers(self.replicas.data_ptr(), self.stride, self.w.data_ptr(),
                            self.v.data_ptr(), self.workspace.data_ptr(), self.workspace.numel(),
                            self.u.data_ptr() if self.u is not None else None)

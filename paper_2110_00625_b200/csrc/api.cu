@@ -271,6 +271,17 @@ mavg_status mavg_workspace_bytes(const mavg_config* cfg, size_t* out_bytes) {
   return MAVG_OK;
 }
 
+mavg_status mavg_workspace_least_bytes(const mavg_config* cfg, size_t* out_bytes) {
+  if (!out_bytes) return fail(&g_create_error, MAVG_ERR_INVALID_ARG, "out_bytes is NULL");
+  *out_bytes = 0;
+  mavg_status st = validate_config(cfg, &g_create_error);
+  if (st != MAVG_OK) return st;
+  Workspace ws;
+  carve_workspace(cfg, &ws);
+  *out_bytes = ws.least;
+  return MAVG_OK;
+}
+
 mavg_status mavg_create(const mavg_config* cfg, const mavg_buffers* buf, mavg_handle* out) {
   if (!out) return fail(&g_create_error, MAVG_ERR_INVALID_ARG, "out is NULL");
   *out = nullptr;
@@ -293,7 +304,7 @@ mavg_status mavg_create(const mavg_config* cfg, const mavg_buffers* buf, mavg_ha
   Workspace ws;
   carve_workspace(cfg, &ws);
   if (buf->workspace_bytes < ws.least)
-    return fail(&g_create_error, MAVG_ERR_BAD_BUFFER, "workspace is smaller than mavg_workspace_bytes");
+    return fail(&g_create_error, MAVG_ERR_BAD_BUFFER, "workspace is smaller than mavg_workspace_least_bytes");
 
   int dev = 0;
   cudaGetLastError();   // a stale non-sticky error of earlier, unrelated calls is not ours

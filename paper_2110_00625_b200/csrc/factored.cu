@@ -1315,6 +1315,8 @@ int fac_steps(const mavg_config* cfg) {
   return enough_rows(cfg, most) && last_plan(cfg).smem <= kLastSmem ? most : 0;
 }
 
+bool fac_reserved(const mavg_config* cfg) { return cfg->learner_momentum == 0.f && fac_steps(cfg) == cfg->K; }
+
 FacLayout fac_layout(const mavg_config* cfg, size_t base) {
   FacLayout t;
   const int L = cfg->n_layers, P = cfg->P, B = cfg->B;

@@ -56,8 +56,10 @@ struct FacState {
 };
 
 // The most steps of a call that a handle's calls may take in this form (0: never; at most the K it was made
-// for), and the scratch for them from `base` on.
+// for), and the scratch for them from `base` on.  fac_reserved: the calls as the handle is made take it, so the
+// workspace size has room for it (up to ten times the plain form's for long rounds of narrow models).
 int fac_steps(const mavg_config* cfg);
+bool fac_reserved(const mavg_config* cfg);
 FacLayout fac_layout(const mavg_config* cfg, size_t base);
 struct TcState;
 mavg_status fac_setup(mavg_ctx* c, TcState* st, std::string* why);

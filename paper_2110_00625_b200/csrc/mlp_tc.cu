@@ -410,9 +410,8 @@ size_t tc_workspace_bytes(const mavg_config* cfg, size_t base, size_t* act_off, 
   *act_off = base;
   const TcLayout t = make_layout(cfg, base, kPlanSmCount);
   *least = t.end;
-  return fac_steps(cfg) ? std::max(t.end, fac_layout(cfg, t.shared_end).end) : t.end;
+  return fac_reserved(cfg) ? std::max(t.end, fac_layout(cfg, t.shared_end).end) : t.end;
 }
-
 
 mavg_status tc_setup(mavg_ctx* c) {
   const mavg_config& cfg = c->cfg;
@@ -620,6 +619,7 @@ mavg_status tc_setup(mavg_ctx* c) {
                         &st->ev_x_free[0], &st->ev_x_free[1]};
   for (cudaEvent_t* ev : evs)
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
+  // (also for calls of fewer steps or another momentum than the handle was made for, where the room is there)
   if (e == cudaSuccess && fac_steps(&cfg) &&
       c->buf.workspace_bytes >= std::max(t.end, fac_layout(&cfg, t.shared_end).end)) {
     const mavg_status fs = fac_setup(c, st, &why);

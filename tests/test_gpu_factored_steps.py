@@ -46,6 +46,13 @@ def _factored(dims, P, K, B, **kw):
     return launches == 1 and K > 1
 
 
+def _takes(dims, P, K, B):
+    g, _ = _handle(dims, P, K, B)
+    r = g.factored()
+    g.close()
+    return r
+
+
 def _q(t):
     return t.bfloat16().float()
 
@@ -127,7 +134,8 @@ def test_the_same_bits_however_it_is_issued(dims, P, K, B):
     # replayed, launch by launch, with copies written eagerly or not, in a handle made for more steps; a second
     # call without a meta-update starts from the learners' own models
     out = []
-    for profiled, defer, more in ((False, True, 0), (True, True, 0), (False, False, 0), (False, True, 3)):
+    spare = next(e for e in (3, 2, 1, 0) if _takes(dims, P, K + e, B))      # (a handle that never does has no room for it)
+    for profiled, defer, more in ((False, True, 0), (True, True, 0), (False, False, 0), (False, True, spare)):
         g, _ = _handle(dims, P, K + more, B, defer_broadcast=defer)
         if more:
             g.set_hparams(K, LR, 1.0, 0.9)
@@ -172,6 +180,32 @@ def test_where_the_form_is_taken():
         ([616, 192, 80, 80, 30], 65, 4, 96, {}, True), ([616, 192, 80, 80, 30], 64, 4, 96, {}, False),
     ]:
         assert _factored(dims, P, K, B, **kw) == want, (dims, P, K, B, kw)
+
+
+def test_a_refused_allocation_leaves_the_plain_form(monkeypatch):
+    # the room for the rows of all steps is not to be had: a handle in the plain form, and the same round as one
+    import ctypes as C
+    dims, P, K, B = SHAPES[-1]
+    g, _ = _handle(dims, P, K, B)
+    full, least = g.workspace.numel(), C.c_size_t()
+    assert g.lib.mavg_workspace_least_bytes(C.byref(g.cfg), C.byref(least)) == 0 and least.value < full
+    g.close()
+    empty = torch.empty
+
+    def refuse(size, *a, **kw):
+        if size == full:
+            raise torch.cuda.OutOfMemoryError("refused")
+        return empty(size, *a, **kw)
+
+    monkeypatch.setattr(torch, "empty", refuse)
+    g, _ = _handle(dims, P, K, B)
+    assert g.workspace.numel() == least.value and not g.factored()
+    monkeypatch.setattr(torch, "empty", empty)
+    plain, _ = _handle(dims, P, K, B, schedule=2)
+    assert abs(g.round(want_loss=True) - plain.round(want_loss=True)) <= 1e-3
+    g.sync(); plain.sync()
+    assert l2_rel(g.v.cpu().numpy(), plain.v.cpu().numpy()) <= 2e-2
+    g.close(); plain.close()
 
 
 def test_a_workspace_of_the_plain_forms_size_keeps_that_form():

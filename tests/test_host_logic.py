@@ -160,3 +160,23 @@ def test_split_masters_take_no_workspace(lib, dims, P, B, total):
     cfg = _cfg(P=P, K=8, n=n, B=B, objective=2, dims=dims, gemm_bf16=1, x_ptr=256, y_ptr=256, n_samples=50000)
     nb = C.c_size_t()
     assert lib.mavg_workspace_bytes(C.byref(cfg), C.byref(nb)) == 0 and nb.value == total
+
+
+@pytest.mark.parametrize("dims,P,K,B,kw,total,least", [
+    # takes rounds in factored form: room for the rows of its steps
+    ([2048, 2048, 10], 64, 64, 64, {}, 7606176768, 754257920),
+    ([3072, 512, 512, 10], 8, 8, 128, {}, 95797248, 83787776),
+    # never does as it was made (too many steps, learner momentum): nothing is reserved
+    ([3072, 512, 512, 10], 8, 64, 128, {}, 83789824, 83789824),
+    ([3072, 512, 512, 10], 8, 8, 128, dict(learner_momentum=0.9), 83787776, 83787776),
+    ([3072, 2048, 2048, 2048, 10], 64, 64, 64, {}, 2889157632, 2889157632),
+    ([3072, 2048, 2048, 2048, 10], 1000, 64, 64, {}, 47326843904, 47326843904),
+])
+def test_scratch_of_factored_rounds_is_reserved_for_handles_that_take_them(lib, dims, P, K, B, kw, total, least):
+    n = sum(dims[i] * dims[i + 1] + dims[i + 1] for i in range(len(dims) - 1))
+    cfg = _cfg(P=P, K=K, n=n, B=B, objective=2, dims=dims, gemm_bf16=1, x_ptr=256, y_ptr=256, n_samples=50000, **kw)
+    full, small = C.c_size_t(), C.c_size_t()
+    assert lib.mavg_workspace_bytes(C.byref(cfg), C.byref(full)) == 0
+    assert lib.mavg_workspace_least_bytes(C.byref(cfg), C.byref(small)) == 0
+    assert lib.mavg_workspace_least_bytes(C.byref(cfg), None) == 1 and lib.mavg_workspace_least_bytes(None, C.byref(C.c_size_t())) == 1
+    assert (full.value, small.value) == (total, least)
