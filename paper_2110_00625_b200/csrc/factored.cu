@@ -1340,11 +1340,11 @@ FacLayout fac_layout(const mavg_config* cfg, size_t base) {
   return t;
 }
 
-mavg_status fac_setup(mavg_ctx* c, TcState* st, std::string* why) {
+void fac_setup(mavg_ctx* c, TcState* st) {
+  std::string* why = nullptr;
   const mavg_config& cfg = c->cfg;
   const int L = cfg.n_layers, P = cfg.P, B = cfg.B;
   FacState* f = new FacState();
-  st->fac = f;
   f->lay = fac_layout(&cfg, st->lay.shared_end);
   f->K = fac_steps(&cfg);
   const FacLayout& t = f->lay;
@@ -1387,21 +1387,20 @@ mavg_status fac_setup(mavg_ctx* c, TcState* st, std::string* why) {
     ok = ok && encode_map(st, &f->s_f[l], bf(t.s[0]), (int)t.s_ld, B, P, t.s_ld, B * t.s_ld, f->fwd[l].cols, why);
     ok = ok && encode_map(st, &f->s_d[l], bf(t.s[1]), (int)t.s_ld, B, P, t.s_ld, B * t.s_ld, f->dgrad[l].cols, why);
   }
-  if (!ok) return MAVG_ERR_CUDA;
   const void* kernels[] = {
       (const void*)k_fac_product<PROD_FWD, 2, false, false>, (const void*)k_fac_product<PROD_FWD, 2, true, false>,
       (const void*)k_fac_product<PROD_RAW, 2, true, false>,  (const void*)k_fac_product<PROD_DGRAD, 1, false, false>,
       (const void*)k_fac_product<PROD_FWD, 2, true, true>,   (const void*)k_fac_product<PROD_DGRAD, 1, false, true>,
       (const void*)k_fac_gram, (const void*)k_fac_last<1>, (const void*)k_fac_last<2>,
       (const void*)k_fac_apply<kApplyStages, kApplyPieces>};
-  for (const void* k : kernels) {
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024);
-    if (e != cudaSuccess) {
-      *why = std::string("factored steps: ") + cudaGetErrorString(e);
-      return MAVG_ERR_CUDA;
-    }
+  for (const void* k : kernels)
+    ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024) == cudaSuccess;
+  if (ok) {
+    st->fac = f;
+  } else {
+    cudaGetLastError();
+    delete f;
   }
-  return MAVG_OK;
 }
 
 bool fac_usable(const mavg_ctx* c) {

@@ -62,7 +62,8 @@ int fac_steps(const mavg_config* cfg);
 bool fac_reserved(const mavg_config* cfg);
 FacLayout fac_layout(const mavg_config* cfg, size_t base);
 struct TcState;
-mavg_status fac_setup(mavg_ctx* c, TcState* st, std::string* why);
+// A tensor map or kernel attribute that is refused leaves the handle the plain form.
+void fac_setup(mavg_ctx* c, TcState* st);
 // The steps of a call that starts from w~ take the factored form.
 bool fac_usable(const mavg_ctx* c);
 cudaError_t fac_local_steps(mavg_ctx* c, int64_t round);

@@ -621,13 +621,8 @@ mavg_status tc_setup(mavg_ctx* c) {
     if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
   // (also for calls of fewer steps or another momentum than the handle was made for, where the room is there)
   if (e == cudaSuccess && fac_steps(&cfg) &&
-      c->buf.workspace_bytes >= std::max(t.end, fac_layout(&cfg, t.shared_end).end)) {
-    const mavg_status fs = fac_setup(c, st, &why);
-    if (fs != MAVG_OK) {
-      c->err = why;
-      return fs;
-    }
-  }
+      c->buf.workspace_bytes >= std::max(t.end, fac_layout(&cfg, t.shared_end).end))
+    fac_setup(c, st);
   if (e == cudaSuccess)
     e = cudaMemsetAsync(ws + t.counters, 0, t.counters_bytes, c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(ws + t.zcount, 0, t.zcount_bytes, c->stream);
