@@ -50,6 +50,7 @@ def test_agrees_with_one_tile_per_block(shape):
     cfg = _cfg(**shape)
     a, *_ = _make(cfg, 0)
     b, *_ = _make(cfg, 2)
+    assert not a.factored()
     a.local_steps(); b.local_steps()
     a.sync(); b.sync()
     la, lb = a.get_losses(), b.get_losses()
@@ -67,8 +68,9 @@ def test_agrees_with_one_tile_per_block(shape):
 
 
 def test_rounds_against_the_oracle(oracle):
-    cfg = _cfg(dims=[1024, 128, 10], P=64, K=2, B=64, S=8192)
+    cfg = _cfg(dims=[1024, 128, 10], P=63, K=2, B=64, S=8192)
     g, x, y, w1 = _make(cfg, 0)
+    assert not g.factored()          # from 8192 rows a round on there are no such products
     o = oracle.Mavg(w1, P=cfg["P"], K=cfg["K"], gamma=cfg["gamma"], mu=cfg["mu"], B=cfg["B"],
                     seed=SEED, objective=oracle.OBJ_MLP, dims=cfg["dims"], bf16=True, x=x, y=y,
                     stride=g.stride)

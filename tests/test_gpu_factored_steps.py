@@ -36,21 +36,16 @@ def _handle(dims, P, K, B, schedule=0, **kw):
     return g, w1
 
 
-def _factored(dims, P, K, B, **kw):
-    """Whether such a handle's rounds take the form: one launch for all hidden weights, none per step."""
+def _takes(dims, P, K, B, **kw):
+    """Whether such a handle's rounds take the form; they then have one launch for all hidden weights, none per step."""
     g, _ = _handle(dims, P, K, B, **kw)
+    takes = g.factored()
     g.set_profiling(True)
     g.round()
     launches = g.get_profile()["wgrad_sgd_gemm"][1]
     g.close()
-    return launches == 1 and K > 1
-
-
-def _takes(dims, P, K, B):
-    g, _ = _handle(dims, P, K, B)
-    r = g.factored()
-    g.close()
-    return r
+    assert K == 1 or takes == (launches == 1), (takes, launches)
+    return takes
 
 
 def _q(t):
@@ -106,7 +101,7 @@ def _reference(dims, P, K, B, w1, x, y, idx):
 
 @pytest.mark.parametrize("dims,P,K,B", SHAPES)
 def test_against_the_same_form_in_torch_and_the_plain_form(dims, P, K, B):
-    assert _factored(dims, P, K, B)
+    assert _takes(dims, P, K, B)
     g, w1 = _handle(dims, P, K, B, defer_broadcast=True)
     idx = [[torch.from_numpy(g.get_batch_indices(1, j, k).astype(np.int64)).cuda() for k in range(1, K + 1)]
            for j in range(P)]
@@ -179,7 +174,7 @@ def test_where_the_form_is_taken():
         ([376, 136, 19], 20, 14, 32, {}, True), ([376, 136, 19], 19, 14, 32, {}, False),
         ([616, 192, 80, 80, 30], 65, 4, 96, {}, True), ([616, 192, 80, 80, 30], 64, 4, 96, {}, False),
     ]:
-        assert _factored(dims, P, K, B, **kw) == want, (dims, P, K, B, kw)
+        assert _takes(dims, P, K, B, **kw) == want, (dims, P, K, B, kw)
 
 
 def test_a_refused_allocation_leaves_the_plain_form(monkeypatch):
@@ -249,3 +244,67 @@ def test_a_weight_that_is_not_finite_spreads_as_in_the_plain_form(dims, P, K, B,
         g.close()
     assert out[0][0] == out[1][0]
     assert np.array_equal(out[0][1], out[1][1]), (out[0][1].mean(), out[1][1].mean())
+
+
+@pytest.mark.parametrize("dims,P,K,B,x_bf16,defer", [([1000, 312, 10], 40, 4, 80, True, True),
+                                                     ([520, 200, 136, 12], 20, 9, 48, False, False),
+                                                     ([1032, 1000, 520, 264, 10], 52, 5, 32, False, True)])
+def test_rounds_of_either_form_on_one_handle(dims, P, K, B, x_bf16, defer):
+    # The forms share scratch, and a factored round leaves the learners' bf16 copies unwritten: every call in turn
+    # leaves what a handle made for it, from the same model, leaves.
+    import paper_2110_00625_b200 as m
+    rng = np.random.default_rng(3)
+    x = torch.from_numpy(rng.standard_normal((4096, dims[0]), dtype=np.float32))
+    y = rng.integers(0, dims[-1], 4096).astype(np.int32)
+
+    def make(w1, K=K, beta=0.0, schedule=0):
+        g = m.Mavg(w1, P=P, K=K, local_lr=LR, mu=0.9, B=B, seed=5, objective=m.OBJ_MLP, dims=dims, gemm_bf16=1, x=x, y=y,
+                   x_bf16=x_bf16, defer_broadcast=defer, learner_momentum=beta, learner_momentum_reset=True,
+                   with_learner_u=True)
+        g.set_schedule(schedule)
+        return g
+
+    def steps_twice(g):
+        g.local_steps(); g.local_steps(); g.meta_update()
+
+    def host(g):
+        w, v = g.w.cpu(), g.v.cpu()
+        g.round_host(w, v)
+        assert torch.equal(w, g.w.cpu()) and torch.equal(v, g.v.cpu())
+
+    def run_out(g):
+        g.set_wait_limit(20_000)
+        g.selftest_wait()
+        with pytest.raises(m.MavgError):
+            g.sync()
+        g.set_wait_limit(0)
+        g.round()
+
+    a = make(m.workloads.mlp_init(dims))
+    turns = [(lambda: None, {}, a.round, "round"),
+             (lambda: a.set_schedule(2), dict(schedule=2), a.round, "round"),
+             (lambda: a.set_schedule(0), {}, a.round, "round"),
+             (lambda: a.set_hparams(1, LR, 1.0, 0.9), dict(K=1), a.round, "round"),
+             (lambda: a.set_hparams(K, LR, 1.0, 0.9), {}, lambda: steps_twice(a), "steps"),
+             (lambda: a.set_learner_momentum(0.9, True), dict(beta=0.9), a.round, "round"),
+             (lambda: a.set_learner_momentum(0.0, True), {}, lambda: host(a), "round"),
+             (lambda: a.set_schedule(2), dict(schedule=2), lambda: host(a), "round"),
+             (lambda: a.set_schedule(0), {}, lambda: run_out(a), "round"),
+             (lambda: None, {}, lambda: host(a), "round")]
+    for turn, (change, kw, call, plain_call) in enumerate(turns):
+        change()
+        w, v, done = a.w.clone(), a.v.clone(), a.get_round()
+        b = make(w.cpu().numpy(), **kw)
+        b.v.copy_(v)
+        b.set_round(done)
+        takes = not kw
+        assert a.factored() == b.factored() == takes, turn
+        call()
+        b.round() if plain_call == "round" else steps_twice(b)
+        a.materialize_replicas(); b.materialize_replicas()
+        a.sync(); b.sync()
+        assert np.array_equal(a.get_losses()[:, :b.K], b.get_losses()), turn
+        for p, q in ((a.w, b.w), (a.v, b.v), (a.replicas[:, :a.n], b.replicas[:, :b.n])):
+            assert torch.equal(p.view(torch.int32), q.view(torch.int32)), turn
+        b.close()
+    a.close()

@@ -25,6 +25,7 @@ def _handle(dims, K, lr, w1=None, schedule=0, **kw):
                gemm_bf16=1, x=x, y=y, x_bf16=True, defer_broadcast=True, **kw)
     g.set_schedule(schedule)
     assert g.get_step_plan()["fwd_with_wgrad"] == len(dims) - 2
+    assert not g.factored()          # rounds that keep no weights between their steps
     return g
 
 
@@ -38,6 +39,7 @@ SHAPES = [[3072, 1024, 512, 10], [3048, 1000, 504, 264, 10], [520, 1024, 1024, 5
 @pytest.mark.parametrize("K", [1, 2, 5])
 @pytest.mark.parametrize("beta", [0.0, 0.9])
 def test_a_step_of_length_zero_keeps_every_bit(dims, K, beta):
+    K = min(K, 8191 // (_learners(dims) * B))
     # local_lr = 0: w <- w + (-0) g leaves every value as it is, whatever steps it goes through;
     # values on and beside the ties of the bf16 rounding, subnormal ones and the largest below 1
     import paper_2110_00625_b200 as m
