@@ -649,27 +649,6 @@ struct LastArgs {
   float gamma;
 };
 
-__device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], const void* p) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_u32(p)) : "memory");
-}
-__device__ __forceinline__ void ldsm_x4_t(uint32_t (&r)[4], const void* p) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(smem_u32(p)) : "memory");
-}
-__device__ __forceinline__ void ldsm_x2(uint32_t (&r)[2], const void* p) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0, %1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(smem_u32(p)) : "memory");
-}
-__device__ __forceinline__ void ldsm_x2_t(uint32_t (&r)[2], const void* p) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0, %1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(smem_u32(p)) : "memory");
-}
-__device__ __forceinline__ void mma16816(float (&d)[4], const uint32_t (&a)[4], const uint32_t (&b)[2]) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
-}
-
 // Elements per row of a shared-memory array of `cols` columns (a multiple of 8): an odd number of 16-byte
 // units, so that eight consecutive rows start in different banks.
 __host__ __device__ constexpr int row_pitch(int cols) { return ((cols >> 3) | 1) << 3; }
@@ -756,8 +735,8 @@ k_fac_last(const LastArgs g) {
       ldsm_x4(a, arow_s + k);
       ldsm_x2(b, wrow_s + k);
       ldsm_x2(bl, wrow_s + k + (size_t)CP * ap);
-      mma16816(d, a, b);
-      mma16816(dl, a, bl);
+      mma_bf16(d, a, b[0], b[1]);
+      mma_bf16(dl, a, bl[0], bl[1]);
     }
 #pragma unroll
     for (int i = 0; i < 4; ++i) d[i] = with_low(d[i], dl[i]);
@@ -831,7 +810,7 @@ k_fac_last(const LastArgs g) {
       for (int m = 0; m < KC; ++m) {
         uint32_t a[4];
         ldsm_x4_t(a, Ds + (size_t)(b0 + (mi >> 1) * 8 + mr) * dp + m * 16 + (mi & 1) * 8);
-        mma16816(d[m], a, b);
+        mma_bf16(d[m], a, b[0], b[1]);
       }
     }
 #pragma unroll
@@ -858,7 +837,7 @@ k_fac_last(const LastArgs g) {
       for (int k = 0; k < KC; ++k) {
         uint32_t a[4];
         ldsm_x4(a, Ds + (size_t)(b0 + (mi & 1) * 8 + mr) * dp + k * 16 + (mi >> 1) * 8);
-        mma16816(d, a, wb[k]);
+        mma_bf16(d, a, wb[k][0], wb[k][1]);
       }
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
@@ -922,25 +901,6 @@ struct ApplyShared {
   uint32_t tmem_slot;
   int abort_flag;
 };
-
-__device__ __forceinline__ void store_3d(const CUtensorMap* m, const void* src, int c0, int c1, int c2) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.global.shared::cta.bulk_group [%0, {%2, %3, %4}], [%1];"
-      ::"l"(reinterpret_cast<uint64_t>(m)), "r"(smem_u32(src)), "r"(c0), "r"(c1), "r"(c2)
-      : "memory");
-}
-
-// Barrier over a group's 128 threads that also ORs a predicate over them.
-__device__ __forceinline__ bool group_any(bool pred, int id) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %1, 0;\n\t"
-      "barrier.red.or.pred p, %2, 128, q;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(r)
-      : "r"((uint32_t)pred), "r"(id)
-      : "memory");
-  return r != 0;
-}
 
 // Persistent: 128 x 256 tiles of W_l, learner by learner (their factors then stay in the L2 while all
 // tiles of the learner read them).  Two accumulators, so that a tile's contraction runs while the tile
@@ -1089,7 +1049,7 @@ k_fac_apply(const __grid_constant__ ApplyArgs g) {
         const uint32_t s = pn % PIECES;
         if (leader) {
           // the store that last read the buffer of the next fetch is done with it
-          asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(kStores) : "memory");
+          tma_store_wait_read<kStores>();
           fetch();
         }
         uint32_t acc[32];
@@ -1108,18 +1068,18 @@ k_fac_apply(const __grid_constant__ ApplyArgs g) {
           *cell = w;
         }
         fence_proxy_async();
-        if ((gone = group_any(failed, 2 + grp))) break;
+        if ((gone = barrier_any(failed, 2 + grp, 128))) break;
         if (leader) {
-          store_3d(&g.w_out[l], mine + (size_t)s * kPieceBytes, n0 + c * kApplyChunk, m0, p);
-          asm volatile("cp.async.bulk.commit_group;" ::: "memory");
+          tma_store_3d(&g.w_out[l], mine + (size_t)s * kPieceBytes, n0 + c * kApplyChunk, m0, p);
+          tma_store_commit();
         }
       }
       tc_fence_before_sync();
       __syncwarp();
-      if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&sh.acc_empty[b])) : "memory");
+      if (lane == 0) mbar_arrive(&sh.acc_empty[b]);
     }
     if (leader) {
-      asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+      tma_store_wait_read<0>();
       if (*abortp) drain_ring(sh.piece_full[grp], (int)fn, PIECES, g.status);
     }
   }

@@ -148,23 +148,8 @@ __device__ __forceinline__ void bulk_commit() {
 __device__ __forceinline__ void bulk_wait_read_all() {
   asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
 }
-__device__ __forceinline__ void mbar_arrive_plain(uint64_t* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(tc::smem_u32(bar)) : "memory");
-}
-// Barrier 1 over the `threads` consumer threads that also ORs a predicate over them: every
-// consumer learns whether any of them gave up a wait, so that they all leave the tile loop in the
-// same iteration and nobody is left behind at a counted barrier.
-__device__ __forceinline__ bool consumers_any(bool pred, int threads) {
-  uint32_t r;
-  asm volatile(
-      "{\n\t.reg .pred p, q;\n\tsetp.ne.u32 q, %1, 0;\n\t"
-      "barrier.red.or.pred p, 1, %2, q;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-      : "=r"(r)
-      : "r"((uint32_t)pred), "r"(threads)
-      : "memory");
-  return r != 0;
-}
-
+// Consumers that give up a wait leave the tile loop together: each tile's first barrier tells all of them
+// (barrier_any), so that nobody is left behind at a counted barrier.
 template <int T, int G, int STAGES, int THREADS>
 __global__ void __launch_bounds__(THREADS + 32)
 k_meta_update_bulk(float* __restrict__ rep, int64_t stride, float* __restrict__ w,
@@ -255,11 +240,11 @@ k_meta_update_bulk(float* __restrict__ rep, int64_t stride, float* __restrict__ 
         }
       }
       __syncwarp();
-      if (lane == 0) mbar_arrive_plain(&empty[s]);
+      if (lane == 0) tc::mbar_arrive(&empty[s]);
     }
     // the result buffers of the tile before last must have been read by their stores
     if (tid == 0) bulk_wait_read_all();
-    if (consumers_any(failed, THREADS)) break;
+    if (tc::barrier_any(failed, 1, THREADS)) break;
 #pragma unroll
     for (int i = 0; i < PER; i += 4) {
       float4 vt = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -276,7 +261,7 @@ k_meta_update_bulk(float* __restrict__ rep, int64_t stride, float* __restrict__ 
       *reinterpret_cast<float4*>(st_out + (size_t)(b * 2 + 1) * T + (i / 4) * THREADS * 4 + tid * 4) = vn;
     }
     __syncwarp();
-    if (lane == 0) mbar_arrive_plain(&wv_empty[b]);
+    if (lane == 0) tc::mbar_arrive(&wv_empty[b]);
     tc::fence_proxy_async();
     asm volatile("bar.sync 1, %0;" ::"n"(THREADS) : "memory");
     if (tid == 0) {

@@ -224,38 +224,18 @@ struct MmaPiece {
   }
 };
 
-__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const __nv_bfloat16* p) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(tc::smem_u32(p)) : "memory");
-}
-__device__ __forceinline__ void ldsm4_t(uint32_t (&r)[4], const __nv_bfloat16* p) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(tc::smem_u32(p)) : "memory");
-}
-__device__ __forceinline__ void ldsm2(uint32_t (&r)[2], const __nv_bfloat16* p) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0, %1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(tc::smem_u32(p)) : "memory");
-}
-__device__ __forceinline__ void ldsm2_t(uint32_t (&r)[2], const __nv_bfloat16* p) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x2.trans.shared.b16 {%0, %1}, [%2];" : "=r"(r[0]), "=r"(r[1]) : "r"(tc::smem_u32(p)) : "memory");
-}
-__device__ __forceinline__ void mma(float (&d)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0, %1, %2, %3}, {%4, %5, %6, %7}, {%8, %9}, {%0, %1, %2, %3};"
-      : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
 // 16 rows x 16 k of the MMA's row operand, 16 columns x 16 k (two of its column operands) from a plane.
 template <bool KC>
 __device__ __forceinline__ void row_operand(uint32_t (&r)[4], const __nv_bfloat16* pl, int row, int k) {
   const int i = threadIdx.x % 32 / 8, j = threadIdx.x % 8;
-  if (KC) ldsm4(r, pl + (row + (i & 1) * 8 + j) * kPitchK + k + (i >> 1) * 8);
-  else ldsm4_t(r, pl + (k + (i >> 1) * 8 + j) * kPitchR + row + (i & 1) * 8);
+  if (KC) tc::ldsm_x4(r, pl + (row + (i & 1) * 8 + j) * kPitchK + k + (i >> 1) * 8);
+  else tc::ldsm_x4_t(r, pl + (k + (i >> 1) * 8 + j) * kPitchR + row + (i & 1) * 8);
 }
 template <bool KC>
 __device__ __forceinline__ void col_operands(uint32_t (&r)[4], const __nv_bfloat16* pl, int row, int k) {
   const int i = threadIdx.x % 32 / 8, j = threadIdx.x % 8;
-  if (KC) ldsm4(r, pl + (row + (i >> 1) * 8 + j) * kPitchK + k + (i & 1) * 8);
-  else ldsm4_t(r, pl + (k + (i & 1) * 8 + j) * kPitchR + row + (i >> 1) * 8);
+  if (KC) tc::ldsm_x4(r, pl + (row + (i >> 1) * 8 + j) * kPitchK + k + (i & 1) * 8);
+  else tc::ldsm_x4_t(r, pl + (k + (i & 1) * 8 + j) * kPitchR + row + (i >> 1) * 8);
 }
 // One slab of the tile.  acc[mt][nt]: 16 x 8 results at rows 32 wm + 16 mt, columns 32 wn + 8 nt; mts, nps: how
 // many 16-row and 16-column groups of the warp's lie inside the result.
@@ -283,18 +263,19 @@ __device__ __forceinline__ void multiply_mma(const __nv_bfloat16* a, const __nv_
 #pragma unroll
       for (int mt = 0; mt < 2; ++mt) {
         if (mt >= mts) break;
-        mma(d[mt][2 * np], fa[mt], fb[0], fb[1]);
-        mma(d[mt][2 * np + 1], fa[mt], fb[2], fb[3]);
+        tc::mma_bf16(d[mt][2 * np], fa[mt], fb[0], fb[1]);
+        tc::mma_bf16(d[mt][2 * np + 1], fa[mt], fb[2], fb[3]);
       }
     }
   }
-  if (!FRESH) return;
+  if constexpr (FRESH) {
 #pragma unroll
-  for (int mt = 0; mt < 2; ++mt)
+    for (int mt = 0; mt < 2; ++mt)
 #pragma unroll
-    for (int nt = 0; nt < 4; ++nt)
+      for (int nt = 0; nt < 4; ++nt)
 #pragma unroll
-      for (int i = 0; i < 4; ++i) acc[mt][nt][i] += own[mt][nt][i];
+        for (int i = 0; i < 4; ++i) acc[mt][nt][i] += own[mt][nt][i];
+  }
 }
 
 // Four finished sums C(m, n .. n+3): the layer's tail and the store.
@@ -709,9 +690,9 @@ __device__ __forceinline__ void mma_tail(const TailArgs& t, int p, int r0, uint8
       float d[4] = {0.f, 0.f, 0.f, 0.f};
       for (int k = k0; k < min(in16, k0 + 64); k += 16) {
         uint32_t fa[4], fb[2];
-        ldsm4(fa, a + ((i8 & 1) * 8 + j8) * ip + k + (i8 >> 1) * 8);
-        ldsm2(fb, w + (size_t)(nt * 8 + j8) * ip + k + (i8 & 1) * 8);
-        mma(d, fa, fb[0], fb[1]);
+        tc::ldsm_x4(fa, a + ((i8 & 1) * 8 + j8) * ip + k + (i8 >> 1) * 8);
+        tc::ldsm_x2(fb, w + (size_t)(nt * 8 + j8) * ip + k + (i8 & 1) * 8);
+        tc::mma_bf16(d, fa, fb[0], fb[1]);
       }
       s[0] += d[0];
       s[1] += d[1];
@@ -737,9 +718,9 @@ __device__ __forceinline__ void mma_tail(const TailArgs& t, int p, int r0, uint8
       float d[4] = {0.f, 0.f, 0.f, 0.f};
       for (int k = k0; k < min(c16, k0 + 64); k += 16) {
         uint32_t fa[4], fb[2];
-        ldsm4(fa, dq + ((i8 & 1) * 8 + j8) * dp + k + (i8 >> 1) * 8);
-        ldsm2_t(fb, w + (size_t)(k + (i8 & 1) * 8 + j8) * ip + nt * 8);
-        mma(d, fa, fb[0], fb[1]);
+        tc::ldsm_x4(fa, dq + ((i8 & 1) * 8 + j8) * dp + k + (i8 >> 1) * 8);
+        tc::ldsm_x2_t(fb, w + (size_t)(k + (i8 & 1) * 8 + j8) * ip + nt * 8);
+        tc::mma_bf16(d, fa, fb[0], fb[1]);
       }
       s[0] += d[0];
       s[1] += d[1];
