@@ -291,32 +291,34 @@ def algorithmic_bytes(cfg, tensor_path, deferred=False, momentum=False, fwd_run_
 
 
 def factored_bytes(cfg, deferred=False, x_bytes=2):
-    """Bytes and flops per ROUND and kernel class of a round in factored form: products take w~ (read once
-    for all learners; the last hidden layer's forward product its low parts too) and the rows of the earlier
-    steps; the hidden layers' weights are written once, at the end."""
+    """Bytes and flops per ROUND and kernel class of a round in factored form: products take w~ (read once for all
+    learners, the forward products its low parts too) and the rows of the earlier steps; the hidden layers'
+    weights are written once, at the end.  "flops" are what the method asks for, two per weight, row and product;
+    "executed_flops" what the form issues: the low parts and the products with the earlier steps' rows besides."""
     dims, P, K, B = cfg["dims"], cfg["P"], cfg["K"], cfg["B"]
     L = len(dims) - 1
     nW = [dims[l] * dims[l + 1] for l in range(L)]
     n = sum(nW) + sum(dims[1:])
-    rows, all_rows = P * B, P * K * B
+    all_rows = P * K * B
     hist = P * B * K * (K - 1) // 2                       # history rows over all steps and learners
     pairs = hist * B                                      # (batch row, history row) pairs
-    fwd = dict(bytes=2 * nW[0] + 2 * 2 * all_rows * dims[0] + 2 * 4 * all_rows * dims[1],   # X W~_1^T, X X^T, base
-               flops=2 * all_rows * nW[0] + 2 * pairs * (dims[0] + dims[1]))
+    hidden = nW[:-1]
+    fwd = dict(bytes=2 * 2 * nW[0] + 2 * 2 * all_rows * dims[0] + 2 * 4 * all_rows * dims[1],   # X W~_1^T, X X^T, base
+               flops=2 * all_rows * sum(hidden),
+               executed_flops=2 * 2 * all_rows * nW[0] + 2 * pairs * (dims[0] + dims[1]))
     fwd["bytes"] += 2 * 2 * pairs + 2 * (hist + all_rows) * dims[1]                          # F_1
-    dgrad = dict(bytes=0, flops=0)
+    dgrad = dict(bytes=0, flops=2 * all_rows * sum(hidden[1:]), executed_flops=0)
     for l in range(1, L - 1):                             # layer l + 1: dims[l] -> dims[l + 1]
-        parts = 2 if l == L - 2 else 1
-        fwd["bytes"] += (K * 2 * parts * nW[l] + 2 * all_rows * (2 * dims[l] + dims[l + 1])
+        fwd["bytes"] += (K * 2 * 2 * nW[l] + 2 * all_rows * (2 * dims[l] + dims[l + 1])
                          + 2 * hist * (dims[l] + dims[l + 1]) + 2 * 2 * pairs)
-        fwd["flops"] += 2 * all_rows * nW[l] * parts + 2 * pairs * (dims[l] + dims[l + 1])
+        fwd["executed_flops"] += 2 * 2 * all_rows * nW[l] + 2 * pairs * (dims[l] + dims[l + 1])
         dgrad["bytes"] += (K * 2 * nW[l] + 2 * all_rows * (2 * dims[l + 1] + 2 * dims[l])
                            + 2 * hist * (dims[l] + dims[l + 1]) + 2 * 2 * pairs)
-        dgrad["flops"] += 2 * all_rows * nW[l] + 2 * pairs * (dims[l] + dims[l + 1])
-    hidden = nW[:-1]
+        dgrad["executed_flops"] += 2 * all_rows * nW[l] + 2 * pairs * (dims[l] + dims[l + 1])
     return {
         "meta_update": dict(bytes=((4 if deferred else 8) * P + 16) * n, flops=0),
-        "batch_gather": dict(bytes=all_rows * dims[0] * (x_bytes + 2), flops=0),
+        # (the low parts of w~ are written beside the batch)
+        "batch_gather": dict(bytes=all_rows * dims[0] * (x_bytes + 2) + 6 * sum(hidden), flops=0),
         "fwd_gemm": fwd,
         "loss": dict(bytes=2 * 2 * all_rows * dims[L - 1] + K * 8 * P * nW[-1], flops=6 * all_rows * nW[-1]),
         "dgrad_gemm": dgrad,
@@ -340,6 +342,8 @@ def kernel_rooflines(per_round, prof, steps, peaks):
             if w["flops"]:
                 e["tflops"] = w["flops"] * steps / sec / 1e12
                 e["frac_tensor"] = e["tflops"] / peaks["bf16_tflops_sustained"]
+                if "executed_flops" in w:
+                    e["executed_tflops"] = w["executed_flops"] * steps / sec / 1e12
             e["bytes_per_launch"] = w["bytes"] * steps / cnt
         out[name] = e
     return out
@@ -609,6 +613,8 @@ def measure_mlp(name, args, m, torch, dist, peaks, world, rank, local, steps, wi
         roof["peak_source"] = peaks["source"]
         roof["bytes_per_launch"] = e["bytes_per_launch"]
         roof["ms_per_launch"] = e["ms_per_launch"]
+        if "executed_tflops" in e:       # "achieved" counts the method's flops only
+            roof["executed_tflops"] = e["executed_tflops"]
         if mode == 1 and not args.learners and not args.beta and not factored:
             roof["traffic"] = NCU_TRAFFIC.get(name, {}).get(dom)
     # the whole round against the HBM roofline: every class's algorithmic bytes / the round's time

@@ -71,11 +71,19 @@ def test_factored_rounds_write_the_weights_once_and_grow_with_the_history():
     R = P * K * B
     assert per["wgrad_sgd_gemm"] == dict(bytes=2 * R * (3072 + 3 * 2048 + 2 * 2048) + 4 * 33 * sum(nW),
                                          flops=2 * R * sum(nW))
-    # a round of one step has no history: the products of the plain form's first step, read once for all
+    # a round of one step has no history: what it executes beyond the method is the low parts of w~
     one = b.factored_bytes(dict(CFG, K=1))
-    assert one["fwd_gemm"]["flops"] == 2 * P * B * (nW[0] + nW[1] + 2 * nW[2])
-    assert one["dgrad_gemm"]["flops"] == 2 * P * B * (nW[1] + nW[2])
+    assert one["fwd_gemm"]["executed_flops"] == 2 * one["fwd_gemm"]["flops"] == 2 * 2 * P * B * sum(nW)
+    assert one["dgrad_gemm"]["executed_flops"] == one["dgrad_gemm"]["flops"] == 2 * P * B * (nW[1] + nW[2])
     # the history of step k is (k - 1) B rows a learner: K (K - 1) / 2 batches in all
-    two, four = (b.factored_bytes(dict(CFG, K=k))["dgrad_gemm"]["flops"] for k in (2, 4))
+    two, four = (b.factored_bytes(dict(CFG, K=k))["dgrad_gemm"]["executed_flops"] for k in (2, 4))
     extra = lambda k, f: f - k * one["dgrad_gemm"]["flops"]
     assert extra(4, four) == 6 * extra(2, two) == 6 * 2 * P * B * B * 2 * (2048 + 2048)
+
+
+def test_factored_rounds_count_the_flops_of_the_method_and_no_others():
+    # whatever the form adds, a round does the plain form's flops
+    b = _bench()
+    plain, fac = b.algorithmic_bytes(CFG, True, deferred=True), b.factored_bytes(CFG, deferred=True)
+    total = lambda per: sum(v["flops"] for v in per.values())
+    assert total(plain) == total(fac) == b.flop_per_sample(CFG["dims"]) * CFG["P"] * CFG["K"] * CFG["B"]
