@@ -197,9 +197,9 @@ __device__ __forceinline__ void load16(uint32_t taddr, bool any, float (&z)[16])
   }
 }
 
-// Bound by the operands' way into the SM and, late in a round, by the history in HBM: P = 32, B = 64, layers of
-// 2048: 20 us in the first step (860 TFLOP/s), 42 us in the sixteenth (another 126 MB of history and 4 MB of
-// Gram rows).  Per-slab divisions in the two issuing threads cost 2 to 6 us of that.
+// Bound by the operands' way into the SM and the tensor pipe and, late in a round, by the history in HBM: P = 32,
+// B = 64, layers of 2048: data gradient 24 us in the first step, 45 us in the sixteenth (another 126 MB of history
+// and 4 MB of Gram rows); forward with both parts of w~ 30 us (1140 TFLOP/s) and 50.  Per-slab divisions in the two issuing threads cost 2 to 6 us of that.
 // grid (column tiles x m_tiles, learner groups).  dgrad with several column tiles: these are a cluster,
 // whose first block adds their bias gradients in rank order.
 // TILES: 16 KB tiles of the MMA's row operand per stage.  LOW (two tiles): the product with w~ reads its low
@@ -1114,7 +1114,7 @@ FacCols cols_for(int P, int B, long row_tiles, int sm_count, int most_learners =
 // Cut of a product that forms its own Gram rows where it can: short launches (a learner per block at most, so
 // that the blocks take the SMs) of at most four row tiles, which with the column tiles are one cluster.
 // us a round with the Gram rows in launches of their own / in the product's: 3072-512-512-10, K = 8, P = 8,
-// B = 128 479 / 455, P = 48, B = 64 861 / 844; 520-200-136-12, P = 20, K = 9, B = 48 367 / 334; six row tiles:
+// B = 128 475 / 469, P = 48, B = 64 876 / 861; 520-200-136-12, P = 20, K = 9, B = 48 372 / 339; six row tiles:
 // 1504-672-672-11, P = 10, K = 8, B = 176 788 / 793; eight: 3072-1024-1024-1024-10, P = 16, K = 8, B = 64
 // 977 / 1288 (clusters of eight blocks of one per SM).
 FacCols product_cols(int P, int B, int rows, int sm_count) {
