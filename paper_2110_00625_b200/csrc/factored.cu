@@ -26,6 +26,7 @@ using namespace gemm;
 
 constexpr int kFacThreads = 320;   // warp 0: TMA producer, warp 1: MMA issuer, warps 2-9: epilogue
 enum { PROD_FWD = 0, PROD_DGRAD = 1, PROD_RAW = 2 };
+constexpr size_t kGramBarBytes = 2 * sizeof(uint64_t);   // static shared memory of a product that forms its Gram rows, beside GemmShared
 
 // Place in a ring of stages and the phase of its barriers, without a division per slab: the one thread that
 // issues the copies and the one that issues the MMAs are on every slab's way.
@@ -894,7 +895,7 @@ struct ApplyArgs {
   int* status;
 };
 template <int STAGES, int PIECES>
-struct ApplyShared {
+struct alignas(16) ApplyShared {            // (whole 16 bytes, as static shared memory is counted)
   uint64_t full_bar[STAGES], empty_bar[STAGES];
   uint64_t acc_full[2], acc_empty[2];
   uint64_t piece_full[2][PIECES];
@@ -1182,7 +1183,7 @@ cudaError_t launch_product(mavg_ctx* c, int cls, const CUtensorMap& w, const CUt
   size_t smem = (size_t)g.stages * stage_bytes + 1024 +
                 (EPI == PROD_DGRAD ? (size_t)2 * g.nl * kBM * sizeof(float) : 0);
   const int cluster = GRAM ? (int)grid.x : EPI == PROD_DGRAD ? g.c_tiles : 1;
-  if (cluster > 1) smem = std::max(smem, tmem_share_bytes(g.tmem_cols, sizeof(GemmShared) + (GRAM ? 2 * sizeof(uint64_t) : 0)));
+  smem = std::max(smem, tmem_share_bytes(g.tmem_cols, sizeof(GemmShared) + (GRAM ? kGramBarBytes : 0)));
   PdlLaunch l(grid, kFacThreads, smem, c->stream, cluster);
   prof_begin(c, cls);
   cudaError_t e = cudaLaunchKernelEx(&l.lc, k_fac_product<EPI, TILES, LOW, GRAM>, w, lo, in, gram ? *gram : in, hist, s, g);
@@ -1201,7 +1202,8 @@ cudaError_t launch_gram(mavg_ctx* c, int cls, const CUtensorMap& hist, const CUt
   g.tmem_cols = tmem_columns(g.BN);
   g.gamma = c->cfg.local_lr;
   g.status = (int*)ws_ptr(c, c->ws.status);
-  PdlLaunch l(grid, kFacThreads, (size_t)g.stages * stage_bytes + 1024, c->stream);
+  PdlLaunch l(grid, kFacThreads, std::max((size_t)g.stages * stage_bytes + 1024, tmem_share_bytes(g.tmem_cols, sizeof(GemmShared))),
+              c->stream);
   prof_begin(c, cls);
   cudaError_t e = cudaLaunchKernelEx(&l.lc, k_fac_gram, hist, b, g);
   prof_end(c);
@@ -1347,14 +1349,17 @@ void fac_setup(mavg_ctx* c, TcState* st) {
     ok = ok && encode_map(st, &f->s_f[l], bf(t.s[0]), (int)t.s_ld, B, P, t.s_ld, B * t.s_ld, f->fwd[l].cols, why);
     ok = ok && encode_map(st, &f->s_d[l], bf(t.s[1]), (int)t.s_ld, B, P, t.s_ld, B * t.s_ld, f->dgrad[l].cols, why);
   }
-  const void* kernels[] = {
-      (const void*)k_fac_product<PROD_FWD, 2, false, false>, (const void*)k_fac_product<PROD_FWD, 2, true, false>,
-      (const void*)k_fac_product<PROD_RAW, 2, true, false>,  (const void*)k_fac_product<PROD_DGRAD, 1, false, false>,
-      (const void*)k_fac_product<PROD_FWD, 2, true, true>,   (const void*)k_fac_product<PROD_DGRAD, 1, false, true>,
-      (const void*)k_fac_gram, (const void*)k_fac_last<1>, (const void*)k_fac_last<2>,
-      (const void*)k_fac_apply<kApplyStages, kApplyPieces>};
-  for (const void* k : kernels)
-    ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, 225 * 1024) == cudaSuccess;
+  // what a block can have beside its static shared memory: all of it, for 512 columns of tensor memory
+  constexpr size_t kFixed = sizeof(GemmShared), kGramFixed = kFixed + kGramBarBytes;
+  const struct { const void* kernel; size_t fixed; } kernels[] = {
+      {(const void*)k_fac_product<PROD_FWD, 2, false, false>, kFixed}, {(const void*)k_fac_product<PROD_FWD, 2, true, false>, kFixed},
+      {(const void*)k_fac_product<PROD_RAW, 2, true, false>, kFixed}, {(const void*)k_fac_product<PROD_DGRAD, 1, false, false>, kFixed},
+      {(const void*)k_fac_product<PROD_FWD, 2, true, true>, kGramFixed}, {(const void*)k_fac_product<PROD_DGRAD, 1, false, true>, kGramFixed},
+      {(const void*)k_fac_gram, kFixed}, {(const void*)k_fac_last<1>, 0}, {(const void*)k_fac_last<2>, 0},
+      {(const void*)k_fac_apply<kApplyStages, kApplyPieces>, sizeof(ApplyShared<kApplyStages, kApplyPieces>)}};
+  for (const auto& k : kernels)
+    ok = ok && cudaFuncSetAttribute(k.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)(kSmSharedBytes - kBlockReservedBytes - k.fixed)) == cudaSuccess;
   if (ok) {
     st->fac = f;
   } else {
@@ -1558,7 +1563,9 @@ cudaError_t fac_local_steps(mavg_ctx* c, int64_t round) {
       g.w_out[l - 1] = st->w32[l];
     }
     g.tiles = g.per_learner * P;
-    PdlLaunch l(dim3((unsigned)std::min(g.tiles, c->sm_count)), kFacThreads, apply_smem(kApplyStages, kApplyPieces),
+    PdlLaunch l(dim3((unsigned)std::min(g.tiles, c->sm_count)), kFacThreads,
+                std::max(apply_smem(kApplyStages, kApplyPieces),
+                         tmem_share_bytes(2 * kApplyBN, sizeof(ApplyShared<kApplyStages, kApplyPieces>))),
                 c->stream);
     prof_begin(c, MAVG_K_WGRAD_SGD);
     e = cudaLaunchKernelEx(&l.lc, k_fac_apply<kApplyStages, kApplyPieces>, g);

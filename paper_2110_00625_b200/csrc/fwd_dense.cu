@@ -184,7 +184,7 @@ cudaError_t launch_fwd_dense(mavg_ctx* c, const DensePlan& pl, const CUtensorMap
   cudaLaunchConfig_t lc{};
   lc.gridDim = dim3((unsigned)(pl.m_tiles * pl.n_tiles));
   lc.blockDim = dim3(kDenseThreads);
-  lc.dynamicSmemBytes = pl.smem;
+  lc.dynamicSmemBytes = std::max(pl.smem, tmem_share_bytes(kDenseCols, sizeof(GemmShared)));
   lc.stream = c->stream;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

@@ -88,18 +88,6 @@ struct GemmShared {
   float colsum[2][kBM];
 };
 
-// Blocks of a cluster wait on one another while they hold tensor memory, and neither tcgen05.alloc nor
-// barrier.cluster.wait has a time limit.  So whatever lies on an SM beside such a block -- of this launch, of another
-// handle's on another stream -- must leave it its columns: the cluster launches that hold tensor memory ask for the
-// same share of an SM's shared memory as of its 512 columns, and blocks that fit by the one then fit by the other.
-// (Blocks that wait on nobody of their own launch give their columns back by themselves.)
-// Returns the least dynamic shared memory of a block of `columns` columns and `fixed` bytes of static shared memory.
-constexpr size_t kSmSharedBytes = 228 * 1024, kBlockReservedBytes = 1024;   // of which a block loses the latter
-__host__ __device__ constexpr size_t tmem_share_bytes(uint32_t columns, size_t fixed) {
-  const size_t share = kSmSharedBytes / 512 * columns;
-  return share > fixed + kBlockReservedBytes ? share - fixed - kBlockReservedBytes : 0;
-}
-
 // Barrier set-up of one tile (one thread): every barrier at phase 0.
 __device__ __forceinline__ void gemm_init_barriers(GemmShared& sh, int stages) {
   for (int s = 0; s < stages; ++s) {

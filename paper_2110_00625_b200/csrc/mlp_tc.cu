@@ -306,6 +306,7 @@ cudaError_t launch_gemm(mavg_ctx* c, int cls, const CUtensorMap& a, const CUtens
   size_t smem = pipe + 1024;
   if (EPI == EPI_FWD_LAST)   // the loss tail reuses the pipeline buffers: logits, dZ, row losses
     smem = std::max(pipe, ((size_t)2 * g.N * g.M + g.N) * sizeof(float)) + 1024;
+  smem = std::max(smem, tmem_share_bytes(pl.tmem_cols, sizeof(GemmShared)));
   dim3 grid((unsigned)(pl.m_tiles * pl.n_tiles * pl.splits), (unsigned)c->cfg.P);
   cudaLaunchConfig_t lc{};
   lc.gridDim = grid;

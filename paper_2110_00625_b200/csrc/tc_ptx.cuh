@@ -294,6 +294,16 @@ __device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&a)[4], 
 }
 
 // ---- tensor memory -----------------------------------------------------------------------------
+// tcgen05.alloc waits, without a time limit, for columns that other blocks of the SM hold, and blocks that hold
+// some may be waiting for others: those of a cluster for one another, a successor's for the kernel before it, with
+// launches of several handles side by side.  So no allocation ever waits: every launch asks for at least the same
+// share of an SM's shared memory as of its 512 columns, and whatever blocks an SM admits have their columns.
+// Returns the least dynamic shared memory of a block of `columns` columns and `fixed` bytes of static shared memory.
+constexpr size_t kSmSharedBytes = 228 * 1024, kBlockReservedBytes = 1024;   // of which a block loses the latter
+__host__ __device__ constexpr size_t tmem_share_bytes(uint32_t columns, size_t fixed) {
+  const size_t share = kSmSharedBytes / 512 * columns;
+  return share > fixed + kBlockReservedBytes ? share - fixed - kBlockReservedBytes : 0;
+}
 __device__ __forceinline__ void tmem_alloc(uint32_t* slot_in_smem, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(
                    smem_u32(slot_in_smem)),

@@ -56,6 +56,11 @@ namespace {
 using namespace tc;
 using namespace wgrad;
 
+// Tensor memory of a block: two accumulators of 32 columns; with a riding forward product a third of B columns behind them.
+__host__ __device__ constexpr uint32_t wgrad_columns(bool fwd_next, int batch) {
+  return !fwd_next ? 64u : (batch <= 64 ? 128u : 256u);
+}
+
 template <bool MOM, bool FWD>
 __global__ void __launch_bounds__(FWD ? kThreadsFwd : kThreads, 1)
 k_wgrad_sgd_stream(const __grid_constant__ CUtensorMap tm_dzt,   // bf16 [P, out, B]  load
@@ -90,8 +95,7 @@ k_wgrad_sgd_stream(const __grid_constant__ CUtensorMap tm_dzt,   // bf16 [P, out
     fence_barrier_init();
     fence_proxy_async();
   }
-  // two accumulators of 32 columns; with fwd_next a third of B columns behind them
-  const uint32_t tmem_cols = !(FWD && g.fwd_next) ? 64u : (g.batch <= 64 ? 128u : 256u);
+  const uint32_t tmem_cols = wgrad_columns(FWD && g.fwd_next, g.batch);
   if (warp == 1) {
     tmem_alloc(&sh.tmem_slot, tmem_cols);
     tmem_relinquish();
@@ -309,7 +313,7 @@ cudaError_t launch_wgrad_multi(mavg_ctx* c, int n, const WgradLayerRef* layers, 
   cudaLaunchConfig_t lc{};
   lc.gridDim = dim3((unsigned)grid);
   lc.blockDim = dim3(kThreads);
-  lc.dynamicSmemBytes = smem;
+  lc.dynamicSmemBytes = std::max(smem, tmem_share_bytes(64, sizeof(WgradShared)));
   lc.stream = c->stream;
   cudaLaunchAttribute at_[1];
   at_[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -355,7 +359,7 @@ cudaError_t launch_wgrad_stream(mavg_ctx* c, const WgradPlan& w, const CUtensorM
   cudaLaunchConfig_t lc{};
   lc.gridDim = dim3((unsigned)w.grid);
   lc.blockDim = dim3(fn ? kThreadsFwd : kThreads);
-  lc.dynamicSmemBytes = w.smem;
+  lc.dynamicSmemBytes = std::max(w.smem, tmem_share_bytes(wgrad_columns(fn != nullptr, c->cfg.B), sizeof(WgradShared)));
   lc.stream = c->stream;
   cudaLaunchAttribute at_[1];
   at_[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;

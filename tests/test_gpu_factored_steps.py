@@ -307,3 +307,36 @@ def test_rounds_of_either_form_on_one_handle(dims, P, K, B, x_bf16, defer):
             assert torch.equal(p.view(torch.int32), q.view(torch.int32)), turn
         b.close()
     a.close()
+
+
+def test_handles_on_streams_of_their_own_side_by_side():
+    # launches of clusters that wait within themselves, of few and of many columns of tensor memory, and a handle in
+    # the plain form, all at once: the bits of each on its own
+    picks = [(SHAPES[6], 0), (SHAPES[1], 0), (([3072, 512, 512, 10], 4, 2, 64), 0), (SHAPES[5], 0), (SHAPES[1], 2)]
+
+    def run(together):
+        handles = []
+        for shape, schedule in picks:
+            torch.cuda.synchronize()
+            stream = torch.cuda.Stream()
+            with torch.cuda.stream(stream):
+                handles.append(_handle(*shape, schedule=schedule, defer_broadcast=True, stream=stream)[0])
+            stream.synchronize()
+        if together:
+            for _ in range(10):
+                for g in handles:
+                    g.round()
+        else:
+            for g in handles:
+                for _ in range(10):
+                    g.round()
+                g.sync()
+        out = []
+        for g in handles:
+            g.sync()
+            out.append((g.w.cpu().numpy().view(np.uint32), g.v.cpu().numpy().view(np.uint32)))
+            g.close()
+        return out
+
+    for alone, beside in zip(run(False), run(True)):
+        assert np.array_equal(alone[0], beside[0]) and np.array_equal(alone[1], beside[1])
