@@ -82,7 +82,8 @@ __device__ __forceinline__ uint4 load8_bf16<float>(const float* src) {
 // both parts (16 bits of the weights).  A rounding of the weights is the same for every sample, step and learner
 // here, where the plain form rounds each learner's own weights at every step, so it does not average out: with
 // one bf16 part v or the mean loss can be further from 64 bits than the plain form's.  Root mean square of
-// v's relative error and of the mean loss's error over 12 seeds, plain / one part / both parts in every hidden layer:
+// v's relative error and of the mean loss's error over 12 seeds (both forms' roundings restated in torch), plain / one
+// part / both parts in every hidden layer:
 //   1000-312-10, P = 40, K = 4, B = 80:            v 3.6e-3 / 3.9e-3 / 0.4e-3, loss 1.1e-4 / 0.7e-4 / 0.4e-4
 //   the same, inputs in [0, 1]:                    v 1.8e-3 / 2.0e-3 / 0.6e-3, loss 2.9e-4 / 3.3e-4 / 0.1e-4
 //   520-200-136-12, P = 20, K = 9, B = 48, [0, 1]: v 3.0e-3 / 3.2e-3 / 2.1e-3, loss 2.1e-4 / 2.4e-4 / 0.3e-4
