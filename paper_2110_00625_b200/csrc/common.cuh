@@ -108,6 +108,7 @@ struct mavg_ctx {
   mavg::Workspace ws;
   std::vector<mavg::MlpLayer> layers;
   void* mlp = nullptr;        // state of the MLP path (owned by mlp files)
+  void* simt = nullptr;       // the same of the path for fp32 and any shapes
   mavg::ShadowMap shadow;     // set by the tensor-core path; dst == nullptr otherwise
   bool shadow_fresh = false;  // the last meta-update wrote the bf16 copy of w~ itself
   // per-launch timing (mavg_set_profiling): one event pair per launch, summed per kernel class

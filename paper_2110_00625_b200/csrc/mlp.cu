@@ -37,11 +37,8 @@ mavg_status mlp_setup(mavg_ctx* c) {
     c->layers.push_back(ly);
   }
   if (use_tensor_cores(&cfg)) return tc_setup(c);
-  cudaError_t e = simt_setup(c);
-  if (e != cudaSuccess) {
-    c->err = std::string("kernel attributes: ") + cudaGetErrorString(e);
-    return MAVG_ERR_CUDA;
-  }
+  const mavg_status st = simt_setup(c);
+  if (st != MAVG_OK) return st;
   small_setup(c);
   return MAVG_OK;
 }
@@ -51,6 +48,7 @@ void mlp_drop_graph(mavg_ctx* c);
 void mlp_teardown(mavg_ctx* c) {
   mlp_drop_graph(c);
   if (c->mlp) tc_teardown(c);
+  if (c->simt) simt_teardown(c);
 }
 
 void mlp_reset_counters(mavg_ctx* c) {

@@ -30,9 +30,10 @@ cudaError_t launch_batch_indices(mavg_ctx* c, int64_t round, int step, int j, in
 cudaError_t launch_sample_gather(mavg_ctx* c, int64_t round, int step, int32_t* idx,
                                  int32_t* labels, __nv_bfloat16* out_bf, __nv_bfloat16* out_bft);
 
-// CUDA-core path (mlp_simt.cu): fp32 arithmetic, or bf16-rounded operands with fp32 FMAs.
+// fp32 arithmetic, or bf16 operands of any shape (mlp_simt.cu).
 size_t simt_workspace_bytes(const mavg_config* cfg, size_t base, size_t* act_off);
-cudaError_t simt_setup(mavg_ctx* c);      // once per handle
+mavg_status simt_setup(mavg_ctx* c);      // once per handle
+void simt_teardown(mavg_ctx* c);
 cudaError_t simt_step(mavg_ctx* c, int64_t round, int step);
 
 // Small models on the CUDA cores (mlp_small.cu): all local steps of a round in one launch.

@@ -419,15 +419,8 @@ mavg_status tc_setup(mavg_ctx* c) {
   TcState* st = new TcState();
   c->mlp = st;
   st->lay = make_layout(&cfg, c->ws.act, kPlanSmCount);
-  void* fn = nullptr;
-  cudaDriverEntryPointQueryResult qres;
-  cudaError_t e = cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &fn, cudaEnableDefault, &qres);
-  if (e != cudaSuccess || !fn || qres != cudaDriverEntryPointSuccess) {
-    c->err = "cuTensorMapEncodeTiled is not available from this driver";
-    cudaGetLastError();
-    return MAVG_ERR_UNSUPPORTED;
-  }
-  st->encode = (EncodeTiledFn)fn;
+  st->encode = tensor_map_encoder(&c->err);
+  if (!st->encode) return MAVG_ERR_UNSUPPORTED;
   const TcLayout& t = st->lay;
   const int L = cfg.n_layers, P = cfg.P, B = cfg.B;
   char* ws = (char*)c->buf.workspace;
@@ -515,7 +508,7 @@ mavg_status tc_setup(mavg_ctx* c) {
   }
   // 227 KB per block in all, of which a few hundred bytes are the kernel's static variables
   constexpr int kMaxDynSmem = 225 * 1024;
-  e = cudaSuccess;
+  cudaError_t e = cudaSuccess;
   const void* kernels[] = {(const void*)k_tc_gemm<EPI_FWD_HIDDEN, 1>, (const void*)k_tc_gemm<EPI_FWD_HIDDEN, 2>,
                            (const void*)k_tc_gemm<EPI_FWD_LAST, 1>,   (const void*)k_tc_gemm<EPI_FWD_LAST, 2>,
                            (const void*)k_tc_gemm<EPI_DGRAD, 1>,      (const void*)k_tc_gemm<EPI_DGRAD, 2>,

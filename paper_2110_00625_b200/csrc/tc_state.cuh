@@ -9,6 +9,7 @@
 #include "factored.cuh"
 #include "fwd_dense.cuh"
 #include "gemm_unit.cuh"
+#include "tensor_map.cuh"
 #include "wgrad_tc.cuh"
 
 namespace mavg {
@@ -47,11 +48,6 @@ struct TcLayout {
 
 
 struct GemmPlan { int m_tiles, n_tiles, splits, kb_per_split, nkb, BN, stages, two_per_sm; uint32_t tmem_cols; };
-
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*,
-                                  const cuuint64_t*, const cuuint64_t*, const cuuint32_t*,
-                                  const cuuint32_t*, CUtensorMapInterleave, CUtensorMapSwizzle,
-                                  CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
 struct TcState {
   TcLayout lay;
@@ -120,21 +116,11 @@ struct TcState {
 };
 
 
-// Tensor [batch, rows, inner] with the given strides (in elements) and box inner x box_rows x box_batch.
 inline bool encode_any(TcState* st, CUtensorMap* m, CUtensorMapDataType dt, int esize, void* ptr,
                 int inner, int rows, int batch, int64_t row_stride, int64_t batch_stride,
                 int box_inner, int box_rows, CUtensorMapSwizzle swz, std::string* why, int box_batch = 1) {
-  cuuint64_t dims[3] = {(cuuint64_t)inner, (cuuint64_t)rows, (cuuint64_t)batch};
-  cuuint64_t strides[2] = {(cuuint64_t)row_stride * esize, (cuuint64_t)batch_stride * esize};
-  cuuint32_t box[3] = {(cuuint32_t)box_inner, (cuuint32_t)box_rows, (cuuint32_t)box_batch};
-  cuuint32_t es[3] = {1, 1, 1};
-  CUresult r = st->encode(m, dt, 3, ptr, dims, strides, box, es, CU_TENSOR_MAP_INTERLEAVE_NONE, swz,
-                          CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-  if (r != CUDA_SUCCESS) {
-    if (why) *why = "cuTensorMapEncodeTiled failed with code " + std::to_string((int)r);
-    return false;
-  }
-  return true;
+  return encode_tiled(st->encode, m, dt, esize, ptr, inner, rows, batch, row_stride, batch_stride, box_inner, box_rows, swz, why,
+                      box_batch);
 }
 
 // bf16 operand of an MMA: 64-element K slabs, 128-byte swizzle.
