@@ -7,6 +7,7 @@
 #include <map>
 #include <mutex>
 #include <set>
+#include <vector>
 #include <new>
 
 #include "common.cuh"
@@ -121,19 +122,9 @@ mavg_status cuda_fail(mavg_ctx* c, cudaError_t e, const char* where) {
     if (e__ != cudaSuccess) return cuda_fail((c), e__, where); \
   } while (0)
 
-// mean of the P*K per-step losses, on the device, into ws.loss_mean
-__global__ void k_mean_loss(const float* __restrict__ losses, int count, float* __restrict__ out) {
-  __shared__ float part[32];
-  float acc = 0.f;
-  for (int i = threadIdx.x; i < count; i += blockDim.x) acc += losses[i];
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    float s = threadIdx.x < (blockDim.x >> 5) ? part[threadIdx.x] : 0.f;
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (threadIdx.x == 0) out[0] = s / (float)count;
-  }
+// mean of the P*K per-step losses
+__global__ void __launch_bounds__(256) k_mean_loss(const float* __restrict__ losses, int count, float* __restrict__ out) {
+  block_mean(losses, count, out);
 }
 
 // A wait that cannot be satisfied: one warp, a barrier that expects an arrival nobody makes.  The
@@ -182,15 +173,20 @@ mavg_status do_meta_update(mavg_ctx* c) {
 
 mavg_status read_mean_loss(mavg_ctx* c, float* mean_loss) {
   if (c->cfg.objective == MAVG_OBJ_MLP) {
-    float* lm = (float*)ws_ptr(c, c->ws.loss_mean);
-    prof_begin(c, MAVG_K_LOSS);
-    k_mean_loss<<<1, 256, 0, c->stream>>>((const float*)ws_ptr(c, c->ws.losses),
-                                          c->cfg.P * c->cfg.K, lm);
-    prof_end(c);
-    CU(c, cudaGetLastError(), "mean-loss kernel");
-    CU(c, cudaMemcpyAsync(mean_loss, lm, sizeof(float), cudaMemcpyDeviceToHost, c->stream),
-       "loss read-back");
+    float* lm = c->mean_dev ? c->mean_dev : (float*)ws_ptr(c, c->ws.loss_mean);
+    if (!c->mean_formed) {
+      prof_begin(c, MAVG_K_LOSS);
+      k_mean_loss<<<1, 256, 0, c->stream>>>((const float*)ws_ptr(c, c->ws.losses),
+                                            c->cfg.P * c->cfg.K, lm);
+      prof_end(c);
+      CU(c, cudaGetLastError(), "mean-loss kernel");
+    }
+    c->mean_formed = false;
+    if (!c->mean_dev)
+      CU(c, cudaMemcpyAsync(mean_loss, lm, sizeof(float), cudaMemcpyDeviceToHost, c->stream),
+         "loss read-back");
     CU(c, cudaStreamSynchronize(c->stream), "stream synchronize");
+    if (c->mean_dev) *mean_loss = *(volatile const float*)c->mean_host;
   } else {
     CU(c, cudaStreamSynchronize(c->stream), "stream synchronize");
     *mean_loss = 0.f;
@@ -239,6 +235,38 @@ bool keep_acquire(int dev, size_t want) {
   cudaGetLastError();
   k.wants.erase(k.wants.find(want));
   return false;
+}
+
+// Words of pinned memory that rounds leave their mean loss in, one per handle: a page for the process, allocated by its
+// first handle (a pinned allocation takes about a millisecond).  A handle that finds none free, or no page, has its mean
+// copied back from the workspace.
+constexpr int kMeanWords = 4096 / sizeof(float);
+std::mutex g_mean_mu;
+float* g_mean_page = nullptr;
+std::vector<float*> g_mean_free;
+
+void mean_word_acquire(float** host, float** dev) {
+  std::lock_guard<std::mutex> lock(g_mean_mu);
+  if (!g_mean_page) {
+    if (cudaHostAlloc((void**)&g_mean_page, kMeanWords * sizeof(float), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
+      cudaGetLastError();
+      g_mean_page = nullptr;
+      return;
+    }
+    for (int i = kMeanWords; i-- > 0;) g_mean_free.push_back(g_mean_page + i);
+  }
+  if (g_mean_free.empty()) return;
+  if (cudaHostGetDevicePointer((void**)dev, g_mean_free.back(), 0) != cudaSuccess) {
+    cudaGetLastError();
+    *dev = nullptr;
+    return;
+  }
+  *host = g_mean_free.back();
+  g_mean_free.pop_back();
+}
+void mean_word_release(float* host) {
+  std::lock_guard<std::mutex> lock(g_mean_mu);
+  g_mean_free.push_back(host);
 }
 
 void keep_release(int dev, size_t want) {
@@ -339,6 +367,7 @@ mavg_status mavg_create(const mavg_config* cfg, const mavg_buffers* buf, mavg_ha
     return MAVG_ERR_CUDA;
   }
   if (cfg->objective == MAVG_OBJ_MLP) {
+    mean_word_acquire(&c->mean_host, &c->mean_dev);
     st = mlp_setup(c);
     if (st == MAVG_OK && mlp_refresh_shared_operands(c) != cudaSuccess) {
       st = MAVG_ERR_CUDA;
@@ -346,6 +375,7 @@ mavg_status mavg_create(const mavg_config* cfg, const mavg_buffers* buf, mavg_ha
     }
     if (st != MAVG_OK) {
       g_create_error = c->err;
+      if (c->mean_host) mean_word_release(c->mean_host);
       mlp_teardown(c);
       delete c;
       return st;
@@ -390,7 +420,9 @@ mavg_status mavg_round(mavg_handle h, float* mean_loss) {
   } else {
     mavg_status st = do_local_steps(h);
     if (st != MAVG_OK) return st;
+    h->mean_wanted = mean_loss != nullptr;
     st = do_meta_update(h);
+    h->mean_wanted = false;
     if (st != MAVG_OK) return st;
   }
   if (mean_loss) return read_mean_loss(h, mean_loss);
@@ -612,6 +644,10 @@ mavg_status mavg_destroy(mavg_handle h) {
     keep_release(h->device, h->l2_keep_want);
   }
   for (cudaEvent_t e : h->ev_pool) cudaEventDestroy(e);
+  if (h->mean_host) {
+    cudaStreamSynchronize(h->stream);              // a round in flight may still write it
+    mean_word_release(h->mean_host);
+  }
   if (h->ev_copy_fork) cudaEventDestroy(h->ev_copy_fork);
   if (h->ev_copy_done) cudaEventDestroy(h->ev_copy_done);
   if (h->s_copy) cudaStreamDestroy(h->s_copy);

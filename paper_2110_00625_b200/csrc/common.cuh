@@ -138,6 +138,10 @@ struct mavg_ctx {
   bool l2_keep = false;
   size_t l2_keep_want = 0;
   int device = 0;
+  // Mean loss of a round: written by the device into this pinned word (null: read back from ws.loss_mean).  mean_wanted: the
+  // meta-update about to be launched may form it on the way, mean_formed: it did.
+  float *mean_host = nullptr, *mean_dev = nullptr;
+  bool mean_wanted = false, mean_formed = false;
   // mavg_round_host: the upload of v runs on a copy stream of its own, next to the local steps
   cudaStream_t s_copy = nullptr;
   cudaEvent_t ev_copy_fork = nullptr, ev_copy_done = nullptr;
@@ -161,6 +165,21 @@ inline MomArgs mom_args(const mavg_ctx* c, bool from_broadcast) {
     m.read_u = (from_broadcast && c->cfg.learner_momentum_reset) ? 0 : 1;
   }
   return m;
+}
+
+// Mean of `count` losses, by 256 threads of a block.
+__device__ __forceinline__ void block_mean(const float* __restrict__ losses, int count, float* out) {
+  __shared__ float part[8];
+  float acc = 0.f;
+  for (int i = threadIdx.x; i < count; i += 256) acc += losses[i];
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    float s = threadIdx.x < 8 ? part[threadIdx.x] : 0.f;
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (threadIdx.x == 0) *out = s / (float)count;
+  }
 }
 
 // Every launcher enqueues on ctx->stream, adds to ctx->launches and returns the CUDA status of

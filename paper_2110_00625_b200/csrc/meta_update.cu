@@ -36,17 +36,25 @@ __device__ __forceinline__ void meta_scalar(float* rep, int64_t stride, float* w
 // broadcast (replica sets far larger than L2) or plain stores (sets the next kernel re-reads).
 // SHADOW: also writes the bf16 copy of the new w~'s weight matrices (see ShadowMap), which saves
 // the separate pass that would read w~ again.
-template <int U, bool STREAM_ST, bool SHADOW = false>
+// MEAN: a block of its own forms the round's mean loss.
+struct MeanArgs { const float* losses; int count; float* out; };
+template <int U, bool STREAM_ST, bool SHADOW = false, bool MEAN = false>
 __global__ void __launch_bounds__(256)
 k_meta_update(float* __restrict__ rep, int64_t stride, float* __restrict__ w,
               float* __restrict__ v, int P, int64_t n, float mu, float zeta, float inv_p,
-              int read_v, int bcast, const ShadowMap sm = ShadowMap()) {
+              int read_v, int bcast, const ShadowMap sm = ShadowMap(), const MeanArgs mean = MeanArgs()) {
+  tc::grid_launch_dependents();
+  tc::grid_dependency_wait();
+  if (MEAN && blockIdx.x == gridDim.x - 1) {
+    block_mean(mean.losses, mean.count, mean.out);
+    return;
+  }
   const int64_t n4 = n >> 2;
   const int64_t stride4 = stride >> 2;
   float4* rep4 = reinterpret_cast<float4*>(rep);
   float4* w4 = reinterpret_cast<float4*>(w);
   float4* v4 = reinterpret_cast<float4*>(v);
-  const int64_t step = (int64_t)gridDim.x * blockDim.x;
+  const int64_t step = (int64_t)(gridDim.x - (MEAN ? 1 : 0)) * blockDim.x;
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n4; q += step) {
     const float4 wt = ld_stream(w4 + q);
     float4 vt = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -363,7 +371,7 @@ cudaError_t launch_meta_update(mavg_ctx* c) {
   const bool big = (size_t)P * (size_t)n * 4 > c->l2_bytes / 2;
   prof_begin(c, MAVG_K_META);
   cudaError_t e = cudaSuccess;
-  c->shadow_fresh = false;
+  c->shadow_fresh = c->mean_formed = false;
   // Shorter vectors leave its blocks few tiles each.  Where the copies are written it still pays for many
   // replicas (us, register / bulk kernel: n = 1.84 M, P = 24 70 / 68, P = 48 136 / 125; n = 2.1 M, P = 64 203 / 182;
   // n = 1.2 M, P = 32 57 / 57, P = 48 88 / 82), not for fewer or below (n = 1.84 M, P = 16 48 / 52; n = 0.9 M, P = 64
@@ -386,10 +394,26 @@ cudaError_t launch_meta_update(mavg_ctx* c) {
                                                                  n, mu, zeta, inv_p, read_v, bcast,
                                                                  c->shadow);
       c->shadow_fresh = true;
-    } else
-      k_meta_update<8, false><<<grid, 256, 0, c->stream>>>(rep, c->buf.replica_stride, w, v, P,
-                                                           n, mu, zeta, inv_p, read_v, bcast);
-    e = cudaGetLastError();
+    } else {
+      // Begins while the small models' one launch of local steps ends, and forms the mean loss on the way where it is
+      // wanted (with the loss copied back after a launch of its own 32-64-10, P = 4, K = 4, B = 32 takes 60 us a round, 50 so).
+      const bool mean = c->mean_wanted && !c->profiling && c->cfg.objective == MAVG_OBJ_MLP;
+      const MeanArgs ma{(const float*)ws_ptr(c, c->ws.losses), P * c->cfg.K,
+                        c->mean_dev ? c->mean_dev : (float*)ws_ptr(c, c->ws.loss_mean)};
+      cudaLaunchConfig_t lc{};
+      lc.gridDim = dim3((unsigned)(grid + (mean ? 1 : 0)));
+      lc.blockDim = dim3(256);
+      lc.stream = c->stream;
+      cudaLaunchAttribute at[1];
+      at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+      at[0].val.programmaticStreamSerializationAllowed = 1;
+      lc.attrs = at;
+      lc.numAttrs = 1;
+      e = cudaLaunchKernelEx(&lc, mean ? k_meta_update<8, false, false, true> : k_meta_update<8, false>, rep,
+                             c->buf.replica_stride, w, v, P, n, mu, zeta, inv_p, read_v, bcast, ShadowMap(), ma);
+      c->mean_formed = mean && e == cudaSuccess;
+    }
+    if (e == cudaSuccess) e = cudaGetLastError();
   }
   prof_end(c);
   return e;

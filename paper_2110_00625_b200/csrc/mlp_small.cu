@@ -7,8 +7,10 @@
 //     block of the cluster as it is produced;
 //   - weight gradients, bias gradients and the SGD step are split by output rows of a layer, the
 //     updated weights again written to every block.
-// Two cluster barriers per step.  Arithmetic as in mlp_simt.cu: fp32 FMAs, operands rounded to bf16
-// first with QUANT.
+// Two cluster barriers per step.  Arithmetic: fp32 FMAs, operands rounded to bf16 first with QUANT.
+// Bound by the latency of dependent instructions, a thousand cycles or two to a phase.  The model comes in in one trip, and
+// the warps that fetch the minibatches take the biases and the loss, beside the weight gradients: 32-64-10, P = 4, K = 4,
+// B = 32 5 us of 55.
 #include <algorithm>
 
 #include "mlp.cuh"
@@ -92,20 +94,29 @@ __device__ __forceinline__ void gather(const SmallArgs& g, float* sm, uint64_t k
   int32_t* label = reinterpret_cast<int32_t*>(sm + g.s.label[buf]);
   int32_t* index = label + g.s.pitch;
   const uint64_t step_key = fold(key, (uint64_t)step);
-  for (int b = t; b < g.B; b += kGather) {
-    const int32_t at = (int32_t)(lo + (int64_t)(((fold(step_key, (uint64_t)b) >> 32) * len) >> 32));
-    index[b] = at;
-    label[b] = g.y[at];
-  }
+  for (int b = t; b < g.B; b += kGather)
+    index[b] = (int32_t)(lo + (int64_t)(((fold(step_key, (uint64_t)b) >> 32) * len) >> 32));
   barrier<kGather, 2>();
   float* x = sm + g.s.x[buf];
-#pragma unroll 4
-  for (int e = t; e < g.B * d; e += kGather) {
-    const int b = quotient(e, g.inv[0]), i = e - b * d;
-    const size_t at = (size_t)index[b] * d + i;
-    x[i * g.s.pitch + b] = g.x_bf16 ? __bfloat162float(((const __nv_bfloat16*)g.x)[at])
-                                    : operand<QUANT>(((const float*)g.x)[at]);
+  int32_t y = 0;                                 // the label of row t travels beside the inputs
+  if (t < g.B) y = g.y[index[t]];
+  const int count = g.B * d;
+  for (int e0 = t; e0 < count; e0 += 8 * kGather) {
+    float v[8];
+    int to[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int e = min(e0 + u * kGather, count - 1), b = quotient(e, g.inv[0]), i = e - b * d;
+      const size_t at = (size_t)index[b] * d + i;
+      v[u] = g.x_bf16 ? __bfloat162float(((const __nv_bfloat16*)g.x)[at]) : operand<QUANT>(((const float*)g.x)[at]);
+      to[u] = i * g.s.pitch + b;
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (e0 + u * kGather < count) x[to[u]] = v[u];
   }
+  if (t < g.B) label[t] = y;
+  for (int b = t + kGather; b < g.B; b += kGather) label[b] = g.y[index[b]];
 }
 
 // out(j, rows) = sum_k A(k, rows) W(j, k) for the block's batch rows; A and out are [feature][pitch],
@@ -208,6 +219,7 @@ template <bool QUANT>
 __global__ void __launch_bounds__(kCompute + kGather)
 k_small_steps(const __grid_constant__ SmallArgs g) {
   extern __shared__ __align__(16) float sm[];
+  tc::grid_launch_dependents();
   tc::grid_dependency_wait();
   const int splits = g.splits, p = blockIdx.x / splits, rank = blockIdx.x % splits;
   const int t = threadIdx.x, pitch = g.s.pitch, L = g.L, B = g.B;
@@ -225,14 +237,26 @@ k_small_steps(const __grid_constant__ SmallArgs g) {
   }
 
   if (computes) {
+    // the whole model, sixteen parameters of a thread in flight
     const float* src = g.src + (size_t)p * g.src_stride;
-    for (int l = 1; l <= L; ++l) {
-      const int in = g.dims[l - 1], out = g.dims[l];
-      float* w = sm + g.s.w[l];
-#pragma unroll 4
-      for (int o = warp; o < out; o += kCompute / 32)
-        for (int i = lane; i < in; i += 32) w[o * (in | 1) + i] = src[g.w_off[l] + o * in + i];
-      for (int o = t; o < out; o += kCompute) sm[g.s.b[l] + o] = src[g.b_off[l] + o];
+    const int n = g.b_off[L] + g.dims[L];
+    for (int e0 = t; e0 < n; e0 += 16 * kCompute) {
+      float v[16];
+#pragma unroll
+      for (int u = 0; u < 16; ++u) v[u] = e0 + u * kCompute < n ? src[e0 + u * kCompute] : 0.f;
+#pragma unroll
+      for (int u = 0; u < 16; ++u) {
+        const int e = e0 + u * kCompute;
+        if (e >= n) break;
+        int l = 1;
+        while (e >= g.b_off[l] + g.dims[l]) ++l;
+        if (e >= g.b_off[l]) {
+          sm[g.s.b[l] + e - g.b_off[l]] = v[u];
+        } else {
+          const int o = quotient(e - g.w_off[l], g.inv[l - 1]), i = e - g.w_off[l] - o * g.dims[l - 1];
+          sm[g.s.w[l] + o * (g.dims[l - 1] | 1) + i] = v[u];
+        }
+      }
     }
     // rows of the last group beyond the batch: zero inputs (their dZ is zero as well)
     for (int e = t; e < g.dims[0] * 4; e += kCompute) {
@@ -331,7 +355,17 @@ k_small_steps(const __grid_constant__ SmallArgs g) {
             else put(wp, v, splits);
           }
         }
-        for (int o = o0 + warp; o < o0 + rows; o += kCompute / 32) {   // from the unrounded dZ
+      }
+    } else {
+      // bias steps (from the unrounded dZ), a warp per output, and the loss
+      MomArgs mom = g.mom;
+      if (step > 1) mom.read_u = 1;
+      float* rep = g.rep + (size_t)p * g.rep_stride;
+      float* u = mom.u ? mom.u + (size_t)p * mom.u_stride : nullptr;
+      for (int l = 1; l <= L; ++l) {
+        const int out = g.dims[l], o0 = out * rank / splits, rows = out * (rank + 1) / splits - o0;
+        const float* dz = sm + g.s.dz[l];
+        for (int o = o0 + warp - kCompute / 32; o < o0 + rows; o += kGather / 32) {
           float s = 0.f;
           for (int b = lane; b < B; b += 32) s += dz[o * pitch + b];
           for (int q = 16; q > 0; q >>= 1) s += __shfl_xor_sync(0xffffffffu, s, q);
@@ -342,12 +376,15 @@ k_small_steps(const __grid_constant__ SmallArgs g) {
           if (last) rep[g.b_off[l] + o] = v;
           else put(sm + g.s.b[l] + o, v, splits);
         }
+        __syncwarp();
       }
-    } else if (rank == 0 && warp == kCompute / 32) {
-      float s = 0.f;
-      for (int b = lane; b < B; b += 32) s += sm[g.s.loss + b];
-      for (int q = 16; q > 0; q >>= 1) s += __shfl_xor_sync(0xffffffffu, s, q);
-      if (lane == 0) g.losses[(size_t)p * g.K + step - 1] = s * inv_b;
+      if (rank == 0 && warp == kCompute / 32) {
+        float s = 0.f;
+        for (int b = lane; b < B; b += 32) s += sm[g.s.loss + b];
+        for (int q = 16; q > 0; q >>= 1) s += __shfl_xor_sync(0xffffffffu, s, q);
+        if (lane == 0) g.losses[(size_t)p * g.K + step - 1] = s * inv_b;
+      }
+      __syncwarp();
     }
     tc::cluster_sync_all();
   }
