@@ -102,6 +102,23 @@ k_simt_begin(const __grid_constant__ GatherArgs g, const __grid_constant__ split
 template <typename Put>
 __device__ __forceinline__ float softmax_row(const float* z, int C, int label, float inv_b, Put put) {
   const int lane = threadIdx.x % 32;
+  if (C <= 128) {                          // four classes a lane, read once
+    float v[4], m = -INFINITY, se = 0.f;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v[q] = lane + 32 * q < C ? z[lane + 32 * q] : -INFINITY;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) m = fmaxf(m, v[q]);
+    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (lane + 32 * q < C) se += expf(v[q] - m);
+    for (int o = 16; o > 0; o >>= 1) se += __shfl_xor_sync(0xffffffffu, se, o);
+    const float lse = m + logf(se);
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      if (lane + 32 * q < C) put(lane + 32 * q, (expf(v[q] - lse) - (lane + 32 * q == label ? 1.f : 0.f)) * inv_b);
+    return lse - z[label];
+  }
   float m = z[lane < C ? lane : 0];
   for (int c = lane + 32; c < C; c += 32) m = fmaxf(m, z[c]);
   for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
@@ -150,13 +167,14 @@ __host__ __device__ constexpr int bf_pitch(int n) { return (((n + 15) / 16 * 16 
 // layer, in one block of 512 threads; the remaining blocks gather the next step's minibatch.  A
 // layer of few classes is latency, not work: as a forward product, a loss and a data gradient it
 // takes three launches with one busy tile column (25 us for 512 x 10, P = 4, B = 100, against
-// 11 here).  The layer's weights are brought into shared memory at once, which exposes one
-// trip to the L2 where reading them class by class exposed a dozen.  For the logits a warp takes
+// 9 here).  The layer's weights and the rows' activations are brought into shared memory at once, which exposes one
+// trip to the L2.  For the logits a warp takes
 // two rows and every fourth group of four classes (lanes along the input width); for the data
 // gradient a thread takes two columns of the input and four rows.
 // Dynamic shared memory: dZ [C][8], logits [8][C], the rows of A_{L-1} [8][in], W_L [C][in].
-// With bf16 operands the two products are warp-level MMAs on bf16 copies (mma_tail): their reads of shared
-// memory were what bounded the launch (333 x 100, P = 6, B = 50: 24 us, 13 now).
+// With bf16 operands the two products are warp-level MMAs on the bf16 planes (mma_tail), whose rows come in by
+// asynchronous copies, with the operands of four MMAs fetched together: 333 x 100, P = 6, B = 50 9 us (24 with FMAs; 14 with
+// the fp32 weights rounded on their way in, 12 with a load, a wait and an MMA at a time and the planes through registers).
 struct TailArgs {
   const __nv_bfloat16* a; int64_t a_plane; // A_{L-1}: planes [P, B, pitch_of(in)]
   const float* w; const float* b; int64_t w_batch;
@@ -182,46 +200,44 @@ __device__ __forceinline__ void mma_tail(const TailArgs& t, int p, int r0, uint8
   __nv_bfloat16* dq = a + 16 * ip;
   float* z = reinterpret_cast<float*>(dq + 16 * dp);
   const float* bias = t.b + (size_t)p * t.w_batch;
-  const int n16 = ((c16 + 16) * ip + 16 * dp) / 8;
-  for (int i = threadIdx.x; i < n16; i += kTailThreads) reinterpret_cast<uint4*>(w)[i] = make_uint4(0, 0, 0, 0);
-  __syncthreads();
-  // rows of `in` of a plane to rows of ip
-  const int pitch = pitch_of(in), units = pitch / 8;
-  auto fill = [&](__nv_bfloat16* dst, const __nv_bfloat16* __restrict__ src, int count) {
-    for (int i0 = threadIdx.x; i0 < count * units; i0 += 4 * kTailThreads) {
-      uint4 v[4];
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-        if (i0 + u * kTailThreads < count * units) v[u] = reinterpret_cast<const uint4*>(src)[i0 + u * kTailThreads];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) {
-        const int i = i0 + u * kTailThreads, r = i / units, k = (i - r * units) * 8;
-        if (i >= count * units) break;
-        if (k + 8 <= in) {
-          *reinterpret_cast<uint4*>(dst + r * ip + k) = v[u];
-        } else {                           // what lies behind a row's end is not its own
-          const uint32_t w4[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
-#pragma unroll
-          for (int j = 0; j < 8; ++j)
-            if (k + j < in) split::put16(dst + r * ip + k + j, w4[j / 2] >> (16 * (j & 1)));
-        }
-      }
+  // Rows of the planes come in as they are, 16 bytes at a time and all on their way at once: what lies behind a row's end
+  // is zero there (products and gathers write it so, W_L's was cleared when the handle was made).  Zeros: the rows'
+  // columns beyond the planes' pitch, rows beyond the last class and the batch rows, and dZ.
+  const int pitch = pitch_of(in), units = pitch / 8, left = in16 - pitch;      // 0 or 8
+  auto fill = [&](__nv_bfloat16* dst, const __nv_bfloat16* __restrict__ src, int count, int padded) {
+    int r = threadIdx.x / units, k = threadIdx.x - r * units;
+    const int dr = kTailThreads / units, dk = kTailThreads - dr * units;
+    while (r < count) {
+      asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tc::smem_u32(dst + r * ip + 8 * k)),
+                   "l"(src + (size_t)r * pitch + 8 * k) : "memory");
+      r += dr;
+      if ((k += dk) >= units) { k -= units; ++r; }
     }
+    if (left)
+      for (int i = threadIdx.x; i < count; i += kTailThreads) *reinterpret_cast<uint4*>(dst + i * ip + pitch) = make_uint4(0, 0, 0, 0);
+    const int n = (padded - count) * ip / 8;
+    for (int i = threadIdx.x; i < n; i += kTailThreads) reinterpret_cast<uint4*>(dst + count * ip)[i] = make_uint4(0, 0, 0, 0);
   };
-  fill(w, t.w16 + (size_t)p * t.w16_batch, C);
-  fill(a, t.a + ((size_t)p * t.B + r0) * pitch, rows);
+  fill(w, t.w16 + (size_t)p * t.w16_batch, C, c16);
+  fill(a, t.a + ((size_t)p * t.B + r0) * pitch, rows, 16);
+  for (int i = threadIdx.x; i < 16 * dp / 8; i += kTailThreads) reinterpret_cast<uint4*>(dq)[i] = make_uint4(0, 0, 0, 0);
+  asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();
   const int i8 = lane / 8, j8 = lane % 8, qr = lane / 4, qc = 2 * (lane % 4);
   for (int nt = warp; nt < (C + 7) / 8; nt += kTailThreads / 32) {
     float s[4] = {0.f, 0.f, 0.f, 0.f};
     for (int k0 = 0; k0 < in16; k0 += 64) {            // 64 inputs' sum on its own: the MMAs cut off, see split_gemm.cuh
       float d[4] = {0.f, 0.f, 0.f, 0.f};
-      for (int k = k0; k < min(in16, k0 + 64); k += 16) {
-        uint32_t fa[4], fb[2];
-        tc::ldsm_x4(fa, a + ((i8 & 1) * 8 + j8) * ip + k + (i8 >> 1) * 8);
-        tc::ldsm_x2(fb, w + (size_t)(nt * 8 + j8) * ip + k + (i8 & 1) * 8);
-        tc::mma_bf16(d, fa, fb[0], fb[1]);
-      }
+      uint32_t fa[4][4], fb[4][2];                     // the operands of four steps together
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (k0 + 16 * u < in16) {
+          tc::ldsm_x4(fa[u], a + ((i8 & 1) * 8 + j8) * ip + k0 + 16 * u + (i8 >> 1) * 8);
+          tc::ldsm_x2(fb[u], w + (size_t)(nt * 8 + j8) * ip + k0 + 16 * u + (i8 & 1) * 8);
+        }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (k0 + 16 * u < in16) tc::mma_bf16(d, fa[u], fb[u][0], fb[u][1]);
       s[0] += d[0];
       s[1] += d[1];
     }
@@ -245,24 +261,27 @@ __device__ __forceinline__ void mma_tail(const TailArgs& t, int p, int r0, uint8
     float s[2] = {0.f, 0.f};
     for (int k0 = 0; k0 < c16; k0 += 64) {             // 64 classes' sum on its own, likewise
       float d[4] = {0.f, 0.f, 0.f, 0.f};
-      for (int k = k0; k < min(c16, k0 + 64); k += 16) {
-        uint32_t fa[4], fb[2];
-        tc::ldsm_x4(fa, dq + ((i8 & 1) * 8 + j8) * dp + k + (i8 >> 1) * 8);
-        tc::ldsm_x2_t(fb, w + (size_t)(k + (i8 & 1) * 8 + j8) * ip + nt * 8);
-        tc::mma_bf16(d, fa, fb[0], fb[1]);
-      }
+      uint32_t fa[4][4], fb[4][2];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (k0 + 16 * u < c16) {
+          tc::ldsm_x4(fa[u], dq + ((i8 & 1) * 8 + j8) * dp + k0 + 16 * u + (i8 >> 1) * 8);
+          tc::ldsm_x2_t(fb[u], w + (size_t)(k0 + 16 * u + (i8 & 1) * 8 + j8) * ip + nt * 8);
+        }
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (k0 + 16 * u < c16) tc::mma_bf16(d, fa[u], fb[u][0], fb[u][1]);
       s[0] += d[0];
       s[1] += d[1];
     }
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int i = nt * 8 + qc + h;
-      if (qr < rows && i < in) {                       // ReLU'(0) = 0
-        const size_t row = (size_t)p * t.B + r0 + qr;
-        const float v = __bfloat162float(a[qr * ip + i]) > 0.f ? s[h] : 0.f;
-        t.dzp[row * in + i] = v;
-        t.dzp_pl[row * pitch + i] = __float2bfloat16_rn(v);
-      }
+    const int i = nt * 8 + qc;
+    if (qr < rows && i < in) {                         // ReLU'(0) = 0
+      const size_t row = (size_t)p * t.B + r0 + qr;
+      const float2 act = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(a + qr * ip + i));
+      const float v0 = act.x > 0.f ? s[0] : 0.f, v1 = act.y > 0.f ? s[1] : 0.f;
+      t.dzp[row * in + i] = v0;
+      if (i + 1 < in) t.dzp[row * in + i + 1] = v1;
+      *reinterpret_cast<__nv_bfloat162*>(t.dzp_pl + row * pitch + i) = __floats2bfloat162_rn(v0, v1);   // (i + 1 == in: 0)
     }
   }
 }
@@ -294,19 +313,32 @@ k_simt_tail(const __grid_constant__ TailArgs t, const __grid_constant__ GatherAr
   const __nv_bfloat16* arow = t.a + ((size_t)p * t.B + r0) * pitch;
   float* w = a + kTailRows * in;
   copy_floats<QUANT>(w, W, C * in);
-  for (int i = threadIdx.x; i < kTailRows * (pitch / 2); i += kTailThreads) {
-    const int r = i / (pitch / 2), k = 2 * (i - r * (pitch / 2));
-    float x0 = 0.f, x1 = 0.f;              // a value is the sum of its planes, the small ones first
-    if (r < rows) {
+  // a value is the sum of its planes, the small ones first; four of a thread's pairs on their way at once
+  const int pairs = pitch / 2;
+  for (int i0 = threadIdx.x; i0 < kTailRows * pairs; i0 += 4 * kTailThreads) {
+    uint32_t h[4][NP];
+    int r[4], k[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int i = i0 + u * kTailThreads;
+      r[u] = i / pairs;
+      k[u] = 2 * (i - r[u] * pairs);
+#pragma unroll
+      for (int q = 0; q < NP; ++q)
+        h[u][q] = r[u] < rows ? *reinterpret_cast<const uint32_t*>(arow + q * t.a_plane + (size_t)r[u] * pitch + k[u]) : 0u;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      if (r[u] >= kTailRows) break;
+      float x0 = 0.f, x1 = 0.f;
 #pragma unroll
       for (int q = NP - 1; q >= 0; --q) {
-        const __nv_bfloat162 h = *reinterpret_cast<const __nv_bfloat162*>(arow + q * t.a_plane + (size_t)r * pitch + k);
-        x0 += __low2float(h);
-        x1 += __high2float(h);
+        x0 += __uint_as_float(h[u][q] << 16);
+        x1 += __uint_as_float(h[u][q] & 0xffff0000u);
       }
+      if (k[u] < in) a[r[u] * in + k[u]] = x0;
+      if (k[u] + 1 < in) a[r[u] * in + k[u] + 1] = x1;
     }
-    if (k < in) a[r * in + k] = x0;
-    if (k + 1 < in) a[r * in + k + 1] = x1;
   }
   __syncthreads();
   {
@@ -732,6 +764,9 @@ mavg_status simt_setup(mavg_ctx* c) {
   }
   if (!ok) return MAVG_ERR_UNSUPPORTED;
   cudaError_t e = cfg.gemm_bf16 ? set_attributes<true>() : set_attributes<false>();
+  // columns beyond the rows of W_L's plane, which mma_tail reads and nobody writes
+  if (e == cudaSuccess && cfg.gemm_bf16 && cfg.dims[L - 1] % 8)
+    e = cudaMemsetAsync(st->buf.w[L], 0, (size_t)(P + 1) * cfg.dims[L] * pitch_of(cfg.dims[L - 1]) * 2, c->stream);
   for (int s = 1; s <= 8 && e == cudaSuccess; ++s) {
     cudaLaunchAttribute at[1];
     cudaLaunchConfig_t lc{};
