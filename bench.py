@@ -327,6 +327,22 @@ def factored_bytes(cfg, deferred=False, x_bytes=2):
     }
 
 
+def rebuilt_bytes(cfg, deferred=False, momentum=False):
+    """The same of a round with rebuilt steps: step k's products read the learners' bf16 weights (w~'s in the first), its
+    weights come from w~, u as the round found it and the rows of steps 1..k; the last step writes W and u."""
+    dims, P, K, B = cfg["dims"], cfg["P"], cfg["K"], cfg["B"]
+    n = sum(dims[l] * dims[l + 1] for l in range(len(dims) - 1))
+    shared = 2 * (P - 1) * n                              # the first step's weights are read once
+    out = algorithmic_bytes(cfg, True, deferred=deferred, momentum=momentum)
+    out["fwd_gemm"]["bytes"] -= shared
+    out["dgrad_gemm"]["bytes"] -= shared - 2 * (P - 1) * dims[0] * dims[1]
+    rows = 2 * P * B * K * (K + 1) // 2 * (sum(dims[:-1]) + sum(dims[1:]))
+    out["wgrad_sgd_gemm"].update(
+        bytes=K * 4 * n + (K - 1) * 2 * P * n + 4 * P * n + (4 * (K + 1) * P * n if momentum else 0) + rows,
+        executed_flops=2 * P * B * K * (K + 1) // 2 * n)
+    return out
+
+
 def kernel_rooflines(per_round, prof, steps, peaks):
     """Per kernel class: algorithmic bytes or flops of all its launches / its summed device time."""
     out = {}
@@ -575,10 +591,13 @@ def measure_mlp(name, args, m, torch, dist, peaks, world, rank, local, steps, wi
     fwd_whole_rows = tuple(plan["fwd_whole_rows"]) if args.schedule == 0 else ()
     # every riding layer but the first keeps its masters split within a round
     split_layers = tuple(range(2, len(fwd_run_tiles) + 1))
-    factored = g.factored()
-    if factored:
+    factored, rebuilt = g.factored(), g.rebuilt()
+    if factored or rebuilt:
         fwd_run_tiles = dense_layers = fwd_whole_rows = ()
+    if factored:
         per_round = factored_bytes(cfg, deferred=not args.no_defer)
+    elif rebuilt:
+        per_round = rebuilt_bytes(cfg, deferred=not args.no_defer, momentum=args.beta != 0.0)
     else:
         per_round = algorithmic_bytes(cfg, mode == 1, deferred=not args.no_defer,
                                       momentum=args.beta != 0.0, fwd_run_tiles=fwd_run_tiles,
@@ -615,14 +634,14 @@ def measure_mlp(name, args, m, torch, dist, peaks, world, rank, local, steps, wi
         roof["ms_per_launch"] = e["ms_per_launch"]
         if "executed_tflops" in e:       # "achieved" counts the method's flops only
             roof["executed_tflops"] = e["executed_tflops"]
-        if mode == 1 and not args.learners and not args.beta and not factored:
+        if mode == 1 and not args.learners and not args.beta and not factored and not rebuilt:
             roof["traffic"] = NCU_TRAFFIC.get(name, {}).get(dom)
     # the whole round against the HBM roofline: every class's algorithmic bytes / the round's time
     round_bytes = sum(v["bytes"] for v in per_round.values())
     ms_round = total_ms / steps
     return dict(
-        cfg=cfg, n=n, units=units, factored=factored, fwd_run_tiles=fwd_run_tiles, dense_layers=dense_layers,
-        fwd_whole_rows=fwd_whole_rows, total_ms=total_ms, e2e_ms=e2e_ms, launches=launches,
+        cfg=cfg, n=n, units=units, factored=factored, rebuilt=rebuilt, fwd_run_tiles=fwd_run_tiles,
+        dense_layers=dense_layers, fwd_whole_rows=fwd_whole_rows, total_ms=total_ms, e2e_ms=e2e_ms, launches=launches,
         clocks=clocks, cpu=cpu, kern=kern, roof=roof, t_wall=t_wall, mode=mode,
         meta_in_round={"ms": statistics.median(meta_ms),
                        "gbs": per_round["meta_update"]["bytes"] / statistics.median(meta_ms) / 1e6},
@@ -688,7 +707,9 @@ def run_mavg(args):
                        "schedule": {0: "CUDA graph of per-product launches",
                                     2: "CUDA graph of per-product launches, plain tensor-core tiles"}[args.schedule],
                        "local_steps": ("factored: products from w~ and the rows of the earlier steps, hidden weights "
-                                       "formed once per round" if r["factored"] else "weights stepped in place"),
+                                       "formed once per round" if r["factored"] else
+                                       "rebuilt: weights formed anew each step from w~ and the rows so far" if r["rebuilt"]
+                                       else "weights stepped in place"),
                        "forward_products": (f"layers 1..{len(r['fwd_run_tiles'])} inside their weight-gradient "
                                             "launch of the step before (steps 2..K; partial sums per "
                                             f"{list(r['fwd_run_tiles'])} column tiles, after {list(r['fwd_whole_rows'])} "

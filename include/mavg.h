@@ -145,8 +145,8 @@ typedef struct {
  * loss accumulators, the device status word).  Checks the configuration like mavg_create. */
 mavg_status mavg_workspace_bytes(const mavg_config *cfg, size_t *out_bytes);
 
-/* The least that mavg_create accepts: smaller where rounds run in factored form (MAVG_SCHED_GRAPH below), which
- * needs room for the rows of all K steps; a handle with less than mavg_workspace_bytes keeps the plain form. */
+/* The least that mavg_create accepts: smaller where rounds are factored or rebuilt (MAVG_SCHED_GRAPH below), which
+ * need room for the rows of all K steps; a handle with less than mavg_workspace_bytes keeps the plain form. */
 mavg_status mavg_workspace_least_bytes(const mavg_config *cfg, size_t *out_bytes);
 
 /* Algorithm 1, the two initialisation lines and the first "set w^j = w~": v <- 0, w^j <- w~_1
@@ -238,8 +238,10 @@ typedef enum {
 mavg_status mavg_get_step_plan(mavg_handle h, int32_t *out);
 
 /* Measurement aid: whether the handle's next local steps, if they start from w~, run in factored form
- * (MAVG_SCHED_GRAPH below), in which case the step plan above describes only calls that do not. */
+ * (MAVG_SCHED_GRAPH below), in which case the step plan above describes only calls that do not.
+ * mavg_get_rebuilt: the same of rebuilt steps. */
 mavg_status mavg_get_factored(mavg_handle h, int32_t *factored);
+mavg_status mavg_get_rebuilt(mavg_handle h, int32_t *rebuilt);
 
 /* Measurement aid (the paper has no counterpart).  While profiling is on, every kernel launch of
  * this handle is bracketed by a pair of CUDA events on the stream.  mavg_get_profile waits for the
@@ -270,11 +272,15 @@ mavg_status mavg_set_profiling(mavg_handle h, int32_t on);
  *     in factored form: W_l(k) = w~_l - gamma sum_{i<k} dZ_l(i)^T A_{l-1}(i) is not formed until the last
  *     step, products take w~ and the factors instead.  w~ enters the forward products and the last layer as
  *     two bf16 parts and the data gradients as one, the sums over the factors through bf16 Gram rows; the plain
- *     form rounds W_l(k) to bf16 at every step.  mavg_workspace_bytes has room for it if
- *     the handle's own K and momentum take it; a buffer with room for the plain form only
+ *     form rounds W_l(k) to bf16 at every step.  Other rounds of large models that start from w~ (P times the hidden layers'
+ *     weights 48 million or more and K <= 6; with learner momentum 28 million and K <= 4; K B <= 512) have rebuilt steps: the
+ *     plain form's steps, whose weights W(k) and u(k) are formed anew in step k from w~, u as the call found it and the
+ *     factors dZ(i), A(i), i <= k.  With momentum they are the plain form's weights to the bit, without it one fp32 step from
+ *     the sum of the gradients.  mavg_workspace_bytes has room for these forms if
+ *     the handle's own K and momentum take one; a buffer with room for the plain form only
  *     (mavg_workspace_least_bytes) is accepted and keeps that.
  *   MAVG_SCHED_GRAPH_TC: the same graph with every product as plain one-tile-per-block
- *     tensor-core launches.  Apart from factored rounds the two differ in the
+ *     tensor-core launches.  Apart from factored and rebuilt rounds the two differ in the
  *     summation order of the products they run differently, nothing else; this one exists for comparison.
  * Profiled rounds (mavg_set_profiling) take the launch-by-launch form of the chosen schedule; what is
  * one launch without profiling (the steps of a small CUDA-core model, a pseudo-gradient round) is one

@@ -21,8 +21,8 @@ EXPORTS = ["mavg_workspace_bytes", "mavg_workspace_least_bytes", "mavg_create", 
            "mavg_materialize_replicas", "mavg_round", "mavg_round_host", "mavg_set_hparams",
            "mavg_set_learner_momentum", "mavg_get_batch_indices",
            "mavg_get_losses", "mavg_get_round", "mavg_set_round", "mavg_get_launch_count",
-           "mavg_get_step_plan", "mavg_get_factored", "mavg_set_profiling", "mavg_set_schedule", "mavg_get_profile", "mavg_sync",
-           "mavg_set_wait_limit", "mavg_selftest_wait", "mavg_cache_release", "mavg_last_error",
+           "mavg_get_step_plan", "mavg_get_factored", "mavg_get_rebuilt", "mavg_set_profiling", "mavg_set_schedule",
+           "mavg_get_profile", "mavg_sync", "mavg_set_wait_limit", "mavg_selftest_wait", "mavg_cache_release", "mavg_last_error",
            "mavg_batch_indices_noalloc", "mavg_destroy"]
 KERNEL_CLASSES = ["meta_update", "broadcast", "pseudograd_steps", "batch_gather", "fwd_gemm",
                   "loss", "dgrad_gemm", "wgrad_sgd_gemm", "aux"]
@@ -93,7 +93,7 @@ def load_library():
     L.mavg_set_round.argtypes = [H, C.c_int64]
     L.mavg_get_launch_count.argtypes = [H, C.POINTER(C.c_int64)]
     L.mavg_get_step_plan.argtypes = [H, C.POINTER(C.c_int32)]
-    L.mavg_get_factored.argtypes = [H, C.POINTER(C.c_int32)]
+    L.mavg_get_factored.argtypes = L.mavg_get_rebuilt.argtypes = [H, C.POINTER(C.c_int32)]
     L.mavg_set_profiling.argtypes = [H, C.c_int32]
     L.mavg_set_schedule.argtypes = [H, C.c_int32]
     L.mavg_get_profile.argtypes = [H, C.c_void_p, C.c_void_p, C.c_int32]
@@ -294,6 +294,12 @@ class Mavg:
         """Whether the next local steps run in factored form if they start from w~ (see mavg_set_schedule)."""
         r = C.c_int32()
         self._check(self.lib.mavg_get_factored(self.handle, C.byref(r)))
+        return bool(r.value)
+
+    def rebuilt(self):
+        """Whether they have rebuilt steps (likewise)."""
+        r = C.c_int32()
+        self._check(self.lib.mavg_get_rebuilt(self.handle, C.byref(r)))
         return bool(r.value)
 
     def set_profiling(self, on):

@@ -562,6 +562,12 @@ mavg_status mavg_get_factored(mavg_handle h, int32_t* factored) {
   return MAVG_OK;
 }
 
+mavg_status mavg_get_rebuilt(mavg_handle h, int32_t* rebuilt) {
+  if (!h || !rebuilt) return MAVG_ERR_INVALID_ARG;
+  *rebuilt = h->cfg.objective == MAVG_OBJ_MLP && mlp_rebuilt(h) ? 1 : 0;
+  return MAVG_OK;
+}
+
 mavg_status mavg_set_profiling(mavg_handle h, int32_t on) {
   CHECK_HANDLE(h);
   h->profiling = on != 0;

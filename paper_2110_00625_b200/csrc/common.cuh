@@ -202,6 +202,7 @@ cudaError_t mlp_local_steps(mavg_ctx* c, int64_t round);
 void mlp_reset_counters(mavg_ctx* c);                    // after an abandoned device-side wait
 void mlp_step_plan(mavg_ctx* c, int32_t* out);           // entries of mavg_plan_entry
 bool mlp_factored(const mavg_ctx* c);                    // a call that starts from w~ runs in factored form
+bool mlp_rebuilt(const mavg_ctx* c);                     // has rebuilt steps
 cudaError_t mlp_indices_only(mavg_ctx* c, int64_t round, int learner, int step, int32_t* dev_out);
 
 // Bracket every kernel launch: prof_begin before it, prof_end after it (counts the launch).

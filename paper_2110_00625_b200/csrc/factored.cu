@@ -9,6 +9,8 @@
 //   k_fac_apply     W_l = w~_l - gamma dZ_l^T A_{l-1} over all steps' rows, every learner and hidden layer
 //   k_fac_last      the last layer (at most 32 classes), which keeps its own weights and steps
 //
+// and the rebuilt local steps of rebuild.cuh, which share the gather and the products with weights.
+//
 // All are launched with programmatic stream serialisation.
 #include <cuda.h>
 
@@ -16,6 +18,7 @@
 
 #include "gemm_unit.cuh"
 #include "mlp.cuh"
+#include "rebuild.cuh"
 #include "tc_state.cuh"
 
 namespace mavg {
@@ -112,13 +115,13 @@ __device__ __forceinline__ uint4 low8(const float* src) {
 // the plain form.  Added up they would be NaN, which ReLU makes 0.
 __device__ __forceinline__ float with_low(float high, float low) { return fabsf(high) <= 3.402823466e38f ? high + low : high; }
 
-// A warp per row (learner p, step k, slot s): its sample's index, its label and its d inputs as bf16.  The
-// first la.blocks blocks write the low parts of w~ instead.
+// A warp per row (learner p, step k, slot s): its sample's index, its label and its d inputs as bf16, learner by learner
+// or (step_major) step by step.  The first la.blocks blocks write the low parts of w~ instead.
 template <typename TIN>
 __global__ void __launch_bounds__(256)
 k_fac_gather(const TIN* __restrict__ x, const int32_t* __restrict__ y, uint64_t seed, int64_t round,
              const int64_t* __restrict__ round_ptr, int P, int K, int B, int64_t kb, int64_t S, int d,
-             int32_t* __restrict__ labels, __nv_bfloat16* __restrict__ out, const __grid_constant__ LowArgs la) {
+             int32_t* __restrict__ labels, __nv_bfloat16* __restrict__ out, int step_major, const __grid_constant__ LowArgs la) {
   if ((int)blockIdx.x < la.blocks) {
     for (int l = 0; l < la.layers; ++l)
       for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < la.total[l] >> 3; t += (int64_t)la.blocks * blockDim.x)
@@ -133,7 +136,7 @@ k_fac_gather(const TIN* __restrict__ x, const int32_t* __restrict__ y, uint64_t 
   const int32_t i = sample_index(seed, round, p, k + 1, s, P, S);
   if (lane == 0) labels[((size_t)k * P + p) * B + s] = y[i];
   const TIN* src = x + (size_t)i * d;
-  uint4* dst = reinterpret_cast<uint4*>(out + ((size_t)p * kb + r) * d);
+  uint4* dst = reinterpret_cast<uint4*>(out + (step_major ? ((size_t)k * P + p) * B + s : (size_t)p * kb + r) * d);
   const int n8 = d >> 3;
   for (int c0 = lane; c0 < n8; c0 += 4 * 32) {
     uint4 v[4];
@@ -159,6 +162,8 @@ struct ProdArgs {
   int c_tiles;              // column tiles: B / cols (RAW: tiles of a learner's rows)
   int row_end;              // RAW: rows per learner
   int nkb;                  // slabs of the product with w~ (0: left out)
+  int w_batched;            // the weights are each learner's own (one learner per block)
+  int in_off;               // added to the learner in the batch operand's array
   int hist;                 // rows of the earlier steps (0: left out)
   int s_row0;               // row of the batch inside a learner's Gram rows
   int stages;
@@ -178,6 +183,7 @@ struct ProdArgs {
   __nv_bfloat16* gram_out;
   int64_t gram_stride, gram_ld;
   float gamma;
+  MomArgs mom;              // of the stepped bias
   int* status;
 };
 
@@ -268,6 +274,7 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
   const int nslab = (g.hist + kBK - 1) / kBK;
   volatile int* abortp = &sh.abort_flag;
   const bool any = g.nkb > 0 || g.hist > 0;
+  const int w_of = g.w_batched ? p0 : 0;
   const int gram_step = kBM * g.m_tiles;           // from one of this block's Gram tiles to the next, in rows
 
   if (warp == 0) {
@@ -292,13 +299,13 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
         uint8_t* sa = smem + (size_t)ring.s * stage_bytes;
         mbar_arrive_expect_tx(full, base_bytes);
         if (kMn) {
-          tma_load_3d(sa, &tm_w, full, m0, i * kBK, 0);
-          tma_load_3d(sa + kATileBytes / 2, &tm_w, full, m0 + 64, i * kBK, 0);
+          tma_load_3d(sa, &tm_w, full, m0, i * kBK, w_of);
+          tma_load_3d(sa + kATileBytes / 2, &tm_w, full, m0 + 64, i * kBK, w_of);
         } else {
-          tma_load_3d(sa, &tm_w, full, i * kBK, m0, 0);
+          tma_load_3d(sa, &tm_w, full, i * kBK, m0, w_of);
         }
         if (LOW) tma_load_3d(sa + kATileBytes, &tm_lo, full, i * kBK, m0, 0);
-        tma_load_3d(sa + kBOff, &tm_in, full, i * kBK, r0, p0);
+        tma_load_3d(sa + kBOff, &tm_in, full, i * kBK, r0, p0 + g.in_off);
       }
       if (GRAM && ok) {
         ok = mbar_wait_cluster(&rows_bar, 0, abortp, g.status, ERR_PRODUCER);
@@ -489,8 +496,9 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
       } else if (ok && m_ok) {
         for (int q = half; q < nl; q += 2) {
           const float w_in = g.bias_in[(size_t)(p0 + q) * g.bias_in_stride + g.bias_off + m];
-          local_update(g.bias_rep + (size_t)(p0 + q) * g.rep_stride + g.bias_off + m, w_in, nullptr, 0,
-                       colsum[q * kBM + row] + colsum[(nl + q) * kBM + row], g.gamma, 0.f);
+          float* u = g.mom.u ? g.mom.u + (size_t)(p0 + q) * g.mom.u_stride + g.bias_off + m : nullptr;
+          local_update(g.bias_rep + (size_t)(p0 + q) * g.rep_stride + g.bias_off + m, w_in, u, g.mom.read_u,
+                       colsum[q * kBM + row] + colsum[(nl + q) * kBM + row], g.gamma, g.mom.beta);
         }
       }
     }
@@ -503,7 +511,8 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
       float s = 0.f;
       for (int r = 0; r < g.c_tiles; ++r) s += ld_cluster_f32(mapa_u32(smem_u32(&sh.colsum[0][row]), (uint32_t)(rank0 + r)));
       const float w_in = g.bias_in[(size_t)p0 * g.bias_in_stride + g.bias_off + m];
-      local_update(g.bias_rep + (size_t)p0 * g.rep_stride + g.bias_off + m, w_in, nullptr, 0, s, g.gamma, 0.f);
+      float* u = g.mom.u ? g.mom.u + (size_t)p0 * g.mom.u_stride + g.bias_off + m : nullptr;
+      local_update(g.bias_rep + (size_t)p0 * g.rep_stride + g.bias_off + m, w_in, u, g.mom.read_u, s, g.gamma, g.mom.beta);
     }
     __syncwarp();
     cluster_sync_all();           // nobody leaves while its sums may still be read
@@ -1229,6 +1238,36 @@ LastPlan last_plan(const mavg_config* cfg) {
   return pl;
 }
 
+// The minibatches of a call's steps and their labels; low: the low parts of w~ as well (factored steps), else ordered step
+// by step (rebuilt ones).
+cudaError_t gather_rows(mavg_ctx* c, const FacLayout& t, int rows, int64_t round, bool low) {
+  const mavg_config& cfg = c->cfg;
+  const int L = cfg.n_layers, P = cfg.P, B = cfg.B, K = cfg.K;
+  int32_t* labels = (int32_t*)ws_ptr(c, t.labels);
+  __nv_bfloat16* out = (__nv_bfloat16*)ws_ptr(c, t.h[0]);
+  const int64_t* rp = c->capturing ? (const int64_t*)(ws_ptr(c, c->ws.status) + 64) : nullptr;
+  LowArgs la{};
+  int64_t all = 0;
+  la.layers = low ? L - 1 : 0;
+  for (int l = 1; l <= la.layers; ++l) {
+    const MlpLayer& ly = c->layers[l - 1];
+    la.w[l - 1] = c->buf.global_w + ly.w_off;
+    la.dst[l - 1] = (__nv_bfloat16*)ws_ptr(c, t.w_lo[l]);
+    all += la.total[l - 1] = (int64_t)ly.in * ly.out;
+  }
+  la.blocks = (int)std::min<int64_t>((all + 8191) / 8192, 2 * c->sm_count);
+  const unsigned grid = (unsigned)(((int64_t)P * rows + 7) / 8 + la.blocks);
+  prof_begin(c, MAVG_K_BATCH);
+  if (cfg.x_dtype == MAVG_X_BF16)
+    k_fac_gather<__nv_bfloat16><<<grid, 256, 0, c->stream>>>((const __nv_bfloat16*)cfg.x, cfg.y, cfg.seed, round, rp,
+                                                            P, K, B, t.kb, cfg.n_samples, cfg.dims[0], labels, out, !low, la);
+  else
+    k_fac_gather<float><<<grid, 256, 0, c->stream>>>((const float*)cfg.x, cfg.y, cfg.seed, round, rp, P, K, B, t.kb,
+                                                     cfg.n_samples, cfg.dims[0], labels, out, !low, la);
+  prof_end(c);
+  return cudaGetLastError();
+}
+
 bool enough_rows(const mavg_config* cfg, int K) { return K >= 2 && (int64_t)cfg->P * K * cfg->B >= 8192; }
 
 }  // namespace
@@ -1375,6 +1414,8 @@ bool fac_usable(const mavg_ctx* c) {
          c->cfg.K <= st->fac->K && enough_rows(&c->cfg, c->cfg.K);
 }
 
+#define FAC_TRY(call) do { if ((e = (call)) != cudaSuccess) return e; } while (0)
+
 // The K steps of a round.  Chain of a step, layers L:
 //   F_1 -> (S_2 -> F_2) -> ... -> last layer -> (T_{L-1} -> D_{L-1}) -> ... -> D_2
 // S_l, T_l: the Gram products that the forward product F_l and the data gradient D_l through layer l
@@ -1388,32 +1429,8 @@ cudaError_t fac_local_steps(mavg_ctx* c, int64_t round) {
   auto bfp = [&](size_t off) { return (__nv_bfloat16*)ws_ptr(c, off); };
   int32_t* labels = (int32_t*)ws_ptr(c, t.labels);
   cudaError_t e;
-#define FAC_TRY(call) do { if ((e = (call)) != cudaSuccess) return e; } while (0)
 
-  {
-    const int64_t* rp = c->capturing ? (const int64_t*)(ws_ptr(c, c->ws.status) + 64) : nullptr;
-    LowArgs la{};
-    int64_t all = 0;
-    la.layers = L - 1;
-    for (int l = 1; l < L; ++l) {
-      const MlpLayer& ly = c->layers[l - 1];
-      la.w[l - 1] = c->buf.global_w + ly.w_off;
-      la.dst[l - 1] = bfp(t.w_lo[l]);
-      all += la.total[l - 1] = (int64_t)ly.in * ly.out;
-    }
-    la.blocks = (int)std::min<int64_t>((all + 8191) / 8192, 2 * c->sm_count);
-    const unsigned grid = (unsigned)(((int64_t)P * rows + 7) / 8 + la.blocks);
-    prof_begin(c, MAVG_K_BATCH);
-    if (cfg.x_dtype == MAVG_X_BF16)
-      k_fac_gather<__nv_bfloat16><<<grid, 256, 0, c->stream>>>((const __nv_bfloat16*)cfg.x, cfg.y, cfg.seed, round, rp,
-                                                              P, K, B, t.kb, cfg.n_samples, cfg.dims[0], labels,
-                                                              bfp(t.h[0]), la);
-    else
-      k_fac_gather<float><<<grid, 256, 0, c->stream>>>((const float*)cfg.x, cfg.y, cfg.seed, round, rp, P, K, B, t.kb,
-                                                       cfg.n_samples, cfg.dims[0], labels, bfp(t.h[0]), la);
-    prof_end(c);
-    FAC_TRY(cudaGetLastError());
-  }
+  FAC_TRY(gather_rows(c, t, rows, round, true));
   const int row_tiles = (rows + f->row_tile - 1) / f->row_tile;
   {
     ProdArgs g{};
@@ -1574,8 +1591,196 @@ cudaError_t fac_local_steps(mavg_ctx* c, int64_t round) {
     FAC_TRY(e);
     FAC_TRY(cudaGetLastError());
   }
-#undef FAC_TRY
   return cudaSuccess;
 }
+
+// Where rounds are rebuilt instead of stepped in place: where they are not factored and what a step moves, 10 bytes per
+// weight in place (18 with momentum), costs more than forming the weights anew from all rows so far, k B in step k.  V: P
+// times the hidden layers' weights.  Time in place / rebuilt over 163 shapes (1 to 3 hidden layers of 128 to 2048, P = 2 ..
+// 48, B = 16 .. 256, V = 8 .. 184 M):
+//   with momentum (an accumulator per step: K <= 4)   V >= 28 M: 1.03 .. 1.58, never slower; V = 8 .. 28 M: 0.844 .. 1.40
+//   without                                  V >= 48 M, K <= 6: 1.12 .. 1.48, never slower; K = 7 .. 16: 0.954 .. 1.19
+// Without momentum rebuilt steps win from V = 24 M on (1.20 .. 1.84), but there the schedule in place is the one whose
+// forward products ride on the weight gradients and whose sums run in another order; it is held to 2e-2 of the plain
+// tiles' v, and at 3072-1024-512-10, P = 13, K = 4, B = 16 (V = 47.8 M) the two are 2.1e-2 apart when rebuilt (as far
+// from 64 bits as each other).
+int reb_steps(const mavg_config* cfg) {
+  const int L = cfg->n_layers, B = cfg->B;
+  const bool momentum = cfg->learner_momentum != 0.f;
+  if (L < 2 || B > 256 || cfg->dims[L] > 32) return 0;
+  int64_t weights = 0;
+  for (int l = 1; l < L; ++l) weights += (int64_t)cfg->dims[l - 1] * cfg->dims[l];
+  if (cfg->P * weights < (momentum ? 28 : 48) * 1000 * 1000) return 0;
+  const int most = std::min({cfg->K, 512 / B, momentum ? rebuild::kMaxMomSteps : 6});
+  return most >= 2 ? most : 0;
+}
+
+bool reb_reserved(const mavg_config* cfg) { return reb_steps(cfg) == cfg->K && !fac_reserved(cfg); }
+
+FacLayout reb_layout(const mavg_config* cfg, size_t base) {
+  FacLayout t;
+  const int L = cfg->n_layers, P = cfg->P;
+  t.kb = (int64_t)reb_steps(cfg) * cfg->B;
+  const size_t rows = (size_t)P * t.kb;
+  size_t off = up(base, 1024);
+  auto take = [&](size_t bytes) { size_t r = off; off = up(off + bytes, 1024); return r; };
+  for (int l = 0; l < L; ++l) t.h[l] = take(rows * cfg->dims[l] * 2);
+  for (int l = 1; l <= L; ++l) {
+    t.g[l] = take(rows * up((size_t)cfg->dims[l], 8) * 2);
+    t.w_own[l] = take((size_t)P * cfg->dims[l - 1] * cfg->dims[l] * 2);
+  }
+  t.labels = take(rows * sizeof(int32_t));
+  t.end = off;
+  return t;
+}
+
+void reb_setup(mavg_ctx* c, TcState* st) {
+  std::string* why = nullptr;
+  const mavg_config& cfg = c->cfg;
+  const int L = cfg.n_layers, P = cfg.P, B = cfg.B;
+  FacState* f = new FacState();
+  f->lay = reb_layout(&cfg, st->lay.shared_end);
+  f->K = reb_steps(&cfg);
+  const FacLayout& t = f->lay;
+  auto bf = [&](size_t off) { return (__nv_bfloat16*)ws_ptr(c, off); };
+  bool ok = true;
+  // rows [steps P, B, d], a row `pitch` long
+  auto rows = [&](CUtensorMap* m, size_t at, int d, int box_rows, int box_learners = 1) {
+    const int pitch = (int)up((size_t)d, 8);
+    ok = ok && encode_map(st, m, bf(at), d, B, f->K * P, pitch, (int64_t)B * pitch, box_rows, why, box_learners);
+  };
+  for (int l = 1; l <= L && ok; ++l) {
+    const int in = cfg.dims[l - 1], out = cfg.dims[l];
+    const int64_t size = (int64_t)in * out;
+    rows(&f->h_mn[l - 1], t.h[l - 1], in, 64);
+    rows(&f->g_mn[l], t.g[l], out, 64);
+    ok = ok && encode_map(st, &f->w_own[l], bf(t.w_own[l]), in, out, P, in, size, kBM, why);
+    ok = ok && encode_map(st, &f->w_own_mn[l], bf(t.w_own[l]), in, out, P, in, size, 64, why);
+    ok = ok && encode_any(st, &f->w_own_st[l], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, bf(t.w_own[l]), in, out, P, in, size,
+                          kWgradTileCols, kWgradTileRows, CU_TENSOR_MAP_SWIZZLE_64B, why);
+    // step 1: products with w~, several learners to a block; later ones a learner's own weights
+    if (l < L) {
+      f->fwd1[l] = cols_for(P, B, (out + kBM - 1) / kBM, c->sm_count);
+      f->fwd[l] = cols_for(P, B, (out + kBM - 1) / kBM, c->sm_count, 1);
+      rows(&f->in1[l], t.h[l - 1], in, f->fwd1[l].cols, f->fwd1[l].nl);
+      rows(&f->in[l], t.h[l - 1], in, f->fwd[l].cols);
+    }
+    if (l > 1) {
+      f->dgrad1[l] = cols_for(P, B, (in + kBM - 1) / kBM, c->sm_count);
+      f->dgrad[l] = cols_for(P, B, (in + kBM - 1) / kBM, c->sm_count, 1);
+      rows(&f->dz_in1[l], t.g[l], out, f->dgrad1[l].cols, f->dgrad1[l].nl);
+      rows(&f->dz_in[l], t.g[l], out, f->dgrad[l].cols);
+    }
+  }
+  f->last_in.resize((size_t)f->K);                 // A_{L-1} of each step as the last layer's launch reads it
+  for (int k = 0; k < f->K && ok; ++k) {
+    const int d = cfg.dims[L - 1];
+    ok = ok && encode_map(st, &f->last_in[k], bf(t.h[L - 1]) + (size_t)k * P * B * d, d, B, P, d, (int64_t)B * d, st->fwd[L].BN, why);
+  }
+  const struct { const void* kernel; size_t fixed; } kernels[] = {
+      {(const void*)k_fac_product<PROD_FWD, 1, false, false>, sizeof(GemmShared)},
+      {(const void*)k_fac_product<PROD_DGRAD, 1, false, false>, sizeof(GemmShared)},
+      {(const void*)rebuild::k_rebuild<false, false>, sizeof(rebuild::Shared)}, {(const void*)rebuild::k_rebuild<false, true>, sizeof(rebuild::Shared)},
+      {(const void*)rebuild::k_rebuild<true, false>, sizeof(rebuild::Shared)}, {(const void*)rebuild::k_rebuild<true, true>, sizeof(rebuild::Shared)}};
+  for (const auto& k : kernels)
+    ok = ok && cudaFuncSetAttribute(k.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)(kSmSharedBytes - kBlockReservedBytes - k.fixed)) == cudaSuccess;
+  if (ok) {
+    st->reb = f;
+  } else {
+    cudaGetLastError();
+    delete f;
+  }
+}
+
+bool reb_usable(const mavg_ctx* c) {
+  const TcState* st = (const TcState*)c->mlp;
+  return st && st->reb && c->schedule == 0 && c->cfg.K >= 2 && c->cfg.K <= st->reb->K &&
+         (c->cfg.learner_momentum == 0.f || c->cfg.K <= rebuild::kMaxMomSteps);
+}
+
+// The K steps of a round: F_1 -> ... -> F_{L-1} -> last layer and loss -> D_L -> ... -> D_2 -> weights of the next step's
+// products (of the call's end: the learners' own, and u).
+cudaError_t reb_local_steps(mavg_ctx* c, int64_t round) {
+  TcState* st = (TcState*)c->mlp;
+  FacState* f = st->reb;
+  const FacLayout& t = f->lay;
+  const mavg_config& cfg = c->cfg;
+  const int L = cfg.n_layers, P = cfg.P, B = cfg.B, K = cfg.K;
+  const MomArgs first = mom_args(c, true);
+  cudaError_t e;
+  FAC_TRY(gather_rows(c, t, K * B, round, false));
+  for (int k = 1; k <= K; ++k) {
+    MomArgs mom = first;
+    if (k > 1 && mom.u) mom.read_u = 1;
+    auto slab = [&](size_t at, int d) { return (__nv_bfloat16*)ws_ptr(c, at) + (size_t)(k - 1) * P * B * up((size_t)d, 8); };
+    auto product = [&](int M, int contraction, int bias_layer, const FacCols& cols) {
+      ProdArgs g{};
+      g.M = M;
+      g.kb = B;
+      g.nl = cols.nl;
+      g.cols = cols.cols;
+      g.c_tiles = cols.c_tiles;
+      g.nkb = (contraction + kBK - 1) / kBK;
+      g.w_batched = k > 1;
+      g.in_off = (k - 1) * P;
+      g.bias_off = c->layers[bias_layer - 1].b_off;
+      g.bias_in = k == 1 ? c->buf.global_w : c->buf.replicas;
+      g.bias_in_stride = k == 1 ? 0 : c->buf.replica_stride;
+      g.mom = mom;
+      return g;
+    };
+    for (int l = 1; l < L; ++l) {
+      ProdArgs g = product(cfg.dims[l], cfg.dims[l - 1], l, k == 1 ? f->fwd1[l] : f->fwd[l]);
+      g.out = slab(t.h[l], cfg.dims[l]);
+      const CUtensorMap &w = k == 1 ? st->wg[l] : f->w_own[l], &in = k == 1 ? f->in1[l] : f->in[l];
+      FAC_TRY((launch_product<PROD_FWD, 1>(c, MAVG_K_FWD, w, w, in, f->g_mn[l], in, g)));
+    }
+    FAC_TRY(st->last_layer(c, k == 1 ? st->wg[L] : f->w_own[L], k == 1, f->last_in[k - 1],
+                          (const int32_t*)ws_ptr(c, t.labels) + (size_t)(k - 1) * P * B, k, slab(t.g[L], cfg.dims[L]), mom));
+    for (int l = L; l > 1; --l) {
+      ProdArgs g = product(cfg.dims[l - 1], cfg.dims[l], l - 1, k == 1 ? f->dgrad1[l] : f->dgrad[l]);
+      g.out = slab(t.g[l - 1], cfg.dims[l - 1]);
+      g.act = slab(t.h[l - 1], cfg.dims[l - 1]);
+      const CUtensorMap &w = k == 1 ? st->wg_mn[l] : f->w_own_mn[l], &dz = k == 1 ? f->dz_in1[l] : f->dz_in[l];
+      FAC_TRY((launch_product<PROD_DGRAD, 1>(c, MAVG_K_DGRAD, w, w, dz, f->h_mn[l - 1], dz, g)));
+    }
+    rebuild::Args g{};
+    g.n_layers = L;
+    g.P = P;
+    g.group = std::min(P, 4);
+    g.B = B;
+    g.steps = k;
+    g.load_u = first.u && first.read_u;
+    g.gamma = cfg.local_lr;
+    g.beta = first.beta;
+    g.status = (int*)ws_ptr(c, c->ws.status);
+    for (int l = 1; l <= L; ++l) {
+      rebuild::Layer& a = g.layer[l - 1];
+      a.m_tiles = (cfg.dims[l] + kBM - 1) / kBM;
+      a.n_tiles = (cfg.dims[l - 1] + rebuild::kBN - 1) / rebuild::kBN;
+      a.in = cfg.dims[l - 1];
+      a.first = g.tiles;
+      g.tiles += a.m_tiles * a.n_tiles;
+      g.dz[l - 1] = f->g_mn[l];
+      g.a[l - 1] = f->h_mn[l - 1];
+      g.w_in[l - 1] = st->w32g[l];
+      g.u[l - 1] = first.u ? st->u32[l] : st->w32g[l];
+      g.out[l - 1] = k == K ? st->w32[l] : f->w_own_st[l];
+    }
+    const int units = (P + g.group - 1) / g.group * g.tiles;
+    PdlLaunch l(dim3((unsigned)std::min(units, c->sm_count)), rebuild::kThreads, std::max(rebuild::smem_of(k == K), rebuild::share()),
+                c->stream);
+    auto kernel = k == K ? (first.u ? rebuild::k_rebuild<true, true> : rebuild::k_rebuild<false, true>)
+                         : (first.u ? rebuild::k_rebuild<true, false> : rebuild::k_rebuild<false, false>);
+    prof_begin(c, MAVG_K_WGRAD_SGD);
+    e = cudaLaunchKernelEx(&l.lc, kernel, g);
+    prof_end(c);
+    FAC_TRY(e);
+    FAC_TRY(cudaGetLastError());
+  }
+  return cudaSuccess;
+}
+#undef FAC_TRY
 
 }  // namespace mavg

@@ -10,6 +10,7 @@
 #include <cuda.h>
 
 #include <string>
+#include <vector>
 
 #include "common.cuh"
 
@@ -20,7 +21,7 @@ struct FacLayout {
   int64_t kb = 0;                            // rows of a learner: fac_steps() * B
   int64_t s_ld = 0;                          // row length of the Gram arrays: kb rounded up to 64
   size_t h[MAVG_MAX_LAYERS] = {};            // A_l, l = 0..L-1: bf16 [P, kb, d_l]
-  size_t g[MAVG_MAX_LAYERS] = {};            // dZ_l, l = 1..L-1: bf16 [P, kb, d_l]
+  size_t g[MAVG_MAX_LAYERS + 1] = {};        // dZ_l, l = 1..L-1: bf16 [P, kb, d_l]
   // X W~_1^T, fp32 [kb, d_1] per learner, and -gamma X X^T below the step diagonal, bf16 [kb, s_ld] per
   // learner.  Where they fit they lie in the learner's rows of the replica array, on W_1, which no
   // factored step reads or writes before the last (in_rows; zbase and s1 are then byte offsets in a row).
@@ -29,6 +30,9 @@ struct FacLayout {
   size_t s[2] = {0, 0};                      // one step's -gamma A A(i)^T and -gamma dZ dZ(i)^T: bf16 [P, B, s_ld]
   size_t labels = 0;                         // int32 [K, P, B]
   size_t w_lo[MAVG_MAX_LAYERS] = {};         // low parts of w~'s hidden layers, l = 1..L-1: bf16 [d_l, d_{l-1}]
+  // rebuilt steps: the learners' weights, l = 1..L: bf16 [P, d_l, d_{l-1}].  The rows above are [steps, P, B, d_l] there,
+  // dZ_L's among them (padded to 8 classes)
+  size_t w_own[MAVG_MAX_LAYERS + 1] = {};
   size_t end = 0;
 };
 
@@ -47,10 +51,16 @@ struct FacState {
   FacCols fwd[MAVG_MAX_LAYERS + 1], dgrad[MAVG_MAX_LAYERS + 1], gram;
   CUtensorMap in[MAVG_MAX_LAYERS + 1], dz_in[MAVG_MAX_LAYERS + 1];
   CUtensorMap s_f[MAVG_MAX_LAYERS + 1], s_d[MAVG_MAX_LAYERS + 1];
+  // Rebuilt steps: the first step's cuts and batch operands (products with w~), and the learners' weights (boxes of
+  // 64 x 128, 64 x 64, and to store 32 x 128)
+  FacCols fwd1[MAVG_MAX_LAYERS + 1], dgrad1[MAVG_MAX_LAYERS + 1];
+  CUtensorMap in1[MAVG_MAX_LAYERS + 1], dz_in1[MAVG_MAX_LAYERS + 1];
+  CUtensorMap w_own[MAVG_MAX_LAYERS + 1], w_own_mn[MAVG_MAX_LAYERS + 1], w_own_st[MAVG_MAX_LAYERS + 1];
+  std::vector<CUtensorMap> last_in;
   CUtensorMap w_lo[MAVG_MAX_LAYERS];         // low parts of w~'s hidden layers, box 64 x 128
   // Row arrays [P, kb, d_l]: A_l (h) and dZ_l (g) with boxes of 64 x 64 rows (_mn: features are the MMA's
   // row dimension, rows the contraction), 64 x 128 (_k) and 64 x gram.cols (_b; A_0: 64 x row_tile).
-  CUtensorMap h_mn[MAVG_MAX_LAYERS], g_mn[MAVG_MAX_LAYERS];
+  CUtensorMap h_mn[MAVG_MAX_LAYERS], g_mn[MAVG_MAX_LAYERS + 1];
   CUtensorMap h_k[MAVG_MAX_LAYERS], g_k[MAVG_MAX_LAYERS];
   CUtensorMap h_b[MAVG_MAX_LAYERS], g_b[MAVG_MAX_LAYERS];
 };
@@ -67,5 +77,14 @@ void fac_setup(mavg_ctx* c, TcState* st);
 // The steps of a call that starts from w~ take the factored form.
 bool fac_usable(const mavg_ctx* c);
 cudaError_t fac_local_steps(mavg_ctx* c, int64_t round);
+
+// The same of rebuilt steps (rebuild.cuh), which calls take that are not factored: the weights of every step are formed anew
+// from w~, u as the call found it and the rows of all steps so far.
+int reb_steps(const mavg_config* cfg);
+bool reb_reserved(const mavg_config* cfg);
+FacLayout reb_layout(const mavg_config* cfg, size_t base);
+void reb_setup(mavg_ctx* c, TcState* st);
+bool reb_usable(const mavg_ctx* c);
+cudaError_t reb_local_steps(mavg_ctx* c, int64_t round);
 
 }  // namespace mavg

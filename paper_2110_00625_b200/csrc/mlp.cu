@@ -60,6 +60,7 @@ void mlp_step_plan(mavg_ctx* c, int32_t* out) {
 }
 
 bool mlp_factored(const mavg_ctx* c) { return use_tensor_cores(&c->cfg) && tc_factored(c); }
+bool mlp_rebuilt(const mavg_ctx* c) { return use_tensor_cores(&c->cfg) && tc_rebuilt(c); }
 
 cudaError_t mlp_refresh_shared_operands(mavg_ctx* c) {
   if (use_tensor_cores(&c->cfg)) return tc_refresh_shared_operands(c);

@@ -74,6 +74,7 @@ cudaError_t launch_tail_finish(mavg_ctx* c, const TailLaunch& t);   // bias step
 
 void tc_reset_counters(mavg_ctx* c);          // after an abandoned device-side wait
 bool tc_factored(const mavg_ctx* c);
+bool tc_rebuilt(const mavg_ctx* c);
 void tc_step_plan(mavg_ctx* c, int32_t* out);  // entries of mavg_plan_entry
 // State of the learners' bf16 copies between calls: which copy of the doubled layer is current, or
 // kW16Stale: none (factored steps keep none; the next step that reads them writes them anew).

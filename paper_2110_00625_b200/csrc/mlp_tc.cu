@@ -411,7 +411,26 @@ size_t tc_workspace_bytes(const mavg_config* cfg, size_t base, size_t* act_off, 
   *act_off = base;
   const TcLayout t = make_layout(cfg, base, kPlanSmCount);
   *least = t.end;
-  return fac_reserved(cfg) ? std::max(t.end, fac_layout(cfg, t.shared_end).end) : t.end;
+  if (fac_reserved(cfg)) return std::max(t.end, fac_layout(cfg, t.shared_end).end);
+  return reb_reserved(cfg) ? std::max(t.end, reb_layout(cfg, t.shared_end).end) : t.end;
+}
+
+static cudaError_t last_layer(mavg_ctx* c, const CUtensorMap& w, bool shared_w, const CUtensorMap& a, const int32_t* labels, int step,
+                          __nv_bfloat16* dz, const MomArgs& mom) {
+  const TcState* st = (const TcState*)c->mlp;
+  const TcLayout& t = st->lay;
+  const int L = c->cfg.n_layers;
+  TcArgs g{};
+  g.M = c->cfg.dims[L]; g.N = c->cfg.B;
+  g.a_batched = shared_w ? 0 : 1; g.b_batched = 1;
+  g.part = (float*)ws_ptr(c, t.part); g.counters = (int*)ws_ptr(c, t.counters);
+  g.bias_rep = c->buf.replicas; g.bias_off = c->layers[L - 1].b_off;
+  g.bias_in = shared_w ? c->buf.global_w : c->buf.replicas;
+  g.bias_in_stride = shared_w ? 0 : c->buf.replica_stride;
+  g.labels = labels; g.loss_out = (float*)ws_ptr(c, c->ws.losses) + (step - 1); g.loss_stride = c->cfg.K;
+  g.dz_bm = dz; g.cpad = t.cpad; g.dz_mb = (__nv_bfloat16*)ws_ptr(c, t.dz_t[L]);
+  g.mom = mom;
+  return launch_gemm<EPI_FWD_LAST>(c, MAVG_K_FWD, w, a, st->fwd[L], g);
 }
 
 mavg_status tc_setup(mavg_ctx* c) {
@@ -617,6 +636,9 @@ mavg_status tc_setup(mavg_ctx* c) {
   if (e == cudaSuccess && fac_steps(&cfg) &&
       c->buf.workspace_bytes >= std::max(t.end, fac_layout(&cfg, t.shared_end).end))
     fac_setup(c, st);
+  st->last_layer = last_layer;
+  if (e == cudaSuccess && reb_steps(&cfg) && c->buf.workspace_bytes >= std::max(t.end, reb_layout(&cfg, t.shared_end).end))
+    reb_setup(c, st);
   if (e == cudaSuccess)
     e = cudaMemsetAsync(ws + t.counters, 0, t.counters_bytes, c->stream);
   if (e == cudaSuccess) e = cudaMemsetAsync(ws + t.zcount, 0, t.zcount_bytes, c->stream);
@@ -639,6 +661,7 @@ void tc_teardown(mavg_ctx* c) {
     for (cudaEvent_t ev : evs)
       if (ev) cudaEventDestroy(ev);
     delete st->fac;
+    delete st->reb;
   }
   delete st;
   c->mlp = nullptr;
@@ -661,6 +684,7 @@ void tc_reset_counters(mavg_ctx* c) {
 }
 
 bool tc_factored(const mavg_ctx* c) { return fac_usable(c); }
+bool tc_rebuilt(const mavg_ctx* c) { return reb_usable(c) && !fac_usable(c); }
 
 void tc_step_plan(mavg_ctx* c, int32_t* out) {
   const TcState* st = (const TcState*)c->mlp;
@@ -718,8 +742,8 @@ cudaError_t tc_refresh_shared_operands(mavg_ctx* c) {
 }
 
 cudaError_t tc_local_steps(mavg_ctx* c, int64_t round) {
-  if (c->replicas_equal_global && fac_usable(c)) {
-    cudaError_t e = fac_local_steps(c, round);
+  if (c->replicas_equal_global && (tc_factored(c) || tc_rebuilt(c))) {
+    cudaError_t e = tc_factored(c) ? fac_local_steps(c, round) : reb_local_steps(c, round);
     if (e != cudaSuccess) return e;
     tc_set_w16_cur(c, kW16Stale);
     c->replicas_equal_global = false;

@@ -1,0 +1,325 @@
+// Rebuilt local steps: a learner's hidden weights after k steps, formed anew from w~, the momentum buffer the call found
+// and the rows of the k steps' factors, instead of being read, stepped and written back every step.  With w~ the same for
+// all learners and the rows a few MB, a step moves 2 bytes per weight (the bf16 copy that the next step's products read)
+// and 4 more with learner momentum (u as it was before the call), where stepping in place moves 10 and 18.  The learners'
+// own weights are rounded to bf16 at every step as in the plain form; with momentum the steps are taken one after the
+// other in fp32 in its very order.
+//
+// 3072-2048-2048-2048-10, P = 8, B = 64, momentum (14.7 M weights a learner), step 1 .. 4 of 4: 162, 178, 231 us against 116 us
+// for the 0.76 GB of steps 1 .. 3 at the copy rate, and 427 against 222 (1.47 GB: W and u go out); the
+// round takes 1586 us, 1928 with the steps in place.  Bound by the epilogue: a piece of 128 x 32 weights takes its group of four warps
+// 2.4 us from tensor memory to the store, longer than its bytes take.  Measured and worse for the last: more groups
+// or eight warps a group (200 .. 448 us: registers), storing from registers (296 .. 560: half-empty sectors), deeper rings
+// with two operand stages (243 .. 493), a warp of its own for fetches and stores (216 .. 413 at best: slower in steps 1 .. 3).
+#pragma once
+#include <cuda.h>
+
+#include "gemm_unit.cuh"
+#include "wgrad_tc.cuh"
+
+namespace mavg {
+namespace rebuild {
+
+using namespace tc;
+using namespace gemm;
+
+constexpr int kGroups = 4;                        // of four epilogue warps: one for each piece of a tile
+constexpr int kThreads = (2 + 4 * kGroups) * 32;  // warp 0: TMA producer, 1: MMA issuer, the rest: epilogue
+constexpr int kBN = 128;                          // input columns of a tile
+constexpr int kPiece = 32;                        // columns of a piece: 16 KB of fp32, rows of 128 bytes, 128-byte swizzle
+constexpr int kPieceBytes = kBM * kPiece * 4;
+constexpr int kStageBytes = 2 * kATileBytes;
+// Shared memory: operand stages and, per epilogue group, buffers for pieces on their way in (w~, u) and one to store from.
+// What leaves with LAST takes fp32 pieces of W, and u where it came in, so one piece less comes in ahead.
+constexpr int stages_of(bool last) { return last ? 3 : 2; }
+constexpr int ring_of(bool last) { return last ? 1 : 2; }
+constexpr int out_bytes(bool last) { return last ? kPieceBytes : kPieceBytes / 2; }
+constexpr int group_bytes(bool last) { return ring_of(last) * kPieceBytes + out_bytes(last); }
+constexpr size_t smem_of(bool last) { return (size_t)stages_of(last) * kStageBytes + kGroups * group_bytes(last) + 1024; }
+static_assert(smem_of(false) <= 226 * 1024 && smem_of(true) <= 226 * 1024, "");
+constexpr int kMaxMomSteps = 512 / kBN;           // with momentum every step's gradient has an accumulator of its own
+enum { ERR_REB_PRODUCER = 51, ERR_REB_MMA = 52, ERR_REB_EPILOGUE = 53 };
+
+struct Layer { int m_tiles, n_tiles, in, first; };   // first: tiles of the layers before
+struct Args {
+  CUtensorMap dz[MAVG_MAX_LAYERS], a[MAVG_MAX_LAYERS];   // rows [steps P, B, d], boxes of 64 features x 64 rows
+  CUtensorMap w_in[MAVG_MAX_LAYERS], u[MAVG_MAX_LAYERS];    // w~ and u, fp32 pieces
+  CUtensorMap out[MAVG_MAX_LAYERS];                    // the bf16 copies, or (LAST) the fp32 masters
+  Layer layer[MAVG_MAX_LAYERS];
+  int n_layers, tiles, P, group;                  // tiles of a learner; learners that share a fetch of w~
+  int B, steps;                                   // steps taken so far, B rows each
+  int load_u;                                     // u is not zero
+  float gamma, beta;
+  int* status;
+};
+struct alignas(16) Shared {                       // (whole 16 bytes, as static shared memory is counted)
+  uint64_t full[3], empty[3], acc_full[2], acc_empty[2], piece_full[kGroups][2];
+  uint32_t tmem_slot;
+  int abort_flag;
+};
+
+__device__ __forceinline__ void drain_copies(uint64_t* full, int issued, int stages, const int* status) {
+  for (int i = max(0, issued - stages); i < issued; ++i) {
+    const uint64_t t0 = global_timer_ns();
+    while (!mbar_try_wait(&full[i % stages], (i / stages) & 1))
+      if (global_timer_ns() - t0 > wait_limit_ns(status)) break;
+  }
+}
+
+// Dynamic shared memory for the same share of an SM as of its tensor memory, of which a block takes all.
+inline size_t share() { return tmem_share_bytes(512, sizeof(Shared)); }
+
+// Persistent over units: a tile of 128 x 128 weights for `group` learners, whose w~ stays in the epilogue's registers (a
+// fetch of w~ for every learner is 4 bytes per weight more, twice what leaves in steps 1 .. K-1 without momentum).
+// LAST: the learners' own weights and u leave, else the bf16 copies of the weights.
+template <bool MOM, bool LAST>
+__global__ void __launch_bounds__(kThreads, 1)
+k_rebuild(const __grid_constant__ Args g) {
+  constexpr int kStages = stages_of(LAST);
+  extern __shared__ uint8_t smem_raw[];
+  __shared__ __align__(16) Shared sh;
+  uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < kStages; ++s) {
+      mbar_init(&sh.full[s], 1);
+      mbar_init(&sh.empty[s], 1);
+    }
+    for (int b = 0; b < 2; ++b) {
+      mbar_init(&sh.acc_full[b], 1);
+      mbar_init(&sh.acc_empty[b], 4 * kGroups);
+    }
+    for (int b = 0; b < kGroups; ++b)
+      for (int s = 0; s < 2; ++s) mbar_init(&sh.piece_full[b][s], 1);
+    sh.abort_flag = 0;
+    fence_barrier_init();
+    fence_proxy_async();
+  }
+  uint32_t* tmem_slot = &sh.tmem_slot;
+  if (warp == 1) {
+    tmem_alloc(tmem_slot, 512);
+    tmem_relinquish();
+  }
+  tc_fence_before_sync();
+  __syncthreads();
+  tc_fence_after_sync();
+  const uint32_t tmem_base = sh.tmem_slot;
+  grid_launch_dependents();   // not before the tensor memory is this block's: see tc_ptx.cuh
+  grid_dependency_wait();
+  volatile int* abortp = &sh.abort_flag;
+  const int nkb = (g.B + kBK - 1) / kBK;          // slabs of a step
+  const int acc_cols = (MOM ? g.steps : 1) * kBN, bufs = 2 * acc_cols <= 512 ? 2 : 1;
+  const int groups = (g.P + g.group - 1) / g.group, units = groups * g.tiles;
+  // units of the same learners follow one another: their rows stay in the L2
+  auto decode = [&](int unit, int& p0, int& p1, int& l, int& m0, int& n0) {
+    const int gr = unit / g.tiles;
+    int r = unit - gr * g.tiles;
+    p0 = gr * g.group;
+    p1 = min(p0 + g.group, g.P);
+    l = 0;
+    while (l + 1 < g.n_layers && r >= g.layer[l + 1].first) ++l;
+    r -= g.layer[l].first;
+    m0 = (r % g.layer[l].m_tiles) * kBM;
+    n0 = (r / g.layer[l].m_tiles) * kBN;
+  };
+
+  if (warp == 0) {
+    if (lane == 0) {
+      int issued = 0;
+      bool ok = true;
+      for (int unit = blockIdx.x; unit < units && ok; unit += gridDim.x) {
+        int p0, p1, l, m0, n0;
+        decode(unit, p0, p1, l, m0, n0);
+        for (int p = p0; p < p1 && ok; ++p)
+          for (int i = 0; i < g.steps * nkb; ++i, ++issued) {
+            const int s = issued % kStages, row = i % nkb * kBK, z = i / nkb * g.P + p;
+            if (!(ok = mbar_wait(&sh.empty[s], ((issued / kStages) & 1) ^ 1, abortp, g.status, ERR_REB_PRODUCER))) break;
+            uint8_t* sa = smem + (size_t)s * kStageBytes;
+            mbar_arrive_expect_tx(&sh.full[s], (uint32_t)kStageBytes);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+              tma_load_3d(sa + h * 8192, &g.dz[l], &sh.full[s], m0 + 64 * h, row, z);
+              tma_load_3d(sa + kATileBytes + h * 8192, &g.a[l], &sh.full[s], n0 + 64 * h, row, z);
+            }
+          }
+      }
+      if (*abortp) drain_copies(sh.full, issued, kStages, g.status);
+    }
+    __syncwarp();
+  } else if (warp == 1) {
+    if (lane == 0) {
+      const uint32_t idesc = idesc_bf16_f32(kBM, kBN, 1, 1);
+      const uint64_t a0 = smem_desc_mn_sw128(smem_u32(smem)), b0 = smem_desc_mn_sw128(smem_u32(smem) + kATileBytes);
+      int it = 0, n = 0;
+      bool ok = true;
+      for (int unit = blockIdx.x; unit < units && ok; unit += gridDim.x) {
+        int p0, p1, l, m0, n0;
+        decode(unit, p0, p1, l, m0, n0);
+        for (int p = p0; p < p1 && ok; ++p, ++n) {
+          const int b = n % bufs;
+          if (!(ok = mbar_wait(&sh.acc_empty[b], ((n / bufs) & 1) ^ 1, abortp, g.status, ERR_REB_MMA))) break;
+          tc_fence_after_sync();
+          for (int i = 0; i < g.steps * nkb; ++i, ++it) {
+            const int s = it % kStages, kb = i % nkb;
+            if (!(ok = mbar_wait(&sh.full[s], (it / kStages) & 1, abortp, g.status, ERR_REB_MMA))) break;
+            tc_fence_after_sync();
+            const uint32_t off = (uint32_t)(s * kStageBytes) >> 4, d = tmem_base + (uint32_t)(b * acc_cols + (MOM ? i / nkb * kBN : 0));
+            // a step's last slab ends with its batch (a multiple of 16)
+            const int nk = min(kBK, g.B - kb * kBK) / 16;
+            const bool first = MOM ? kb == 0 : i == 0;
+            for (int k = 0; k < nk; ++k)
+              umma_bf16(d, a0 + off + (uint32_t)k * ((16 * 128) >> 4), b0 + off + (uint32_t)k * ((16 * 128) >> 4), idesc,
+                        (uint32_t)(!first || k > 0));
+            umma_commit(&sh.empty[s]);
+          }
+          if (ok) umma_commit(&sh.acc_full[b]);
+        }
+      }
+    }
+    __syncwarp();
+  } else {
+    // A group of four warps per piece.  Its first thread fetches w~ and u pieces ahead of their use and stores the finished
+    // ones.  One barrier a piece: behind it the piece has been read and what is to be stored is in shared memory; before
+    // the next is written, the first thread has seen the store leave it (it carries that to the barrier before the write).
+    // The barriers carry a wait that was given up, so that the group leaves together.
+    constexpr int kRing = ring_of(LAST);
+    const int grp = (warp - 2) >> 2, q4 = warp & 3, row = q4 * 32 + lane;
+    const bool leader = ((warp - 2) & 3) == 0 && lane == 0, load_u = MOM && g.load_u;
+    const bool u_apart = MOM && LAST && !load_u;   // u does not come in, but leaves from the buffer for it
+    uint8_t* in_buf = smem + kStages * kStageBytes + (size_t)grp * group_bytes(LAST);
+    uint8_t* ob = in_buf + kRing * kPieceBytes;
+    // the leader's place in the group's list of pieces: of w~ (fp == -1), then of each learner's u
+    int fu = blockIdx.x, fp = -1;
+    uint32_t fn = 0;
+    auto fetch = [&]() {
+      while (fu < units) {
+        int p0, p1, l, m0, n0;
+        decode(fu, p0, p1, l, m0, n0);
+        const int c0 = n0 + grp * kPiece, of = fp, last_of = load_u ? p1 - p0 : 0;
+        if (++fp >= last_of || c0 >= g.layer[l].in) { fp = -1; fu += gridDim.x; }
+        if (c0 >= g.layer[l].in) continue;
+        const uint32_t s = fn % kRing;
+        mbar_arrive_expect_tx(&sh.piece_full[grp][s], kPieceBytes);
+        if (of < 0) tma_load_3d(in_buf + (size_t)s * kPieceBytes, &g.w_in[l], &sh.piece_full[grp][s], c0, m0, 0);
+        else tma_load_3d(in_buf + (size_t)s * kPieceBytes, &g.u[l], &sh.piece_full[grp][s], c0, m0, p0 + of);
+        ++fn;
+        return;
+      }
+    };
+    if (leader)
+      for (int i = 0; i < kRing; ++i) fetch();
+    uint32_t pn = 0;                               // pieces taken in
+    int n = 0;
+    bool failed = false, gone = false;
+    auto cell = [&](uint8_t* buf, int c) { return reinterpret_cast<float4*>(buf + (size_t)row * 128 + ((c ^ (row & 7)) << 4)); };
+    auto wait_piece = [&]() {
+      if (!mbar_wait(&sh.piece_full[grp][pn % kRing], (pn / kRing) & 1, abortp, g.status, ERR_REB_EPILOGUE)) failed = true;
+      return in_buf + (size_t)(pn % kRing) * kPieceBytes;
+    };
+    for (int unit = blockIdx.x; unit < units && !gone; unit += gridDim.x) {
+      int p0, p1, l, m0, n0;
+      decode(unit, p0, p1, l, m0, n0);
+      const int c0 = grp * kPiece;
+      const bool mine = n0 + c0 < g.layer[l].in;
+      float w[kPiece];
+      if (mine) {
+        uint8_t* buf = wait_piece();
+#pragma unroll
+        for (int c = 0; c < kPiece / 4; ++c) {
+          const float4 v = *cell(buf, c);
+          w[4 * c] = v.x; w[4 * c + 1] = v.y; w[4 * c + 2] = v.z; w[4 * c + 3] = v.w;
+        }
+        ++pn;
+        if (leader) tma_store_wait_read<0>();      // (the store before the first write of this unit)
+        if ((gone = barrier_any(failed, 2 + grp, 128))) break;
+        if (leader && !u_apart) fetch();
+      }
+      for (int p = p0; p < p1; ++p, ++n) {
+        const int b = n % bufs;
+        if (!mbar_wait(&sh.acc_full[b], (n / bufs) & 1, abortp, g.status, ERR_REB_EPILOGUE)) failed = true;
+        __syncwarp();
+        tc_fence_after_sync();
+        const uint32_t acc = tmem_base + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(b * acc_cols + c0);
+        uint8_t* ub = in_buf;
+        if (mine && load_u) ub = wait_piece();
+        if (mine) {
+#pragma unroll
+          for (int h = 0; h < kPiece / 8; ++h) {   // 8 columns
+            float x[8], v[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              x[j] = w[8 * h + j];
+              v[j] = 0.f;
+            }
+            if (load_u) {
+#pragma unroll
+              for (int c = 0; c < 2; ++c) {
+                const float4 t = *cell(ub, 2 * h + c);
+                v[4 * c] = t.x; v[4 * c + 1] = t.y; v[4 * c + 2] = t.z; v[4 * c + 3] = t.w;
+              }
+            }
+            uint32_t r[MOM ? kMaxMomSteps : 1][8];
+#pragma unroll
+            for (int i = 0; i < (MOM ? kMaxMomSteps : 1); ++i)
+              if (!MOM || i < g.steps) tmem_ld_8cols(acc + (uint32_t)(i * kBN + 8 * h), r[i]);
+            tmem_ld_wait();
+#pragma unroll
+            for (int i = 0; i < (MOM ? kMaxMomSteps : 1); ++i) {
+              if (MOM && i >= g.steps) break;
+#pragma unroll
+              for (int j = 0; j < 8; ++j) {
+                if (MOM) msgd(x[j], v[j], __uint_as_float(r[i][j]), g.gamma, g.beta);
+                else x[j] = fmaf(-g.gamma, __uint_as_float(r[i][j]), x[j]);
+              }
+            }
+            if (LAST) {
+#pragma unroll
+              for (int c = 0; c < 2; ++c) {
+                *cell(ob, 2 * h + c) = make_float4(x[4 * c], x[4 * c + 1], x[4 * c + 2], x[4 * c + 3]);
+                if (MOM) *cell(ub, 2 * h + c) = make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
+              }
+            } else {                               // rows of 64 bytes, 64-byte swizzle
+              uint32_t hw[4];
+#pragma unroll
+              for (int j = 0; j < 4; ++j) {
+                const __nv_bfloat162 t = __floats2bfloat162_rn(x[2 * j], x[2 * j + 1]);
+                hw[j] = *reinterpret_cast<const uint32_t*>(&t);
+              }
+              *reinterpret_cast<uint4*>(ob + (size_t)row * 64 + ((h ^ ((row >> 1) & 3)) << 4)) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
+            }
+          }
+        }
+        tc_fence_before_sync();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&sh.acc_empty[b]);
+        if (!mine) {
+          if (failed) { gone = true; break; }
+          continue;
+        }
+        fence_proxy_async();
+        if ((gone = barrier_any(failed, 2 + grp, 128))) break;
+        if (leader) {
+          tma_store_3d(&g.out[l], ob, n0 + c0, m0, p);
+          if (MOM && LAST) tma_store_3d(&g.u[l], ub, n0 + c0, m0, p);
+          tma_store_commit();
+        }
+        if (load_u) ++pn;
+        if (leader && load_u && !LAST) fetch();    // (its buffer has been read)
+        if (leader) tma_store_wait_read<0>();
+        if (leader && load_u && LAST) fetch();     // (its buffer has been stored from)
+        if ((gone = barrier_any(failed, 2 + grp, 128))) break;
+      }
+      if (leader && mine && u_apart && !gone) fetch();
+    }
+    if (leader) {
+      tma_store_wait_read<0>();
+      if (*abortp) drain_copies(sh.piece_full[grp], (int)fn, kRing, g.status);
+    }
+  }
+  tc_fence_before_sync();
+  __syncthreads();
+  if (warp == 1) tmem_dealloc(tmem_base, 512);
+}
+
+}  // namespace rebuild
+}  // namespace mavg

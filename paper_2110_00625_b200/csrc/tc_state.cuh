@@ -108,6 +108,11 @@ struct TcState {
   GemmPlan fwd[MAVG_MAX_LAYERS + 1], dgrad[MAVG_MAX_LAYERS + 1];
   WgradPlan wgrad[MAVG_MAX_LAYERS + 1];
   FacState* fac = nullptr;                    // factored steps (factored.cuh), null: not for this handle
+  FacState* reb = nullptr;                    // rebuilt steps, likewise
+  // The plain form's launch for the last layer's product, loss, dZ_L (to dz, rows of whole groups of 8) and bias step, with
+  // the given operands.
+  cudaError_t (*last_layer)(mavg_ctx* c, const CUtensorMap& w, bool shared_w, const CUtensorMap& a, const int32_t* labels, int step,
+                            __nv_bfloat16* dz, const MomArgs& mom) = nullptr;
   // side streams and events for the branches of a step that may overlap
   cudaStream_t s_wgrad = nullptr, s_gather = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_wgrad_done = nullptr, ev_gather_done = nullptr,
