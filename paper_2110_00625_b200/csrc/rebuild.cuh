@@ -5,12 +5,14 @@
 // own weights are rounded to bf16 at every step as in the plain form; with momentum the steps are taken one after the
 // other in fp32 in its very order.
 //
-// 3072-2048-2048-2048-10, P = 8, B = 64, momentum (14.7 M weights a learner), step 1 .. 4 of 4: 162, 178, 231 us against 116 us
-// for the 0.76 GB of steps 1 .. 3 at the copy rate, and 427 against 222 (1.47 GB: W and u go out); the
-// round takes 1586 us, 1928 with the steps in place.  Bound by the epilogue: a piece of 128 x 32 weights takes its group of four warps
-// 2.4 us from tensor memory to the store, longer than its bytes take.  Measured and worse for the last: more groups
-// or eight warps a group (200 .. 448 us: registers), storing from registers (296 .. 560: half-empty sectors), deeper rings
-// with two operand stages (243 .. 493), a warp of its own for fetches and stores (216 .. 413 at best: slower in steps 1 .. 3).
+// 3072-2048-2048-2048-10, P = 8, B = 64, momentum (14.7 M weights a learner), step 1 .. 4 of 4: 146, 158, 225 us against 116 us
+// for the 0.76 GB of steps 1 .. 3 at the copy rate, and 370 against 222 (1.47 GB: W and u go out); the round takes 1463 us,
+// 1928 with the steps in place.  What bounds steps 1 .. 3 is what an SM takes in from the L2, about 49 GB/s: 32 KB of operands
+// per tile and step so far beside 64 KB of u, 95, 127 and 158 us.  The last step waits for its stores and, with all of
+// tensor memory taken by one learner's four gradients, for the next learner's.  Registers: four steps' accumulators of
+// 8 columns at once spilled (166, 184, 236 and 437 us), two at once do not.  Measured and worse: more groups, or eight
+// warps a group; storing from registers (296 .. 560 us: half-empty sectors); deeper rings with two operand stages; in the
+// last step pieces of 16 columns, two in turn (400); the copies in and out by warps of their own (137, 151, 238 and 423).
 #pragma once
 #include <cuda.h>
 
@@ -56,6 +58,7 @@ struct alignas(16) Shared {                       // (whole 16 bytes, as static 
   uint64_t full[3], empty[3], acc_full[2], acc_empty[2], piece_full[kGroups][2];
   uint32_t tmem_slot;
   int abort_flag;
+  int fetch_unit[kGroups], fetch_p[kGroups], fetched[kGroups];   // a group's place in its list of pieces to fetch
 };
 
 __device__ __forceinline__ void drain_copies(uint64_t* full, int issued, int stages, const int* status) {
@@ -189,25 +192,31 @@ k_rebuild(const __grid_constant__ Args g) {
     uint8_t* in_buf = smem + kStages * kStageBytes + (size_t)grp * group_bytes(LAST);
     uint8_t* ob = in_buf + kRing * kPieceBytes;
     // the leader's place in the group's list of pieces: of w~ (fp == -1), then of each learner's u
-    int fu = blockIdx.x, fp = -1;
-    uint32_t fn = 0;
+    // (in shared memory: it is seldom looked at, and registers are short)
     auto fetch = [&]() {
+      int fu = sh.fetch_unit[grp], fp = sh.fetch_p[grp];
       while (fu < units) {
         int p0, p1, l, m0, n0;
         decode(fu, p0, p1, l, m0, n0);
         const int c0 = n0 + grp * kPiece, of = fp, last_of = load_u ? p1 - p0 : 0;
         if (++fp >= last_of || c0 >= g.layer[l].in) { fp = -1; fu += gridDim.x; }
         if (c0 >= g.layer[l].in) continue;
-        const uint32_t s = fn % kRing;
+        const uint32_t s = (uint32_t)sh.fetched[grp]++ % kRing;
+        sh.fetch_unit[grp] = fu;
+        sh.fetch_p[grp] = fp;
         mbar_arrive_expect_tx(&sh.piece_full[grp][s], kPieceBytes);
         if (of < 0) tma_load_3d(in_buf + (size_t)s * kPieceBytes, &g.w_in[l], &sh.piece_full[grp][s], c0, m0, 0);
         else tma_load_3d(in_buf + (size_t)s * kPieceBytes, &g.u[l], &sh.piece_full[grp][s], c0, m0, p0 + of);
-        ++fn;
         return;
       }
+      sh.fetch_unit[grp] = fu;
     };
-    if (leader)
+    if (leader) {
+      sh.fetch_unit[grp] = blockIdx.x;
+      sh.fetch_p[grp] = -1;
+      sh.fetched[grp] = 0;
       for (int i = 0; i < kRing; ++i) fetch();
+    }
     uint32_t pn = 0;                               // pieces taken in
     int n = 0;
     bool failed = false, gone = false;
@@ -258,19 +267,26 @@ k_rebuild(const __grid_constant__ Args g) {
                 v[4 * c] = t.x; v[4 * c + 1] = t.y; v[4 * c + 2] = t.z; v[4 * c + 3] = t.w;
               }
             }
-            uint32_t r[MOM ? kMaxMomSteps : 1][8];
+            if (MOM) {                             // two steps at a time: more accumulators in flight do not fit the registers
 #pragma unroll
-            for (int i = 0; i < (MOM ? kMaxMomSteps : 1); ++i)
-              if (!MOM || i < g.steps) tmem_ld_8cols(acc + (uint32_t)(i * kBN + 8 * h), r[i]);
-            tmem_ld_wait();
+              for (int i = 0; i < kMaxMomSteps; i += 2) {
+                if (i >= g.steps) break;
+                uint32_t r[2][8];
+                tmem_ld_8cols(acc + (uint32_t)(i * kBN + 8 * h), r[0]);
+                if (i + 1 < g.steps) tmem_ld_8cols(acc + (uint32_t)((i + 1) * kBN + 8 * h), r[1]);
+                tmem_ld_wait();
 #pragma unroll
-            for (int i = 0; i < (MOM ? kMaxMomSteps : 1); ++i) {
-              if (MOM && i >= g.steps) break;
+                for (int j = 0; j < 8; ++j) msgd(x[j], v[j], __uint_as_float(r[0][j]), g.gamma, g.beta);
+                if (i + 1 < g.steps)
 #pragma unroll
-              for (int j = 0; j < 8; ++j) {
-                if (MOM) msgd(x[j], v[j], __uint_as_float(r[i][j]), g.gamma, g.beta);
-                else x[j] = fmaf(-g.gamma, __uint_as_float(r[i][j]), x[j]);
+                  for (int j = 0; j < 8; ++j) msgd(x[j], v[j], __uint_as_float(r[1][j]), g.gamma, g.beta);
               }
+            } else {
+              uint32_t r[8];
+              tmem_ld_8cols(acc + (uint32_t)(8 * h), r);
+              tmem_ld_wait();
+#pragma unroll
+              for (int j = 0; j < 8; ++j) x[j] = fmaf(-g.gamma, __uint_as_float(r[j]), x[j]);
             }
             if (LAST) {
 #pragma unroll
@@ -292,10 +308,7 @@ k_rebuild(const __grid_constant__ Args g) {
         tc_fence_before_sync();
         __syncwarp();
         if (lane == 0) mbar_arrive(&sh.acc_empty[b]);
-        if (!mine) {
-          if (failed) { gone = true; break; }
-          continue;
-        }
+        if (!mine) continue;                       // (a wait given up here is carried by the next barrier)
         fence_proxy_async();
         if ((gone = barrier_any(failed, 2 + grp, 128))) break;
         if (leader) {
@@ -313,7 +326,7 @@ k_rebuild(const __grid_constant__ Args g) {
     }
     if (leader) {
       tma_store_wait_read<0>();
-      if (*abortp) drain_copies(sh.piece_full[grp], (int)fn, kRing, g.status);
+      if (*abortp) drain_copies(sh.piece_full[grp], sh.fetched[grp], kRing, g.status);
     }
   }
   tc_fence_before_sync();
