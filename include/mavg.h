@@ -273,7 +273,7 @@ mavg_status mavg_set_profiling(mavg_handle h, int32_t on);
  *     step, products take w~ and the factors instead.  w~ enters the forward products and the last layer as
  *     two bf16 parts and the data gradients as one, the sums over the factors through bf16 Gram rows; the plain
  *     form rounds W_l(k) to bf16 at every step.  Other rounds of large models that start from w~ (P times the hidden layers'
- *     weights 48 million or more and K <= 6; with learner momentum 28 million and K <= 4; K B <= 512) have rebuilt steps: the
+ *     weights 48 million or more and K <= 6; with learner momentum 20 million and K <= 4; K B <= 512) have rebuilt steps: the
  *     plain form's steps, whose weights W(k) and u(k) are formed anew in step k from w~, u as the call found it and the
  *     factors dZ(i), A(i), i <= k.  With momentum they are the plain form's weights to the bit, without it one fp32 step from
  *     the sum of the gradients.  mavg_workspace_bytes has room for these forms if

@@ -1596,9 +1596,9 @@ cudaError_t fac_local_steps(mavg_ctx* c, int64_t round) {
 
 // Where rounds are rebuilt instead of stepped in place: where they are not factored and what a step moves, 10 bytes per
 // weight in place (18 with momentum), costs more than forming the weights anew from all rows so far, k B in step k.  V: P
-// times the hidden layers' weights.  Time in place / rebuilt over 163 shapes (1 to 3 hidden layers of 128 to 2048, P = 2 ..
+// times the hidden layers' weights.  Time in place / rebuilt over 323 shapes (1 to 3 hidden layers of 128 to 2048, P = 2 ..
 // 48, B = 16 .. 256, V = 8 .. 184 M):
-//   with momentum (an accumulator per step: K <= 4)   V >= 28 M: 1.03 .. 1.58, never slower; V = 8 .. 28 M: 0.844 .. 1.40
+//   with momentum (an accumulator per step: K <= 4)   V >= 20 M: 1.03 .. 1.58, never slower; V = 8 .. 20 M: 0.797 .. 1.40
 //   without                                  V >= 48 M, K <= 6: 1.12 .. 1.48, never slower; K = 7 .. 16: 0.954 .. 1.19
 // Without momentum rebuilt steps win from V = 24 M on (1.20 .. 1.84), but there the schedule in place is the one whose
 // forward products ride on the weight gradients and whose sums run in another order; it is held to 2e-2 of the plain
@@ -1610,7 +1610,7 @@ int reb_steps(const mavg_config* cfg) {
   if (L < 2 || B > 256 || cfg->dims[L] > 32) return 0;
   int64_t weights = 0;
   for (int l = 1; l < L; ++l) weights += (int64_t)cfg->dims[l - 1] * cfg->dims[l];
-  if (cfg->P * weights < (momentum ? 28 : 48) * 1000 * 1000) return 0;
+  if (cfg->P * weights < (momentum ? 20 : 48) * 1000 * 1000) return 0;
   const int most = std::min({cfg->K, 512 / B, momentum ? rebuild::kMaxMomSteps : 6});
   return most >= 2 ? most : 0;
 }

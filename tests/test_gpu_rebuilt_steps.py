@@ -39,7 +39,7 @@ def _steps_from_own_weights(g):                   # the second call does not sta
 
 
 @pytest.mark.parametrize("dims,P,K,B,beta,reset,defer,calls", [
-    ([520, 264, 136, 10], 168, 3, 16, 0.9, False, True, _rounds),
+    ([520, 264, 136, 10], 118, 3, 16, 0.9, False, True, _rounds),
     ([520, 264, 136, 10], 170, 2, 16, 0.9, True, False, _rounds),
     ([520, 264, 136, 10], 167, 4, 80, 0.5, False, False, _rounds),
     ([1000, 520, 32], 55, 2, 48, 0.9, False, True, _steps_from_own_weights),
