@@ -36,25 +36,16 @@ __device__ __forceinline__ void meta_scalar(float* rep, int64_t stride, float* w
 // broadcast (replica sets far larger than L2) or plain stores (sets the next kernel re-reads).
 // SHADOW: also writes the bf16 copy of the new w~'s weight matrices (see ShadowMap), which saves
 // the separate pass that would read w~ again.
-// MEAN: a block of its own forms the round's mean loss.
-struct MeanArgs { const float* losses; int count; float* out; };
-template <int U, bool STREAM_ST, bool SHADOW = false, bool MEAN = false>
-__global__ void __launch_bounds__(256)
-k_meta_update(float* __restrict__ rep, int64_t stride, float* __restrict__ w,
-              float* __restrict__ v, int P, int64_t n, float mu, float zeta, float inv_p,
-              int read_v, int bcast, const ShadowMap sm = ShadowMap(), const MeanArgs mean = MeanArgs()) {
-  tc::grid_launch_dependents();
-  tc::grid_dependency_wait();
-  if (MEAN && blockIdx.x == gridDim.x - 1) {
-    block_mean(mean.losses, mean.count, mean.out);
-    return;
-  }
+template <int U, bool STREAM_ST, bool SHADOW>
+__device__ __forceinline__ void meta_vectors(float* __restrict__ rep, int64_t stride, float* __restrict__ w,
+                                             float* __restrict__ v, int P, int64_t n, float mu, float zeta, float inv_p,
+                                             int read_v, int bcast, const ShadowMap& sm, int blocks) {
   const int64_t n4 = n >> 2;
   const int64_t stride4 = stride >> 2;
   float4* rep4 = reinterpret_cast<float4*>(rep);
   float4* w4 = reinterpret_cast<float4*>(w);
   float4* v4 = reinterpret_cast<float4*>(v);
-  const int64_t step = (int64_t)(gridDim.x - (MEAN ? 1 : 0)) * blockDim.x;
+  const int64_t step = (int64_t)blocks * blockDim.x;
   for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < n4; q += step) {
     const float4 wt = ld_stream(w4 + q);
     float4 vt = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -104,6 +95,29 @@ k_meta_update(float* __restrict__ rep, int64_t stride, float* __restrict__ w,
   if (blockIdx.x == 0 && threadIdx.x < (n & 3))
     meta_scalar(rep, stride, w, v, P, (n4 << 2) + threadIdx.x, mu, zeta, inv_p, read_v != 0,
                 bcast != 0);
+}
+
+template <int U, bool STREAM_ST, bool SHADOW = false>
+__global__ void __launch_bounds__(256)
+k_meta_update(float* __restrict__ rep, int64_t stride, float* __restrict__ w,
+              float* __restrict__ v, int P, int64_t n, float mu, float zeta, float inv_p,
+              int read_v, int bcast, const ShadowMap sm = ShadowMap()) {
+  meta_vectors<U, STREAM_ST, SHADOW>(rep, stride, w, v, P, n, mu, zeta, inv_p, read_v, bcast, sm, gridDim.x);
+}
+
+// Launched before a model's local steps have ended; MEAN: a block of its own forms the round's mean loss.
+template <bool MEAN>
+__global__ void __launch_bounds__(256)
+k_meta_update_early(float* __restrict__ rep, int64_t stride, float* __restrict__ w,
+                    float* __restrict__ v, int P, int64_t n, float mu, float zeta, float inv_p,
+                    int read_v, int bcast, const float* __restrict__ losses, int count, float* mean) {
+  tc::grid_launch_dependents();
+  tc::grid_dependency_wait();
+  if (MEAN && blockIdx.x == gridDim.x - 1) {
+    block_mean(losses, count, mean);
+    return;
+  }
+  meta_vectors<8, false, false>(rep, stride, w, v, P, n, mu, zeta, inv_p, read_v, bcast, ShadowMap(), gridDim.x - (MEAN ? 1 : 0));
 }
 
 // Algorithm 1's "set w^j = w~" on its own (initialisation, resume), optionally with v <- 0.
@@ -394,23 +408,28 @@ cudaError_t launch_meta_update(mavg_ctx* c) {
                                                                  n, mu, zeta, inv_p, read_v, bcast,
                                                                  c->shadow);
       c->shadow_fresh = true;
+    } else if (const bool mean = c->mean_wanted && !c->profiling; c->cfg.objective != MAVG_OBJ_MLP || (P > 16 && !mean)) {
+      k_meta_update<8, false><<<grid, 256, 0, c->stream>>>(rep, c->buf.replica_stride, w, v, P,
+                                                           n, mu, zeta, inv_p, read_v, bcast);
     } else {
-      // Begins while the small models' one launch of local steps ends, and forms the mean loss on the way where it is
-      // wanted (with the loss copied back after a launch of its own 32-64-10, P = 4, K = 4, B = 32 takes 60 us a round, 50 so).
-      const bool mean = c->mean_wanted && !c->profiling && c->cfg.objective == MAVG_OBJ_MLP;
-      const MeanArgs ma{(const float*)ws_ptr(c, c->ws.losses), P * c->cfg.K,
-                        c->mean_dev ? c->mean_dev : (float*)ws_ptr(c, c->ws.loss_mean)};
+      // Begins while a model's local steps end, and forms the mean loss on the way where it is wanted (with the loss copied
+      // back after a launch of its own 32-64-10, P = 4, K = 4, B = 32 takes 60 us a round, 50 so).  With many learners the
+      // blocks that wait take room from the steps (64-128-10, P = 40, K = 4, B = 32 89.2 / 91.8 us).  Meta-updates that follow
+      // one another do not: some gain (n = 1.28 M, P = 4 10.5 / 9.4 us a launch, n = 201 K, P = 12 6.2 / 5.4), others lose
+      // as much where the L2 holds the set (n = 562 K, P = 11 10.6 / 12.1; n = 353 K, P = 25 12.9 / 15.2).
       cudaLaunchConfig_t lc{};
       lc.gridDim = dim3((unsigned)(grid + (mean ? 1 : 0)));
       lc.blockDim = dim3(256);
       lc.stream = c->stream;
       cudaLaunchAttribute at[1];
       at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-      at[0].val.programmaticStreamSerializationAllowed = 1;
+      at[0].val.programmaticStreamSerializationAllowed = P <= 16;
       lc.attrs = at;
       lc.numAttrs = 1;
-      e = cudaLaunchKernelEx(&lc, mean ? k_meta_update<8, false, false, true> : k_meta_update<8, false>, rep,
-                             c->buf.replica_stride, w, v, P, n, mu, zeta, inv_p, read_v, bcast, ShadowMap(), ma);
+      e = cudaLaunchKernelEx(&lc, mean ? k_meta_update_early<true> : k_meta_update_early<false>, rep,
+                             c->buf.replica_stride, w, v, P, n, mu, zeta, inv_p, read_v, bcast,
+                             (const float*)ws_ptr(c, c->ws.losses), P * c->cfg.K,
+                             c->mean_dev ? c->mean_dev : (float*)ws_ptr(c, c->ws.loss_mean));
       c->mean_formed = mean && e == cudaSuccess;
     }
     if (e == cudaSuccess) e = cudaGetLastError();
