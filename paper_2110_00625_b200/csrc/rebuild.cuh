@@ -5,8 +5,8 @@
 // own weights are rounded to bf16 at every step as in the plain form; with momentum the steps are taken one after the
 // other in fp32 in its very order.
 //
-// 3072-2048-2048-2048-10, P = 8, B = 64, momentum (14.7 M weights a learner), step 1 .. 4 of 4: 146, 158, 225 us against 116 us
-// for the 0.76 GB of steps 1 .. 3 at the copy rate, and 370 against 222 (1.47 GB: W and u go out); the round takes 1463 us,
+// 3072-2048-2048-2048-10, P = 8, B = 64, momentum (14.7 M weights a learner), step 1 .. 4 of 4: 145, 164, 194 us against 116 us
+// for the 0.76 GB of steps 1 .. 3 at the copy rate, and 386 against 222 (1.47 GB: W and u go out); the round takes 1447 us,
 // 1928 with the steps in place.  What bounds steps 1 .. 3 is what an SM takes in from the L2, about 49 GB/s: 32 KB of operands
 // per tile and step so far beside 64 KB of u, 95, 127 and 158 us.  The last step waits for its stores and, with all of
 // tensor memory taken by one learner's four gradients, for the next learner's.  Registers: four steps' accumulators of
@@ -55,7 +55,7 @@ struct Args {
   int* status;
 };
 struct alignas(16) Shared {                       // (whole 16 bytes, as static shared memory is counted)
-  uint64_t full[3], empty[3], acc_full[2], acc_empty[2], piece_full[kGroups][2];
+  uint64_t full[3], empty[3], acc_full[4], acc_empty[4], piece_full[kGroups][2];
   uint32_t tmem_slot;
   int abort_flag;
   int fetch_unit[kGroups], fetch_p[kGroups], fetched[kGroups];   // a group's place in its list of pieces to fetch
@@ -88,7 +88,7 @@ k_rebuild(const __grid_constant__ Args g) {
       mbar_init(&sh.full[s], 1);
       mbar_init(&sh.empty[s], 1);
     }
-    for (int b = 0; b < 2; ++b) {
+    for (int b = 0; b < 4; ++b) {
       mbar_init(&sh.acc_full[b], 1);
       mbar_init(&sh.acc_empty[b], 4 * kGroups);
     }
@@ -111,7 +111,9 @@ k_rebuild(const __grid_constant__ Args g) {
   grid_dependency_wait();
   volatile int* abortp = &sh.abort_flag;
   const int nkb = (g.B + kBK - 1) / kBK;          // slabs of a step
-  const int acc_cols = (MOM ? g.steps : 1) * kBN, bufs = 2 * acc_cols <= 512 ? 2 : 1;
+  // Tensor memory as a ring of four accumulators: with momentum a learner takes one per step, else one (a learner's at
+  // a time, twice where they fit twice: 146, 158, 225 and 370 us, the round 1463)
+  const int accs = MOM ? g.steps : 1;
   const int groups = (g.P + g.group - 1) / g.group, units = groups * g.tiles;
   // units of the same learners follow one another: their rows stay in the L2
   auto decode = [&](int unit, int& p0, int& p1, int& l, int& m0, int& n0) {
@@ -158,25 +160,25 @@ k_rebuild(const __grid_constant__ Args g) {
       for (int unit = blockIdx.x; unit < units && ok; unit += gridDim.x) {
         int p0, p1, l, m0, n0;
         decode(unit, p0, p1, l, m0, n0);
-        for (int p = p0; p < p1 && ok; ++p, ++n) {
-          const int b = n % bufs;
-          if (!(ok = mbar_wait(&sh.acc_empty[b], ((n / bufs) & 1) ^ 1, abortp, g.status, ERR_REB_MMA))) break;
-          tc_fence_after_sync();
+        for (int p = p0; p < p1 && ok; ++p)
           for (int i = 0; i < g.steps * nkb; ++i, ++it) {
-            const int s = it % kStages, kb = i % nkb;
+            const int s = it % kStages, kb = i % nkb, b = n & 3;
+            const bool first = MOM ? kb == 0 : i == 0, last = MOM ? kb == nkb - 1 : i == g.steps * nkb - 1;
+            if (first && !(ok = mbar_wait(&sh.acc_empty[b], ((n >> 2) & 1) ^ 1, abortp, g.status, ERR_REB_MMA))) break;
             if (!(ok = mbar_wait(&sh.full[s], (it / kStages) & 1, abortp, g.status, ERR_REB_MMA))) break;
             tc_fence_after_sync();
-            const uint32_t off = (uint32_t)(s * kStageBytes) >> 4, d = tmem_base + (uint32_t)(b * acc_cols + (MOM ? i / nkb * kBN : 0));
+            const uint32_t off = (uint32_t)(s * kStageBytes) >> 4, d = tmem_base + (uint32_t)(b * kBN);
             // a step's last slab ends with its batch (a multiple of 16)
             const int nk = min(kBK, g.B - kb * kBK) / 16;
-            const bool first = MOM ? kb == 0 : i == 0;
             for (int k = 0; k < nk; ++k)
               umma_bf16(d, a0 + off + (uint32_t)k * ((16 * 128) >> 4), b0 + off + (uint32_t)k * ((16 * 128) >> 4), idesc,
                         (uint32_t)(!first || k > 0));
             umma_commit(&sh.empty[s]);
+            if (last) {
+              umma_commit(&sh.acc_full[b]);
+              ++n;
+            }
           }
-          if (ok) umma_commit(&sh.acc_full[b]);
-        }
       }
     }
     __syncwarp();
@@ -218,7 +220,7 @@ k_rebuild(const __grid_constant__ Args g) {
       for (int i = 0; i < kRing; ++i) fetch();
     }
     uint32_t pn = 0;                               // pieces taken in
-    int n = 0;
+    int n = 0;                                     // accumulators taken before this learner's
     bool failed = false, gone = false;
     auto cell = [&](uint8_t* buf, int c) { return reinterpret_cast<float4*>(buf + (size_t)row * 128 + ((c ^ (row & 7)) << 4)); };
     auto wait_piece = [&]() {
@@ -243,12 +245,12 @@ k_rebuild(const __grid_constant__ Args g) {
         if ((gone = barrier_any(failed, 2 + grp, 128))) break;
         if (leader && !u_apart) fetch();
       }
-      for (int p = p0; p < p1; ++p, ++n) {
-        const int b = n % bufs;
-        if (!mbar_wait(&sh.acc_full[b], (n / bufs) & 1, abortp, g.status, ERR_REB_EPILOGUE)) failed = true;
+      for (int p = p0; p < p1; ++p, n += accs) {
+        for (int i = n; i < n + accs; ++i)
+          if (!mbar_wait(&sh.acc_full[i & 3], (i >> 2) & 1, abortp, g.status, ERR_REB_EPILOGUE)) failed = true;
         __syncwarp();
         tc_fence_after_sync();
-        const uint32_t acc = tmem_base + ((uint32_t)(q4 * 32) << 16) + (uint32_t)(b * acc_cols + c0);
+        const uint32_t acc = tmem_base + ((uint32_t)(q4 * 32) << 16) + (uint32_t)c0;
         uint8_t* ub = in_buf;
         if (mine && load_u) ub = wait_piece();
         if (mine) {
@@ -272,8 +274,8 @@ k_rebuild(const __grid_constant__ Args g) {
               for (int i = 0; i < kMaxMomSteps; i += 2) {
                 if (i >= g.steps) break;
                 uint32_t r[2][8];
-                tmem_ld_8cols(acc + (uint32_t)(i * kBN + 8 * h), r[0]);
-                if (i + 1 < g.steps) tmem_ld_8cols(acc + (uint32_t)((i + 1) * kBN + 8 * h), r[1]);
+                tmem_ld_8cols(acc + (uint32_t)(((n + i) & 3) * kBN + 8 * h), r[0]);
+                if (i + 1 < g.steps) tmem_ld_8cols(acc + (uint32_t)(((n + i + 1) & 3) * kBN + 8 * h), r[1]);
                 tmem_ld_wait();
 #pragma unroll
                 for (int j = 0; j < 8; ++j) msgd(x[j], v[j], __uint_as_float(r[0][j]), g.gamma, g.beta);
@@ -283,7 +285,7 @@ k_rebuild(const __grid_constant__ Args g) {
               }
             } else {
               uint32_t r[8];
-              tmem_ld_8cols(acc + (uint32_t)(8 * h), r);
+              tmem_ld_8cols(acc + (uint32_t)((n & 3) * kBN + 8 * h), r);
               tmem_ld_wait();
 #pragma unroll
               for (int j = 0; j < 8; ++j) x[j] = fmaf(-g.gamma, __uint_as_float(r[j]), x[j]);
@@ -307,7 +309,8 @@ k_rebuild(const __grid_constant__ Args g) {
         }
         tc_fence_before_sync();
         __syncwarp();
-        if (lane == 0) mbar_arrive(&sh.acc_empty[b]);
+        if (lane == 0)
+          for (int i = n; i < n + accs; ++i) mbar_arrive(&sh.acc_empty[i & 3]);
         if (!mine) continue;                       // (a wait given up here is carried by the next barrier)
         fence_proxy_async();
         if ((gone = barrier_any(failed, 2 + grp, 128))) break;
