@@ -33,20 +33,28 @@ enum { ERR_SPLIT_PRODUCER = 41, ERR_SPLIT_MMA = 42, ERR_SPLIT_EPILOGUE = 43 };
 
 __host__ __device__ constexpr int pitch_of(int d) { return (d + 7) / 8 * 8; }
 
-// Two neighbours as NP bf16 planes.  Round to nearest leaves at most half a unit to the next plane.  An infinite
-// or overflowing first part stands alone: what it leaves over would be NaN.
+// Two neighbours as NP bf16 planes.  Round to nearest leaves at most half a unit to the next plane.  The first of three is
+// the largest finite bf16 number where a finite value rounds beyond it (from 3.39e38 on), which leaves 16 bits to the other
+// two; that of an infinite value is infinite and stands alone: what it leaves over would be NaN.
 template <int NP>
 __device__ __forceinline__ void split2(float a, float b, uint32_t (&pl)[NP]) {
 #pragma unroll
   for (int i = 0; i < NP; ++i) {
-    const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
-    pl[i] = *reinterpret_cast<const uint32_t*>(&h);
+    if (NP > 1 && i == 0) {
+      asm("cvt.rn.satfinite.bf16x2.f32 %0, %1, %2;" : "=r"(pl[i]) : "f"(b), "f"(a));
+    } else {
+      const __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
+      pl[i] = *reinterpret_cast<const uint32_t*>(&h);
+    }
     if (i + 1 < NP) {
-      a -= __low2float(h);
-      b -= __high2float(h);
-      if (i == 0) {
-        a = fabsf(a) <= 3.402823466e38f ? a : 0.f;
-        b = fabsf(b) <= 3.402823466e38f ? b : 0.f;
+      a -= __uint_as_float(pl[i] << 16);
+      b -= __uint_as_float(pl[i] & 0xffff0000u);
+      if (i == 0) {                                // the next number up is the infinite one
+        const bool ia = fabsf(a) == INFINITY, ib = fabsf(b) == INFINITY;
+        if (ia) pl[i] += 1u;
+        if (ib) pl[i] += 0x10000u;
+        a = ia ? 0.f : a;
+        b = ib ? 0.f : b;
       }
     }
   }

@@ -18,14 +18,14 @@ SHAPES = [                                  # dims, B, P
 ]
 
 
-def _pair(oracle, mode, dims, B, P, beta, w1=None, x=None):
+def _pair(oracle, mode, dims, B, P, beta, w1=None, x=None, K=2):
     import paper_2110_00625_b200 as m
     rng = np.random.default_rng(B)
     S = 60 * P + 7
     x = rng.standard_normal((S, dims[0]), dtype=np.float32) if x is None else x
     y = rng.integers(0, dims[-1], size=len(x)).astype(np.int32)
     w1 = m.workloads.mlp_init(dims) if w1 is None else w1
-    kw = dict(P=P, K=2, mu=0.9, B=B, seed=11, dims=dims, x=x, y=y)
+    kw = dict(P=P, K=K, mu=0.9, B=B, seed=11, dims=dims, x=x, y=y)
     g = m.Mavg(w1, local_lr=0.01, objective=m.OBJ_MLP, gemm_bf16=mode, learner_momentum=beta, defer_broadcast=P == 1, **kw)
     o = oracle.Mavg(w1, gamma=0.01, objective=oracle.OBJ_MLP, bf16=mode != 0, beta=beta, stride=g.stride, **kw)
     return g, o
@@ -78,5 +78,36 @@ def test_infinite_weights_reach_no_more_than_their_own_unit(oracle, dims, B, P, 
     rep[:, at] = 0.0
     want = want.copy()
     want[:, at] = 0.0
+    assert l2_rel(rep, want) <= 1e-6
+    g.close()
+
+
+@pytest.mark.parametrize("value", [3.4e38, -3.4e38, np.finfo(np.float32).max])
+@pytest.mark.parametrize("dims,B,P", [([300, 200, 70, 10], 32, 2), ([301, 200, 70, 10], 300, 1)])
+def test_the_largest_fp32_values_are_finite_ones(oracle, dims, B, P, value):
+    # above 3.39e38 a value rounds to a bf16 infinity, whose product with a zero is NaN: weights of layers 1 and 2 whose
+    # inputs are zero (where they are not, the unit is dead), and inputs whose weights are
+    import paper_2110_00625_b200 as m
+    x = np.random.default_rng(3).standard_normal((100, dims[0])).astype(np.float32)
+    x[0::2, 5] = 0.0
+    x[1::2, 5] = -1e-30 * np.sign(value)
+    x[0::3, 9] = value
+    w1 = m.workloads.mlp_init(dims)
+    W1, b1 = w1[:dims[1] * dims[0]].reshape(dims[1], dims[0]), w1[dims[1] * dims[0]:][:dims[1]]
+    W2 = w1[dims[1] * (dims[0] + 1):][:dims[2] * dims[1]].reshape(dims[2], dims[1])
+    W1[7, 5] = W2[3, 11] = value
+    W1[:, 9] = 0.0
+    b1[11] = -1e9                                # unit 11 is dead
+    g, o = _pair(oracle, 0, dims, B, P, 0.0, w1, x, K=1)
+    g.local_steps()
+    losses, _ = o.local_steps()
+    g.sync()
+    assert np.isfinite(losses).all() and l2_rel(g.get_losses(), losses) <= 1e-6
+    rep, want = g.replicas[:, :g.n].cpu().numpy(), o.replicas[:, :g.n].copy()
+    large = [np.flatnonzero(w1 == np.float32(value)), np.arange(dims[1]) * dims[0] + 9]
+    assert (rep[:, large[0]] == np.float32(value)).all() and (want[:, large[0]] == np.float32(value)).all()
+    assert np.abs(want[:, large[1]]).max() > 1e30 and l2_rel(rep[:, large[1]], want[:, large[1]]) <= 6e-6   # a step, as above
+    for at in large + [np.array([dims[1] * dims[0] + 11])]:
+        rep[:, at] = want[:, at] = 0.0
     assert l2_rel(rep, want) <= 1e-6
     g.close()
