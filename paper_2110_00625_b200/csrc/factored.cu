@@ -1695,8 +1695,8 @@ void reb_setup(mavg_ctx* c, TcState* st) {
 
 bool reb_usable(const mavg_ctx* c) {
   const TcState* st = (const TcState*)c->mlp;
-  return st && st->reb && c->schedule == 0 && c->cfg.K >= 2 && c->cfg.K <= st->reb->K &&
-         (c->cfg.learner_momentum == 0.f || c->cfg.K <= rebuild::kMaxMomSteps);
+  // by the momentum and K of now, which may not be those the handle was made with
+  return st && st->reb && c->schedule == 0 && c->cfg.K <= st->reb->K && reb_steps(&c->cfg) == c->cfg.K;
 }
 
 // The K steps of a round: F_1 -> ... -> F_{L-1} -> last layer and loss -> D_L -> ... -> D_2 -> weights of the next step's

@@ -60,3 +60,31 @@ def test_without_momentum_one_step_from_the_sum_of_the_gradients(dims, P, K, B):
     # One fp32 rounding of the weights instead of K; v (the mean displacement) differs where a weight rounds to the other
     # bf16 neighbour: the two forms' spread is that of any other order of sums, 2^-8 of v at these sizes, and twice that.
     assert max(_pair(dims, P, K, B, 0.0, False, True, lambda g: g.round())) < 2 ** -7
+
+
+def test_by_the_momentum_and_steps_of_now():
+    import paper_2110_00625_b200 as m
+    dims, P, B = [3072, 1024, 512, 10], 10, 64       # 37 M hidden weights: with momentum only
+    x = torch.randn(2000, dims[0], device="cuda")
+    y = torch.randint(0, dims[-1], (2000,), device="cuda").int()
+    w1 = m.workloads.mlp_init(dims)
+    kw = dict(P=P, local_lr=0.002, mu=0.9, B=B, seed=3, objective=m.OBJ_MLP, dims=dims, gemm_bf16=1, x=x, y=y, x_bf16=True,
+              with_learner_u=True)
+    g = m.Mavg(w1, K=4, learner_momentum=0.9, **kw)
+    rebuilt = [g.rebuilt()]
+    for beta, K in ((0.9, 3), (0.0, 4), (0.5, 4), (0.0, 2), (0.5, 1), (0.5, 6), (0.5, 2)):
+        g.set_learner_momentum(beta)
+        g.set_hparams(K, 0.002, 1.0, 0.9)
+        rebuilt.append(g.rebuilt())
+        w = g.w.clone()
+        g.set_round(0)
+        g.v.zero_()
+        g.u.zero_()
+        g.round()
+        h = m.Mavg(w, K=K, learner_momentum=beta, **kw)
+        h.round()
+        for a, b in zip((g.w, g.v, g.replicas[:, :g.n], g.u[:, :g.n]), (h.w, h.v, h.replicas[:, :h.n], h.u[:, :h.n])):
+            assert torch.equal(a, b)
+        h.close()
+    assert rebuilt == [True, True, False, True, False, False, False, True]
+    g.close()
