@@ -273,14 +273,14 @@ mavg_status mavg_set_profiling(mavg_handle h, int32_t on);
  *     step, products take w~ and the factors instead.  w~ enters the forward products and the last layer as
  *     two bf16 parts and the data gradients as one, the sums over the factors through bf16 Gram rows; the plain
  *     form rounds W_l(k) to bf16 at every step.  Other rounds of large models that start from w~ (P times the hidden layers'
- *     weights 48 million or more and K <= 6; with learner momentum 20 million and K <= 4; K B <= 512) have rebuilt steps: the
- *     plain form's steps, whose weights W(k) and u(k) are formed anew in step k from w~, u as the call found it and the
- *     factors dZ(i), A(i), i <= k.  With momentum they are the plain form's weights to the bit, without it one fp32 step from
- *     the sum of the gradients.  mavg_workspace_bytes has room for these forms if
+ *     weights 48 million or more, with learner momentum 20 million; K <= 4 and K B <= 512, without momentum also K <= 6 and
+ *     K B <= 384) may have rebuilt steps (mavg_get_rebuilt): the plain form's steps, whose weights W(k) and u(k) are formed
+ *     anew in step k from w~, u as the call found it and the factors dZ(i), A(i), i <= k, with the plain form's sums in its
+ *     order and so its results to the bit.  mavg_workspace_bytes has room for these forms if
  *     the handle's own K and momentum take one; a buffer with room for the plain form only
  *     (mavg_workspace_least_bytes) is accepted and keeps that.
  *   MAVG_SCHED_GRAPH_TC: the same graph with every product as plain one-tile-per-block
- *     tensor-core launches.  Apart from factored and rebuilt rounds the two differ in the
+ *     tensor-core launches.  Apart from factored rounds the two differ in the
  *     summation order of the products they run differently, nothing else; this one exists for comparison.
  * Profiled rounds (mavg_set_profiling) take the launch-by-launch form of the chosen schedule; what is
  * one launch without profiling (the steps of a small CUDA-core model, a pseudo-gradient round) is one

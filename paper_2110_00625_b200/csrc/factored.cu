@@ -9,7 +9,7 @@
 //   k_fac_apply     W_l = w~_l - gamma dZ_l^T A_{l-1} over all steps' rows, every learner and hidden layer
 //   k_fac_last      the last layer (at most 32 classes), which keeps its own weights and steps
 //
-// and the rebuilt local steps of rebuild.cuh, which share the gather and the products with weights.
+// and the rebuilt local steps of rebuild.cuh, which share the gather; their products are the plain form's launches.
 //
 // All are launched with programmatic stream serialisation.
 #include <cuda.h>
@@ -28,7 +28,7 @@ using namespace tc;
 using namespace gemm;
 
 constexpr int kFacThreads = 320;   // warp 0: TMA producer, warp 1: MMA issuer, warps 2-9: epilogue
-enum { PROD_FWD = 0, PROD_DGRAD = 1, PROD_RAW = 2 };
+enum { PROD_FWD = 0, PROD_DGRAD = 1, PROD_RAW = 2, PROD_DGRAD_STEP = 3 };
 constexpr size_t kGramBarBytes = 2 * sizeof(uint64_t);   // static shared memory of a product that forms its Gram rows, beside GemmShared
 
 // Place in a ring of stages and the phase of its barriers, without a division per slab: the one thread that
@@ -163,7 +163,6 @@ struct ProdArgs {
   int row_end;              // RAW: rows per learner
   int nkb;                  // slabs of the product with w~ (0: left out)
   int w_batched;            // the weights are each learner's own (one learner per block)
-  int in_off;               // added to the learner in the batch operand's array
   int hist;                 // rows of the earlier steps (0: left out)
   int s_row0;               // row of the batch inside a learner's Gram rows
   int stages;
@@ -183,7 +182,7 @@ struct ProdArgs {
   __nv_bfloat16* gram_out;
   int64_t gram_stride, gram_ld;
   float gamma;
-  MomArgs mom;              // of the stepped bias
+  MomArgs mom;              // of the stepped bias (PROD_DGRAD_STEP)
   int* status;
 };
 
@@ -233,7 +232,7 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
   // A stage: the w~ tile (LOW: and its low part), then the batch operand; or TILES history slabs in the
   // tiles' places, with their Gram rows where the batch operand is.
   static_assert(!LOW || TILES == 2, "");
-  constexpr bool kMn = EPI == PROD_DGRAD;          // w~ is read MN-major
+  constexpr bool kStep = EPI == PROD_DGRAD_STEP, kMn = EPI == PROD_DGRAD || kStep;   // kMn: the weights are read MN-major
   constexpr int kBOff = TILES * kATileBytes;
   const int stage_bytes = product_stage_bytes(TILES, EPI == PROD_RAW ? 1 : TILES, g.nl, g.cols), s_bytes = g.cols * kBK * 2;
   __shared__ __align__(8) uint64_t gram_bar, rows_bar;     // GRAM: Gram sums complete; Gram rows in global memory
@@ -305,7 +304,7 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
           tma_load_3d(sa, &tm_w, full, i * kBK, m0, w_of);
         }
         if (LOW) tma_load_3d(sa + kATileBytes, &tm_lo, full, i * kBK, m0, 0);
-        tma_load_3d(sa + kBOff, &tm_in, full, i * kBK, r0, p0 + g.in_off);
+        tma_load_3d(sa + kBOff, &tm_in, full, i * kBK, r0, p0);
       }
       if (GRAM && ok) {
         ok = mbar_wait_cluster(&rows_bar, 0, abortp, g.status, ERR_PRODUCER);
@@ -441,9 +440,59 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     };
 #pragma unroll
     for (int j = 0; j < 16; ++j) { zb[j] = 0.f; act[j] = __float2bfloat16_rn(0.f); }
-    fetch(half * 16);
+    if (!kStep) fetch(half * 16);
     const bool ok = !any || mbar_wait_warp(&sh.acc_bar, 0, abortp, g.status, ERR_EPILOGUE);
-    if (ok) {
+    if (kStep && ok) {
+      // The bias step's sums in the order of the plain form's tile: a sum over every second 32 columns of a learner, from
+      // the first, and one over the others.  One learner: a sum to each half of the warps; several: a learner, both sums.
+      tc_fence_after_sync();
+      const uint32_t lane_addr = tmem_base + ((uint32_t)(q4 * 32) << 16);
+      const int groups = g.cols / 16;
+      int q = nl > 1 ? half : 0, which = nl > 1 ? 0 : half, gr = 2 * which;
+      float s = 0.f;
+      auto settle = [&] {                          // on to a group of 16 columns that exists, or behind the last learner
+        while (q < nl && gr >= groups) {
+          colsum[(which * nl + q) * kBM + row] = s;
+          s = 0.f;
+          if (nl > 1 && which == 0) {
+            which = 1;
+          } else {
+            q += nl > 1 ? 2 : 1;
+            which = nl > 1 ? 0 : half;
+          }
+          gr = 2 * which;
+        }
+      };
+      auto place = [&] { return ((size_t)(p0 + q) * g.kb + r0 + 16 * gr) * g.M + m; };
+      auto fetch_act = [&] {
+        if (m_ok && q < nl) {
+          const size_t at = place();
+#pragma unroll
+          for (int j = 0; j < 16; ++j) act[j] = g.act[at + (size_t)j * g.M];
+        }
+      };
+      settle();
+      fetch_act();
+#pragma unroll 1
+      while (q < nl) {
+        const size_t at = place();
+        float z[16];
+        load16(lane_addr + (uint32_t)(q * g.cols + 16 * gr), true, z);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) {
+          z[j] = __bfloat162float(act[j]) > 0.f ? z[j] : 0.f;        // ReLU'(0) = 0
+          s += z[j];
+        }
+        gr += gr & 1 ? 3 : 1;
+        settle();
+        fetch_act();
+        if (m_ok) {
+#pragma unroll
+          for (int j = 0; j < 16; ++j) g.out[at + (size_t)j * g.M] = __float2bfloat16_rn(z[j]);
+        }
+      }
+    }
+    if (!kStep && ok) {
       tc_fence_after_sync();
       const uint32_t lane_addr = tmem_base + ((uint32_t)(q4 * 32) << 16);
 #pragma unroll 1
@@ -487,7 +536,7 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
         }
       }
     }
-    if (EPI == PROD_DGRAD) {
+    if (kMn) {
       // bias step of the layer below, b[m] -= gamma * sum_b dZ[b, m]: the two warps that share a row add
       // their sums in a fixed order
       epilogue_barrier();
@@ -496,7 +545,7 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
       } else if (ok && m_ok) {
         for (int q = half; q < nl; q += 2) {
           const float w_in = g.bias_in[(size_t)(p0 + q) * g.bias_in_stride + g.bias_off + m];
-          float* u = g.mom.u ? g.mom.u + (size_t)(p0 + q) * g.mom.u_stride + g.bias_off + m : nullptr;
+          float* u = kStep && g.mom.u ? g.mom.u + (size_t)(p0 + q) * g.mom.u_stride + g.bias_off + m : nullptr;
           local_update(g.bias_rep + (size_t)(p0 + q) * g.rep_stride + g.bias_off + m, w_in, u, g.mom.read_u,
                        colsum[q * kBM + row] + colsum[(nl + q) * kBM + row], g.gamma, g.mom.beta);
         }
@@ -511,8 +560,7 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
       float s = 0.f;
       for (int r = 0; r < g.c_tiles; ++r) s += ld_cluster_f32(mapa_u32(smem_u32(&sh.colsum[0][row]), (uint32_t)(rank0 + r)));
       const float w_in = g.bias_in[(size_t)p0 * g.bias_in_stride + g.bias_off + m];
-      float* u = g.mom.u ? g.mom.u + (size_t)p0 * g.mom.u_stride + g.bias_off + m : nullptr;
-      local_update(g.bias_rep + (size_t)p0 * g.rep_stride + g.bias_off + m, w_in, u, g.mom.read_u, s, g.gamma, g.mom.beta);
+      local_update(g.bias_rep + (size_t)p0 * g.rep_stride + g.bias_off + m, w_in, nullptr, 0, s, g.gamma, 0.f);
     }
     __syncwarp();
     cluster_sync_all();           // nobody leaves while its sums may still be read
@@ -1191,7 +1239,7 @@ cudaError_t launch_product(mavg_ctx* c, int cls, const CUtensorMap& w, const CUt
   g.low_col = (uint32_t)(GRAM ? gram_columns(g.cols, g.m_tiles, g.hist) : g.nl * g.cols);
   g.tmem_cols = tmem_columns((int)g.low_col + (LOW ? g.nl * g.cols : 0));
   size_t smem = (size_t)g.stages * stage_bytes + 1024 +
-                (EPI == PROD_DGRAD ? (size_t)2 * g.nl * kBM * sizeof(float) : 0);
+                (EPI == PROD_DGRAD || EPI == PROD_DGRAD_STEP ? (size_t)2 * g.nl * kBM * sizeof(float) : 0);
   const int cluster = GRAM ? (int)grid.x : EPI == PROD_DGRAD ? g.c_tiles : 1;
   smem = std::max(smem, tmem_share_bytes(g.tmem_cols, sizeof(GemmShared) + (GRAM ? kGramBarBytes : 0)));
   PdlLaunch l(grid, kFacThreads, smem, c->stream, cluster);
@@ -1596,14 +1644,13 @@ cudaError_t fac_local_steps(mavg_ctx* c, int64_t round) {
 
 // Where rounds are rebuilt instead of stepped in place: where they are not factored and what a step moves, 10 bytes per
 // weight in place (18 with momentum), costs more than forming the weights anew from all rows so far, k B in step k.  V: P
-// times the hidden layers' weights.  Time in place / rebuilt over 323 shapes (1 to 3 hidden layers of 128 to 2048, P = 2 ..
-// 48, B = 16 .. 256, V = 8 .. 184 M):
-//   with momentum (an accumulator per step: K <= 4)   V >= 20 M: 1.03 .. 1.58, never slower; V = 8 .. 20 M: 0.797 .. 1.40
-//   without                                  V >= 48 M, K <= 6: 1.12 .. 1.48, never slower; K = 7 .. 16: 0.954 .. 1.19
-// Without momentum rebuilt steps win from V = 24 M on (1.20 .. 1.84), but there the schedule in place is the one whose
-// forward products ride on the weight gradients and whose sums run in another order; it is held to 2e-2 of the plain
-// tiles' v, and at 3072-1024-512-10, P = 13, K = 4, B = 16 (V = 47.8 M) the two are 2.1e-2 apart when rebuilt (as far
-// from 64 bits as each other).
+// times the hidden layers' weights.  Time in place / rebuilt over 340 shapes (1 to 3 hidden layers of 128 to 2048, P = 2 ..
+// 48, B = 16 .. 256, V = 12 .. 190 M):
+//   with momentum (all steps' accumulators at once: K <= 4)   V >= 20 M: 1.003 .. 1.57; V = 12 .. 20 M: 0.92 .. 1.31
+//   without, V >= 48 M        K <= 4: 1.07 .. 1.50; K = 5, 6: 1.05 .. 1.21 up to 384 rows a learner, 0.969 at 480
+//            V = 20 .. 48 M   K <= 4: 0.949 .. 1.36; K = 5, 6: 0.866 .. 1.24
+// Where the forward products ride on the weight gradients in place, K = 5 takes 1.02 and 1.04 times as long rebuilt:
+// four steps at most there (reb_usable).
 int reb_steps(const mavg_config* cfg) {
   const int L = cfg->n_layers, B = cfg->B;
   const bool momentum = cfg->learner_momentum != 0.f;
@@ -1611,7 +1658,7 @@ int reb_steps(const mavg_config* cfg) {
   int64_t weights = 0;
   for (int l = 1; l < L; ++l) weights += (int64_t)cfg->dims[l - 1] * cfg->dims[l];
   if (cfg->P * weights < (momentum ? 20 : 48) * 1000 * 1000) return 0;
-  const int most = std::min({cfg->K, 512 / B, momentum ? rebuild::kMaxMomSteps : 6});
+  const int most = std::min({cfg->K, 512 / B, momentum || cfg->K * B > 384 ? 4 : 6});
   return most >= 2 ? most : 0;
 }
 
@@ -1628,7 +1675,9 @@ FacLayout reb_layout(const mavg_config* cfg, size_t base) {
   for (int l = 1; l <= L; ++l) {
     t.g[l] = take(rows * up((size_t)cfg->dims[l], 8) * 2);
     t.w_own[l] = take((size_t)P * cfg->dims[l - 1] * cfg->dims[l] * 2);
+    if (l < L) t.act_t[l] = take((size_t)P * cfg->B * cfg->dims[l] * 2);
   }
+  t.dz_t = take((size_t)P * cfg->B * *std::max_element(cfg->dims + 1, cfg->dims + L) * 2);
   t.labels = take(rows * sizeof(int32_t));
   t.end = off;
   return t;
@@ -1644,47 +1693,64 @@ void reb_setup(mavg_ctx* c, TcState* st) {
   const FacLayout& t = f->lay;
   auto bf = [&](size_t off) { return (__nv_bfloat16*)ws_ptr(c, off); };
   bool ok = true;
-  // rows [steps P, B, d], a row `pitch` long
-  auto rows = [&](CUtensorMap* m, size_t at, int d, int box_rows, int box_learners = 1) {
+  // rows [n, B, d], a row `pitch` long
+  auto rows = [&](CUtensorMap* m, __nv_bfloat16* at, int d, int n, int box_rows, int box_learners = 1) {
     const int pitch = (int)up((size_t)d, 8);
-    ok = ok && encode_map(st, m, bf(at), d, B, f->K * P, pitch, (int64_t)B * pitch, box_rows, why, box_learners);
+    ok = ok && encode_map(st, m, at, d, B, n, pitch, (int64_t)B * pitch, box_rows, why, box_learners);
   };
+  // Products of k_fac_product where it sums in the plain form's order: over the whole contraction, and for a bias step
+  // over the whole batch; the others are the plain form's launches, whose data gradients read A_{l-1} transposed.
+  // (3072-2048-2048-2048-10, P = 8, B = 64: data gradients of a step 50 us, 57 as the plain form's launches; 1080-576-576-32,
+  // P = 26, B = 176 27 and 32.)
+  for (int l = 2; l <= L; ++l) {
+    const int m_tiles = (cfg.dims[l - 1] + kBM - 1) / kBM;
+    f->dgrad1[l] = cols_for(P, B, m_tiles, c->sm_count);
+    f->dgrad[l] = cols_for(P, B, m_tiles, c->sm_count, 1);
+    f->own_dgrad[l] = st->dgrad[l].splits == 1 && f->dgrad1[l].c_tiles == 1 && f->dgrad[l].c_tiles == 1;
+  }
+  for (int l = 1; l < L; ++l) {
+    const int m_tiles = (cfg.dims[l] + kBM - 1) / kBM;
+    f->fwd1[l] = cols_for(P, B, m_tiles, c->sm_count);
+    f->fwd[l] = cols_for(P, B, m_tiles, c->sm_count, 1);
+    for (int first = 0; first < 2; ++first) {
+      const FwdForm form = fwd_form(st, l, first);
+      const bool rides = !first && l <= st->fuse_upto;   // the plain form's product rides on a launch, with whole sums
+      f->own_fwd[first][l] = (rides || form == FwdForm::DENSE || (form == FwdForm::TILES && st->fwd[l].splits == 1)) &&
+                             ((l + 1 == L && st->tail_ok) || f->own_dgrad[l + 1]);
+      ok = ok && (!rides || f->own_fwd[first][l]);
+    }
+  }
+  f->step_in.resize((size_t)f->K * (MAVG_MAX_LAYERS + 1));
+  f->step_dz.resize(f->step_in.size());
   for (int l = 1; l <= L && ok; ++l) {
     const int in = cfg.dims[l - 1], out = cfg.dims[l];
     const int64_t size = (int64_t)in * out;
-    rows(&f->h_mn[l - 1], t.h[l - 1], in, 64);
-    rows(&f->g_mn[l], t.g[l], out, 64);
+    rows(&f->h_mn[l - 1], bf(t.h[l - 1]), in, f->K * P, 64);
+    rows(&f->g_mn[l], bf(t.g[l]), out, f->K * P, 64);
     ok = ok && encode_map(st, &f->w_own[l], bf(t.w_own[l]), in, out, P, in, size, kBM, why);
     ok = ok && encode_map(st, &f->w_own_mn[l], bf(t.w_own[l]), in, out, P, in, size, 64, why);
     ok = ok && encode_any(st, &f->w_own_st[l], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, bf(t.w_own[l]), in, out, P, in, size,
                           kWgradTileCols, kWgradTileRows, CU_TENSOR_MAP_SWIZZLE_64B, why);
-    // step 1: products with w~, several learners to a block; later ones a learner's own weights
-    if (l < L) {
-      f->fwd1[l] = cols_for(P, B, (out + kBM - 1) / kBM, c->sm_count);
-      f->fwd[l] = cols_for(P, B, (out + kBM - 1) / kBM, c->sm_count, 1);
-      rows(&f->in1[l], t.h[l - 1], in, f->fwd1[l].cols, f->fwd1[l].nl);
-      rows(&f->in[l], t.h[l - 1], in, f->fwd[l].cols);
-    }
-    if (l > 1) {
-      f->dgrad1[l] = cols_for(P, B, (in + kBM - 1) / kBM, c->sm_count);
-      f->dgrad[l] = cols_for(P, B, (in + kBM - 1) / kBM, c->sm_count, 1);
-      rows(&f->dz_in1[l], t.g[l], out, f->dgrad1[l].cols, f->dgrad1[l].nl);
-      rows(&f->dz_in[l], t.g[l], out, f->dgrad[l].cols);
+    for (int k = 1; k <= f->K && ok; ++k) {
+      const size_t at = (size_t)(k - 1) * (MAVG_MAX_LAYERS + 1) + l;
+      __nv_bfloat16* a = bf(t.h[l - 1]) + (size_t)(k - 1) * P * B * in;
+      const FwdForm form = l < L ? fwd_form(st, l, k == 1) : FwdForm::TILES;
+      const FacCols &fc = k == 1 ? f->fwd1[l] : f->fwd[l], &dc = k == 1 ? f->dgrad1[l] : f->dgrad[l];
+      if (l < L && f->own_fwd[k == 1][l]) rows(&f->step_in[at], a, in, P, fc.cols, fc.nl);
+      else if (form == FwdForm::DENSE) ok = encode_map(st, &f->step_in[at], a, in, P * B, 1, in, (int64_t)P * B * in, kDenseCols, why);
+      else rows(&f->step_in[at], a, in, P, form == FwdForm::SPLIT ? B : st->fwd[l].BN);
+      __nv_bfloat16* dz = bf(t.g[l]) + (size_t)(k - 1) * P * B * up((size_t)out, 8);
+      if (l > 1 && f->own_dgrad[l]) rows(&f->step_dz[at], dz, out, P, dc.cols, dc.nl);
+      else if (l > 1) rows(&f->step_dz[at], dz, out, P, st->dgrad[l].BN);
     }
   }
-  f->last_in.resize((size_t)f->K);                 // A_{L-1} of each step as the last layer's launch reads it
-  for (int k = 0; k < f->K && ok; ++k) {
-    const int d = cfg.dims[L - 1];
-    ok = ok && encode_map(st, &f->last_in[k], bf(t.h[L - 1]) + (size_t)k * P * B * d, d, B, P, d, (int64_t)B * d, st->fwd[L].BN, why);
-  }
-  const struct { const void* kernel; size_t fixed; } kernels[] = {
-      {(const void*)k_fac_product<PROD_FWD, 1, false, false>, sizeof(GemmShared)},
-      {(const void*)k_fac_product<PROD_DGRAD, 1, false, false>, sizeof(GemmShared)},
-      {(const void*)rebuild::k_rebuild<false, false>, sizeof(rebuild::Shared)}, {(const void*)rebuild::k_rebuild<false, true>, sizeof(rebuild::Shared)},
-      {(const void*)rebuild::k_rebuild<true, false>, sizeof(rebuild::Shared)}, {(const void*)rebuild::k_rebuild<true, true>, sizeof(rebuild::Shared)}};
-  for (const auto& k : kernels)
-    ok = ok && cudaFuncSetAttribute(k.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)(kSmSharedBytes - kBlockReservedBytes - k.fixed)) == cudaSuccess;
+  for (const void* k : {(const void*)k_fac_product<PROD_FWD, 1, false, false>, (const void*)k_fac_product<PROD_DGRAD_STEP, 1, false, false>})
+    ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)(kSmSharedBytes - kBlockReservedBytes - sizeof(GemmShared))) == cudaSuccess;
+  for (const void* k : {(const void*)rebuild::k_rebuild<false, false>, (const void*)rebuild::k_rebuild<false, true>,
+                        (const void*)rebuild::k_rebuild<true, false>, (const void*)rebuild::k_rebuild<true, true>})
+    ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    (int)(kSmSharedBytes - kBlockReservedBytes - sizeof(rebuild::Shared))) == cudaSuccess;
   if (ok) {
     st->reb = f;
   } else {
@@ -1696,11 +1762,14 @@ void reb_setup(mavg_ctx* c, TcState* st) {
 bool reb_usable(const mavg_ctx* c) {
   const TcState* st = (const TcState*)c->mlp;
   // by the momentum and K of now, which may not be those the handle was made with
-  return st && st->reb && c->schedule == 0 && c->cfg.K <= st->reb->K && reb_steps(&c->cfg) == c->cfg.K;
+  return st && st->reb && c->schedule == 0 && c->cfg.K <= st->reb->K && reb_steps(&c->cfg) == c->cfg.K &&
+         (c->cfg.K <= 4 || !st->fuse_upto);
 }
 
 // The K steps of a round: F_1 -> ... -> F_{L-1} -> last layer and loss -> D_L -> ... -> D_2 -> weights of the next step's
-// products (of the call's end: the learners' own, and u).
+// products (of the call's end: the learners' own, and u).  Every sum is formed in the plain form's order, so that the two
+// give the same bits: another order moves operands across a bf16 rounding boundary, and after a few steps v is 1e-3 to
+// 1e-2 off and single rows of u more than their size.
 cudaError_t reb_local_steps(mavg_ctx* c, int64_t round) {
   TcState* st = (TcState*)c->mlp;
   FacState* f = st->reb;
@@ -1714,36 +1783,60 @@ cudaError_t reb_local_steps(mavg_ctx* c, int64_t round) {
     MomArgs mom = first;
     if (k > 1 && mom.u) mom.read_u = 1;
     auto slab = [&](size_t at, int d) { return (__nv_bfloat16*)ws_ptr(c, at) + (size_t)(k - 1) * P * B * up((size_t)d, 8); };
-    auto product = [&](int M, int contraction, int bias_layer, const FacCols& cols) {
+    StepOperands o{};
+    o.step = k;
+    o.shared_w = k == 1;
+    o.mom = mom;
+    const CUtensorMap* in = &f->step_in[(size_t)(k - 1) * (MAVG_MAX_LAYERS + 1)];
+    const CUtensorMap* dz = &f->step_dz[(size_t)(k - 1) * (MAVG_MAX_LAYERS + 1)];
+    auto operands = [&](int l, const CUtensorMap* w, const CUtensorMap* x, size_t out, int out_layer, size_t out_t) {
+      o.l = l;
+      o.w = w;
+      o.in = x;
+      o.out_bm = slab(out, cfg.dims[out_layer]);
+      o.out_mb = (__nv_bfloat16*)ws_ptr(c, out_t);
+    };
+    auto own = [&](const FacCols& cols, int contraction, int bias_layer) {
       ProdArgs g{};
-      g.M = M;
+      g.M = cfg.dims[bias_layer];
       g.kb = B;
       g.nl = cols.nl;
       g.cols = cols.cols;
       g.c_tiles = cols.c_tiles;
       g.nkb = (contraction + kBK - 1) / kBK;
       g.w_batched = k > 1;
-      g.in_off = (k - 1) * P;
       g.bias_off = c->layers[bias_layer - 1].b_off;
       g.bias_in = k == 1 ? c->buf.global_w : c->buf.replicas;
       g.bias_in_stride = k == 1 ? 0 : c->buf.replica_stride;
       g.mom = mom;
+      g.out = o.out_bm;
       return g;
     };
     for (int l = 1; l < L; ++l) {
-      ProdArgs g = product(cfg.dims[l], cfg.dims[l - 1], l, k == 1 ? f->fwd1[l] : f->fwd[l]);
-      g.out = slab(t.h[l], cfg.dims[l]);
-      const CUtensorMap &w = k == 1 ? st->wg[l] : f->w_own[l], &in = k == 1 ? f->in1[l] : f->in[l];
-      FAC_TRY((launch_product<PROD_FWD, 1>(c, MAVG_K_FWD, w, w, in, f->g_mn[l], in, g)));
+      operands(l, k == 1 ? &st->wg[l] : &f->w_own[l], in + l, t.h[l], l, t.act_t[l]);
+      if (f->own_fwd[k == 1][l])
+        FAC_TRY((launch_product<PROD_FWD, 1>(c, MAVG_K_FWD, *o.w, *o.w, *o.in, f->g_mn[l], *o.in,
+                                             own(k == 1 ? f->fwd1[l] : f->fwd[l], cfg.dims[l - 1], l))));
+      else
+        FAC_TRY(st->run_forward(c, o));
     }
-    FAC_TRY(st->last_layer(c, k == 1 ? st->wg[L] : f->w_own[L], k == 1, f->last_in[k - 1],
-                          (const int32_t*)ws_ptr(c, t.labels) + (size_t)(k - 1) * P * B, k, slab(t.g[L], cfg.dims[L]), mom));
-    for (int l = L; l > 1; --l) {
-      ProdArgs g = product(cfg.dims[l - 1], cfg.dims[l], l - 1, k == 1 ? f->dgrad1[l] : f->dgrad[l]);
-      g.out = slab(t.g[l - 1], cfg.dims[l - 1]);
-      g.act = slab(t.h[l - 1], cfg.dims[l - 1]);
-      const CUtensorMap &w = k == 1 ? st->wg_mn[l] : f->w_own_mn[l], &dz = k == 1 ? f->dz_in1[l] : f->dz_in[l];
-      FAC_TRY((launch_product<PROD_DGRAD, 1>(c, MAVG_K_DGRAD, w, w, dz, f->h_mn[l - 1], dz, g)));
+    operands(L, k == 1 ? &st->wg[L] : &f->w_own[L], in + L, t.g[L - 1], L - 1, t.dz_t);
+    o.labels = (const int32_t*)ws_ptr(c, t.labels) + (size_t)(k - 1) * P * B;
+    o.dz_bm = slab(t.g[L], cfg.dims[L]);
+    o.a_bm = slab(t.h[L - 1], cfg.dims[L - 1]);
+    o.w16 = k == 1 ? (const __nv_bfloat16*)ws_ptr(c, st->lay.w16g) + st->lay.sh_off[L - 1] : (const __nv_bfloat16*)ws_ptr(c, t.w_own[L]);
+    o.w16_stride = k == 1 ? 0 : (int64_t)cfg.dims[L - 1] * cfg.dims[L];
+    FAC_TRY(st->run_last_layer(c, o));
+    for (int l = st->tail_ok ? L - 1 : L; l > 1; --l) {
+      operands(l, k == 1 ? &st->wg_mn[l] : &f->w_own_mn[l], dz + l, t.g[l - 1], l - 1, t.dz_t);
+      o.mask_mb = (const __nv_bfloat16*)ws_ptr(c, t.act_t[l - 1]);
+      if (f->own_dgrad[l]) {
+        ProdArgs g = own(k == 1 ? f->dgrad1[l] : f->dgrad[l], cfg.dims[l], l - 1);
+        g.act = slab(t.h[l - 1], cfg.dims[l - 1]);
+        FAC_TRY((launch_product<PROD_DGRAD_STEP, 1>(c, MAVG_K_DGRAD, *o.w, *o.w, *o.in, f->h_mn[l - 1], *o.in, g)));
+      } else {
+        FAC_TRY(st->run_dgrad(c, o));
+      }
     }
     rebuild::Args g{};
     g.n_layers = L;

@@ -33,6 +33,7 @@ struct FacLayout {
   // rebuilt steps: the learners' weights, l = 1..L: bf16 [P, d_l, d_{l-1}].  The rows above are [steps, P, B, d_l] there,
   // dZ_L's among them (padded to 8 classes)
   size_t w_own[MAVG_MAX_LAYERS + 1] = {};
+  size_t act_t[MAVG_MAX_LAYERS] = {}, dz_t = 0;   // A_l, l = 1..L-1, of the step at hand, and a dZ_l: bf16 [P, d_l, B]
   size_t end = 0;
 };
 
@@ -51,12 +52,13 @@ struct FacState {
   FacCols fwd[MAVG_MAX_LAYERS + 1], dgrad[MAVG_MAX_LAYERS + 1], gram;
   CUtensorMap in[MAVG_MAX_LAYERS + 1], dz_in[MAVG_MAX_LAYERS + 1];
   CUtensorMap s_f[MAVG_MAX_LAYERS + 1], s_d[MAVG_MAX_LAYERS + 1];
-  // Rebuilt steps: the first step's cuts and batch operands (products with w~), and the learners' weights (boxes of
-  // 64 x 128, 64 x 64, and to store 32 x 128)
+  // Rebuilt steps: the learners' weights (boxes of 64 x 128, 64 x 64, and to store 32 x 128) and each step's batch operands:
+  // A_{l-1} and dZ_l of step k at [(k - 1) (MAVG_MAX_LAYERS + 1) + l].  fwd1, dgrad1: cuts of the first step's products, with
+  // w~; own_fwd (of the first step at [1]), own_dgrad: the products are k_fac_product's, not the plain form's launches
   FacCols fwd1[MAVG_MAX_LAYERS + 1], dgrad1[MAVG_MAX_LAYERS + 1];
-  CUtensorMap in1[MAVG_MAX_LAYERS + 1], dz_in1[MAVG_MAX_LAYERS + 1];
+  bool own_fwd[2][MAVG_MAX_LAYERS + 1] = {}, own_dgrad[MAVG_MAX_LAYERS + 1] = {};
   CUtensorMap w_own[MAVG_MAX_LAYERS + 1], w_own_mn[MAVG_MAX_LAYERS + 1], w_own_st[MAVG_MAX_LAYERS + 1];
-  std::vector<CUtensorMap> last_in;
+  std::vector<CUtensorMap> step_in, step_dz;
   CUtensorMap w_lo[MAVG_MAX_LAYERS];         // low parts of w~'s hidden layers, box 64 x 128
   // Row arrays [P, kb, d_l]: A_l (h) and dZ_l (g) with boxes of 64 x 64 rows (_mn: features are the MMA's
   // row dimension, rows the contraction), 64 x 128 (_k) and 64 x gram.cols (_b; A_0: 64 x row_tile).

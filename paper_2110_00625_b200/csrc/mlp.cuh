@@ -60,7 +60,9 @@ struct TailLaunch {
   const int32_t* labels;
   float* loss_out;
   int loss_stride;
-  __nv_bfloat16* dz_t;           // out: dZ_L^T [P, C, B]
+  __nv_bfloat16* dz_t;           // out: dZ_L^T [P, C, B], and where given dZ_L [P, B, cpad]
+  __nv_bfloat16* dz_bm;
+  int cpad;
   __nv_bfloat16* dzp_bm;         // out: dZ_{L-1} [P, B, in] and its transpose [P, in, B]
   __nv_bfloat16* dzp_mb;
   float* part;                   // scratch of tail_fused_part_bytes()

@@ -407,31 +407,121 @@ bool tc_shapes_ok(const mavg_config* cfg, std::string* why) {
   return true;
 }
 
+namespace {
+
+// Small problems (a few dozen weight tiles per SM in the largest layer): one persistent launch
+// takes the weight gradients of all layers, instead of one launch per layer on a side stream.
+bool wgrad_merges(const mavg_config* cfg, int sm_count, const WgradPlan* w) {
+  if (cfg->n_layers < 2 || (long)cfg->P * w[1].m_tiles * w[1].n_tiles > 64L * sm_count) return false;
+  for (int l = 2; l <= cfg->n_layers; ++l)
+    if (w[l].slots != w[1].slots || w[l].a_bufs != w[1].a_bufs) return false;
+  return true;
+}
+
+// Plans of the weight-gradient launches that can take the next step's forward product along, of layers 1..n: n.
+int riding_plans(const mavg_config* cfg, const TcLayout& t, int sm_count, bool momentum, bool streaming, WgradPlan* f) {
+  if (cfg->B > 128) return 0;
+  for (int l = 1; l < cfg->n_layers; ++l) {
+    f[l] = plan_wgrad_stream(cfg->dims[l], cfg->dims[l - 1], cfg->B, cfg->P, sm_count, momentum, streaming, true, t.lo_stride[l] > 0);
+    const size_t need = (size_t)cfg->P * f[l].m_tiles * f[l].n_chunks * cfg->B * kBM * sizeof(float);
+    if (f[l].slots < 2 || need > t.zpart_bytes || (size_t)cfg->P * f[l].m_tiles * sizeof(int) > t.zcount_bytes) return l - 1;
+  }
+  return cfg->n_layers - 1;
+}
+
+// Whether every sum of those products runs over a whole row, in the order of a product of its own.
+bool whole_sums(int P, int riding, const WgradPlan* f) {
+  for (int l = 1; l <= riding; ++l)
+    if (f[l].n_chunks > 1 && f[l].whole_rows < P * f[l].m_tiles) return false;
+  return true;
+}
+
+// Whether a handle's rounds may be rebuilt, from the configuration alone (their masters are beyond the L2).
+bool may_rebuild(const mavg_config* cfg, const TcLayout& t) {
+  WgradPlan w[MAVG_MAX_LAYERS + 1], f[MAVG_MAX_LAYERS + 1];
+  const bool momentum = cfg->learner_momentum != 0.f;
+  for (int l = 1; l <= cfg->n_layers; ++l)
+    w[l] = plan_wgrad_stream(cfg->dims[l], cfg->dims[l - 1], cfg->B, cfg->P, kPlanSmCount, momentum, true);
+  if (wgrad_merges(cfg, kPlanSmCount, w)) return true;
+  const int riding = riding_plans(cfg, t, kPlanSmCount, momentum, true, f);
+  return whole_sums(cfg->P, riding, f) && (cfg->K <= 4 || !riding);
+}
+
+}  // namespace
+
 size_t tc_workspace_bytes(const mavg_config* cfg, size_t base, size_t* act_off, size_t* least) {
   *act_off = base;
   const TcLayout t = make_layout(cfg, base, kPlanSmCount);
   *least = t.end;
   if (fac_reserved(cfg)) return std::max(t.end, fac_layout(cfg, t.shared_end).end);
-  return reb_reserved(cfg) ? std::max(t.end, reb_layout(cfg, t.shared_end).end) : t.end;
+  return reb_reserved(cfg) && may_rebuild(cfg, t) ? std::max(t.end, reb_layout(cfg, t.shared_end).end) : t.end;
 }
 
-static cudaError_t last_layer(mavg_ctx* c, const CUtensorMap& w, bool shared_w, const CUtensorMap& a, const int32_t* labels, int step,
-                          __nv_bfloat16* dz, const MomArgs& mom) {
+namespace {
+
+TcArgs product_args(mavg_ctx* c, const StepOperands& o, int features, int bias_layer) {
+  const TcLayout& t = ((const TcState*)c->mlp)->lay;
+  TcArgs g{};
+  g.M = features; g.N = c->cfg.B;
+  g.a_batched = o.shared_w ? 0 : 1; g.b_batched = 1;
+  g.part = (float*)ws_ptr(c, t.part); g.counters = (int*)ws_ptr(c, t.counters);
+  g.bias_rep = c->buf.replicas; g.bias_off = c->layers[bias_layer - 1].b_off;
+  g.bias_in = o.shared_w ? c->buf.global_w : c->buf.replicas;
+  g.bias_in_stride = o.shared_w ? 0 : c->buf.replica_stride;
+  g.out_bm = o.out_bm; g.out_mb = o.out_mb;
+  g.mom = o.mom;
+  return g;
+}
+
+cudaError_t forward(mavg_ctx* c, const StepOperands& o) {
+  const TcState* st = (const TcState*)c->mlp;
+  const MlpLayer& ly = c->layers[o.l - 1];
+  const FwdForm form = c->schedule == 0 ? fwd_form(st, o.l, o.shared_w) : FwdForm::TILES;
+  if (form == FwdForm::DENSE)
+    return launch_fwd_dense(c, st->dense[o.l], *o.w, *o.in, ly.out, c->buf.global_w + ly.b_off, o.out_bm, o.out_mb);
+  const TcArgs g = product_args(c, o, ly.out, o.l);
+  return form == FwdForm::SPLIT ? launch_gemm_ks(c, *o.w, *o.in, st->fwd_ks[o.l], g)
+                                : launch_gemm<EPI_FWD_HIDDEN>(c, MAVG_K_FWD, *o.w, *o.in, st->fwd[o.l], g);
+}
+
+TailLaunch tail_launch(mavg_ctx* c, const StepOperands& o) {
+  const TcLayout& t = ((const TcState*)c->mlp)->lay;
+  TailLaunch tl{};
+  tl.a_bm = o.a_bm;
+  tl.w16 = o.w16; tl.w16_stride = o.w16_stride;
+  tl.shared_w = o.shared_w;
+  tl.labels = o.labels;
+  tl.loss_out = (float*)ws_ptr(c, c->ws.losses) + (o.step - 1); tl.loss_stride = c->cfg.K;
+  tl.dz_t = (__nv_bfloat16*)ws_ptr(c, t.dz_t[o.l]);
+  tl.dz_bm = o.dz_bm; tl.cpad = t.cpad;
+  tl.dzp_bm = o.out_bm; tl.dzp_mb = o.out_mb;
+  tl.part = (float*)ws_ptr(c, t.tail_part);
+  tl.mom = o.mom;
+  return tl;
+}
+
+cudaError_t last_layer(mavg_ctx* c, const StepOperands& o) {
   const TcState* st = (const TcState*)c->mlp;
   const TcLayout& t = st->lay;
-  const int L = c->cfg.n_layers;
-  TcArgs g{};
-  g.M = c->cfg.dims[L]; g.N = c->cfg.B;
-  g.a_batched = shared_w ? 0 : 1; g.b_batched = 1;
-  g.part = (float*)ws_ptr(c, t.part); g.counters = (int*)ws_ptr(c, t.counters);
-  g.bias_rep = c->buf.replicas; g.bias_off = c->layers[L - 1].b_off;
-  g.bias_in = shared_w ? c->buf.global_w : c->buf.replicas;
-  g.bias_in_stride = shared_w ? 0 : c->buf.replica_stride;
-  g.labels = labels; g.loss_out = (float*)ws_ptr(c, c->ws.losses) + (step - 1); g.loss_stride = c->cfg.K;
-  g.dz_bm = dz; g.cpad = t.cpad; g.dz_mb = (__nv_bfloat16*)ws_ptr(c, t.dz_t[L]);
-  g.mom = mom;
-  return launch_gemm<EPI_FWD_LAST>(c, MAVG_K_FWD, w, a, st->fwd[L], g);
+  if (st->tail_ok && c->schedule == 0) {
+    const TailLaunch tl = tail_launch(c, o);
+    const cudaError_t e = launch_tail_fused(c, tl);
+    return e != cudaSuccess ? e : launch_tail_finish(c, tl);
+  }
+  TcArgs g = product_args(c, o, c->cfg.dims[o.l], o.l);
+  g.labels = o.labels; g.loss_out = (float*)ws_ptr(c, c->ws.losses) + (o.step - 1); g.loss_stride = c->cfg.K;
+  g.dz_bm = o.dz_bm; g.cpad = t.cpad; g.dz_mb = (__nv_bfloat16*)ws_ptr(c, t.dz_t[o.l]);
+  return launch_gemm<EPI_FWD_LAST>(c, MAVG_K_FWD, *o.w, *o.in, st->fwd[o.l], g);
 }
+
+cudaError_t dgrad(mavg_ctx* c, const StepOperands& o) {
+  TcArgs g = product_args(c, o, c->cfg.dims[o.l - 1], o.l - 1);
+  g.mask_mb = o.mask_mb;
+  g.a_mn = 1;
+  return launch_gemm<EPI_DGRAD>(c, MAVG_K_DGRAD, *o.w, *o.in, ((const TcState*)c->mlp)->dgrad[o.l], g);
+}
+
+}  // namespace
 
 mavg_status tc_setup(mavg_ctx* c) {
   const mavg_config& cfg = c->cfg;
@@ -536,41 +626,27 @@ mavg_status tc_setup(mavg_ctx* c) {
     if (e == cudaSuccess)
       e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem);
   if (e == cudaSuccess) e = wgrad_stream_prepare();
-  // Small problems (a few dozen weight tiles per SM in the largest layer): one persistent launch
-  // takes the weight gradients of all layers, instead of one launch per layer on a side stream.
-  {
-    const WgradPlan& w1 = st->wgrad[1];
-    st->wgrad_merged = L >= 2 && (long)P * w1.m_tiles * w1.n_tiles <= 64L * c->sm_count;
-    for (int l = 2; l <= L; ++l)
-      if (st->wgrad[l].slots != w1.slots || st->wgrad[l].a_bufs != w1.a_bufs) st->wgrad_merged = false;
-  }
+  st->wgrad_merged = wgrad_merges(&cfg, c->sm_count, st->wgrad);
   // Where the weight gradients are launches of their own, the launch of layer l can take the
   // next step's forward product of layer l along (layers 1..fuse_upto, a prefix of the hidden
   // layers): its plan gets room for the next step's input tile and long runs, and the input
   // buffers get a view with 32-column boxes.
   st->fuse_upto = 0;
-  if (!st->wgrad_merged && L >= 2 && B <= 128 && ok) {
-    for (int l = 1; l < L; ++l) {
-      const int in = cfg.dims[l - 1], out = cfg.dims[l];
-      const WgradPlan w = plan_wgrad_stream(out, in, B, P, c->sm_count, st->wgrad_mom,
-                                            !masters_fit_l2(c), true, t.lo_stride[l] > 0);
-      const size_t need = (size_t)P * w.m_tiles * w.n_chunks * B * kBM * sizeof(float);
-      if (w.slots < 2 || need > t.zpart_bytes || (size_t)P * w.m_tiles * sizeof(int) > t.zcount_bytes)
-        break;
-      bool enc = true;
-      for (int i = 0; i < 2 && enc; ++i) {
-        const size_t src = l == 1 ? t.xg[i] : (i == 0 ? t.act[l - 1] : t.act_b[l - 1]);
-        enc = encode_any(st, &st->a_next[l][i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, bf(src), in, B,
-                         P, in, (int64_t)B * in, kWgradTileCols, B, CU_TENSOR_MAP_SWIZZLE_64B, &why);
-      }
-      if (enc && t.lo_stride[l] > 0)
-        enc = encode_any(st, &st->lo16[l], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, bf(t.lo16[l]), in, out, P,
-                         in, t.lo_stride[l], kWgradTileCols, kWgradTileRows, CU_TENSOR_MAP_SWIZZLE_64B,
-                         &why);
-      if (!enc) break;
-      st->wgrad_f[l] = w;
-      st->fuse_upto = l;
+  const int riding = st->wgrad_merged ? 0 : riding_plans(&cfg, t, c->sm_count, st->wgrad_mom, !masters_fit_l2(c), st->wgrad_f);
+  for (int l = 1; l <= riding && ok; ++l) {
+    const int in = cfg.dims[l - 1], out = cfg.dims[l];
+    bool enc = true;
+    for (int i = 0; i < 2 && enc; ++i) {
+      const size_t src = l == 1 ? t.xg[i] : (i == 0 ? t.act[l - 1] : t.act_b[l - 1]);
+      enc = encode_any(st, &st->a_next[l][i], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, bf(src), in, B,
+                       P, in, (int64_t)B * in, kWgradTileCols, B, CU_TENSOR_MAP_SWIZZLE_64B, &why);
     }
+    if (enc && t.lo_stride[l] > 0)
+      enc = encode_any(st, &st->lo16[l], CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, bf(t.lo16[l]), in, out, P,
+                       in, t.lo_stride[l], kWgradTileCols, kWgradTileRows, CU_TENSOR_MAP_SWIZZLE_64B,
+                       &why);
+    if (!enc) break;
+    st->fuse_upto = l;
   }
   // First step of a round: the hidden layers' forward products as one dense product each, where
   // that gives enough tiles (the input buffers seen as one [P*B, in] array).
@@ -636,8 +712,10 @@ mavg_status tc_setup(mavg_ctx* c) {
   if (e == cudaSuccess && fac_steps(&cfg) &&
       c->buf.workspace_bytes >= std::max(t.end, fac_layout(&cfg, t.shared_end).end))
     fac_setup(c, st);
-  st->last_layer = last_layer;
-  if (e == cudaSuccess && reb_steps(&cfg) && c->buf.workspace_bytes >= std::max(t.end, reb_layout(&cfg, t.shared_end).end))
+  st->run_forward = forward;
+  st->run_last_layer = last_layer;
+  st->run_dgrad = dgrad;
+  if (e == cudaSuccess && reb_steps(&cfg) && whole_sums(P, st->fuse_upto, st->wgrad_f) && c->buf.workspace_bytes >= std::max(t.end, reb_layout(&cfg, t.shared_end).end))
     reb_setup(c, st);
   if (e == cudaSuccess)
     e = cudaMemsetAsync(ws + t.counters, 0, t.counters_bytes, c->stream);
@@ -769,14 +847,11 @@ cudaError_t tc_step(mavg_ctx* c, int64_t round, int step) {
   TcState* st = (TcState*)c->mlp;
   const TcLayout& t = st->lay;
   const mavg_config& cfg = c->cfg;
-  const int B = cfg.B, L = cfg.n_layers, K = cfg.K;
+  const int L = cfg.n_layers, K = cfg.K;
   char* ws = (char*)c->buf.workspace;
   auto bfp = [&](size_t off) { return (__nv_bfloat16*)(ws + off); };
   int32_t* idx = (int32_t*)ws_ptr(c, c->ws.idx);
   int32_t* labels = (int32_t*)ws_ptr(c, c->ws.labels);
-  float* losses = (float*)ws_ptr(c, c->ws.losses);
-  float* part = (float*)(ws + t.part);
-  int* counters = (int*)(ws + t.counters);
   const bool shared_w = c->replicas_equal_global;   // first step after a (re-)broadcast
   const MomArgs mom = mom_args(c, shared_w);
   const bool overlap = !c->profiling;
@@ -860,40 +935,28 @@ cudaError_t tc_step(mavg_ctx* c, int64_t round, int step) {
   }
 
   for (int l = 1; l <= L; ++l) {
-    const MlpLayer& ly = c->layers[l - 1];
-    TcArgs g{};
-    g.M = ly.out; g.N = B;
-    g.a_batched = shared_w ? 0 : 1; g.b_batched = 1;
-    g.part = part; g.counters = counters;
-    g.bias_rep = c->buf.replicas; g.bias_off = ly.b_off;
-    g.bias_in = shared_w ? c->buf.global_w : c->buf.replicas;
-    g.bias_in_stride = shared_w ? 0 : c->buf.replica_stride;
-    const CUtensorMap& wm = shared_w ? st->wg[l] : w_k(l);
-    const CUtensorMap& am = l == 1 ? st->x_in[xb] : act_in(l);
+    StepOperands o{};
+    o.l = l; o.step = step;
+    o.shared_w = shared_w;
+    o.w = shared_w ? &st->wg[l] : &w_k(l);
+    o.in = l == 1 ? &st->x_in[xb] : &act_in(l);
+    o.labels = labels_b;
+    o.mom = mom;
     if (l <= done) {
       // A_l of this step came out of the previous step's weight-gradient launch of this layer
-    } else if (l < L && shared_w && c->schedule == 0 && st->dense[l].ok) {
-      // every learner holds w~: one dense product over the batch rows of all learners
-      TC_TRY(launch_fwd_dense(c, st->dense[l], st->wg[l], st->in2d[l][l == 1 ? xb : ab], ly.out,
-                              c->buf.global_w + ly.b_off, act_of(l, ab), act_t_of(l, ab)));
     } else if (l < L) {
-      g.out_bm = act_of(l, ab); g.out_mb = act_t_of(l, ab);
-      if (c->schedule == 0 && st->fwd_ks[l].splits > 1)
-        TC_TRY(launch_gemm_ks(c, wm, l == 1 ? st->x_in_ks[xb] : act_in_ks(l), st->fwd_ks[l], g));
-      else
-        TC_TRY(launch_gemm<EPI_FWD_HIDDEN>(c, MAVG_K_FWD, wm, am, st->fwd[l], g));
+      const FwdForm form = c->schedule == 0 ? fwd_form(st, l, shared_w) : FwdForm::TILES;
+      if (form == FwdForm::DENSE) o.in = &st->in2d[l][l == 1 ? xb : ab];   // the batch rows of all learners
+      else if (form == FwdForm::SPLIT) o.in = l == 1 ? &st->x_in_ks[xb] : &act_in_ks(l);
+      o.out_bm = act_of(l, ab); o.out_mb = act_t_of(l, ab);
+      TC_TRY(forward(c, o));
     } else if (fused_tail) {
       // last layer forward, loss, dZ_L and dgrad_L in one CUDA-core kernel
-      TailLaunch tl{};
-      tl.a_bm = L >= 2 ? act_of(L - 1, ab) : bfp(t.xg[xb]);
-      tl.w16 = (shared_w ? bfp(t.w16g) : bfp(t.w16)) + t.sh_off[L - 1];
-      tl.w16_stride = shared_w ? 0 : t.n16;
-      tl.shared_w = shared_w;
-      tl.labels = labels_b; tl.loss_out = losses + (step - 1); tl.loss_stride = K;
-      tl.dz_t = bfp(t.dz_t[L]);
-      if (L >= 2) { tl.dzp_bm = bfp(t.dz[L - 1]); tl.dzp_mb = bfp(t.dz_t[L - 1]); }
-      tl.part = (float*)(ws + t.tail_part);
-      tl.mom = mom;
+      o.a_bm = L >= 2 ? act_of(L - 1, ab) : bfp(t.xg[xb]);
+      o.w16 = (shared_w ? bfp(t.w16g) : bfp(t.w16)) + t.sh_off[L - 1];
+      o.w16_stride = shared_w ? 0 : t.n16;
+      if (L >= 2) { o.out_bm = bfp(t.dz[L - 1]); o.out_mb = bfp(t.dz_t[L - 1]); }
+      const TailLaunch tl = tail_launch(c, o);
       TC_TRY(launch_tail_fused(c, tl));
       // bias steps and loss: beside the backward pass, joined at the end of the step
       if (overlap) {
@@ -916,10 +979,8 @@ cudaError_t tc_step(mavg_ctx* c, int64_t round, int step) {
         TC_TRY(launch_tail_finish(c, tl));
       }
     } else {
-      g.labels = labels_b; g.loss_out = losses + (step - 1); g.loss_stride = K;
-      g.dz_bm = bfp(t.dz[L]); g.cpad = t.cpad; g.dz_mb = bfp(t.dz_t[L]);
-      g.mom = mom;
-      TC_TRY(launch_gemm<EPI_FWD_LAST>(c, MAVG_K_FWD, wm, am, st->fwd[l], g));
+      o.dz_bm = bfp(t.dz[L]);
+      TC_TRY(last_layer(c, o));
     }
   }
   // the labels of this step have been consumed: the next step's gather may run now
@@ -938,20 +999,15 @@ cudaError_t tc_step(mavg_ctx* c, int64_t round, int step) {
   for (int l = L; l >= 1; --l) {
     const MlpLayer& ly = c->layers[l - 1];
     if (l > 1 && !(fused_tail && l == L)) {
-      const MlpLayer& below = c->layers[l - 2];
-      TcArgs g{};
-      g.M = ly.in; g.N = B;
-      g.a_batched = shared_w ? 0 : 1; g.b_batched = 1;
-      g.part = part; g.counters = counters;
-      g.bias_rep = c->buf.replicas; g.bias_off = below.b_off;
-      g.bias_in = shared_w ? c->buf.global_w : c->buf.replicas;
-      g.bias_in_stride = shared_w ? 0 : c->buf.replica_stride;
-      g.out_bm = bfp(t.dz[l - 1]); g.out_mb = bfp(t.dz_t[l - 1]);
-      g.mask_mb = act_t_of(l - 1, ab);
-      g.a_mn = 1;
-      g.mom = mom;
-      TC_TRY(launch_gemm<EPI_DGRAD>(c, MAVG_K_DGRAD, shared_w ? st->wg_mn[l] : w_mn(l),
-                                    st->dz[l], st->dgrad[l], g));
+      StepOperands o{};
+      o.l = l; o.step = step;
+      o.shared_w = shared_w;
+      o.w = shared_w ? &st->wg_mn[l] : &w_mn(l);
+      o.in = &st->dz[l];
+      o.out_bm = bfp(t.dz[l - 1]); o.out_mb = bfp(t.dz_t[l - 1]);
+      o.mask_mb = act_t_of(l - 1, ab);
+      o.mom = mom;
+      TC_TRY(dgrad(c, o));
     }
     const CUtensorMap& bm = l == 1 ? st->x_in_t[xb] : act_in_t(l);
     if (merged) continue;        // all layers' weight gradients follow in one launch

@@ -1,9 +1,9 @@
 // Rebuilt local steps: a learner's hidden weights after k steps, formed anew from w~, the momentum buffer the call found
 // and the rows of the k steps' factors, instead of being read, stepped and written back every step.  With w~ the same for
 // all learners and the rows a few MB, a step moves 2 bytes per weight (the bf16 copy that the next step's products read)
-// and 4 more with learner momentum (u as it was before the call), where stepping in place moves 10 and 18.  The learners'
-// own weights are rounded to bf16 at every step as in the plain form; with momentum the steps are taken one after the
-// other in fp32 in its very order.
+// and 4 more with learner momentum (u as it was before the call), where stepping in place moves 10 and 18.  The steps are
+// taken one after the other in fp32, each from its own gradient's sum, and the weights are rounded to bf16 at every step: the
+// plain form's numbers, to the bit.
 //
 // 3072-2048-2048-2048-10, P = 8, B = 64, momentum (14.7 M weights a learner), step 1 .. 4 of 4: 145, 164, 194 us against 116 us
 // for the 0.76 GB of steps 1 .. 3 at the copy rate, and 386 against 222 (1.47 GB: W and u go out); the round takes 1447 us,
@@ -13,6 +13,8 @@
 // 8 columns at once spilled (166, 184, 236 and 437 us), two at once do not.  Measured and worse: more groups, or eight
 // warps a group; storing from registers (296 .. 560 us: half-empty sectors); deeper rings with two operand stages; in the
 // last step pieces of 16 columns, two in turn (400); the copies in and out by warps of their own (137, 151, 238 and 423).
+// Without momentum an accumulator is read and given back at a time (two at a time: 1.04 times as long over 25 shapes).  All
+// steps' gradients in one accumulator took 0.76 to 1 of the time but rounded the weights once, and not at every step.
 #pragma once
 #include <cuda.h>
 
@@ -39,7 +41,9 @@ constexpr int out_bytes(bool last) { return last ? kPieceBytes : kPieceBytes / 2
 constexpr int group_bytes(bool last) { return ring_of(last) * kPieceBytes + out_bytes(last); }
 constexpr size_t smem_of(bool last) { return (size_t)stages_of(last) * kStageBytes + kGroups * group_bytes(last) + 1024; }
 static_assert(smem_of(false) <= 226 * 1024 && smem_of(true) <= 226 * 1024, "");
-constexpr int kMaxMomSteps = 512 / kBN;           // with momentum every step's gradient has an accumulator of its own
+constexpr int kAccs = 512 / kBN;                  // every step's gradient has an accumulator of its own
+constexpr int kMaxMomSteps = kAccs;               // with momentum all of a learner's are taken together
+static_assert(kMaxMomSteps == 4, "reb_steps");
 enum { ERR_REB_PRODUCER = 51, ERR_REB_MMA = 52, ERR_REB_EPILOGUE = 53 };
 
 struct Layer { int m_tiles, n_tiles, in, first; };   // first: tiles of the layers before
@@ -111,9 +115,9 @@ k_rebuild(const __grid_constant__ Args g) {
   grid_dependency_wait();
   volatile int* abortp = &sh.abort_flag;
   const int nkb = (g.B + kBK - 1) / kBK;          // slabs of a step
-  // Tensor memory as a ring of four accumulators: with momentum a learner takes one per step, else one (a learner's at
-  // a time, twice where they fit twice: 146, 158, 225 and 370 us, the round 1463)
-  const int accs = MOM ? g.steps : 1;
+  // Tensor memory as a ring of four accumulators, of which a learner takes one per step (a learner's at a time, twice
+  // where they fit twice: 146, 158, 225 and 370 us, the round 1463)
+  const int accs = g.steps;
   const int groups = (g.P + g.group - 1) / g.group, units = groups * g.tiles;
   // units of the same learners follow one another: their rows stay in the L2
   auto decode = [&](int unit, int& p0, int& p1, int& l, int& m0, int& n0) {
@@ -163,7 +167,7 @@ k_rebuild(const __grid_constant__ Args g) {
         for (int p = p0; p < p1 && ok; ++p)
           for (int i = 0; i < g.steps * nkb; ++i, ++it) {
             const int s = it % kStages, kb = i % nkb, b = n & 3;
-            const bool first = MOM ? kb == 0 : i == 0, last = MOM ? kb == nkb - 1 : i == g.steps * nkb - 1;
+            const bool first = kb == 0, last = kb == nkb - 1;
             if (first && !(ok = mbar_wait(&sh.acc_empty[b], ((n >> 2) & 1) ^ 1, abortp, g.status, ERR_REB_MMA))) break;
             if (!(ok = mbar_wait(&sh.full[s], (it / kStages) & 1, abortp, g.status, ERR_REB_MMA))) break;
             tc_fence_after_sync();
@@ -187,12 +191,13 @@ k_rebuild(const __grid_constant__ Args g) {
     // ones.  One barrier a piece: behind it the piece has been read and what is to be stored is in shared memory; before
     // the next is written, the first thread has seen the store leave it (it carries that to the barrier before the write).
     // The barriers carry a wait that was given up, so that the group leaves together.
-    constexpr int kRing = ring_of(LAST);
+    constexpr int kRing = MOM ? ring_of(LAST) : 1;   // (without momentum w~'s pieces alone come in)
     const int grp = (warp - 2) >> 2, q4 = warp & 3, row = q4 * 32 + lane;
     const bool leader = ((warp - 2) & 3) == 0 && lane == 0, load_u = MOM && g.load_u;
     const bool u_apart = MOM && LAST && !load_u;   // u does not come in, but leaves from the buffer for it
     uint8_t* in_buf = smem + kStages * kStageBytes + (size_t)grp * group_bytes(LAST);
-    uint8_t* ob = in_buf + kRing * kPieceBytes;
+    uint8_t* ob = in_buf + ring_of(LAST) * kPieceBytes;
+    uint8_t* between = LAST ? ob : in_buf + kPieceBytes;   // not MOM: weights after four steps, each thread's own
     // the leader's place in the group's list of pieces: of w~ (fp == -1), then of each learner's u
     // (in shared memory: it is seldom looked at, and registers are short)
     auto fetch = [&]() {
@@ -227,6 +232,19 @@ k_rebuild(const __grid_constant__ Args g) {
       if (!mbar_wait(&sh.piece_full[grp][pn % kRing], (pn / kRing) & 1, abortp, g.status, ERR_REB_EPILOGUE)) failed = true;
       return in_buf + (size_t)(pn % kRing) * kPieceBytes;
     };
+    auto put_fp32 = [&](uint8_t* buf, int h, const float (&x)[8]) {
+#pragma unroll
+      for (int c = 0; c < 2; ++c) *cell(buf, 2 * h + c) = make_float4(x[4 * c], x[4 * c + 1], x[4 * c + 2], x[4 * c + 3]);
+    };
+    auto put_bf16 = [&](int h, const float (&x)[8]) {   // rows of 64 bytes, 64-byte swizzle
+      uint32_t hw[4];
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const __nv_bfloat162 t = __floats2bfloat162_rn(x[2 * j], x[2 * j + 1]);
+        hw[j] = *reinterpret_cast<const uint32_t*>(&t);
+      }
+      *reinterpret_cast<uint4*>(ob + (size_t)row * 64 + ((h ^ ((row >> 1) & 3)) << 4)) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
+    };
     for (int unit = blockIdx.x; unit < units && !gone; unit += gridDim.x) {
       int p0, p1, l, m0, n0;
       decode(unit, p0, p1, l, m0, n0);
@@ -246,32 +264,32 @@ k_rebuild(const __grid_constant__ Args g) {
         if (leader && !u_apart) fetch();
       }
       for (int p = p0; p < p1; ++p, n += accs) {
-        for (int i = n; i < n + accs; ++i)
-          if (!mbar_wait(&sh.acc_full[i & 3], (i >> 2) & 1, abortp, g.status, ERR_REB_EPILOGUE)) failed = true;
-        __syncwarp();
-        tc_fence_after_sync();
         const uint32_t acc = tmem_base + ((uint32_t)(q4 * 32) << 16) + (uint32_t)c0;
         uint8_t* ub = in_buf;
-        if (mine && load_u) ub = wait_piece();
-        if (mine) {
+        if (MOM) {                                 // all of the learner's accumulators together
+          for (int i = n; i < n + accs; ++i)
+            if (!mbar_wait(&sh.acc_full[i & 3], (i >> 2) & 1, abortp, g.status, ERR_REB_EPILOGUE)) failed = true;
+          __syncwarp();
+          tc_fence_after_sync();
+          if (mine && load_u) ub = wait_piece();
+          if (mine) {
 #pragma unroll
-          for (int h = 0; h < kPiece / 8; ++h) {   // 8 columns
-            float x[8], v[8];
+            for (int h = 0; h < kPiece / 8; ++h) {   // 8 columns
+              float x[8], v[8];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-              x[j] = w[8 * h + j];
-              v[j] = 0.f;
-            }
-            if (load_u) {
-#pragma unroll
-              for (int c = 0; c < 2; ++c) {
-                const float4 t = *cell(ub, 2 * h + c);
-                v[4 * c] = t.x; v[4 * c + 1] = t.y; v[4 * c + 2] = t.z; v[4 * c + 3] = t.w;
+              for (int j = 0; j < 8; ++j) {
+                x[j] = w[8 * h + j];
+                v[j] = 0.f;
               }
-            }
-            if (MOM) {                             // two steps at a time: more accumulators in flight do not fit the registers
+              if (load_u) {
 #pragma unroll
-              for (int i = 0; i < kMaxMomSteps; i += 2) {
+                for (int c = 0; c < 2; ++c) {
+                  const float4 t = *cell(ub, 2 * h + c);
+                  v[4 * c] = t.x; v[4 * c + 1] = t.y; v[4 * c + 2] = t.z; v[4 * c + 3] = t.w;
+                }
+              }
+#pragma unroll
+              for (int i = 0; i < kMaxMomSteps; i += 2) {   // two steps at a time: more accumulators in flight do not fit the registers
                 if (i >= g.steps) break;
                 uint32_t r[2][8];
                 tmem_ld_8cols(acc + (uint32_t)(((n + i) & 3) * kBN + 8 * h), r[0]);
@@ -283,34 +301,60 @@ k_rebuild(const __grid_constant__ Args g) {
 #pragma unroll
                   for (int j = 0; j < 8; ++j) msgd(x[j], v[j], __uint_as_float(r[1][j]), g.gamma, g.beta);
               }
-            } else {
-              uint32_t r[8];
-              tmem_ld_8cols(acc + (uint32_t)((n & 3) * kBN + 8 * h), r);
-              tmem_ld_wait();
+              if (LAST) {
 #pragma unroll
-              for (int j = 0; j < 8; ++j) x[j] = fmaf(-g.gamma, __uint_as_float(r[j]), x[j]);
-            }
-            if (LAST) {
-#pragma unroll
-              for (int c = 0; c < 2; ++c) {
-                *cell(ob, 2 * h + c) = make_float4(x[4 * c], x[4 * c + 1], x[4 * c + 2], x[4 * c + 3]);
-                if (MOM) *cell(ub, 2 * h + c) = make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
+                for (int c = 0; c < 2; ++c) {
+                  *cell(ob, 2 * h + c) = make_float4(x[4 * c], x[4 * c + 1], x[4 * c + 2], x[4 * c + 3]);
+                  *cell(ub, 2 * h + c) = make_float4(v[4 * c], v[4 * c + 1], v[4 * c + 2], v[4 * c + 3]);
+                }
+              } else {
+                put_bf16(h, x);
               }
-            } else {                               // rows of 64 bytes, 64-byte swizzle
-              uint32_t hw[4];
-#pragma unroll
-              for (int j = 0; j < 4; ++j) {
-                const __nv_bfloat162 t = __floats2bfloat162_rn(x[2 * j], x[2 * j + 1]);
-                hw[j] = *reinterpret_cast<const uint32_t*>(&t);
-              }
-              *reinterpret_cast<uint4*>(ob + (size_t)row * 64 + ((h ^ ((row >> 1) & 3)) << 4)) = make_uint4(hw[0], hw[1], hw[2], hw[3]);
             }
           }
+          tc_fence_before_sync();
+          __syncwarp();
+          if (lane == 0)
+            for (int i = n; i < n + accs; ++i) mbar_arrive(&sh.acc_empty[i & 3]);
+        } else {                                   // up to four at a time; between the fours the weights stay in shared memory
+          for (int done = 0; done < accs; done += kAccs) {
+            const int begin = n + done, end = n + min(done + kAccs, accs);
+            for (int i = begin; i < end; ++i)
+              if (!mbar_wait(&sh.acc_full[i & 3], (i >> 2) & 1, abortp, g.status, ERR_REB_EPILOGUE)) failed = true;
+            __syncwarp();
+            tc_fence_after_sync();
+            if (mine) {
+#pragma unroll
+              for (int h = 0; h < kPiece / 8; ++h) {
+                float x[8];
+#pragma unroll
+                for (int j = 0; j < 8; ++j) x[j] = w[8 * h + j];
+                if (done > 0) {
+#pragma unroll
+                  for (int c = 0; c < 2; ++c) {
+                    const float4 t = *cell(between, 2 * h + c);
+                    x[4 * c] = t.x; x[4 * c + 1] = t.y; x[4 * c + 2] = t.z; x[4 * c + 3] = t.w;
+                  }
+                }
+#pragma unroll 1
+                for (int i = begin; i < end; ++i) {
+                  uint32_t r[8];
+                  tmem_ld_8cols(acc + (uint32_t)((i & 3) * kBN + 8 * h), r);
+                  tmem_ld_wait();
+#pragma unroll
+                  for (int j = 0; j < 8; ++j) x[j] = fmaf(-g.gamma, __uint_as_float(r[j]), x[j]);
+                }
+                if (LAST) put_fp32(ob, h, x);
+                else if (end < n + accs) put_fp32(between, h, x);
+                else put_bf16(h, x);
+              }
+            }
+            tc_fence_before_sync();
+            __syncwarp();
+            if (lane == 0)
+              for (int i = begin; i < end; ++i) mbar_arrive(&sh.acc_empty[i & 3]);
+          }
         }
-        tc_fence_before_sync();
-        __syncwarp();
-        if (lane == 0)
-          for (int i = n; i < n + accs; ++i) mbar_arrive(&sh.acc_empty[i & 3]);
         if (!mine) continue;                       // (a wait given up here is carried by the next barrier)
         fence_proxy_async();
         if ((gone = barrier_any(failed, 2 + grp, 128))) break;

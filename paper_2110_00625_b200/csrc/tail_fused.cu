@@ -35,6 +35,8 @@ struct TailArgs {
   float* loss_out;               // loss_out[p * loss_stride]
   int loss_stride;
   __nv_bfloat16* dz_t;           // dZ_L transposed [P, C, B]
+  __nv_bfloat16* dz_bm;          // and as [P, B, cpad], or null
+  int cpad;
   __nv_bfloat16* dzp_bm;         // dZ_{L-1} [P, B, in]     (null for a one-layer model)
   __nv_bfloat16* dzp_mb;         // dZ_{L-1} transposed [P, in, B]
   float* part;                   // [P, blocks, in + C + 1] partial sums
@@ -150,6 +152,7 @@ k_last_layer_fused(const TailArgs g) {
       const float gr = (__expf(v - lse) - (l == yb ? 1.f : 0.f)) * (1.0f / (float)B);
       z[r][l] = gr;
       zq[l][r] = __bfloat162float(__float2bfloat16_rn(gr));
+      if (g.dz_bm) g.dz_bm[((size_t)p * B + r0 + r) * g.cpad + l] = __float2bfloat16_rn(gr);
     }
   }
   __syncthreads();
@@ -287,6 +290,8 @@ TailArgs tail_args(mavg_ctx* c, const TailLaunch& t) {
   g.loss_out = t.loss_out;
   g.loss_stride = t.loss_stride;
   g.dz_t = t.dz_t;
+  g.dz_bm = t.dz_bm;
+  g.cpad = t.cpad;
   g.dzp_bm = L >= 2 ? t.dzp_bm : nullptr;
   g.dzp_mb = L >= 2 ? t.dzp_mb : nullptr;
   g.part = t.part;

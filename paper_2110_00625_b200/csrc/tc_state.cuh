@@ -49,6 +49,25 @@ struct TcLayout {
 
 struct GemmPlan { int m_tiles, n_tiles, splits, kb_per_split, nkb, BN, stages, two_per_sm; uint32_t tmem_cols; };
 
+// Operands of one product of a step: layer l's forward product, or the data gradient through it.
+struct StepOperands {
+  int l, step;
+  bool shared_w;                              // the weights are w~, for all learners
+  const CUtensorMap *w, *in;                  // weights; batch operand, boxes of the launch's own height
+  __nv_bfloat16 *out_bm, *out_mb;             // A_l or dZ_{l-1}: [P, B, d] and [P, d, B]
+  const __nv_bfloat16* mask_mb;               // data gradient: A_{l-1} [P, d, B]
+  // last layer: labels, dZ_L [P, B, cpad]; where it is the fused kernel (out_* are dZ_{L-1} then) its rows and weights
+  const int32_t* labels;
+  __nv_bfloat16* dz_bm;
+  const __nv_bfloat16 *a_bm, *w16;
+  int64_t w16_stride;
+  MomArgs mom;
+};
+
+// How the forward product of a hidden layer is launched in schedule 0: for all learners at once, by clusters that split
+// the contraction, or tile by tile.
+enum class FwdForm { DENSE, SPLIT, TILES };
+
 struct TcState {
   TcLayout lay;
   EncodeTiledFn encode = nullptr;
@@ -109,10 +128,10 @@ struct TcState {
   WgradPlan wgrad[MAVG_MAX_LAYERS + 1];
   FacState* fac = nullptr;                    // factored steps (factored.cuh), null: not for this handle
   FacState* reb = nullptr;                    // rebuilt steps, likewise
-  // The plain form's launch for the last layer's product, loss, dZ_L (to dz, rows of whole groups of 8) and bias step, with
-  // the given operands.
-  cudaError_t (*last_layer)(mavg_ctx* c, const CUtensorMap& w, bool shared_w, const CUtensorMap& a, const int32_t* labels, int step,
-                            __nv_bfloat16* dz, const MomArgs& mom) = nullptr;
+  // The plain form's launches of a step's products, for rebuilt steps, which bring operands of their own (mlp_tc.cu)
+  cudaError_t (*run_forward)(mavg_ctx* c, const StepOperands& o) = nullptr;
+  cudaError_t (*run_last_layer)(mavg_ctx* c, const StepOperands& o) = nullptr;
+  cudaError_t (*run_dgrad)(mavg_ctx* c, const StepOperands& o) = nullptr;
   // side streams and events for the branches of a step that may overlap
   cudaStream_t s_wgrad = nullptr, s_gather = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_wgrad_done = nullptr, ev_gather_done = nullptr,
@@ -120,6 +139,9 @@ struct TcState {
               ev_x_free[2] = {nullptr, nullptr};
 };
 
+inline FwdForm fwd_form(const TcState* st, int l, bool shared_w) {
+  return shared_w && st->dense[l].ok ? FwdForm::DENSE : st->fwd_ks[l].splits > 1 ? FwdForm::SPLIT : FwdForm::TILES;
+}
 
 inline bool encode_any(TcState* st, CUtensorMap* m, CUtensorMapDataType dt, int esize, void* ptr,
                 int inner, int rows, int batch, int64_t row_stride, int64_t batch_stride,

@@ -1,30 +1,38 @@
-"""Rebuilt local steps (weights formed anew each step from w~, u and the steps' rows) against the plain form, which steps
-each learner's weights in place: one and several row and column tiles, ragged ones, batches of whole and part slabs, one
-accumulator buffer and two, u zero, reset and carried over."""
+"""Rebuilt local steps (weights formed anew each step from w~, u and the steps' rows) are the plain form's, which steps each
+learner's weights in place, to the bit: one and several row and column tiles, ragged ones, batches of whole and part slabs, u
+zero, reset and carried over, more steps than accumulators; first steps of all learners at once, products split over a
+cluster or over blocks, forward products that ride on the plain form's weight gradients, the fused last layer."""
 import pytest
 import torch
 
 pytestmark = pytest.mark.gpu
 
 
-def _pair(dims, P, K, B, beta, reset, defer, calls, seed=0):
+def _run(dims, P, K, B, beta, reset, defer, calls, rebuilt, how):
+    """The state after `calls`.  The plain form of the same settings: a handle made for one step (how == "steps"), without
+    the momentum that would make it one for rebuilt steps ("momentum"), or the plain tiles where these sum alike ("tiles")."""
     import paper_2110_00625_b200 as m
-    gen = torch.Generator(device="cuda").manual_seed(seed)
+    gen = torch.Generator(device="cuda").manual_seed(0)
     x = torch.randn(4000, dims[0], generator=gen, device="cuda")
     y = torch.randint(0, dims[-1], (4000,), generator=gen, device="cuda").int()
-    w1 = m.workloads.mlp_init(dims, seed=seed)
-    out = []
-    for schedule in (0, 2):
-        g = m.Mavg(w1, P=P, K=K, local_lr=0.002, mu=0.9, B=B, seed=3, objective=m.OBJ_MLP, dims=dims, gemm_bf16=1, x=x, y=y,
-                   x_bf16=True, defer_broadcast=defer, learner_momentum=beta, learner_momentum_reset=reset)
-        g.set_schedule(schedule)
-        assert g.rebuilt() == (schedule == 0)
-        calls(g)
-        g.sync()
-        out.append((g.v.clone(), g.w.clone(), g.replicas[:, :g.n].clone(),
-                    g.u[:, :g.n].clone() if beta else g.v.clone(), torch.from_numpy(g.get_losses().copy())))
-        g.close()
-    return [((a.double() - b.double()).norm() / b.double().norm()).item() for a, b in zip(*out)]
+    late_momentum, late_steps = not rebuilt and how == "momentum", not rebuilt and how == "steps"
+    g = m.Mavg(m.workloads.mlp_init(dims), P=P, K=1 if late_steps else K, local_lr=0.002, mu=0.9, B=B, seed=3,
+               objective=m.OBJ_MLP, dims=dims, gemm_bf16=1, x=x, y=y, x_bf16=True, defer_broadcast=defer,
+               learner_momentum=0.0 if late_momentum else beta, learner_momentum_reset=reset, with_learner_u=beta != 0)
+    if late_steps:
+        g.set_hparams(K, 0.002, 1.0, 0.9)
+    if late_momentum:
+        g.set_learner_momentum(beta, reset)
+    if not rebuilt and how == "tiles":
+        g.set_schedule(2)
+    assert g.rebuilt() == rebuilt and not g.factored()
+    calls(g)
+    g.sync()
+    out = [g.v.clone(), g.w.clone(), g.replicas[:, :g.n].clone(), torch.from_numpy(g.get_losses().copy())]
+    if beta:
+        out.append(g.u[:, :g.n].clone())
+    g.close()
+    return out
 
 
 def _rounds(g):
@@ -38,28 +46,27 @@ def _steps_from_own_weights(g):                   # the second call does not sta
     g.local_steps()
 
 
-@pytest.mark.parametrize("dims,P,K,B,beta,reset,defer,calls", [
-    ([520, 264, 136, 10], 118, 3, 16, 0.9, False, True, _rounds),
-    ([520, 264, 136, 10], 170, 2, 16, 0.9, True, False, _rounds),
-    ([520, 264, 136, 10], 167, 4, 80, 0.5, False, False, _rounds),
-    ([1000, 520, 32], 55, 2, 48, 0.9, False, True, _steps_from_own_weights),
-    ([784, 128, 3], 281, 2, 256, 0.9, False, False, _rounds),
-    ([2048, 2048, 2048, 10], 13, 2, 144, 0.9, False, False, _rounds),
-    ([3072, 2048, 2048, 2048, 10], 8, 4, 64, 0.9, False, True, _rounds),
+@pytest.mark.parametrize("dims,P,K,B,beta,reset,defer,calls,how", [
+    ([520, 264, 136, 10], 118, 3, 16, 0.9, False, True, _rounds, "momentum"),
+    ([520, 264, 136, 10], 170, 2, 16, 0.9, True, False, _rounds, "momentum"),
+    ([520, 264, 136, 10], 167, 4, 80, 0.5, False, False, _rounds, "momentum"),
+    ([1000, 520, 32], 55, 2, 48, 0.9, False, True, _steps_from_own_weights, "momentum"),
+    ([784, 128, 3], 281, 2, 256, 0.9, False, False, _rounds, "momentum"),
+    ([3072, 1024, 512, 10], 10, 4, 64, 0.9, False, True, _rounds, "momentum"),
+    ([2424, 776, 32], 18, 3, 48, 0.9, False, True, _rounds, "momentum"),
+    ([2048, 2048, 2048, 10], 13, 2, 144, 0.9, False, False, _rounds, "steps"),
+    ([3072, 2048, 2048, 2048, 10], 8, 4, 64, 0.9, False, True, _rounds, "steps"),
+    ([2056, 1000, 32], 24, 2, 160, 0.0, False, True, _rounds, "tiles"),
+    ([1120, 1304, 1304, 1304, 10], 10, 6, 16, 0.0, False, True, _rounds, "steps"),
+    ([1352, 1984, 1984, 1984, 10], 9, 6, 48, 0.0, False, False, _rounds, "steps"),
+    ([1416, 1800, 1800, 1800, 32], 7, 2, 48, 0.0, False, True, _steps_from_own_weights, "steps"),
+    ([3072, 2048, 2048, 2048, 10], 8, 3, 64, 0.0, False, True, _rounds, "steps"),
+    ([2488, 608, 608, 32], 27, 2, 48, 0.0, False, False, _rounds, "steps"),
 ])
-def test_with_momentum_the_steps_are_the_plain_ones(dims, P, K, B, beta, reset, defer, calls):
-    # The same fp32 steps in the same order, from sums whose terms are the same: the order of a sum's parts differs in a
-    # few places (1e-7 of a gradient), and where that moves a weight across a bf16 rounding boundary (1 in 2^15 of them, a
-    # 2^-9 of the weight) the next step's gradient moves by 2^-9 2^-7.5 = 1e-5 at most.
-    assert max(_pair(dims, P, K, B, beta, reset, defer, calls)) < 1e-5
-
-
-@pytest.mark.parametrize("dims,P,K,B", [([2056, 512, 264, 10], 41, 6, 32), ([2056, 1000, 32], 24, 2, 160),
-                                        ([3072, 1000, 520, 10], 14, 4, 128), ([3072, 2048, 2048, 2048, 10], 8, 3, 64)])
-def test_without_momentum_one_step_from_the_sum_of_the_gradients(dims, P, K, B):
-    # One fp32 rounding of the weights instead of K; v (the mean displacement) differs where a weight rounds to the other
-    # bf16 neighbour: the two forms' spread is that of any other order of sums, 2^-8 of v at these sizes, and twice that.
-    assert max(_pair(dims, P, K, B, 0.0, False, True, lambda g: g.round())) < 2 ** -7
+def test_the_steps_are_the_plain_ones(dims, P, K, B, beta, reset, defer, calls, how):
+    got, want = (_run(dims, P, K, B, beta, reset, defer, calls, rebuilt, how) for rebuilt in (True, False))
+    for a, b in zip(got, want):
+        assert torch.equal(a, b)
 
 
 def test_by_the_momentum_and_steps_of_now():
