@@ -9,9 +9,10 @@
 // layer 1's forward product, 22 here; 55 for the weight gradients, 24 to 32 here); 1000-333-100, P = 6, K = 4, B = 50 with
 // bf16 operands: 140 us, 170 with warp-level MMAs.  Relative error of one step's gradients against 64 bits (2-norm, weight
 // matrices of layers 1, 2, .. in units of 1e-7, FMA chains / here): 3072-512-512-10, B = 100 2.8 3.2 2.8 / 1.8 1.8 2.4;
-// inputs in [0, 1] 1.9 3.0 2.9 / 1.9 1.9 2.0; 2900-130-800-77, B = 31 2.8 3.8 3.4 / 2.1 2.4 2.1; 1501-799-99, B = 129
-// 2.6 2.6 / 1.9 2.3; 300-700-100-3, B = 160, [0, 1] 2.0 1.9 2.1 / 1.6 1.4 1.4.  With two slabs to an accumulator of a
-// forward product 2.8 3.0 3.4 where it is 1.9 1.9 2.0.
+// inputs in [0, 1] 1.9 2.8 2.8 / 1.9 1.8 1.9, B = 192 2.3 2.8 2.9 / 1.6 1.5 1.6, B = 256 2.4 2.9 2.8 / 1.9 1.8 1.9, B = 300
+// 2.6 3.0 3.0 / 1.7 1.6 1.6; 2900-130-800-77, B = 31 2.8 3.8 3.4 / 2.1 2.4 2.1; 1501-799-99, B = 129 2.5 2.8 / 1.9 2.0;
+// 301-131-66-5, B = 256, [0, 1] 2.2 2.2 2.4 / 1.7 1.5 1.5; 700-300-10, B = 512, [0, 1] 3.1 3.3 / 1.5 1.5.  With two slabs to
+// an accumulator of a forward product 2.8 3.0 3.4 where it is 1.9 1.9 2.0.
 // A step is L-1 forward launches, one for the whole last layer up to its data gradient (which
 // also gathers the next step's minibatch), L-2 data gradients and one for the weight gradients,
 // bias gradients and SGD steps of all layers.  While a deferred re-broadcast is outstanding the first
@@ -580,11 +581,12 @@ cudaError_t launch_product(mavg_ctx* c, int cls, const CUtensorMap& w, bool shar
 // split than the kernel before it has to wait until the SM is empty.
 template <bool QUANT>
 cudaError_t set_attributes() {
-  constexpr int NP = kPlanes<QUANT>;
+  constexpr int NP = kPlanes<QUANT>, kTwo = NP == 3 ? 2 : 1;
   const struct { const void* kernel; size_t smem; } kernels[] = {
       {(const void*)split::k_split_product<NP, false>, kSplitSmem}, {(const void*)split::k_split_product<NP, true>, kSplitSmem},
-      {(const void*)split::k_split_wgrad<NP, false, false>, kSplitSmem}, {(const void*)split::k_split_wgrad<NP, true, false>, kSplitSmem},
-      {(const void*)split::k_split_wgrad<NP, false, true>, kSplitSmem}, {(const void*)split::k_split_wgrad<NP, true, true>, kSplitSmem},
+      {(const void*)split::k_split_wgrad<NP, false, 1>, kSplitSmem}, {(const void*)split::k_split_wgrad<NP, true, 1>, kSplitSmem},
+      {(const void*)split::k_split_wgrad<NP, false, kTwo>, kSplitSmem}, {(const void*)split::k_split_wgrad<NP, true, kTwo>, kSplitSmem},
+      {(const void*)split::k_split_wgrad<NP, false, split::kManyChains>, kSplitSmem}, {(const void*)split::k_split_wgrad<NP, true, split::kManyChains>, kSplitSmem},
       {(const void*)k_simt_begin<QUANT>, 0}, {(const void*)k_simt_loss<QUANT>, 0}, {(const void*)k_simt_tail<QUANT>, kTailSmem}};
   for (const auto& k : kernels) {
     cudaError_t e = cudaFuncSetAttribute(k.kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
@@ -725,10 +727,12 @@ cudaError_t step_impl(mavg_ctx* c, int64_t round, int step) {
   w.stages = std::min(split::kMaxStages, (int)((kSplitSmem - 1024) / split::wgrad_stage_bytes(NP)));
   const size_t smem = std::max((size_t)w.stages * split::wgrad_stage_bytes(NP) + 1024,
                                split::tmem_share_bytes(NP == 3 ? 512 : 256, sizeof(split::Barriers)));
-  const bool many = B > split::kChainSlabs * split::kSlab;
-  auto kernel = many ? (mom.u ? split::k_split_wgrad<NP, true, true> : split::k_split_wgrad<NP, false, true>)
-                     : (mom.u ? split::k_split_wgrad<NP, true, false> : split::k_split_wgrad<NP, false, false>);
-  return launch(c, MAVG_K_WGRAD_SGD, kernel, dim3((unsigned)std::min(w.tiles, c->sm_count)), split::wgrad_threads(many), 1, smem, w);
+  constexpr int kTwo = NP == 3 ? 2 : 1;              // (one plane: never two)
+  const int chains = split::wgrad_chains(NP, B);
+  auto pick = [&](auto one, auto two, auto many) { return chains == 1 ? one : chains == 2 ? two : many; };
+  auto kernel = mom.u ? pick(split::k_split_wgrad<NP, true, 1>, split::k_split_wgrad<NP, true, kTwo>, split::k_split_wgrad<NP, true, split::kManyChains>)
+                      : pick(split::k_split_wgrad<NP, false, 1>, split::k_split_wgrad<NP, false, kTwo>, split::k_split_wgrad<NP, false, split::kManyChains>);
+  return launch(c, MAVG_K_WGRAD_SGD, kernel, dim3((unsigned)std::min(w.tiles, c->sm_count)), split::wgrad_threads(chains), 1, smem, w);
 }
 
 }  // namespace

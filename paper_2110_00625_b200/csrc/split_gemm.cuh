@@ -3,7 +3,7 @@
 // products of two such sums the six largest are formed, x0 y0 in one accumulator and the other five in another, and
 // what is left out is below 2^-25 of |x| |y|.  With bf16 operands (NP = 1) there is one plane and one accumulator.
 // The tensor cores cut a sum off where they add to it, always towards zero, so an accumulator takes one slab of 64
-// contraction elements (of a weight gradient four); the epilogue warps then add it to fp32 registers, rounded to
+// contraction elements (of a weight gradient two or four); the epilogue warps then add it to fp32 registers, rounded to
 // nearest, while the next goes into the other accumulator.  Against 64 bits: see mlp_simt.cu.
 //
 // Operands are kept as planes [NP][matrices, rows, pitch] (pitch: the width to a multiple of 8), which TMA reads in
@@ -26,9 +26,20 @@ constexpr int kMaxN = 128;                        // columns: four accumulators 
 constexpr int kMaxStages = 6;
 // Warp 0: TMA producer, 1: MMA issuer, then the epilogue; of a weight gradient two more for the biases and the loss.
 constexpr int kProductEpi = 8, kProductThreads = (2 + kProductEpi) * 32;
-constexpr int wgrad_epi(bool many) { return many ? 8 : 16; }
-constexpr int wgrad_threads(bool many) { return (4 + wgrad_epi(many)) * 32; }
-constexpr int kChainSlabs = 4;                    // of a weight gradient: slabs in one accumulator
+// Slabs of a weight gradient in one accumulator, and how many accumulators a sum takes: one, two that the epilogue adds where
+// it uses them, or kManyChains, added one after the other to registers.  fp32 with four slabs to an accumulator: a sum of
+// 160 like terms was 1.32 times as far from 64 bits as a chain of FMAs (192: 1.35; two slabs: 1.02 and 0.96), gradients of
+// 301-131-66-5 with inputs in [0, 1] at B = 256 up to 1.21 times (0.75).  3072-512-512-10, P = 4, K = 4 takes 408 us a round
+// at B = 160 (four slabs 377; two with sums in registers 436), 475 at 256 (438, 489).  bf16 operands are what limits one
+// plane: four slabs, whose sums the accumulator cuts off less often than the former warp-level MMAs theirs.
+constexpr int chain_slabs(int np) { return np == 3 ? 2 : 4; }
+constexpr int kManyChains = 0;
+constexpr int wgrad_chains(int np, int B) {
+  const int chain = chain_slabs(np) * kSlab;
+  return B <= chain ? 1 : np == 3 && B <= 2 * chain ? 2 : kManyChains;
+}
+constexpr int wgrad_epi(int chains) { return chains == kManyChains ? 8 : 16; }
+constexpr int wgrad_threads(int chains) { return (4 + wgrad_epi(chains)) * 32; }
 enum { ERR_SPLIT_PRODUCER = 41, ERR_SPLIT_MMA = 42, ERR_SPLIT_EPILOGUE = 43 };
 
 __host__ __device__ constexpr int pitch_of(int d) { return (d + 7) / 8 * 8; }
@@ -444,15 +455,16 @@ struct Weights {
 
 // Weight gradients, SGD steps, bias steps of all layers and the losses: persistent over tiles of 128 inputs x 128
 // outputs, dW^T = A^T dZ, so that the lanes of a warp finish neighbours of a row of W.  A tile's weights are fetched
-// while the tile before it is finished.  MANY: batches of more than kChainSlabs slabs, whose sums meet in registers; up
-// to there an accumulator takes the whole batch and is read where it is used, which leaves registers for twice the warps.
+// while the tile before it is finished.  CHAINS: see wgrad_chains; without sums in registers there is room for twice the warps.
 // Bound by what an SM takes in (three planes: 154 KB a tile at B = 100) and by the epilogue's stores: 3072-512-512-10,
 // P = 4, B = 100 32 us, 24 in a call's last step, which writes no planes.  On the way: eight warps with sums in registers 46,
 // biases summed by the epilogue 40, weights fetched at the tile's own beginning 44, a word at a time 46.
-template <int NP, bool MOM, bool MANY>
-__global__ void __launch_bounds__(wgrad_threads(MANY), 1)
+template <int NP, bool MOM, int CHAINS>
+__global__ void __launch_bounds__(wgrad_threads(CHAINS), 1)
 k_split_wgrad(const __grid_constant__ WgradArgs g) {
-  constexpr int kEpi = wgrad_epi(MANY), kStep = MANY ? 32 : 64, kGroups = kMaxN / kStep;
+  constexpr bool MANY = CHAINS == kManyChains;
+  constexpr int kChainSlabs = chain_slabs(NP);
+  constexpr int kEpi = wgrad_epi(CHAINS), kStep = MANY ? 32 : 64, kGroups = kMaxN / kStep;
   extern __shared__ uint8_t smem_raw[];
   __shared__ __align__(16) Barriers sh;
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -608,12 +620,12 @@ k_split_wgrad(const __grid_constant__ WgradArgs g) {
       next = tile_at(t + gridDim.x);
       const int l = x.l, p = x.p, o0 = x.o0;
       const WgradLayer& ly = g.layer[l];
-      const int N = columns(l, o0), outs = min(N, ly.out - o0);
+      const int N = columns(l, o0);
       const size_t w_at = w_place(x);
       const uint32_t low = lane_addr + (uint32_t)((2 + (tile & 1)) * kMaxN);
       const int c = 16 * ((warp - 2) >> 2);
       Sums<kStep> sums;                            // (not MANY: unused)
-      int b = chain & 1;
+      int b = CHAINS == 2 ? 0 : chain & 1;
       if (MANY) {
         sums.clear();
         for (int s = 0; s < slabs; s += kChainSlabs, ++chain) {
@@ -628,8 +640,9 @@ k_split_wgrad(const __grid_constant__ WgradArgs g) {
         }
       } else {
         ok = mbar_wait_warp(&sh.acc_full[b], (chain >> 1) & 1, abortp, g.status, ERR_SPLIT_EPILOGUE);
+        if (CHAINS == 2 && ok) ok = mbar_wait_warp(&sh.acc_full[1], (chain >> 1) & 1, abortp, g.status, ERR_SPLIT_EPILOGUE);
         tc_fence_after_sync();
-        ++chain;
+        chain += CHAINS;
       }
       if (barrier_any(!ok, 1, kEpi * 32)) break;   // a wait that was given up: all leave together
       const int pitch = pitch_of(ly.in);
@@ -646,6 +659,12 @@ k_split_wgrad(const __grid_constant__ WgradArgs g) {
           } else {
             uint32_t r[16], rl[16];
             tmem_ld_16cols(lane_addr + (uint32_t)(b * kMaxN + c + kStep * gr), r);
+            if (CHAINS == 2) {                     // (both accumulators are this tile's)
+              tmem_ld_16cols(lane_addr + (uint32_t)(kMaxN + c + kStep * gr), rl);
+              tmem_ld_wait();
+#pragma unroll
+              for (int j = 0; j < 16; ++j) r[j] = __float_as_uint(__uint_as_float(r[j]) + __uint_as_float(rl[j]));
+            }
             if (NP == 3) tmem_ld_16cols(low + (uint32_t)(c + kStep * gr), rl);
             tmem_ld_wait();
 #pragma unroll
@@ -664,6 +683,7 @@ k_split_wgrad(const __grid_constant__ WgradArgs g) {
         tc_fence_before_sync();
         __syncwarp();
         if (lane == 0) mbar_arrive(&sh.acc_empty[b]);
+        if (CHAINS == 2 && lane == 0) mbar_arrive(&sh.acc_empty[1]);
       }
     }
   }
