@@ -175,6 +175,7 @@ mavg_status read_mean_loss(mavg_ctx* c, float* mean_loss) {
   if (c->cfg.objective == MAVG_OBJ_MLP) {
     float* lm = c->mean_dev ? c->mean_dev : (float*)ws_ptr(c, c->ws.loss_mean);
     if (!c->mean_formed) {
+      c->mean_in_flight = true;
       prof_begin(c, MAVG_K_LOSS);
       k_mean_loss<<<1, 256, 0, c->stream>>>((const float*)ws_ptr(c, c->ws.losses),
                                             c->cfg.P * c->cfg.K, lm);
@@ -186,6 +187,7 @@ mavg_status read_mean_loss(mavg_ctx* c, float* mean_loss) {
       CU(c, cudaMemcpyAsync(mean_loss, lm, sizeof(float), cudaMemcpyDeviceToHost, c->stream),
          "loss read-back");
     CU(c, cudaStreamSynchronize(c->stream), "stream synchronize");
+    c->mean_in_flight = false;
     if (c->mean_dev) *mean_loss = *(volatile const float*)c->mean_host;
   } else {
     CU(c, cudaStreamSynchronize(c->stream), "stream synchronize");
@@ -650,10 +652,8 @@ mavg_status mavg_destroy(mavg_handle h) {
     keep_release(h->device, h->l2_keep_want);
   }
   for (cudaEvent_t e : h->ev_pool) cudaEventDestroy(e);
-  if (h->mean_host) {
-    cudaStreamSynchronize(h->stream);              // a round in flight may still write it
-    mean_word_release(h->mean_host);
-  }
+  // (a round that failed between the launch and its end may still write the word: it is not given out again)
+  if (h->mean_host && !h->mean_in_flight) mean_word_release(h->mean_host);
   if (h->ev_copy_fork) cudaEventDestroy(h->ev_copy_fork);
   if (h->ev_copy_done) cudaEventDestroy(h->ev_copy_done);
   if (h->s_copy) cudaStreamDestroy(h->s_copy);

@@ -139,9 +139,10 @@ struct mavg_ctx {
   size_t l2_keep_want = 0;
   int device = 0;
   // Mean loss of a round: written by the device into this pinned word (null: read back from ws.loss_mean).  mean_wanted: the
-  // meta-update about to be launched may form it on the way, mean_formed: it did.
+  // meta-update about to be launched may form it on the way, mean_formed: it did.  mean_in_flight: a launch that writes it has
+  // not been waited for.
   float *mean_host = nullptr, *mean_dev = nullptr;
-  bool mean_wanted = false, mean_formed = false;
+  bool mean_wanted = false, mean_formed = false, mean_in_flight = false;
   // mavg_round_host: the upload of v runs on a copy stream of its own, next to the local steps
   cudaStream_t s_copy = nullptr;
   cudaEvent_t ev_copy_fork = nullptr, ev_copy_done = nullptr;

@@ -431,6 +431,7 @@ cudaError_t launch_meta_update(mavg_ctx* c) {
                              (const float*)ws_ptr(c, c->ws.losses), P * c->cfg.K,
                              c->mean_dev ? c->mean_dev : (float*)ws_ptr(c, c->ws.loss_mean));
       c->mean_formed = mean && e == cudaSuccess;
+      if (c->mean_formed) c->mean_in_flight = true;
     }
     if (e == cudaSuccess) e = cudaGetLastError();
   }
