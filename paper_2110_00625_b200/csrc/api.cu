@@ -240,7 +240,7 @@ bool keep_acquire(int dev, size_t want) {
 }
 
 // Words of pinned memory that rounds leave their mean loss in, one per handle: a page for the process, allocated by its
-// first handle (a pinned allocation takes about a millisecond).  A handle that finds none free, or no page, has its mean
+// first handle (a pinned allocation takes about a millisecond) and kept until it exits.  A handle that finds none free, or no page, has its mean
 // copied back from the workspace.
 constexpr int kMeanWords = 4096 / sizeof(float);
 std::mutex g_mean_mu;
@@ -250,7 +250,12 @@ std::vector<float*> g_mean_free;
 void mean_word_acquire(float** host, float** dev) {
   std::lock_guard<std::mutex> lock(g_mean_mu);
   if (!g_mean_page) {
-    if (cudaHostAlloc((void**)&g_mean_page, kMeanWords * sizeof(float), cudaHostAllocMapped | cudaHostAllocPortable) != cudaSuccess) {
+    // (it has nothing to do with a stream that is being captured, but would break the capture unless it says so)
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    const cudaError_t e = cudaHostAlloc((void**)&g_mean_page, kMeanWords * sizeof(float), cudaHostAllocMapped | cudaHostAllocPortable);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) {
       cudaGetLastError();
       g_mean_page = nullptr;
       return;
