@@ -37,10 +37,8 @@ mavg_status mlp_setup(mavg_ctx* c) {
     c->layers.push_back(ly);
   }
   if (use_tensor_cores(&cfg)) return tc_setup(c);
-  const mavg_status st = simt_setup(c);
-  if (st != MAVG_OK) return st;
-  small_setup(c);
-  return MAVG_OK;
+  small_setup(c);                                // where it is taken nothing of the other path is ever launched
+  return c->small_splits ? MAVG_OK : simt_setup(c);
 }
 
 void mlp_drop_graph(mavg_ctx* c);

@@ -19,6 +19,9 @@
 // step of a round reads the weights from w~ and writes the results to the replicas, so its P copies
 // are never needed.
 #include <algorithm>
+#include <array>
+#include <map>
+#include <mutex>
 
 #include "mlp.cuh"
 #include "split_gemm.cuh"
@@ -499,7 +502,7 @@ size_t carve(const mavg_config* cfg, char* base, SimtBuffers* sb) {
 struct SimtState {
   SimtBuffers buf;
   int n_tiles, N;                          // batch tiles of a product
-  int resident[9];                         // clusters of that many product blocks the GPU holds at once
+  int resident[9];                         // resident_clusters()
   CUtensorMap x[2], x_mn[2];
   CUtensorMap a[MAVG_MAX_LAYERS + 1], a_mn[MAVG_MAX_LAYERS + 1], dz[MAVG_MAX_LAYERS + 1], dz_mn[MAVG_MAX_LAYERS + 1];
   CUtensorMap w[MAVG_MAX_LAYERS + 1], w_mn[MAVG_MAX_LAYERS + 1];   // boxes of 64 x 128, 64 x 64
@@ -577,24 +580,74 @@ cudaError_t launch_product(mavg_ctx* c, int cls, const CUtensorMap& w, bool shar
                 split::kProductThreads, g.splits, sh.smem, w, x, g);
 }
 
-// Every kernel of a step asks for the same split of the SM's memory: a launch that needs another
-// split than the kernel before it has to wait until the SM is empty.
+typedef void (*WgradKernel)(split::WgradArgs);
 template <bool QUANT>
-cudaError_t set_attributes() {
-  constexpr int NP = kPlanes<QUANT>, kTwo = NP == 3 ? 2 : 1;
-  const struct { const void* kernel; size_t smem; } kernels[] = {
-      {(const void*)split::k_split_product<NP, false>, kSplitSmem}, {(const void*)split::k_split_product<NP, true>, kSplitSmem},
-      {(const void*)split::k_split_wgrad<NP, false, 1>, kSplitSmem}, {(const void*)split::k_split_wgrad<NP, true, 1>, kSplitSmem},
-      {(const void*)split::k_split_wgrad<NP, false, kTwo>, kSplitSmem}, {(const void*)split::k_split_wgrad<NP, true, kTwo>, kSplitSmem},
-      {(const void*)split::k_split_wgrad<NP, false, split::kManyChains>, kSplitSmem}, {(const void*)split::k_split_wgrad<NP, true, split::kManyChains>, kSplitSmem},
-      {(const void*)k_simt_begin<QUANT>, 0}, {(const void*)k_simt_loss<QUANT>, 0}, {(const void*)k_simt_tail<QUANT>, kTailSmem}};
+WgradKernel wgrad_kernel(int B, bool momentum) {
+  constexpr int NP = kPlanes<QUANT>, kTwo = NP == 3 ? 2 : 1;   // (one plane: never two)
+  const int chains = split::wgrad_chains(NP, B);
+  auto pick = [&](auto one, auto two, auto many) { return chains == 1 ? one : chains == 2 ? two : many; };
+  return momentum ? pick(split::k_split_wgrad<NP, true, 1>, split::k_split_wgrad<NP, true, kTwo>, split::k_split_wgrad<NP, true, split::kManyChains>)
+                  : pick(split::k_split_wgrad<NP, false, 1>, split::k_split_wgrad<NP, false, kTwo>, split::k_split_wgrad<NP, false, split::kManyChains>);
+}
+
+// Every kernel of a step asks for the same split of the SM's memory: a launch that needs another
+// split than the kernel before it has to wait until the SM is empty.  Only kernels that the handle's steps launch are asked
+// for: the first call for one loads it (1000-333-100 with bf16 operands: a process's first handle takes 9.6 ms, 10.7 with all).
+template <bool QUANT>
+cudaError_t set_attributes(const mavg_ctx* c) {
+  constexpr int NP = kPlanes<QUANT>;
+  const mavg_config& cfg = c->cfg;
+  const bool tail = product_layers(&cfg) < cfg.n_layers;
+  const struct { const void* kernel; size_t smem; bool used; } kernels[] = {
+      {(const void*)split::k_split_product<NP, false>, kSplitSmem, true},
+      {(const void*)split::k_split_product<NP, true>, kSplitSmem, !tail || cfg.n_layers > 2},
+      {(const void*)wgrad_kernel<QUANT>(cfg.B, false), kSplitSmem, true},
+      {(const void*)wgrad_kernel<QUANT>(cfg.B, true), kSplitSmem, c->buf.learner_u != nullptr},
+      {(const void*)k_simt_begin<QUANT>, 0, true}, {(const void*)k_simt_loss<QUANT>, 0, !tail}, {(const void*)k_simt_tail<QUANT>, kTailSmem, tail}};
   for (const auto& k : kernels) {
+    if (!k.used) continue;
     cudaError_t e = cudaFuncSetAttribute(k.kernel, cudaFuncAttributePreferredSharedMemoryCarveout,
                                          cudaSharedmemCarveoutMaxShared);
     if (e == cudaSuccess && k.smem) e = cudaFuncSetAttribute(k.kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;
+}
+
+// Clusters of s product blocks that the GPU holds at once, at [s]; 0 where the query is refused: such a split is not taken.
+// Asked once per device and shape of a product (one or three planes, batch tiles of 16 to 128 rows).
+void resident_clusters(int device, int np, int N, int (&resident)[9]) {
+  static std::mutex mu;
+  static std::map<std::array<int, 3>, std::array<int, 9>> known;
+  std::lock_guard<std::mutex> lock(mu);
+  const std::array<int, 3> key{device, np, N};
+  auto it = known.find(key);
+  std::array<int, 9> got{};
+  if (it != known.end()) {
+    got = it->second;
+  } else {
+    bool all = true;
+    for (int s = 2; s <= 8; ++s) {
+      cudaLaunchAttribute at[1];
+      cudaLaunchConfig_t lc{};
+      at[0].id = cudaLaunchAttributeClusterDimension;
+      at[0].val.clusterDim.x = (unsigned)s;
+      at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+      lc.gridDim = dim3((unsigned)s);
+      lc.blockDim = dim3(split::kProductThreads);
+      lc.dynamicSmemBytes = product_shape(np, N).smem;
+      lc.attrs = at;
+      lc.numAttrs = 1;
+      const cudaError_t e = np == 1 ? cudaOccupancyMaxActiveClusters(&got[s], split::k_split_product<1, false>, &lc)
+                                    : cudaOccupancyMaxActiveClusters(&got[s], split::k_split_product<3, false>, &lc);
+      if (e == cudaSuccess) continue;
+      cudaGetLastError();
+      got[s] = 0;
+      all = false;
+    }
+    if (all) known[key] = got;
+  }
+  for (int s = 0; s <= 8; ++s) resident[s] = got[s];
 }
 
 template <bool QUANT>
@@ -727,12 +780,8 @@ cudaError_t step_impl(mavg_ctx* c, int64_t round, int step) {
   w.stages = std::min(split::kMaxStages, (int)((kSplitSmem - 1024) / split::wgrad_stage_bytes(NP)));
   const size_t smem = std::max((size_t)w.stages * split::wgrad_stage_bytes(NP) + 1024,
                                split::tmem_share_bytes(NP == 3 ? 512 : 256, sizeof(split::Barriers)));
-  constexpr int kTwo = NP == 3 ? 2 : 1;              // (one plane: never two)
-  const int chains = split::wgrad_chains(NP, B);
-  auto pick = [&](auto one, auto two, auto many) { return chains == 1 ? one : chains == 2 ? two : many; };
-  auto kernel = mom.u ? pick(split::k_split_wgrad<NP, true, 1>, split::k_split_wgrad<NP, true, kTwo>, split::k_split_wgrad<NP, true, split::kManyChains>)
-                      : pick(split::k_split_wgrad<NP, false, 1>, split::k_split_wgrad<NP, false, kTwo>, split::k_split_wgrad<NP, false, split::kManyChains>);
-  return launch(c, MAVG_K_WGRAD_SGD, kernel, dim3((unsigned)std::min(w.tiles, c->sm_count)), split::wgrad_threads(chains), 1, smem, w);
+  return launch(c, MAVG_K_WGRAD_SGD, wgrad_kernel<QUANT>(B, mom.u != nullptr), dim3((unsigned)std::min(w.tiles, c->sm_count)),
+                split::wgrad_threads(split::wgrad_chains(NP, B)), 1, smem, w);
 }
 
 }  // namespace
@@ -767,24 +816,11 @@ mavg_status simt_setup(mavg_ctx* c) {
     if (l <= product_layers(&cfg)) map(&st->w[l], &st->w_mn[l], st->buf.w[l], cfg.dims[l - 1], cfg.dims[l], P + 1, split::kTile);
   }
   if (!ok) return MAVG_ERR_UNSUPPORTED;
-  cudaError_t e = cfg.gemm_bf16 ? set_attributes<true>() : set_attributes<false>();
+  cudaError_t e = cfg.gemm_bf16 ? set_attributes<true>(c) : set_attributes<false>(c);
   // columns beyond the rows of W_L's plane, which mma_tail reads and nobody writes
   if (e == cudaSuccess && cfg.gemm_bf16 && cfg.dims[L - 1] % 8)
     e = cudaMemsetAsync(st->buf.w[L], 0, (size_t)(P + 1) * cfg.dims[L] * pitch_of(cfg.dims[L - 1]) * 2, c->stream);
-  for (int s = 1; s <= 8 && e == cudaSuccess; ++s) {
-    cudaLaunchAttribute at[1];
-    cudaLaunchConfig_t lc{};
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)s;
-    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
-    lc.gridDim = dim3((unsigned)s);
-    lc.blockDim = dim3(split::kProductThreads);
-    lc.dynamicSmemBytes = product_shape(np, st->N).smem;
-    lc.attrs = at;
-    lc.numAttrs = 1;
-    if (cfg.gemm_bf16) e = cudaOccupancyMaxActiveClusters(&st->resident[s], split::k_split_product<1, false>, &lc);
-    else e = cudaOccupancyMaxActiveClusters(&st->resident[s], split::k_split_product<3, false>, &lc);
-  }
+  if (e == cudaSuccess) resident_clusters(c->device, np, st->N, st->resident);
   if (e == cudaSuccess) return MAVG_OK;
   c->err = std::string("kernel attributes: ") + cudaGetErrorString(e);
   return MAVG_ERR_CUDA;
