@@ -146,7 +146,9 @@ typedef struct {
 mavg_status mavg_workspace_bytes(const mavg_config *cfg, size_t *out_bytes);
 
 /* The least that mavg_create accepts: smaller where rounds are factored or rebuilt (MAVG_SCHED_GRAPH below), which
- * need room for the rows of all K steps; a handle with less than mavg_workspace_bytes keeps the plain form. */
+ * need room for the rows of all K steps; a handle with less than mavg_workspace_bytes keeps the plain form.  Smaller too
+ * for several learners with gemm_bf16 0 or 2, whose weights are kept a second time as operands (6 or 2 bytes each): a handle
+ * with less takes the local steps some learners at a time, one at the least, with the same results. */
 mavg_status mavg_workspace_least_bytes(const mavg_config *cfg, size_t *out_bytes);
 
 /* Algorithm 1, the two initialisation lines and the first "set w^j = w~": v <- 0, w^j <- w~_1

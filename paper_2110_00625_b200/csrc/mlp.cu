@@ -19,7 +19,7 @@ mavg_status mlp_validate(const mavg_config* cfg, std::string* why) {
 
 size_t mlp_workspace_bytes(const mavg_config* cfg, Workspace* ws, size_t base) {
   if (use_tensor_cores(cfg)) return tc_workspace_bytes(cfg, base, &ws->act, &ws->least);
-  return ws->least = simt_workspace_bytes(cfg, base, &ws->act);
+  return simt_workspace_bytes(cfg, base, &ws->act, &ws->least);
 }
 
 mavg_status mlp_setup(mavg_ctx* c) {
@@ -71,12 +71,7 @@ __global__ void k_set_round(int64_t* dst, int64_t round) { *dst = round; }
 
 cudaError_t run_steps(mavg_ctx* c, int64_t round) {
   if (use_tensor_cores(&c->cfg)) return tc_local_steps(c, round);
-  for (int k = 1; k <= c->cfg.K; ++k) {
-    cudaError_t e = simt_step(c, round, k);
-    if (e != cudaSuccess) return e;
-    c->replicas_equal_global = false;
-  }
-  return cudaSuccess;
+  return simt_local_steps(c, round);
 }
 
 void drop_graph(mavg_ctx* c) {

@@ -31,12 +31,13 @@ cudaError_t launch_sample_gather(mavg_ctx* c, int64_t round, int step, int32_t* 
                                  int32_t* labels, __nv_bfloat16* out_bf, __nv_bfloat16* out_bft);
 
 // fp32 arithmetic, or bf16 operands of any shape (mlp_simt.cu).
-size_t simt_workspace_bytes(const mavg_config* cfg, size_t base, size_t* act_off);
+size_t simt_workspace_bytes(const mavg_config* cfg, size_t base, size_t* act_off, size_t* least);
 mavg_status simt_setup(mavg_ctx* c);      // once per handle
 void simt_teardown(mavg_ctx* c);
-cudaError_t simt_step(mavg_ctx* c, int64_t round, int step);
+cudaError_t simt_local_steps(mavg_ctx* c, int64_t round);    // all K of them
 
 // Small models on the CUDA cores (mlp_small.cu): all local steps of a round in one launch.
+bool small_always(const mavg_config* cfg);   // taken whenever the device grants the launch
 void small_setup(mavg_ctx* c);            // once per handle: c->small_splits > 0 where it is used
 cudaError_t small_local_steps(mavg_ctx* c, int64_t round);
 

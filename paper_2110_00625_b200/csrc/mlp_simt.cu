@@ -42,10 +42,10 @@ struct GatherArgs {
   const void* x; int x_bf16;
   const int32_t* y;
   uint64_t seed; int64_t round; const int64_t* round_ptr;
-  int step, P, B, d;
+  int step, P, p0, n, B, d;            // learners p0 .. p0 + n - 1 of P
   int64_t S;
-  __nv_bfloat16* out; int64_t plane;   // planes [P, B, pitch_of(d)]
-  int32_t* labels;                     // [P, B]
+  __nv_bfloat16* out; int64_t plane;   // planes [n, B, pitch_of(d)]
+  int32_t* labels;                     // [n, B]
 };
 
 // One sampled row: index, label and the row itself.
@@ -55,7 +55,7 @@ __device__ __forceinline__ void gather_row(const GatherArgs& g, int row) {
   __shared__ int32_t sidx;
   if (threadIdx.x == 0) {
     const int64_t round = g.round_ptr ? *g.round_ptr : g.round;
-    sidx = sample_index(g.seed, round, row / g.B, g.step, row % g.B, g.P, g.S);
+    sidx = sample_index(g.seed, round, g.p0 + row / g.B, g.step, row % g.B, g.P, g.S);
     g.labels[row] = g.y[sidx];
   }
   __syncthreads();
@@ -94,11 +94,11 @@ __global__ void __launch_bounds__(256)
 k_simt_begin(const __grid_constant__ GatherArgs g, const __grid_constant__ split::SplitWeights w) {
   tc::grid_launch_dependents();
   tc::grid_dependency_wait();
-  if ((int)blockIdx.x < g.P * g.B) {
+  if ((int)blockIdx.x < g.n * g.B) {
     gather_row<QUANT>(g, blockIdx.x);
     return;
   }
-  const int row = ((int)blockIdx.x - g.P * g.B) * 8 + (int)threadIdx.x / 32;
+  const int row = ((int)blockIdx.x - g.n * g.B) * 8 + (int)threadIdx.x / 32;
   if (row < w.copies * w.first[w.L]) split::split_weight_row<kPlanes<QUANT>>(w, row);
 }
 
@@ -442,6 +442,7 @@ k_simt_loss(const float* __restrict__ logits, const int32_t* __restrict__ labels
 }
 
 // ---------------------------------------------------------------------------------- host side
+// (P: the learners that take their steps together)
 struct SimtBuffers {
   __nv_bfloat16* xg[2];                    // planes [P, B, pitch]: the minibatch, alternate steps
   int32_t* labels[2];                      // [P, B]
@@ -471,8 +472,8 @@ int product_layers(const mavg_config* cfg) {
 // Layers whose weights are kept as planes: those, and with bf16 operands the last one (mma_tail).
 int plane_layers(const mavg_config* cfg) { return cfg->gemm_bf16 ? cfg->n_layers : product_layers(cfg); }
 
-size_t carve(const mavg_config* cfg, char* base, SimtBuffers* sb) {
-  const size_t rows = (size_t)cfg->P * cfg->B;
+size_t carve(const mavg_config* cfg, int learners, char* base, SimtBuffers* sb) {
+  const size_t rows = (size_t)learners * cfg->B;
   const int np = cfg->gemm_bf16 ? kPlanes<true> : kPlanes<false>;
   size_t off = 0;
   auto take = [&](size_t bytes) {
@@ -493,7 +494,7 @@ size_t carve(const mavg_config* cfg, char* base, SimtBuffers* sb) {
     sb->dz_f[l] = (float*)take(rows * cfg->dims[l] * 4);
   }
   for (int l = 1; l <= plane_layers(cfg); ++l)
-    sb->w[l] = (__nv_bfloat16*)take((size_t)np * (cfg->P + 1) * cfg->dims[l] * pitch_of(cfg->dims[l - 1]) * 2);
+    sb->w[l] = (__nv_bfloat16*)take((size_t)np * (learners + 1) * cfg->dims[l] * pitch_of(cfg->dims[l - 1]) * 2);
   return off;
 }
 
@@ -501,6 +502,7 @@ size_t carve(const mavg_config* cfg, char* base, SimtBuffers* sb) {
 // weight gradients (boxes of 64 x 64).
 struct SimtState {
   SimtBuffers buf;
+  int group;                               // learners that take their steps together: all of them where the scratch has room
   int n_tiles, N;                          // batch tiles of a product
   int resident[9];                         // resident_clusters()
   CUtensorMap x[2], x_mn[2];
@@ -549,11 +551,11 @@ ProductShape product_shape(int np, int N) {
 
 // Forward product or data gradient.
 template <bool QUANT, bool DGRAD>
-cudaError_t launch_product(mavg_ctx* c, int cls, const CUtensorMap& w, bool shared_w, const CUtensorMap& x, split::ProductArgs g) {
+cudaError_t launch_product(mavg_ctx* c, int cls, int n, const CUtensorMap& w, bool shared_w, const CUtensorMap& x, split::ProductArgs g) {
   constexpr int NP = kPlanes<QUANT>;
   const SimtState* st = (const SimtState*)c->simt;
   const ProductShape sh = product_shape(NP, st->N);
-  g.P = c->cfg.P;
+  g.P = st->group;
   g.B = c->cfg.B;
   g.N = st->N;
   g.n_tiles = st->n_tiles;
@@ -570,13 +572,13 @@ cudaError_t launch_product(mavg_ctx* c, int cls, const CUtensorMap& w, bool shar
   // P = 4, K = 2, B = 42 143 / 134, 322-266-305-5, P = 2, K = 3, B = 37 151 / 138; with at most four blocks to a tile
   // 3072-512-512-10, P = 4, K = 4, B = 100 403 for 381.
   const int slabs = (g.K + split::kSlab - 1) / split::kSlab;
-  const int64_t tiles = (int64_t)g.m_tiles * g.n_tiles * g.P;
+  const int64_t tiles = (int64_t)g.m_tiles * g.n_tiles * c->cfg.P;   // (of all learners: the same sums in groups)
   g.splits = 1;
   for (int s = 2; s <= 8 && slabs >= s; ++s)
     if (tiles <= st->resident[s]) g.splits = s;
   g.per_split = (slabs + g.splits - 1) / g.splits;
   g.splits = (slabs + g.per_split - 1) / g.per_split;
-  return launch(c, cls, split::k_split_product<NP, DGRAD>, dim3((unsigned)(g.splits * g.m_tiles * g.n_tiles), 1, (unsigned)g.P),
+  return launch(c, cls, split::k_split_product<NP, DGRAD>, dim3((unsigned)(g.splits * g.m_tiles * g.n_tiles), 1, (unsigned)n),
                 split::kProductThreads, g.splits, sh.smem, w, x, g);
 }
 
@@ -650,28 +652,30 @@ void resident_clusters(int device, int np, int N, int (&resident)[9]) {
   for (int s = 0; s <= 8; ++s) resident[s] = got[s];
 }
 
+// A step of the learners p0 .. p0 + n - 1.
 template <bool QUANT>
-cudaError_t step_impl(mavg_ctx* c, int64_t round, int step) {
+cudaError_t step_impl(mavg_ctx* c, int64_t round, int step, int p0, int n) {
   constexpr int NP = kPlanes<QUANT>;
   const mavg_config& cfg = c->cfg;
-  const int P = cfg.P, B = cfg.B, L = cfg.n_layers;
+  const int B = cfg.B, L = cfg.n_layers;
   const SimtState* st = (const SimtState*)c->simt;
+  const int G = st->group;
   const SimtBuffers& sb = st->buf;
-  auto plane_of = [&](int d) { return (int64_t)P * B * pitch_of(d); };
+  auto plane_of = [&](int d) { return (int64_t)G * B * pitch_of(d); };
   const int cur = step & 1;
   GatherArgs ga{};
   ga.x = cfg.x; ga.x_bf16 = cfg.x_dtype == MAVG_X_BF16;
   ga.y = cfg.y; ga.seed = cfg.seed; ga.round = round;
   ga.round_ptr = c->capturing ? (const int64_t*)(ws_ptr(c, c->ws.status) + 64) : nullptr;
-  ga.step = step; ga.P = P; ga.B = B; ga.d = cfg.dims[0]; ga.S = cfg.n_samples;
+  ga.step = step; ga.P = cfg.P; ga.p0 = p0; ga.n = n; ga.B = B; ga.d = cfg.dims[0]; ga.S = cfg.n_samples;
   ga.out = sb.xg[cur]; ga.plane = plane_of(cfg.dims[0]); ga.labels = sb.labels[cur];
   GatherArgs next = ga;
   next.step = step + 1; next.out = sb.xg[cur ^ 1]; next.labels = sb.labels[cur ^ 1];
-  const int gather_rows = step < cfg.K ? P * B : 0;
+  const int gather_rows = step < cfg.K ? n * B : 0;
   cudaError_t e;
   // the weights before this step
-  float* rep = c->buf.replicas;
   const int64_t rs = c->buf.replica_stride;
+  float* rep = c->buf.replicas + p0 * rs;
   const float* win = starts_from_global(c) ? c->buf.global_w : rep;
   const int64_t ws = starts_from_global(c) ? 0 : rs;
   const bool shared_w = starts_from_global(c);
@@ -679,20 +683,21 @@ cudaError_t step_impl(mavg_ctx* c, int64_t round, int step) {
   if (step == 1) {
     split::SplitWeights w{};
     w.L = plane_layers(&cfg);
-    w.copies = shared_w ? 1 : P;
+    w.copies = shared_w ? 1 : n;
     w.src_batch = ws;
     for (int l = 1; l <= w.L; ++l) {
       w.src[l - 1] = win + c->layers[l - 1].w_off;
-      w.dst[l - 1] = sb.w[l] + (shared_w ? P * w_matrix(l) : 0);
+      w.dst[l - 1] = sb.w[l] + (shared_w ? G * w_matrix(l) : 0);
       w.dst_batch[l - 1] = w_matrix(l);
-      w.dst_plane[l - 1] = (P + 1) * w_matrix(l);
+      w.dst_plane[l - 1] = (G + 1) * w_matrix(l);
       w.in[l - 1] = cfg.dims[l - 1];
       w.first[l] = w.first[l - 1] + cfg.dims[l];
     }
-    const int64_t blocks = (int64_t)P * B + ((int64_t)w.copies * w.first[w.L] + 7) / 8;
+    const int64_t blocks = (int64_t)n * B + ((int64_t)w.copies * w.first[w.L] + 7) / 8;
     if ((e = launch(c, MAVG_K_BATCH, k_simt_begin<QUANT>, dim3((unsigned)blocks), 256, 1, 0, ga, w)) != cudaSuccess) return e;
   }
-  const MomArgs mom = mom_args(c, c->replicas_equal_global);
+  MomArgs mom = mom_args(c, c->replicas_equal_global);
+  if (mom.u) mom.u += p0 * mom.u_stride;
   auto a_in = [&](int l) { return l == 1 ? sb.xg[cur] : sb.a[l - 1]; };
   const MlpLayer& top = c->layers[L - 1];
   const bool tail = product_layers(&cfg) < L;
@@ -705,14 +710,14 @@ cudaError_t step_impl(mavg_ctx* c, int64_t round, int step) {
     g.hidden = l < L;
     if (l < L) g.out = sb.a[l];
     else g.out_f = sb.logits;
-    if ((e = launch_product<QUANT, false>(c, MAVG_K_FWD, st->w[l], shared_w, l == 1 ? st->x[cur] : st->a[l - 1], g)) != cudaSuccess) return e;
+    if ((e = launch_product<QUANT, false>(c, MAVG_K_FWD, n, st->w[l], shared_w, l == 1 ? st->x[cur] : st->a[l - 1], g)) != cudaSuccess) return e;
   }
   if (tail) {
     TailArgs t{};
     t.a = a_in(L); t.a_plane = plane_of(top.in);
     t.w = win + top.w_off; t.b = win + top.b_off; t.w_batch = ws;
     t.labels = sb.labels[cur];
-    t.P = P; t.B = B; t.in = top.in; t.C = top.out; t.row_blocks = (B + kTailRows - 1) / kTailRows;
+    t.P = n; t.B = B; t.in = top.in; t.C = top.out; t.row_blocks = (B + kTailRows - 1) / kTailRows;
     t.row_loss = sb.row_loss; t.dz = sb.dz_f[L];
     t.dz_pl = sb.dz[L]; t.dz_plane = plane_of(top.out);
     if (L >= 2) {
@@ -722,14 +727,14 @@ cudaError_t step_impl(mavg_ctx* c, int64_t round, int step) {
     }
     // few classes on very wide rows: their padding to 16 would not fit
     t.mma = QUANT && tail_smem(t.in, t.C, true) <= kTailSmem;
-    t.w16 = sb.w[L] + (shared_w ? P * w_matrix(L) : 0);
+    t.w16 = sb.w[L] + (shared_w ? G * w_matrix(L) : 0);
     t.w16_batch = shared_w ? 0 : w_matrix(L);
-    if ((e = launch(c, MAVG_K_LOSS, k_simt_tail<QUANT>, dim3((unsigned)(P * t.row_blocks + gather_rows)),
+    if ((e = launch(c, MAVG_K_LOSS, k_simt_tail<QUANT>, dim3((unsigned)(n * t.row_blocks + gather_rows)),
                     kTailThreads, 1, tail_smem(t.in, t.C, t.mma), t, next)) != cudaSuccess)
       return e;
   } else {
-    if ((e = launch(c, MAVG_K_LOSS, k_simt_loss<QUANT>, dim3((unsigned)(P + gather_rows)), 1024, 1, 0,
-                    (const float*)sb.logits, (const int32_t*)sb.labels[cur], P, B, top.out, sb.row_loss,
+    if ((e = launch(c, MAVG_K_LOSS, k_simt_loss<QUANT>, dim3((unsigned)(n + gather_rows)), 1024, 1, 0,
+                    (const float*)sb.logits, (const int32_t*)sb.labels[cur], n, B, top.out, sb.row_loss,
                     sb.dz_f[L], sb.dz[L], plane_of(top.out), next)) != cudaSuccess)
       return e;
   }
@@ -739,16 +744,16 @@ cudaError_t step_impl(mavg_ctx* c, int64_t round, int step) {
     g.M = ly.in; g.K = ly.out;
     g.out = sb.dz[l - 1]; g.out_f = sb.dz_f[l - 1];
     g.act = sb.a[l - 1]; g.pitch = pitch_of(ly.in);
-    if ((e = launch_product<QUANT, true>(c, MAVG_K_DGRAD, st->w_mn[l], shared_w, st->dz[l], g)) != cudaSuccess) return e;
+    if ((e = launch_product<QUANT, true>(c, MAVG_K_DGRAD, n, st->w_mn[l], shared_w, st->dz[l], g)) != cudaSuccess) return e;
   }
   split::WgradArgs w{};
-  w.L = L; w.P = P; w.B = B;
+  w.L = L; w.P = G; w.B = B;
   w.write_planes = step < cfg.K;
   // Tiles of 128 x 64 where wider ones would leave SMs without any (us a round, 128 / 64 wide: 322-266-305-5, P = 2,
   // K = 3, B = 37 160 / 151, 357-761-217-96, P = 1, K = 4, B = 149 261 / 250; beyond the line 437-425-42, P = 6, K = 4,
   // B = 36 103 / 110, 3072-512-512-10, P = 4, K = 4, B = 100 382 / 394: a narrow tile takes in half as much again).
   int64_t wide = 0;
-  for (const MlpLayer& ly : c->layers) wide += (int64_t)((ly.in + 127) / 128) * ((ly.out + 127) / 128) * P;
+  for (const MlpLayer& ly : c->layers) wide += (int64_t)((ly.in + 127) / 128) * ((ly.out + 127) / 128) * cfg.P;
   w.bn = wide <= c->sm_count ? 64 : 128;
   for (int l = 1; l <= L; ++l) {
     const MlpLayer& ly = c->layers[l - 1];
@@ -765,16 +770,16 @@ cudaError_t step_impl(mavg_ctx* c, int64_t round, int step) {
     if (l <= plane_layers(&cfg)) {
       g.w16 = sb.w[l];
       g.w16_batch = w_matrix(l);
-      g.w16_plane = (P + 1) * w_matrix(l);
+      g.w16_plane = (G + 1) * w_matrix(l);
     }
-    w.tiles += g.i_tiles * g.o_tiles * P;
+    w.tiles += g.i_tiles * g.o_tiles * n;
   }
   w.w_in = win; w.w_in_batch = ws;
   w.rep = rep; w.rep_stride = rs;
   w.mom = mom;
   w.gamma = cfg.local_lr;
   w.row_loss = sb.row_loss;
-  w.loss_out = (float*)ws_ptr(c, c->ws.losses) + (step - 1);
+  w.loss_out = (float*)ws_ptr(c, c->ws.losses) + (size_t)p0 * cfg.K + (step - 1);
   w.loss_stride = cfg.K;
   w.status = (int*)ws_ptr(c, c->ws.status);
   w.stages = std::min(split::kMaxStages, (int)((kSplitSmem - 1024) / split::wgrad_stage_bytes(NP)));
@@ -786,20 +791,35 @@ cudaError_t step_impl(mavg_ctx* c, int64_t round, int step) {
 
 }  // namespace
 
-size_t simt_workspace_bytes(const mavg_config* cfg, size_t base, size_t* act_off) {
+size_t simt_workspace_bytes(const mavg_config* cfg, size_t base, size_t* act_off, size_t* least) {
   *act_off = base;
   SimtBuffers sb;
-  return base + carve(cfg, nullptr, &sb);
+  *least = base + carve(cfg, 1, nullptr, &sb);
+  // (models whose steps are one launch use none of it unless that launch is refused)
+  return small_always(cfg) ? *least : base + carve(cfg, cfg->P, nullptr, &sb);
 }
 
 mavg_status simt_setup(mavg_ctx* c) {
   const mavg_config& cfg = c->cfg;
-  const int L = cfg.n_layers, P = cfg.P, B = cfg.B, np = cfg.gemm_bf16 ? kPlanes<true> : kPlanes<false>;
+  const int L = cfg.n_layers, B = cfg.B, np = cfg.gemm_bf16 ? kPlanes<true> : kPlanes<false>;
   const EncodeTiledFn encode = tensor_map_encoder(&c->err);
   if (!encode) return MAVG_ERR_UNSUPPORTED;
   SimtState* st = new SimtState();
   c->simt = st;
-  carve(&cfg, ws_ptr(c, c->ws.act), &st->buf);
+  // The planes of the learners' weights are 1.5 times the replica array with fp32 operands: where the scratch has room for
+  // fewer learners' they take their steps in groups, one after the other.
+  const size_t room = c->buf.workspace_bytes - c->ws.act;
+  int P = cfg.P;
+  if (carve(&cfg, P, nullptr, &st->buf) > room) {
+    int fits = 1;
+    while (P - fits > 1) {
+      const int half = fits + (P - fits) / 2;
+      (carve(&cfg, half, nullptr, &st->buf) > room ? P : fits) = half;
+    }
+    P = (cfg.P + (cfg.P + fits - 1) / fits - 1) / ((cfg.P + fits - 1) / fits);   // of as many groups, the most even
+  }
+  st->group = P;
+  carve(&cfg, P, ws_ptr(c, c->ws.act), &st->buf);
   st->n_tiles = (B + split::kMaxN - 1) / split::kMaxN;
   st->N = ((B + st->n_tiles - 1) / st->n_tiles + 15) / 16 * 16;
   bool ok = true;
@@ -831,8 +851,19 @@ void simt_teardown(mavg_ctx* c) {
   c->simt = nullptr;
 }
 
-cudaError_t simt_step(mavg_ctx* c, int64_t round, int step) {
-  return c->cfg.gemm_bf16 ? step_impl<true>(c, round, step) : step_impl<false>(c, round, step);
+cudaError_t simt_local_steps(mavg_ctx* c, int64_t round) {
+  const bool from_broadcast = c->replicas_equal_global;
+  const int group = ((const SimtState*)c->simt)->group;
+  cudaError_t e = cudaSuccess;
+  for (int p0 = 0; p0 < c->cfg.P && e == cudaSuccess; p0 += group) {
+    c->replicas_equal_global = from_broadcast;
+    const int n = std::min(group, c->cfg.P - p0);
+    for (int k = 1; k <= c->cfg.K && e == cudaSuccess; ++k) {
+      e = c->cfg.gemm_bf16 ? step_impl<true>(c, round, k, p0, n) : step_impl<false>(c, round, k, p0, n);
+      c->replicas_equal_global = false;
+    }
+  }
+  return e;
 }
 
 }  // namespace mavg

@@ -485,6 +485,8 @@ static bool small_fits(const mavg_config* cfg) {
   return cfg->gemm_bf16 != 1 && layout(cfg).floats * sizeof(float) <= kSmallSmem;
 }
 
+bool small_always(const mavg_config* cfg) { return cfg->n <= 4096 && small_fits(cfg); }
+
 // Splits: the widest cluster that every block still has a group of rows for and of which the GPU holds
 // all P at once (a cluster's blocks share one GPC, so that is fewer than SMs / S).
 // The path is taken for models of at most 4096 parameters and, up to what shared memory holds, where
@@ -513,7 +515,7 @@ void small_setup(mavg_ctx* c) {
     cudaGetLastError();
     return;
   }
-  if (cfg.n <= 4096 || (splits >= 4 && cfg.n * cfg.B <= (int64_t)110000 * splits)) c->small_splits = splits;
+  if (small_always(&cfg) || (splits >= 4 && cfg.n * cfg.B <= (int64_t)110000 * splits)) c->small_splits = splits;
 }
 
 cudaError_t small_local_steps(mavg_ctx* c, int64_t round) {
