@@ -1862,8 +1862,7 @@ cudaError_t reb_local_steps(mavg_ctx* c, int64_t round) {
       g.out[l - 1] = k == K ? st->w32[l] : f->w_own_st[l];
     }
     const int units = (P + g.group - 1) / g.group * g.tiles;
-    PdlLaunch l(dim3((unsigned)std::min(units, c->sm_count)), rebuild::kThreads, std::max(rebuild::smem_of(k == K), rebuild::share()),
-                c->stream);
+    PdlLaunch l(dim3((unsigned)std::min(units, c->sm_count)), rebuild::kThreads, rebuild::launch_bytes(k == K), c->stream);
     auto kernel = k == K ? (first.u ? rebuild::k_rebuild<true, true> : rebuild::k_rebuild<false, true>)
                          : (first.u ? rebuild::k_rebuild<true, false> : rebuild::k_rebuild<false, false>);
     prof_begin(c, MAVG_K_WGRAD_SGD);

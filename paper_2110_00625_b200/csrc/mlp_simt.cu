@@ -535,26 +535,12 @@ cudaError_t launch(mavg_ctx* c, int cls, void (*kernel)(Params...), dim3 grid, i
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-constexpr size_t kSplitSmem = split::kSmSharedBytes - split::kBlockReservedBytes - sizeof(split::Barriers);
-
-// What a product's launch asks of an SM.
-struct ProductShape { int stages; uint32_t tmem_cols; size_t smem; };
-ProductShape product_shape(int np, int N) {
-  ProductShape s{0, 32, 0};
-  while ((int)s.tmem_cols < (np == 3 ? 3 : 2) * N) s.tmem_cols <<= 1;
-  const int stage = split::product_stage_bytes(np, N);
-  s.stages = std::min(split::kMaxStages, (int)((kSplitSmem - 1024) / stage));
-  s.smem = std::max((size_t)s.stages * stage, (size_t)(N / 16 + 7) * 16 * split::kTile * 4) + 1024;
-  s.smem = std::max(s.smem, split::tmem_share_bytes(s.tmem_cols, sizeof(split::Barriers)));
-  return s;
-}
-
 // Forward product or data gradient.
 template <bool QUANT, bool DGRAD>
 cudaError_t launch_product(mavg_ctx* c, int cls, int n, const CUtensorMap& w, bool shared_w, const CUtensorMap& x, split::ProductArgs g) {
   constexpr int NP = kPlanes<QUANT>;
   const SimtState* st = (const SimtState*)c->simt;
-  const ProductShape sh = product_shape(NP, st->N);
+  const split::LaunchShape sh = split::product_shape(NP, st->N);
   g.P = st->group;
   g.B = c->cfg.B;
   g.N = st->N;
@@ -601,10 +587,10 @@ cudaError_t set_attributes(const mavg_ctx* c) {
   const mavg_config& cfg = c->cfg;
   const bool tail = product_layers(&cfg) < cfg.n_layers;
   const struct { const void* kernel; size_t smem; bool used; } kernels[] = {
-      {(const void*)split::k_split_product<NP, false>, kSplitSmem, true},
-      {(const void*)split::k_split_product<NP, true>, kSplitSmem, !tail || cfg.n_layers > 2},
-      {(const void*)wgrad_kernel<QUANT>(cfg.B, false), kSplitSmem, true},
-      {(const void*)wgrad_kernel<QUANT>(cfg.B, true), kSplitSmem, c->buf.learner_u != nullptr},
+      {(const void*)split::k_split_product<NP, false>, split::kSmem, true},
+      {(const void*)split::k_split_product<NP, true>, split::kSmem, !tail || cfg.n_layers > 2},
+      {(const void*)wgrad_kernel<QUANT>(cfg.B, false), split::kSmem, true},
+      {(const void*)wgrad_kernel<QUANT>(cfg.B, true), split::kSmem, c->buf.learner_u != nullptr},
       {(const void*)k_simt_begin<QUANT>, 0, true}, {(const void*)k_simt_loss<QUANT>, 0, !tail}, {(const void*)k_simt_tail<QUANT>, kTailSmem, tail}};
   for (const auto& k : kernels) {
     if (!k.used) continue;
@@ -637,7 +623,7 @@ void resident_clusters(int device, int np, int N, int (&resident)[9]) {
       at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
       lc.gridDim = dim3((unsigned)s);
       lc.blockDim = dim3(split::kProductThreads);
-      lc.dynamicSmemBytes = product_shape(np, N).smem;
+      lc.dynamicSmemBytes = split::product_shape(np, N).smem;
       lc.attrs = at;
       lc.numAttrs = 1;
       const cudaError_t e = np == 1 ? cudaOccupancyMaxActiveClusters(&got[s], split::k_split_product<1, false>, &lc)
@@ -782,11 +768,10 @@ cudaError_t step_impl(mavg_ctx* c, int64_t round, int step, int p0, int n) {
   w.loss_out = (float*)ws_ptr(c, c->ws.losses) + (size_t)p0 * cfg.K + (step - 1);
   w.loss_stride = cfg.K;
   w.status = (int*)ws_ptr(c, c->ws.status);
-  w.stages = std::min(split::kMaxStages, (int)((kSplitSmem - 1024) / split::wgrad_stage_bytes(NP)));
-  const size_t smem = std::max((size_t)w.stages * split::wgrad_stage_bytes(NP) + 1024,
-                               split::tmem_share_bytes(NP == 3 ? 512 : 256, sizeof(split::Barriers)));
+  const split::LaunchShape shape = split::wgrad_shape(NP);
+  w.stages = shape.stages;
   return launch(c, MAVG_K_WGRAD_SGD, wgrad_kernel<QUANT>(B, mom.u != nullptr), dim3((unsigned)std::min(w.tiles, c->sm_count)),
-                split::wgrad_threads(split::wgrad_chains(NP, B)), 1, smem, w);
+                split::wgrad_threads(split::wgrad_chains(NP, B)), 1, shape.smem, w);
 }
 
 }  // namespace

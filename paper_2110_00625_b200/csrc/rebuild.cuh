@@ -73,8 +73,11 @@ __device__ __forceinline__ void drain_copies(uint64_t* full, int issued, int sta
   }
 }
 
-// Dynamic shared memory for the same share of an SM as of its tensor memory, of which a block takes all.
-inline size_t share() { return tmem_share_bytes(512, sizeof(Shared)); }
+// Dynamic shared memory of a launch: at least the same share of an SM as of its tensor memory, of which a block takes all.
+inline size_t launch_bytes(bool last) {
+  const size_t share = tmem_share_bytes(512, sizeof(Shared));
+  return smem_of(last) > share ? smem_of(last) : share;
+}
 
 // Persistent over units: a tile of 128 x 128 weights for `group` learners, whose w~ stays in the epilogue's registers (a
 // fetch of w~ for every learner is 4 bytes per weight more, twice what leaves in steps 1 .. K-1 without momentum).

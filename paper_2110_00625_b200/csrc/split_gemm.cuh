@@ -11,6 +11,8 @@
 #pragma once
 #include <cuda.h>
 
+#include <algorithm>
+
 #include "common.cuh"
 #include "tc_ptx.cuh"
 
@@ -691,6 +693,21 @@ k_split_wgrad(const __grid_constant__ WgradArgs g) {
   __syncthreads();
   if (warp == 1) tmem_dealloc(tmem_base, NP == 3 ? 512 : 256);
 }
+
+// What a launch asks of an SM.
+constexpr size_t kSmem = kSmSharedBytes - kBlockReservedBytes - sizeof(Barriers);
+struct LaunchShape { int stages; uint32_t tmem_cols; size_t smem; };
+inline LaunchShape launch_shape(int stage_bytes, uint32_t tmem_cols, size_t least) {
+  LaunchShape s{std::min(kMaxStages, (int)((kSmem - 1024) / stage_bytes)), tmem_cols, 0};
+  s.smem = std::max({(size_t)s.stages * stage_bytes + 1024, least, tmem_share_bytes(tmem_cols, sizeof(Barriers))});
+  return s;
+}
+inline LaunchShape product_shape(int np, int N) {
+  uint32_t cols = 32;
+  while ((int)cols < (np == 3 ? 3 : 2) * N) cols <<= 1;
+  return launch_shape(product_stage_bytes(np, N), cols, (size_t)(N / 16 + 7) * 16 * kTile * 4 + 1024);   // the sums a block receives
+}
+inline LaunchShape wgrad_shape(int np) { return launch_shape(wgrad_stage_bytes(np), np == 3 ? 512 : 256, 0); }
 
 // The weights that a call's first step finds, as planes: a warp per row of a matrix.
 struct SplitWeights {

@@ -339,6 +339,7 @@ def _fused_handle(dims, K, **kw):
     g = m.Mavg(w1, P=FUSED_P, K=K, local_lr=cfg["gamma"], mu=cfg["mu"], B=FUSED_B,
                seed=m.workloads.BASE_SEED, objective=m.OBJ_MLP, dims=dims, gemm_bf16=1,
                x=x, y=y, x_bf16=True, **kw)
+    assert not g.rebuilt()                # rounds without weight gradients that a product could ride on
     return g, cfg, x, y, w1
 
 

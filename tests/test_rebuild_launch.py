@@ -14,7 +14,7 @@ MAIN = r'''
 using namespace mavg;
 int main() {
   for (bool last : {false, true})
-    printf("%zu %zu %zu\n", sizeof(rebuild::Shared), std::max(rebuild::smem_of(last), rebuild::share()), tc::tmem_share_bytes(32, 0));
+    printf("%zu %zu %zu %zu\n", sizeof(rebuild::Shared), rebuild::launch_bytes(last), rebuild::smem_of(last), tc::tmem_share_bytes(32, 0));
 }
 '''
 
@@ -27,8 +27,8 @@ def test_its_shared_memory_is_its_share_of_an_sm(tmp_path):
     src.write_text(MAIN)
     subprocess.run([B.NVCC, *B.FLAGS, "-I", CSRC, str(src), "-o", str(exe)], check=True)
     for line in subprocess.run([str(exe)], capture_output=True, text=True, check=True).stdout.splitlines():
-        fixed, dynamic, least = map(int, line.split())
-        assert fixed % 16 == 0 and fixed + dynamic <= 227 * 1024
+        fixed, dynamic, used, least = map(int, line.split())
+        assert fixed % 16 == 0 and fixed + dynamic <= 227 * 1024 and used <= dynamic
         # all 512 columns: beside it not even a block of the fewest columns fits
         assert fixed + dynamic + 1024 + least + 1024 > 228 * 1024
 
@@ -38,5 +38,3 @@ def test_it_takes_its_columns_before_the_next_kernel_may_begin():
     body = text[text.index("tmem_alloc("):text.index("tmem_dealloc(")]
     assert body.index("grid_launch_dependents()") < body.index("grid_dependency_wait()")
     assert text.count("tmem_alloc(") == 1
-    host = open(os.path.join(CSRC, "factored.cu")).read()
-    assert "std::max(rebuild::smem_of(k == K), rebuild::share())" in host
