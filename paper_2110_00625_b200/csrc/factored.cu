@@ -55,16 +55,6 @@ __device__ __forceinline__ void part_mma(uint32_t d, uint64_t adesc, uint32_t a_
 }
 constexpr uint32_t kStepK = 2, kStepMn = (16 * 128) >> 4;
 
-// Copies that were issued before a wait was given up get a bounded chance to land before the block retires:
-// the last `stages` of `issued`.
-__device__ __forceinline__ void drain_ring(uint64_t* full_bar, int issued, int stages, const int* status) {
-  for (int i = max(0, issued - stages); i < issued; ++i) {
-    const uint64_t t0 = global_timer_ns();
-    while (!mbar_try_wait(&full_bar[i % stages], (i / stages) & 1))
-      if (global_timer_ns() - t0 > wait_limit_ns(status)) break;
-  }
-}
-
 // ------------------------------------------------------------------------------------- gather
 
 template <typename TIN>
@@ -323,7 +313,7 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
             tma_load_3d(sa + kBOff + h * s_bytes, &tm_s, full, (i + h) * kBK, s_row, p0 + q);
           }
         }
-      if (*abortp) drain_ring(sh.full_bar, issued, stages, g.status);
+      if (*abortp) drain_copies(sh.full_bar, issued, stages, g.status);
     }
     __syncwarp();
   } else if (warp == 1) {
@@ -641,7 +631,7 @@ k_fac_gram(const __grid_constant__ CUtensorMap tm_hist, const __grid_constant__ 
         tma_load_3d(sa, &tm_hist, full, i * kBK, s0, p);
         tma_load_3d(sa + kATileBytes, &tm_b, full, i * kBK, r0, p);
       }
-      if (*abortp) drain_ring(sh.full_bar, issued, stages, g.status);
+      if (*abortp) drain_copies(sh.full_bar, issued, stages, g.status);
     }
     __syncwarp();
   } else if (warp == 1) {
@@ -1039,7 +1029,7 @@ k_fac_apply(const __grid_constant__ ApplyArgs g) {
             tma_load_3d(sa + kATileBytes + h * 8192, tm_b, full, n0 + 64 * h, i * kBK, p);
         }
       }
-      if (*abortp) drain_ring(sh.full_bar, issued, STAGES, g.status);
+      if (*abortp) drain_copies(sh.full_bar, issued, STAGES, g.status);
     }
     __syncwarp();
   } else if (warp == 1) {
@@ -1139,7 +1129,7 @@ k_fac_apply(const __grid_constant__ ApplyArgs g) {
     }
     if (leader) {
       tma_store_wait_read<0>();
-      if (*abortp) drain_ring(sh.piece_full[grp], (int)fn, PIECES, g.status);
+      if (*abortp) drain_copies(sh.piece_full[grp], (int)fn, PIECES, g.status);
     }
   }
   tc_fence_before_sync();

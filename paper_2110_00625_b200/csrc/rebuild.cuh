@@ -65,14 +65,6 @@ struct alignas(16) Shared {                       // (whole 16 bytes, as static 
   int fetch_unit[kGroups], fetch_p[kGroups], fetched[kGroups];   // a group's place in its list of pieces to fetch
 };
 
-__device__ __forceinline__ void drain_copies(uint64_t* full, int issued, int stages, const int* status) {
-  for (int i = max(0, issued - stages); i < issued; ++i) {
-    const uint64_t t0 = global_timer_ns();
-    while (!mbar_try_wait(&full[i % stages], (i / stages) & 1))
-      if (global_timer_ns() - t0 > wait_limit_ns(status)) break;
-  }
-}
-
 // Dynamic shared memory of a launch: at least the same share of an SM as of its tensor memory, of which a block takes all.
 inline size_t launch_bytes(bool last) {
   const size_t share = tmem_share_bytes(512, sizeof(Shared));

@@ -126,15 +126,6 @@ __device__ __forceinline__ void init_barriers(Barriers& sh, int stages, int epil
   fence_barrier_init();
   fence_proxy_async();
 }
-// Copies in flight when a wait was given up get a bounded chance to land before the block retires.
-__device__ __forceinline__ void drain_copies(Barriers& sh, int issued, int stages, const int* status) {
-  for (int i = max(0, issued - stages); i < issued; ++i) {
-    const uint64_t t0 = global_timer_ns();
-    while (!mbar_try_wait(&sh.full[i % stages], (i / stages) & 1))
-      if (global_timer_ns() - t0 > wait_limit_ns(status)) break;
-  }
-}
-
 // This thread's sums: tensor-memory lane 32 (warp % 4) + lane, 16 of every STEP columns.
 template <int STEP>
 struct Sums {
@@ -238,7 +229,7 @@ k_split_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant_
           tma_load_3d(sa + NP * kTileBytes + (size_t)q * N * kSlab * 2, &tm_x, &sh.full[s], k0, n0, q * g.P + p);
         }
       }
-      if (*abortp) drain_copies(sh, issued, stages, g.status);
+      if (*abortp) drain_copies(sh.full, issued, stages, g.status);
     }
     __syncwarp();
   } else if (warp == 1) {
@@ -520,7 +511,7 @@ k_split_wgrad(const __grid_constant__ WgradArgs g) {
           }
         }
       }
-      if (*abortp) drain_copies(sh, issued, stages, g.status);
+      if (*abortp) drain_copies(sh.full, issued, stages, g.status);
     }
     __syncwarp();
   } else if (warp == 1) {

@@ -75,6 +75,15 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volati
   return true;
 }
 
+// Copies in flight when a wait was given up get a bounded chance to land before the block retires.  full: the ring's barriers.
+__device__ __forceinline__ void drain_copies(uint64_t* full, int issued, int stages, const int* status) {
+  for (int i = max(0, issued - stages); i < issued; ++i) {
+    const uint64_t t0 = global_timer_ns();
+    while (!mbar_try_wait(&full[i % stages], (i / stages) & 1))
+      if (global_timer_ns() - t0 > wait_limit_ns(status)) break;
+  }
+}
+
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
