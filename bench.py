@@ -700,8 +700,8 @@ def run_mavg(args):
             "vs_baseline": None, "dtype": "bf16" if r["mode"] else "f32", "data": "synthetic",
             "config": {"workload": workload_label(args.workload, cfg),
                        "global_batch": cfg["P"] * cfg["B"], "parallelism": "replicas only",
-                       "gemm": {1: "tcgen05 tensor cores", 2: "CUDA cores, bf16-rounded operands",
-                                0: "CUDA cores fp32"}[r["mode"]],
+                       "gemm": {1: "tcgen05 tensor cores", 2: "tcgen05 or CUDA cores by size, bf16-rounded operands",
+                                0: "fp32: three bf16 planes on tcgen05, or CUDA cores by size"}[r["mode"]],
                        "defer_broadcast": not args.no_defer, "learner_momentum": args.beta,
                        "l2_keep": bool(args.l2_keep),
                        "schedule": {0: "CUDA graph of per-product launches",
@@ -749,7 +749,7 @@ def main():
     ap.add_argument("--warmup", type=int, default=3)
     ap.add_argument("--impl", default="mavg", choices=["mavg", "reference"])
     ap.add_argument("--gemm", type=int, default=1, choices=[1, 2],
-                    help="1: tensor cores (default); 2: CUDA cores with bf16-rounded operands")
+                    help="1: tensor cores (default); 2: bf16-rounded operands, any shape")
     ap.add_argument("--workload", default=WORKLOAD, choices=["C2", "C4", "C5"],
                     help="C4 (large MLP) is the benchmark workload; C2 (CIFAR-shaped MLP) as the "
                          "main workload, or C5 (pseudo-gradient round at 25.6 M parameters) alone")

@@ -85,7 +85,9 @@ typedef struct {
    * [W_1 (dims[1] x dims[0], row-major), b_1, W_2, b_2, ...]. */
   int32_t n_layers;
   int32_t dims[MAVG_MAX_LAYERS + 1];
-  int32_t gemm_bf16; /* 0: fp32 FMA arithmetic throughout.  1: every matrix-product operand
+  int32_t gemm_bf16; /* 0: fp32 operands and sums throughout (in matrix products each operand as the sum of
+                        three bf16 numbers, which holds it exactly from 2^-110 up; of a product at most about
+                        2^-24 is left out).  1: every matrix-product operand
                         (weights, activations, dZ) rounded to bf16 (nearest-even), fp32
                         accumulation, fp32 master weights, bias, ReLU, softmax and SGD in fp32 */
   float pseudo_grad_sigma; /* PSEUDOGRAD: standard deviation of the variates */
@@ -103,7 +105,7 @@ typedef struct {
                         and the next local step the replica array then holds the previous round's
                         learner models; mavg_materialize_replicas writes the copies on request.
                         What a program writes into the replica rows between two rounds: an MLP handle
-                        on the CUDA cores (gemm_bf16 0 or 2) starts its learners from the rows
+                        with gemm_bf16 0 or 2 starts its learners from the rows
                         wherever they hold the copies (always with 0, after
                         mavg_materialize_replicas with 1); a tensor-core or pseudo-gradient handle
                         starts them from w~. */
@@ -258,7 +260,7 @@ typedef enum {
   MAVG_K_LOSS = 5,      /* softmax cross-entropy and loss reductions; the fused last-layer kernel */
   MAVG_K_DGRAD = 6,     /* backward-data GEMMs (+ReLU mask, bias step) */
   MAVG_K_WGRAD_SGD = 7, /* backward-weight GEMMs fused with the SGD step; all K local steps of a
-                           small CUDA-core model, which are one launch */
+                           small model (gemm_bf16 0 or 2), which are one launch */
   MAVG_K_AUX = 8,       /* operand copies (bf16 shadows) */
   MAVG_K_COUNT = 9
 } mavg_kernel_class;
@@ -285,7 +287,7 @@ mavg_status mavg_set_profiling(mavg_handle h, int32_t on);
  *     tensor-core launches.  Apart from factored rounds the two differ in the
  *     summation order of the products they run differently, nothing else; this one exists for comparison.
  * Profiled rounds (mavg_set_profiling) take the launch-by-launch form of the chosen schedule; what is
- * one launch without profiling (the steps of a small CUDA-core model, a pseudo-gradient round) is one
+ * one launch without profiling (the steps of a small model, a pseudo-gradient round) is one
  * launch with it. */
 typedef enum { MAVG_SCHED_GRAPH = 0, MAVG_SCHED_GRAPH_TC = 2 } mavg_schedule;
 mavg_status mavg_set_schedule(mavg_handle h, int32_t mode);

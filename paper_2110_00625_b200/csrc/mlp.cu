@@ -1,5 +1,5 @@
 // MLP learner level: layout bookkeeping and the per-round loop over the K local steps of
-// Algorithm 1, dispatching each step to the tensor-core or the CUDA-core kernels.
+// Algorithm 1, dispatched to the bf16 tensor-core path, the path for fp32 and any shapes, or the small-model kernel.
 #include "mlp.cuh"
 
 namespace mavg {
@@ -134,7 +134,7 @@ cudaError_t mlp_local_steps(mavg_ctx* c, int64_t round) {
   // start elsewhere (local steps called twice in a row), profiled rounds and handles whose
   // capture failed once take the launch-by-launch path.
   if (c->small_splits) return small_local_steps(c, round);
-  // The graph of a CUDA-core handle reads w~ with defer_broadcast and the replica array without; a
+  // The graph of an fp32 or odd-shaped model reads w~ with defer_broadcast and the replica array without; a
   // deferred round whose copies were written on request starts from them, outside the graph.
   const bool usual_start = c->replicas_equal_global &&
                            (use_tensor_cores(&c->cfg) || c->replicas_materialized == !c->cfg.defer_broadcast);

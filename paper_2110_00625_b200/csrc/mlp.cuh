@@ -18,7 +18,7 @@ __device__ __forceinline__ int32_t sample_index(uint64_t seed, int64_t round, in
   return (int32_t)(lo + (int64_t)((u * (uint64_t)(hi - lo)) >> 32));
 }
 
-// Where the CUDA-core paths find the learners' models at the start of a round: in w~ while a deferred
+// Where the paths of gemm_bf16 0 and 2 find the learners' models at the start of a round: in w~ while a deferred
 // re-broadcast has not been carried out, in the replica array otherwise (whose rows a program may have
 // edited since they were written).
 inline bool starts_from_global(const mavg_ctx* c) {

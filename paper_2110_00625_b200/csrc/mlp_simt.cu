@@ -5,9 +5,9 @@
 //   SGD       W_l <- W_l - gamma dW_l, b_l <- b_l - gamma db_l    (Algorithm 1's local update)
 // The products run on tcgen05 with fp32 operands as three bf16 planes, or with QUANT on the operands rounded to bf16
 // (nearest-even) as one, which makes this path compute the same thing as the tensor-core path (split_gemm.cuh).
-// Rounds of 3072-512-512-10, P = 4, K = 4, B = 100 in fp32: 380 us, 570 with chains of FMAs on the CUDA cores (53 us for
+// Rounds of 3072-512-512-10, P = 4, K = 4, B = 100 in fp32: 366 us, 570 with chains of FMAs on the CUDA cores (53 us for
 // layer 1's forward product, 22 here; 55 for the weight gradients, 24 to 32 here); 1000-333-100, P = 6, K = 4, B = 50 with
-// bf16 operands: 140 us, 170 with warp-level MMAs.  Relative error of one step's gradients against 64 bits (2-norm, weight
+// bf16 operands: 127 us, 170 with warp-level MMAs.  Relative error of one step's gradients against 64 bits (2-norm, weight
 // matrices of layers 1, 2, .. in units of 1e-7, FMA chains / here): 3072-512-512-10, B = 100 2.8 3.2 2.8 / 1.8 1.8 2.4;
 // inputs in [0, 1] 1.9 2.8 2.8 / 1.9 1.8 1.9, B = 192 2.3 2.8 2.9 / 1.6 1.5 1.6, B = 256 2.4 2.9 2.8 / 1.9 1.8 1.9, B = 300
 // 2.6 3.0 3.0 / 1.7 1.6 1.6; 2900-130-800-77, B = 31 2.8 3.8 3.4 / 2.1 2.4 2.1; 1501-799-99, B = 129 2.5 2.8 / 1.9 2.0;

@@ -491,10 +491,13 @@ bool small_always(const mavg_config* cfg) { return cfg->n <= 4096 && small_fits(
 // all P at once (a cluster's blocks share one GPC, so that is fewer than SMs / S).
 // The path is taken for models of at most 4096 parameters and, up to what shared memory holds, where
 // at least four blocks share a learner and a block's products are at most 110 000 multiply-adds each.
-// Measured against a launch per product, K = 4, us a round: 32-64-10, B = 32: P = 4 43 / 64, P = 100
-// 84 / 158, P = 300 226 / 358; 80-128-16, B = 32, P = 4 (8 blocks, 50 000) 66 / 84; 80-128-128-16,
-// B = 32, P = 4 (116 000) 109 / 147; beyond the line 80-128-16, B = 48, P = 16 (149 000) 105 / 100;
-// with one block a learner 80-128-16, B = 4 94 / 74, and 80-128-128-16, B = 16, P = 300 833 / 535.
+// Measured against a launch per product, 150 models with K = 1, 4 or 8 and P = 1 .. 300: up to 4096 parameters 1.18 .. 4.3
+// times as fast (32-64-10, K = 4, B = 32, us a round: P = 4 32 / 75, P = 100 78 / 165, P = 300 179 / 423); beyond, in fp32
+// 1.00 .. 2.6 (80-128-16, B = 32, P = 4 55 / 83; B = 48, P = 16, 74 600 a block, 95 / 94); with bf16 operands, whose
+// launches have a plane to each operand, 1.03 .. 1.6 up to 25 000 a block and 0.76 .. 1.25 above (52-112-126-10, P = 8,
+// K = 4, B = 20 148 / 112).  What the lines leave to the launches would be 0.60 .. 2.3 with one to three blocks a learner
+// (80-128-128-16, B = 16, P = 300 800 / 569; 78-57-13, P = 123, K = 8, B = 61 251 / 575) and 1.2 beyond 110 000
+// (80-128-128-16, B = 32, P = 4 107 / 129).
 // A device or driver that refuses one of the calls here leaves the handle the launch per product.
 void small_setup(mavg_ctx* c) {
   const mavg_config& cfg = c->cfg;

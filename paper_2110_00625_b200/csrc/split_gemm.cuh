@@ -1,7 +1,7 @@
 // Matrix products of models whose widths, batch or arithmetic the bf16 path does not take (mlp_simt.cu), on
-// tcgen05.  An fp32 operand is the exact sum of three bf16 numbers, x = x0 + x1 + x2 (NP = 3 planes); of the nine
-// products of two such sums the six largest are formed, x0 y0 in one accumulator and the other five in another, and
-// what is left out is below 2^-25 of |x| |y|.  With bf16 operands (NP = 1) there is one plane and one accumulator.
+// tcgen05.  An fp32 operand is the sum of three bf16 numbers, x = x0 + x1 + x2 (NP = 3 planes), exactly from 2^-110
+// up; of the nine products of two such sums the six largest are formed, x0 y0 in one accumulator and the other five in
+// another, and what is left out, x1 y2 + x2 y1 + x2 y2, is at most about 2^-24 of |x| |y|.  With bf16 operands (NP = 1) there is one plane and one accumulator.
 // The tensor cores cut a sum off where they add to it, always towards zero, so an accumulator takes one slab of 64
 // contraction elements (of a weight gradient two or four); the epilogue warps then add it to fp32 registers, rounded to
 // nearest, while the next goes into the other accumulator.  Against 64 bits: see mlp_simt.cu.
