@@ -8,17 +8,20 @@ import torch
 pytestmark = pytest.mark.gpu
 
 
-def _run(dims, P, K, B, beta, reset, defer, calls, rebuilt, how):
+def _run(dims, P, K, B, beta, reset, defer, calls, rebuilt, how, odd=(), with_u=False):
     """The state after `calls`.  The plain form of the same settings: a handle made for one step (how == "steps"), without
     the momentum that would make it one for rebuilt steps ("momentum"), or the plain tiles where these sum alike ("tiles")."""
     import paper_2110_00625_b200 as m
     gen = torch.Generator(device="cuda").manual_seed(0)
     x = torch.randn(4000, dims[0], generator=gen, device="cuda")
     y = torch.randint(0, dims[-1], (4000,), generator=gen, device="cuda").int()
+    w1 = m.workloads.mlp_init(dims)
+    for at, value in odd:
+        w1[at] = value
     late_momentum, late_steps = not rebuilt and how == "momentum", not rebuilt and how == "steps"
-    g = m.Mavg(m.workloads.mlp_init(dims), P=P, K=1 if late_steps else K, local_lr=0.002, mu=0.9, B=B, seed=3,
+    g = m.Mavg(w1, P=P, K=1 if late_steps else K, local_lr=0.002, mu=0.9, B=B, seed=3,
                objective=m.OBJ_MLP, dims=dims, gemm_bf16=1, x=x, y=y, x_bf16=True, defer_broadcast=defer,
-               learner_momentum=0.0 if late_momentum else beta, learner_momentum_reset=reset, with_learner_u=beta != 0)
+               learner_momentum=0.0 if late_momentum else beta, learner_momentum_reset=reset, with_learner_u=with_u or beta != 0)
     if late_steps:
         g.set_hparams(K, 0.002, 1.0, 0.9)
     if late_momentum:
@@ -67,6 +70,31 @@ def test_the_steps_are_the_plain_ones(dims, P, K, B, beta, reset, defer, calls, 
     got, want = (_run(dims, P, K, B, beta, reset, defer, calls, rebuilt, how) for rebuilt in (True, False))
     for a, b in zip(got, want):
         assert torch.equal(a, b)
+
+
+def _profiled(g):
+    g.set_profiling(True)
+    _rounds(g)
+
+
+@pytest.mark.parametrize("dims,P,K,B,beta,how", [([3072, 1024, 512, 10], 10, 4, 64, 0.9, "momentum"),
+                                                 ([1120, 1304, 1304, 1304, 10], 10, 6, 16, 0.0, "steps")])
+def test_launch_by_launch_and_with_a_buffer_for_momentum(dims, P, K, B, beta, how):
+    want = _run(dims, P, K, B, beta, False, True, _rounds, False, how)
+    for calls, with_u in ((_profiled, False), (_rounds, True)):
+        for a, b in zip(_run(dims, P, K, B, beta, False, True, calls, True, how, with_u=with_u), want):
+            assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("dims,P,K,B,beta,how", [([3072, 1024, 512, 10], 10, 3, 64, 0.9, "momentum"),
+                                                 ([1416, 1800, 1800, 1800, 32], 7, 2, 48, 0.0, "steps")])
+@pytest.mark.parametrize("value", [float("inf"), float("-inf"), float("nan"), 3.4e38])
+def test_what_is_not_finite_spreads_as_in_the_plain_form(dims, P, K, B, beta, how, value):
+    odd = [(7 * dims[0] + 5, value), (dims[1] * (dims[0] + 1) + 11 * dims[1] + 3, value)]   # in W_1 and W_2
+    got, want = (_run(dims, P, K, B, beta, False, True, lambda g: g.round(), rebuilt, how, odd) for rebuilt in (True, False))
+    assert not all(torch.isfinite(t).all() for t in want)
+    for a, b in zip(got, want):
+        assert torch.equal(a.isnan(), b.isnan()) and torch.equal(a.nan_to_num(nan=0.0), b.nan_to_num(nan=0.0))
 
 
 def test_by_the_momentum_and_steps_of_now():
