@@ -28,7 +28,7 @@ using namespace tc;
 using namespace gemm;
 
 constexpr int kFacThreads = 320;   // warp 0: TMA producer, warp 1: MMA issuer, warps 2-9: epilogue
-enum { PROD_FWD = 0, PROD_DGRAD = 1, PROD_RAW = 2, PROD_DGRAD_STEP = 3 };
+enum { PROD_FWD = 0, PROD_DGRAD = 1, PROD_RAW = 2, PROD_DGRAD_STEP = 3, PROD_FWD_RUNS = 4 };
 constexpr size_t kGramBarBytes = 2 * sizeof(uint64_t);   // static shared memory of a product that forms its Gram rows, beside GemmShared
 
 // Place in a ring of stages and the phase of its barriers, without a division per slab: the one thread that
@@ -153,6 +153,9 @@ struct ProdArgs {
   int row_end;              // RAW: rows per learner
   int nkb;                  // slabs of the product with w~ (0: left out)
   int w_batched;            // the weights are each learner's own (one learner per block)
+  // PROD_FWD_RUNS: sums of `run` groups of 16 contraction elements each, `runs` of them, added in ascending order; the first
+  // whole_rows pairs of learner and row tile take one sum
+  int run, runs, whole_rows;
   int hist;                 // rows of the earlier steps (0: left out)
   int s_row0;               // row of the batch inside a learner's Gram rows
   int stages;
@@ -223,6 +226,7 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
   // tiles' places, with their Gram rows where the batch operand is.
   static_assert(!LOW || TILES == 2, "");
   constexpr bool kStep = EPI == PROD_DGRAD_STEP, kMn = EPI == PROD_DGRAD || kStep;   // kMn: the weights are read MN-major
+  constexpr bool kRuns = EPI == PROD_FWD_RUNS, kFwd = EPI == PROD_FWD || kRuns;
   constexpr int kBOff = TILES * kATileBytes;
   const int stage_bytes = product_stage_bytes(TILES, EPI == PROD_RAW ? 1 : TILES, g.nl, g.cols), s_bytes = g.cols * kBK * 2;
   __shared__ __align__(8) uint64_t gram_bar, rows_bar;     // GRAM: Gram sums complete; Gram rows in global memory
@@ -264,6 +268,7 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
   volatile int* abortp = &sh.abort_flag;
   const bool any = g.nkb > 0 || g.hist > 0;
   const int w_of = g.w_batched ? p0 : 0;
+  const int runs = kRuns && p0 * g.m_tiles + m_tile >= g.whole_rows ? g.runs : 1;
   const int gram_step = kBM * g.m_tiles;           // from one of this block's Gram tiles to the next, in rows
 
   if (warp == 0) {
@@ -344,7 +349,14 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
         if (!(ok = mbar_wait(&sh.full_bar[ring.s], ring.ph, abortp, g.status, ERR_MMA))) break;
         tc_fence_after_sync();
         const uint32_t off = (uint32_t)ring.s * unit;
-        slab_mma(tmem_base, a_base + off, kStepA, b_base + off, kStepK, idesc_base, i > 0);
+        if (kRuns && runs > 1) {
+          for (int k = 0; k < kBK / 16; ++k) {       // (what lies behind the last run's elements is zero)
+            const int at = i * (kBK / 16) + k, r = min(at / g.run, runs - 1);
+            umma_bf16(tmem_base + (uint32_t)(r * N), a_base + off + kStepA * k, b_base + off + kStepK * k, idesc_base, (uint32_t)(at > r * g.run));
+          }
+        } else {
+          slab_mma(tmem_base, a_base + off, kStepA, b_base + off, kStepK, idesc_base, i > 0);
+        }
         if (LOW) slab_mma(tmem_base + g.low_col, a_base + off + (kATileBytes >> 4), kStepA, b_base + off, kStepK, idesc_base, i > 0);
         umma_commit(&sh.empty_bar[ring.s]);
       }
@@ -404,7 +416,7 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
     // What a group of columns needs besides the accumulator (the fp32 base of layer 1, the activations that
     // gate dZ) is in flight while the group before it, or the main loop, is still at work.
     const int end = EPI == PROD_RAW ? min(g.cols, g.row_end - r0) : nl * g.cols;
-    const bool add_base = EPI == PROD_FWD && g.zbase != nullptr;
+    const bool add_base = kFwd && g.zbase != nullptr;
     float zb[16], bias_next = 0.f;
     __nv_bfloat16 act[16];
     auto locate = [&](int c0, size_t& at, size_t& z_at, int& q) {
@@ -418,7 +430,7 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
       int q;
       if (!m_ok || c0 >= end) return;
       locate(c0, at, z_at, q);
-      if (EPI == PROD_FWD) bias_next = g.bias_in[(size_t)(p0 + q) * g.bias_in_stride + g.bias_off + m];
+      if (kFwd) bias_next = g.bias_in[(size_t)(p0 + q) * g.bias_in_stride + g.bias_off + m];
       if (add_base) {
 #pragma unroll
         for (int j = 0; j < 16; ++j) zb[j] = __ldg(g.zbase + z_at + (size_t)j * g.M);
@@ -492,13 +504,22 @@ k_fac_product(const __grid_constant__ CUtensorMap tm_w, const __grid_constant__ 
         locate(c0, at, z_at, q);
         float z[16];
         load16(lane_addr + (uint32_t)c0, any, z);
+        if (kRuns && runs > 1) {
+#pragma unroll 1
+          for (int r = 1; r < runs; ++r) {
+            float t[16];
+            load16(lane_addr + (uint32_t)(r * N + c0), true, t);
+#pragma unroll
+            for (int j = 0; j < 16; ++j) z[j] += t[j];
+          }
+        }
         if (LOW) {
           float low[16];
           load16(lane_addr + g.low_col + (uint32_t)c0, any, low);
 #pragma unroll
           for (int j = 0; j < 16; ++j) z[j] = with_low(z[j], low[j]);
         }
-        if (EPI == PROD_FWD) {
+        if (kFwd) {
 #pragma unroll
           for (int j = 0; j < 16; ++j) z[j] = (add_base ? z[j] + zb[j] : z[j]) + bias_next;
           fetch(c0 + 32);
@@ -1224,10 +1245,10 @@ cudaError_t launch_product(mavg_ctx* c, int cls, const CUtensorMap& w, const CUt
   const int stage_bytes = product_stage_bytes(TILES, EPI == PROD_RAW ? 1 : TILES, g.nl, g.cols);
   const dim3 grid((unsigned)(g.m_tiles * g.c_tiles), (unsigned)((g.P + g.nl - 1) / g.nl));
   const int hist_stages = ((g.hist + kBK - 1) / kBK + TILES - 1) / TILES;
-  g.stages = stages_for(std::max(1, g.gram_nkb + g.nkb + g.nl * hist_stages), stage_bytes, (long)grid.x * grid.y,
-                        c->sm_count);
   g.low_col = (uint32_t)(GRAM ? gram_columns(g.cols, g.m_tiles, g.hist) : g.nl * g.cols);
-  g.tmem_cols = tmem_columns((int)g.low_col + (LOW ? g.nl * g.cols : 0));
+  g.tmem_cols = tmem_columns(EPI == PROD_FWD_RUNS ? g.runs * g.cols : (int)g.low_col + (LOW ? g.nl * g.cols : 0));
+  g.stages = stages_for(std::max(1, g.gram_nkb + g.nkb + g.nl * hist_stages), stage_bytes,
+                        EPI == PROD_FWD_RUNS && g.tmem_cols > 256 ? 1 : (long)grid.x * grid.y, c->sm_count);
   size_t smem = (size_t)g.stages * stage_bytes + 1024 +
                 (EPI == PROD_DGRAD || EPI == PROD_DGRAD_STEP ? (size_t)2 * g.nl * kBM * sizeof(float) : 0);
   const int cluster = GRAM ? (int)grid.x : EPI == PROD_DGRAD ? g.c_tiles : 1;
@@ -1639,8 +1660,8 @@ cudaError_t fac_local_steps(mavg_ctx* c, int64_t round) {
 //   with momentum (all steps' accumulators at once: K <= 4)   V >= 20 M: 1.003 .. 1.57; V = 12 .. 20 M: 0.92 .. 1.31
 //   without, V >= 48 M        K <= 4: 1.07 .. 1.50; K = 5, 6: 1.05 .. 1.21 up to 384 rows a learner, 0.969 at 480
 //            V = 20 .. 48 M   K <= 4: 0.949 .. 1.36; K = 5, 6: 0.866 .. 1.24
-// Where the forward products ride on the weight gradients in place, K = 5 takes 1.02 and 1.04 times as long rebuilt:
-// four steps at most there (reb_usable).
+// Where the forward products ride on the weight gradients in place (280 shapes more): with momentum 1.07 .. 1.44; without
+// K = 2, 3 1.04 .. 1.51, K = 4 1.09 .. 1.22 up to 64 batch rows and 0.897 .. 1.08 above, K = 5 0.965 and 0.981 (reb_riding).
 int reb_steps(const mavg_config* cfg) {
   const int L = cfg->n_layers, B = cfg->B;
   const bool momentum = cfg->learner_momentum != 0.f;
@@ -1650,6 +1671,10 @@ int reb_steps(const mavg_config* cfg) {
   if (cfg->P * weights < (momentum ? 20 : 48) * 1000 * 1000) return 0;
   const int most = std::min({cfg->K, 512 / B, momentum || cfg->K * B > 384 ? 4 : 6});
   return most >= 2 ? most : 0;
+}
+
+bool reb_riding(const mavg_config* cfg) {
+  return cfg->learner_momentum != 0.f || cfg->K <= 3 || (cfg->K == 4 && cfg->B <= 64);
 }
 
 bool reb_reserved(const mavg_config* cfg) { return reb_steps(cfg) == cfg->K && !fac_reserved(cfg); }
@@ -1688,8 +1713,8 @@ void reb_setup(mavg_ctx* c, TcState* st) {
     const int pitch = (int)up((size_t)d, 8);
     ok = ok && encode_map(st, m, at, d, B, n, pitch, (int64_t)B * pitch, box_rows, why, box_learners);
   };
-  // Products of k_fac_product where it sums in the plain form's order: over the whole contraction, and for a bias step
-  // over the whole batch; the others are the plain form's launches, whose data gradients read A_{l-1} transposed.
+  // Products of k_fac_product where it sums in the plain form's order: over the whole contraction, or over the runs of a
+  // product that rides on a weight gradient there, and for a bias step over the whole batch; the others are the plain form's launches, whose data gradients read A_{l-1} transposed.
   // (3072-2048-2048-2048-10, P = 8, B = 64: data gradients of a step 50 us, 57 as the plain form's launches; 1080-576-576-32,
   // P = 26, B = 176 27 and 32.)
   for (int l = 2; l <= L; ++l) {
@@ -1704,10 +1729,12 @@ void reb_setup(mavg_ctx* c, TcState* st) {
     f->fwd[l] = cols_for(P, B, m_tiles, c->sm_count, 1);
     for (int first = 0; first < 2; ++first) {
       const FwdForm form = fwd_form(st, l, first);
-      const bool rides = !first && l <= st->fuse_upto;   // the plain form's product rides on a launch, with whole sums
+      // the plain form's product rides on a launch, with sums over whole rows or, added up, over runs of them
+      const bool rides = !first && l <= st->fuse_upto;
+      if (rides && partial_sums(P, st->wgrad_f[l])) f->runs[l] = st->wgrad_f[l].n_chunks;
       f->own_fwd[first][l] = (rides || form == FwdForm::DENSE || (form == FwdForm::TILES && st->fwd[l].splits == 1)) &&
                              ((l + 1 == L && st->tail_ok) || f->own_dgrad[l + 1]);
-      ok = ok && (!rides || f->own_fwd[first][l]);
+      ok = ok && (!rides || (f->own_fwd[first][l] && f->runs[l] * f->fwd[l].cols <= 512));
     }
   }
   f->step_in.resize((size_t)f->K * (MAVG_MAX_LAYERS + 1));
@@ -1734,7 +1761,8 @@ void reb_setup(mavg_ctx* c, TcState* st) {
       else if (l > 1) rows(&f->step_dz[at], dz, out, P, st->dgrad[l].BN);
     }
   }
-  for (const void* k : {(const void*)k_fac_product<PROD_FWD, 1, false, false>, (const void*)k_fac_product<PROD_DGRAD_STEP, 1, false, false>})
+  for (const void* k : {(const void*)k_fac_product<PROD_FWD, 1, false, false>, (const void*)k_fac_product<PROD_FWD_RUNS, 1, false, false>,
+                        (const void*)k_fac_product<PROD_DGRAD_STEP, 1, false, false>})
     ok = ok && cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                     (int)(kSmSharedBytes - kBlockReservedBytes - sizeof(GemmShared))) == cudaSuccess;
   for (const void* k : {(const void*)rebuild::k_rebuild<false, false>, (const void*)rebuild::k_rebuild<false, true>,
@@ -1753,7 +1781,7 @@ bool reb_usable(const mavg_ctx* c) {
   const TcState* st = (const TcState*)c->mlp;
   // by the momentum and K of now, which may not be those the handle was made with
   return st && st->reb && c->schedule == 0 && c->cfg.K <= st->reb->K && reb_steps(&c->cfg) == c->cfg.K &&
-         (c->cfg.K <= 4 || !st->fuse_upto);
+         (!st->fuse_upto || reb_riding(&c->cfg));
 }
 
 // The K steps of a round: F_1 -> ... -> F_{L-1} -> last layer and loss -> D_L -> ... -> D_2 -> weights of the next step's
@@ -1804,11 +1832,19 @@ cudaError_t reb_local_steps(mavg_ctx* c, int64_t round) {
     };
     for (int l = 1; l < L; ++l) {
       operands(l, k == 1 ? &st->wg[l] : &f->w_own[l], in + l, t.h[l], l, t.act_t[l]);
-      if (f->own_fwd[k == 1][l])
-        FAC_TRY((launch_product<PROD_FWD, 1>(c, MAVG_K_FWD, *o.w, *o.w, *o.in, f->g_mn[l], *o.in,
-                                             own(k == 1 ? f->fwd1[l] : f->fwd[l], cfg.dims[l - 1], l))));
-      else
+      if (!f->own_fwd[k == 1][l]) {
         FAC_TRY(st->run_forward(c, o));
+        continue;
+      }
+      ProdArgs g = own(k == 1 ? f->fwd1[l] : f->fwd[l], cfg.dims[l - 1], l);
+      if (k > 1 && f->runs[l] > 1) {
+        g.run = 2 * st->wgrad_f[l].chunk;            // (tiles of 32 columns)
+        g.runs = f->runs[l];
+        g.whole_rows = st->wgrad_f[l].whole_rows;
+        FAC_TRY((launch_product<PROD_FWD_RUNS, 1>(c, MAVG_K_FWD, *o.w, *o.w, *o.in, f->g_mn[l], *o.in, g)));
+      } else {
+        FAC_TRY((launch_product<PROD_FWD, 1>(c, MAVG_K_FWD, *o.w, *o.w, *o.in, f->g_mn[l], *o.in, g)));
+      }
     }
     operands(L, k == 1 ? &st->wg[L] : &f->w_own[L], in + L, t.g[L - 1], L - 1, t.dz_t);
     o.labels = (const int32_t*)ws_ptr(c, t.labels) + (size_t)(k - 1) * P * B;

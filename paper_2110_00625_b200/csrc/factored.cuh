@@ -57,6 +57,7 @@ struct FacState {
   // w~; own_fwd (of the first step at [1]), own_dgrad: the products are k_fac_product's, not the plain form's launches
   FacCols fwd1[MAVG_MAX_LAYERS + 1], dgrad1[MAVG_MAX_LAYERS + 1];
   bool own_fwd[2][MAVG_MAX_LAYERS + 1] = {}, own_dgrad[MAVG_MAX_LAYERS + 1] = {};
+  int runs[MAVG_MAX_LAYERS + 1] = {};        // partial sums of a forward product after the first step's (0, 1: none)
   CUtensorMap w_own[MAVG_MAX_LAYERS + 1], w_own_mn[MAVG_MAX_LAYERS + 1], w_own_st[MAVG_MAX_LAYERS + 1];
   std::vector<CUtensorMap> step_in, step_dz;
   CUtensorMap w_lo[MAVG_MAX_LAYERS];         // low parts of w~'s hidden layers, box 64 x 128
@@ -83,6 +84,7 @@ cudaError_t fac_local_steps(mavg_ctx* c, int64_t round);
 // The same of rebuilt steps (rebuild.cuh), which calls take that are not factored: the weights of every step are formed anew
 // from w~, u as the call found it and the rows of all steps so far.
 int reb_steps(const mavg_config* cfg);
+bool reb_riding(const mavg_config* cfg);       // also where the plain form's forward products ride on its weight gradients
 bool reb_reserved(const mavg_config* cfg);
 FacLayout reb_layout(const mavg_config* cfg, size_t base);
 void reb_setup(mavg_ctx* c, TcState* st);

@@ -429,10 +429,10 @@ int riding_plans(const mavg_config* cfg, const TcLayout& t, int sm_count, bool m
   return cfg->n_layers - 1;
 }
 
-// Whether every sum of those products runs over a whole row, in the order of a product of its own.
-bool whole_sums(int P, int riding, const WgradPlan* f) {
+// Whether rebuilt steps can form those products' sums in their order: partial sums have columns of tensor memory.
+bool sums_fit(const mavg_config* cfg, int riding, const WgradPlan* f) {
   for (int l = 1; l <= riding; ++l)
-    if (f[l].n_chunks > 1 && f[l].whole_rows < P * f[l].m_tiles) return false;
+    if (partial_sums(cfg->P, f[l]) && f[l].n_chunks * cfg->B > 512) return false;
   return true;
 }
 
@@ -444,7 +444,7 @@ bool may_rebuild(const mavg_config* cfg, const TcLayout& t) {
     w[l] = plan_wgrad_stream(cfg->dims[l], cfg->dims[l - 1], cfg->B, cfg->P, kPlanSmCount, momentum, true);
   if (wgrad_merges(cfg, kPlanSmCount, w)) return true;
   const int riding = riding_plans(cfg, t, kPlanSmCount, momentum, true, f);
-  return whole_sums(cfg->P, riding, f) && (cfg->K <= 4 || !riding);
+  return sums_fit(cfg, riding, f) && (!riding || reb_riding(cfg));
 }
 
 }  // namespace
@@ -715,7 +715,7 @@ mavg_status tc_setup(mavg_ctx* c) {
   st->run_forward = forward;
   st->run_last_layer = last_layer;
   st->run_dgrad = dgrad;
-  if (e == cudaSuccess && reb_steps(&cfg) && whole_sums(P, st->fuse_upto, st->wgrad_f) && c->buf.workspace_bytes >= std::max(t.end, reb_layout(&cfg, t.shared_end).end))
+  if (e == cudaSuccess && reb_steps(&cfg) && sums_fit(&cfg, st->fuse_upto, st->wgrad_f) && c->buf.workspace_bytes >= std::max(t.end, reb_layout(&cfg, t.shared_end).end))
     reb_setup(c, st);
   if (e == cudaSuccess)
     e = cudaMemsetAsync(ws + t.counters, 0, t.counters_bytes, c->stream);

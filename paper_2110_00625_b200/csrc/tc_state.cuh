@@ -143,6 +143,9 @@ inline FwdForm fwd_form(const TcState* st, int l, bool shared_w) {
   return shared_w && st->dense[l].ok ? FwdForm::DENSE : st->fwd_ks[l].splits > 1 ? FwdForm::SPLIT : FwdForm::TILES;
 }
 
+// Whether a forward product that rides on a weight-gradient launch is formed in several sums.
+inline bool partial_sums(int P, const WgradPlan& w) { return w.n_chunks > 1 && w.whole_rows < P * w.m_tiles; }
+
 inline bool encode_any(TcState* st, CUtensorMap* m, CUtensorMapDataType dt, int esize, void* ptr,
                 int inner, int rows, int batch, int64_t row_stride, int64_t batch_stride,
                 int box_inner, int box_rows, CUtensorMapSwizzle swz, std::string* why, int box_batch = 1) {

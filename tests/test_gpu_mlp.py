@@ -336,10 +336,12 @@ def _fused_handle(dims, K, **kw):
     cfg.update(dims=dims, P=FUSED_P, K=K, B=FUSED_B, S=4096)
     x, y = m.workloads.make_dataset(cfg, S=cfg["S"])
     w1 = m.workloads.mlp_init(cfg["dims"])
-    g = m.Mavg(w1, P=FUSED_P, K=K, local_lr=cfg["gamma"], mu=cfg["mu"], B=FUSED_B,
+    # made for one step: rebuilt rounds, whose weight gradients no product rides on, are for handles of two steps and more
+    g = m.Mavg(w1, P=FUSED_P, K=1, local_lr=cfg["gamma"], mu=cfg["mu"], B=FUSED_B,
                seed=m.workloads.BASE_SEED, objective=m.OBJ_MLP, dims=dims, gemm_bf16=1,
                x=x, y=y, x_bf16=True, **kw)
-    assert not g.rebuilt()                # rounds without weight gradients that a product could ride on
+    g.set_hparams(K, cfg["gamma"], 1.0, cfg["mu"])
+    assert not g.rebuilt()
     return g, cfg, x, y, w1
 
 

@@ -65,6 +65,11 @@ def _steps_from_own_weights(g):                   # the second call does not sta
     ([1416, 1800, 1800, 1800, 32], 7, 2, 48, 0.0, False, True, _steps_from_own_weights, "steps"),
     ([3072, 2048, 2048, 2048, 10], 8, 3, 64, 0.0, False, True, _rounds, "steps"),
     ([2488, 608, 608, 32], 27, 2, 48, 0.0, False, False, _rounds, "steps"),
+    ([3072, 1024, 512, 10], 14, 4, 16, 0.0, False, True, _rounds, "steps"),          # riding products in partial sums
+    ([2816, 1184, 1184, 1184, 10], 24, 2, 96, 0.0, False, False, _rounds, "steps"),
+    ([3072, 2048, 10], 13, 4, 16, 0.9, False, True, _rounds, "steps"),                # some rows whole, the others not
+    ([3048, 1000, 504, 264, 10], 13, 3, 32, 0.9, False, True, _rounds, "steps"),      # ragged
+    ([1632, 1024, 512, 10], 24, 2, 32, 0.9, False, True, _rounds, "steps"),           # runs of an odd number of tiles
 ])
 def test_the_steps_are_the_plain_ones(dims, P, K, B, beta, reset, defer, calls, how):
     got, want = (_run(dims, P, K, B, beta, reset, defer, calls, rebuilt, how) for rebuilt in (True, False))

@@ -21,8 +21,12 @@ def _handle(dims, K, lr, w1=None, schedule=0, **kw):
     x = rng.standard_normal((1024, dims[0]), dtype=np.float32)
     y = rng.integers(0, dims[-1], size=1024).astype(np.int32)
     w1 = m.workloads.mlp_init(dims) if w1 is None else w1
-    g = m.Mavg(w1, P=_learners(dims), K=K, local_lr=lr, mu=0.9, B=B, seed=3, objective=m.OBJ_MLP, dims=dims,
+    # made for one step where its losses' room allows more: steps in place, not rebuilt
+    late = _learners(dims) * K <= 64
+    g = m.Mavg(w1, P=_learners(dims), K=1 if late else K, local_lr=lr, mu=0.9, B=B, seed=3, objective=m.OBJ_MLP, dims=dims,
                gemm_bf16=1, x=x, y=y, x_bf16=True, defer_broadcast=True, **kw)
+    g.set_hparams(K, lr, 1.0, 0.9)
+    assert not (late and g.rebuilt())
     g.set_schedule(schedule)
     assert g.get_step_plan()["fwd_with_wgrad"] == len(dims) - 2
     assert not g.factored()          # rounds that keep no weights between their steps
@@ -55,7 +59,7 @@ def test_a_step_of_length_zero_keeps_every_bit(dims, K, beta):
     # zeros of either sign become +0: keep them out
     w1 = np.where(bits << 1 == 0, np.uint32(0x3c000000), bits).view(np.float32)
     g = _handle(dims, K, 0.0, w1=w1, learner_momentum=beta)
-    for _ in range(2):               # the second call does not start from w~: its steps are in place, not rebuilt
+    for _ in range(2):               # the second call does not start from w~: its steps are in place in any case
         g.local_steps()
         g.sync()
         rep = g.replicas[:, :g.n].cpu().numpy().view(np.uint32)

@@ -10,14 +10,14 @@ pytestmark = pytest.mark.gpu
 
 def _run(dims, P, profiled, schedule, beta=0.0):
     import paper_2110_00625_b200 as m
-    B, K = 16, 4
+    B, K = 16, 5                     # (up to four steps may be rebuilt, where nothing rides)
     rng = np.random.default_rng(5)
     x = rng.standard_normal((1024, dims[0]), dtype=np.float32)
     y = rng.integers(0, dims[-1], size=1024).astype(np.int32)
     g = m.Mavg(m.workloads.mlp_init(dims), P=P, K=K, local_lr=0.01, mu=0.9, B=B, seed=3,
                objective=m.OBJ_MLP, dims=dims, gemm_bf16=1, x=x, y=y, x_bf16=True,
                defer_broadcast=True, learner_momentum=beta)
-    assert g.get_step_plan()["fwd_with_wgrad"] == len(dims) - 2
+    assert g.get_step_plan()["fwd_with_wgrad"] == len(dims) - 2 and not g.rebuilt()
     g.set_schedule(schedule)
     g.set_profiling(profiled)
     losses = [g.round(want_loss=True) for _ in range(2)]
